@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-        if (warp == 0 && lane == 0) {
+        if (warp == 0 && elect_one()) {
             bool ok = true;
             int nk = 0, nv = 0, qn = 0, dn = 0, sn = 0;   // fills so far: K, V, Q ring, dO ring, statistics ring
             auto wait_empty = [&](int bar, int use) {
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                     ++sn;
                 }
             }
-        } else if (warp == 1 && lane == 0) {
+        } else if (warp == 1 && elect_one()) {
             constexpr uint32_t idescT = umma_idesc(128, 128, 0, 0);
             constexpr uint32_t idescD = umma_idesc(128, HD, 0, 1);
             bool ok = true;
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-        if (warp == 0 && lane == 0) {
+        if (warp == 0 && elect_one()) {
             bool ok = true;
             int nq = 0, nd = 0, kn = 0, vn = 0;   // fills so far: Q, dO, K ring, V ring (= gate ring)
             auto wait_empty = [&](int bar, int use) {
@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
                     ++vn;
                 }
             }
-        } else if (warp == 1 && lane == 0) {
+        } else if (warp == 1 && elect_one()) {
             constexpr uint32_t idescS = umma_idesc(128, 128, 0, 0);
             constexpr uint32_t idescD = umma_idesc(128, HD, 0, 1);
             bool ok = true;

@@ -149,7 +149,7 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
-        if (warp == 0 && lane == 0) {
+        if (warp == 0 && elect_one()) {
             // ------------------------------------------------------------ TMA producer
             bool ok = true;
             int nq = 0;                       // query operands issued so far (all work items)
@@ -205,7 +205,7 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                     load_kv(sV, B_VFULL, B_VEMPTY, x, vf, &tm.v, HD, s * p.Lp + J * kTile);
                 }
             }
-        } else if (warp == 1 && lane == 0) {
+        } else if (warp == 1 && elect_one()) {
             // ------------------------------------------------------------ MMA issuer
             // a negative scale is applied as a sign flip of the logits here (negate-A bit), its magnitude in the softmax
             const uint32_t idescS = umma_idesc(128, 128, 0, 0) | (p.scale < 0.f ? (1u << 13) : 0u);
@@ -217,6 +217,7 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
             auto issue_s = [&](int x, int qs, int ks, int kdim, bool acc) {   // ks >= 2: a V slot
                 // (descriptors advance by their low word only: 32 bytes per step, the next panel after four steps)
                 uint32_t a_lo = umma_desc_lo(smem_u32(sQ + qs * kSlotBytes), 16), b_lo = umma_desc_lo(smem_u32(sK + ks * kSlotBytes), 16);
+#pragma unroll
                 for (int kk = 0; kk < kdim / 16; ++kk) {
                     umma_ss(tmem + x * 128, umma_desc_join(a_lo), umma_desc_join(b_lo), idescS, (acc || kk > 0) ? 1u : 0u);
                     const uint32_t step = (kk & 3) == 3 ? (kPanelBytes - 96u) >> 4 : 2u;
