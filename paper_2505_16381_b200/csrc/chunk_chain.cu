@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     const int grid = (int)gridDim.x;
 
     if (warp == 8) {
-    if (lane == 0) {
+    if (elect_one()) {
     // ------------------------------------------------------------------ leader: TMA loads and every product
     bool ok = true;
     uint32_t ph[7] = {0, 0, 0, 0, 0, 0, 0};
@@ -99,24 +99,24 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         // ---- phase 0: dXq = lower(-(dQl U^T + s dSd Y^T)) -> cA, while the previous chunk's results are still leaving
         // the other columns; then dw = -Y dKr - U dP^T
         if (!wait(B_LOAD)) break;
-        mma_call(tmem + cA, sa(1), OP_K, sa(0), OP_K, KD, 128, false);
-        mma_call(tmem + cA, sa(3), OP_MN, sa(2), OP_MN, K8, 128, true);          // slot 2 holds Y^T
+        mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(1), sa(0), false);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cA, sa(3), sa(2), true);          // slot 2 holds Y^T
         if (chunk != (int)blockIdx.x && !wait(B_R1)) break;                      // the previous chunk's dw has left cDW
         if (!wait(B_LOAD2)) break;
-        mma_call(tmem + cDW, sa(2), OP_MN, sa(5), OP_MN, K8, HD, false, true);
-        mma_call(tmem + cDW, sa(0), OP_K, sa(6), OP_K, KD, HD, true, true);
+        mma<OP_MN, OP_MN, K8, HD, true>(tmem + cDW, sa(2), sa(5), false);
+        mma<OP_K, OP_K, KD, HD, true>(tmem + cDW, sa(0), sa(6), true);
         umma_commit(&bars[B_MMA]);
         // ---- phase 1: dY = -(W dKr^T + Xq^T s dSd) -> cA,  dU = -(Xq^T dQl + W dP) -> cB.  dU's products read no tile
         // that the workers are writing and go to their own columns: they run underneath the read-out of dXq.
         if (!wait(B_MMA)) break;
         mbar_expect_tx(&bars[B_LOAD], kTileB);
         tma_tile(slot(2), &tm.xqn, &bars[B_LOAD], kT, r0);
-        mma_call(tmem + cB, sa(4), OP_K, sa(6), OP_MN, KD, HD, false);           // W dP needs no new tile
+        mma<OP_K, OP_MN, KD, HD>(tmem + cB, sa(4), sa(6), false);           // W dP needs no new tile
         if (!wait(B_LOAD)) break;
-        mma_call(tmem + cB, sa(2), OP_MN, sa(1), OP_MN, K8, HD, true, true);     // slot 2 holds -Xq: negated back
+        mma<OP_MN, OP_MN, K8, HD, true>(tmem + cB, sa(2), sa(1), true);     // slot 2 holds -Xq: negated back
         if (!wait(B_R0)) break;                                                  // dXq has left cA
-        mma_call(tmem + cA, sa(4), OP_K, sa(5), OP_K, KD, 128, false);
-        mma_call(tmem + cA, sa(2), OP_MN, sa(3), OP_K, K8, 128, true, true);
+        mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(4), sa(5), false);
+        mma<OP_MN, OP_K, K8, 128, true>(tmem + cA, sa(2), sa(3), true);
         umma_commit(&bars[B_MMA]);
         // ---- phase 2: dT = lower(dY Xk^T + dU W^T) -> cA, and phase 3 right behind it (the same dY and dU tiles and T~):
         // dXk = strictLower(T~^T dY) -> cB,  dw += T~^T dU.  (s dSd)^T is not needed again before phase 5, where it is
@@ -127,14 +127,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tma_tile(slot(1), &tm.th, &bars[B_LOAD], kT, r0);
         tma_tile(slot(3), &tm.tl, &bars[B_LOAD], kT, r0);
         if (!wait(B_R1)) break;                                                  // dY, dU tiles
-        mma_call(tmem + cA, sa(6), OP_K, sa(4), OP_K, KD, 128, false);           // dU W^T needs no new tile
+        mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(6), sa(4), false);           // dU W^T needs no new tile
         if (!wait(B_LOAD)) break;
-        mma_call(tmem + cA, sa(5), OP_K, sa(2), OP_K, K8, 128, true);
+        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(5), sa(2), true);
         umma_commit(&bars[B_MMA]);
-        mma_call(tmem + cB, sa(1), OP_MN, sa(5), OP_MN, K8, 128, false);
-        mma_call(tmem + cB, sa(3), OP_MN, sa(5), OP_MN, K8, 128, true);
-        mma_call(tmem + cDW, sa(1), OP_MN, sa(6), OP_MN, K8, HD, true);
-        mma_call(tmem + cDW, sa(3), OP_MN, sa(6), OP_MN, K8, HD, true);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cB, sa(1), sa(5), false);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cB, sa(3), sa(5), true);
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(1), sa(6), true);
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(3), sa(6), true);
         umma_commit(&bars[B_MMA2]);
         // ---- phase 4: M = Ainv^T dT -> cG;  tmp = M D;  dA = strictLower(-tmp Ainv^T) -> cA;  W W^T -> cB (for dbeta)
         if (!wait(B_MMA) || !wait(B_MMA2)) break;
@@ -143,17 +143,17 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tma_tile(slot(6), &tm.al, &bars[B_LOAD], kT, r0);
         if (!wait(B_LOAD)) break;
         if (!wait(B_R0)) break;                                                  // dT hi, lo tiles
-        mma_call(tmem + cG, sa(1), OP_MN, sa(2), OP_MN, K8, 128, false);
-        mma_call(tmem + cG, sa(6), OP_MN, sa(2), OP_MN, K8, 128, true);
-        mma_call(tmem + cG, sa(1), OP_MN, sa(3), OP_MN, K8, 128, true);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(1), sa(2), false);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(6), sa(2), true);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(1), sa(3), true);
         umma_commit(&bars[B_MMA]);
         if (!wait(B_R1)) break;                                                  // dXk has left cB
-        mma_call(tmem + cB, sa(4), OP_K, sa(4), OP_K, KD, 128, false);          // retires with the next group
+        mma<OP_K, OP_K, KD, 128>(tmem + cB, sa(4), sa(4), false);          // retires with the next group
         if (!wait(B_MMA)) break;
         if (!wait(B_R0)) break;                                                  // tmp hi, lo tiles
-        mma_call(tmem + cA, sa(2), OP_K, sa(1), OP_K, K8, 128, false);
-        mma_call(tmem + cA, sa(2), OP_K, sa(6), OP_K, K8, 128, true);
-        mma_call(tmem + cA, sa(3), OP_K, sa(1), OP_K, K8, 128, true);
+        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(2), sa(1), false);
+        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(2), sa(6), true);
+        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(3), sa(1), true);
         umma_commit(&bars[B_MMA]);
         // ---- phase 5: dq -> cB, dk -> cG and the rest of dw, in three groups.  K and Q replace Ainv hi / lo, (s dSd)^T
         // returns.  First the products that need neither dGm nor the columns that dbeta still reads; when they have
@@ -163,17 +163,17 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tma_tile(slot(3), &tm.dsdt, &bars[B_LOAD], kT, r0);
         tma_tile(slot(6), &tm.q, &bars[B_LOAD], HD, r0);
         tma_tile(slot(1), &tm.k, &bars[B_LOAD], HD, r0);
-        mma_call(tmem + cG, sa(5), OP_MN, sa(4), OP_MN, K8, HD, false);          // dXk^T W needs no new tile
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cG, sa(5), sa(4), false);          // dXk^T W needs no new tile
         if (!wait(B_LOAD)) break;
-        mma_call(tmem + cG, sa(3), OP_K, sa(6), OP_MN, K8, HD, true);            // s dSd^T Q
-        mma_call(tmem + cDW, sa(0), OP_MN, sa(6), OP_MN, K8, HD, true);          // dXq^T Q
-        mma_call(tmem + cDW, sa(5), OP_K, sa(1), OP_MN, K8, HD, true);           // dXk K
+        mma<OP_K, OP_MN, K8, HD>(tmem + cG, sa(3), sa(6), true);            // s dSd^T Q
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(0), sa(6), true);          // dXq^T Q
+        mma<OP_K, OP_MN, K8, HD>(tmem + cDW, sa(5), sa(1), true);           // dXk K
         umma_commit(&bars[B_MMA2]);
         if (!wait(B_R1)) break;                                                  // dGm hi tile; W W^T has left cB
-        mma_call(tmem + cB, sa(3), OP_MN, sa(1), OP_MN, K8, HD, false);          // s dSd K
-        mma_call(tmem + cB, sa(0), OP_K, sa(4), OP_MN, K8, HD, true);            // dXq W
-        mma_call(tmem + cDW, sa(2), OP_K, sa(4), OP_MN, K8, HD, true);           // dGm W
-        mma_call(tmem + cDW, sa(2), OP_MN, sa(4), OP_MN, K8, HD, true);          // dGm^T W
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cB, sa(3), sa(1), false);          // s dSd K
+        mma<OP_K, OP_MN, K8, HD>(tmem + cB, sa(0), sa(4), true);            // dXq W
+        mma<OP_K, OP_MN, K8, HD>(tmem + cDW, sa(2), sa(4), true);           // dGm W
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(2), sa(4), true);          // dGm^T W
         umma_commit(&bars[B_MMA]);
         if (!wait(B_MMA2)) break;
         // (the last two products cannot start before the second group has left the pipe anyway: the next chunk's tiles are
@@ -182,8 +182,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         if (!wait(B_MMA)) break;
         if (next < nchunks) first_loads_a(next);                                 // slots 0 - 3 and 6 are free
         if (!wait(B_R0)) break;                                                  // dGm lo tile (over dXk)
-        mma_call(tmem + cDW, sa(5), OP_K, sa(4), OP_MN, K8, HD, true);
-        mma_call(tmem + cDW, sa(5), OP_MN, sa(4), OP_MN, K8, HD, true);
+        mma<OP_K, OP_MN, K8, HD>(tmem + cDW, sa(5), sa(4), true);
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(5), sa(4), true);
         umma_commit(&bars[B_MMA2]);
         if (!wait(B_MMA2)) break;
         if (next < nchunks) first_loads_b(next);                                 // and the other two

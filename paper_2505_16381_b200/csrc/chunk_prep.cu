@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
     if (warp >= kWorkers / 32) {
         // ------------------------------------------------------------------ issuer
         asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
-        if (tid == kWorkers) {
+        if (warp == kWorkers / 32 && elect_one()) {
             auto wait = [&](int b, uint32_t par) { return mbar_wait(&bars[b], par, abort_flag, ST_PREP); };
             auto load = [&](int chunk) {
                 mbar_expect_tx(&bars[B_LOAD], (KEYS ? 2 : 3) * kT * HD * 2);
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                 ok = wait(B_LOAD, 0);
                 if (ok) {
                     tc_fence_after_sync();
-                    mma_small(tmem + 0, aW_, OP_K, aW_, OP_K, KS, 128, false);
+                    mma<OP_K, OP_K, KS, 128>(tmem + 0, aW_, aW_, false);
                     umma_commit(&bars[B_GM]);
                 }
             }
@@ -150,28 +150,28 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                 // Xq, Xk: their columns held the previous chunk's W^T U and Xq U
                 if (it > 0 && !wait(R_E3, par ^ 1)) break;
                 tc_fence_after_sync();
-                if (!KEYS) mma_small(tmem + 128, aQ, OP_K, aW, OP_K, KS, 128, false);
-                mma_small(tmem + 256, aW, OP_K, aK, OP_K, KS, 128, false);
+                if (!KEYS) mma<OP_K, OP_K, KS, 128>(tmem + 128, aQ, aW, false);
+                mma<OP_K, OP_K, KS, 128>(tmem + 256, aW, aK, false);
                 umma_commit(&bars[B_XQK]);
                 // last merge level of the triangular inverse: T = C A^-1, then B^-1 T, as bf16 pairs (64 x 64 x 64 each; the
                 // eight 8 KB operand tiles sit in the Q / K slots, whose products have retired by then)
                 if (!wait(R_M1, par)) break;
                 tc_fence_after_sync();
-                mma_small(tmem + 0, aQ, OP_K, aQ + 2 * kInvTileB, OP_MN, 4, 64, false);
-                mma_small(tmem + 0, aQ, OP_K, aQ + 3 * kInvTileB, OP_MN, 4, 64, true);
-                mma_small(tmem + 0, aQ + kInvTileB, OP_K, aQ + 2 * kInvTileB, OP_MN, 4, 64, true);
+                mma<OP_K, OP_MN, 4, 64>(tmem + 0, aQ, aQ + 2 * kInvTileB, false);
+                mma<OP_K, OP_MN, 4, 64>(tmem + 0, aQ, aQ + 3 * kInvTileB, true);
+                mma<OP_K, OP_MN, 4, 64>(tmem + 0, aQ + kInvTileB, aQ + 2 * kInvTileB, true);
                 umma_commit(&bars[B_M1]);
                 if (!wait(R_M2, par)) break;
                 tc_fence_after_sync();
-                mma_small(tmem + 64, aQ + 4 * kInvTileB, OP_K, aQ + 6 * kInvTileB, OP_MN, 4, 64, false);
-                mma_small(tmem + 64, aQ + 4 * kInvTileB, OP_K, aQ + 7 * kInvTileB, OP_MN, 4, 64, true);
-                mma_small(tmem + 64, aQ + 5 * kInvTileB, OP_K, aQ + 6 * kInvTileB, OP_MN, 4, 64, true);
+                mma<OP_K, OP_MN, 4, 64>(tmem + 64, aQ + 4 * kInvTileB, aQ + 6 * kInvTileB, false);
+                mma<OP_K, OP_MN, 4, 64>(tmem + 64, aQ + 4 * kInvTileB, aQ + 7 * kInvTileB, true);
+                mma<OP_K, OP_MN, 4, 64>(tmem + 64, aQ + 5 * kInvTileB, aQ + 6 * kInvTileB, true);
                 umma_commit(&bars[B_M2]);
                 // U = T~ W  (lo x lo terms are dropped everywhere)
                 if (!wait(R_TT, par)) break;
                 tc_fence_after_sync();
-                mma_small(tmem + 0, aQ, OP_K, aW, OP_MN, 8, HD, false);
-                mma_small(tmem + 0, aK, OP_K, aW, OP_MN, 8, HD, true);
+                mma<OP_K, OP_MN, 8, HD>(tmem + 0, aQ, aW, false);
+                mma<OP_K, OP_MN, 8, HD>(tmem + 0, aK, aW, true);
                 umma_commit(&bars[B_U]);
                 if (SAVE) {   // the tiles kept for the chain rule leave through TMA stores, straight from the operand slots
                     store(&tm.th, sQK, kT, chunk);
@@ -184,9 +184,9 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                     store(&tm.xk, sBig + 2 * kTileB, kT, chunk);
                     tma_store_commit();
                 }
-                mma_small(tmem + 384, aQ, OP_K, aBig + 2 * kTileB, OP_MN, 8, 128, false);
-                mma_small(tmem + 384, aK, OP_K, aBig + 2 * kTileB, OP_MN, 8, 128, true);
-                mma_small(tmem + 384, aQ, OP_K, aBig + 3 * kTileB, OP_MN, 8, 128, true);
+                mma<OP_K, OP_MN, 8, 128>(tmem + 384, aQ, aBig + 2 * kTileB, false);
+                mma<OP_K, OP_MN, 8, 128>(tmem + 384, aK, aBig + 2 * kTileB, true);
+                mma<OP_K, OP_MN, 8, 128>(tmem + 384, aQ, aBig + 3 * kTileB, true);
                 // B_Y lets the workers overwrite T~ (with U) and Xk (with Y): the stores must have read them
                 if (SAVE) tma_store_wait_read();
                 umma_commit(&bars[B_Y]);
@@ -194,12 +194,12 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                 if (!wait(R_U, par)) break;
                 tc_fence_after_sync();
                 if (!KEYS) {
-                    mma_small(tmem + 256, aBig, OP_K, aQ, OP_MN, 8, HD, false);
-                    mma_small(tmem + 256, aBig + kTileB, OP_K, aQ, OP_MN, 8, HD, true);
-                    mma_small(tmem + 256, aBig, OP_K, aK, OP_MN, 8, HD, true);
+                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, aBig, aQ, false);
+                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, aBig + kTileB, aQ, true);
+                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, aBig, aK, true);
                 }
-                mma_small(tmem + 128, aW, OP_MN, aQ, OP_MN, 8, HD, false);
-                mma_small(tmem + 128, aW, OP_MN, aK, OP_MN, 8, HD, true);
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, aW, aQ, false);
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, aW, aK, true);
                 umma_commit(&bars[B_G3A]);
                 if (SAVE) {
                     store(&tm.u, sQK, HD, chunk);
@@ -208,8 +208,8 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                 // Y^T W
                 if (!wait(R_Y, par)) break;
                 tc_fence_after_sync();
-                mma_small(tmem + 384, aBig + 2 * kTileB, OP_MN, aW, OP_MN, 8, HD, false);
-                mma_small(tmem + 384, aBig + 3 * kTileB, OP_MN, aW, OP_MN, 8, HD, true);
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, aBig + 2 * kTileB, aW, false);
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, aBig + 3 * kTileB, aW, true);
                 umma_commit(&bars[B_G3B]);
                 // next chunk: once this chunk's last product has retired every tile slot is free
                 const int next = chunk + (int)gridDim.x;
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                     load(next);
                     if (!wait(B_LOAD, par ^ 1)) break;
                     tc_fence_after_sync();
-                    mma_small(tmem + 0, aW, OP_K, aW, OP_K, KS, 128, false);
+                    mma<OP_K, OP_K, KS, 128>(tmem + 0, aW, aW, false);
                     umma_commit(&bars[B_GM]);
                 }
             }

@@ -63,6 +63,11 @@ __device__ __forceinline__ void loads_wait(Ctx& c) {
     if (!mbar_wait(&c.bars[0], c.ph_load, c.abort_flag, ST_LEVELS)) c.ok = false;
     c.ph_load ^= 1;
 }
+// The thread that issues a group of products: one lane of warp 0, unless a thread of that warp has given up.  The warp must
+// be converged up to a wait (the vote joins it again).
+__device__ __forceinline__ bool leader(const Ctx& c) {
+    return c.warp == 0 && __all_sync(0xffffffffu, c.ok) && elect_one();
+}
 __device__ __forceinline__ void publish() {
     fence_proxy_async_smem();
     tc_fence_before_sync();
@@ -109,7 +114,7 @@ __global__ void __launch_bounds__(256, 1) dyadic_fwd_kernel(const __grid_constan
     const long mat_lo = p.lv.dy_off[p.l] / (HD * HD) + (long)s * cnt + 2 * b;        // right factor; left is +1
     const long mat_out = p.lv.dy_off[p.l + 1] / (HD * HD) + (long)s * cnt2 + b;
     uint8_t* sm = c.smem;
-    if (c.tid == 0) {
+    if (c.warp == 0 && elect_one()) {
         mbar_expect_tx(&c.bars[0], 4 * kT * HD * 2);
         tma_tile(sm + 0 * kTileB, &tm.dyh, &c.bars[0], HD, (int)((mat_lo + 1) * HD));
         tma_tile(sm + 1 * kTileB, &tm.dyl, &c.bars[0], HD, (int)((mat_lo + 1) * HD));
@@ -117,12 +122,12 @@ __global__ void __launch_bounds__(256, 1) dyadic_fwd_kernel(const __grid_constan
         tma_tile(sm + 3 * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat_lo * HD));
     }
     loads_wait(c);
-    if (c.tid == 0 && c.ok) {
+    if (leader(c)) {
         tc_fence_after_sync();
         const uint32_t a = smem_u32(sm);
-        mma(c.tmem, a, OP_K, a + 2 * kTileB, OP_MN, HD / 16, HD, false);
-        mma(c.tmem, a, OP_K, a + 3 * kTileB, OP_MN, HD / 16, HD, true);
-        mma(c.tmem, a + kTileB, OP_K, a + 2 * kTileB, OP_MN, HD / 16, HD, true);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, false);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 3 * kTileB, true);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a + kTileB, a + 2 * kTileB, true);
         umma_commit(&c.bars[1]);
     }
     mma_wait(c);
@@ -165,12 +170,12 @@ __global__ void __launch_bounds__(256, 1) dyadic_fused_kernel(const __grid_const
     // acc(col) = left (slots a, a + 1) x right (slots b, b + 1), the lo x lo term left out
     auto product = [&](uint32_t col, int a, int b) {
         publish();   // operands written by this CTA's threads are visible, and nobody still reads the accumulator
-        if (c.tid == 0 && c.ok) {
+        if (leader(c)) {
             tc_fence_after_sync();
             const uint32_t base = smem_u32(sm);
-            mma(c.tmem + col, base + a * kTileB, OP_K, base + b * kTileB, OP_MN, HD / 16, HD, false);
-            mma(c.tmem + col, base + a * kTileB, OP_K, base + (b + 1) * kTileB, OP_MN, HD / 16, HD, true);
-            mma(c.tmem + col, base + (a + 1) * kTileB, OP_K, base + b * kTileB, OP_MN, HD / 16, HD, true);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + a * kTileB, base + b * kTileB, false);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + a * kTileB, base + (b + 1) * kTileB, true);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + (a + 1) * kTileB, base + b * kTileB, true);
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
@@ -215,13 +220,13 @@ __global__ void __launch_bounds__(256, 1) dyadic_fused_kernel(const __grid_const
     __syncthreads();
     // part 1 announces all four tiles and fetches the right factor, part 2 the left one (its slots free up later)
     auto request_a1 = [&](int k, int b_) {
-        if (c.tid != 0) return;
+        if (c.warp != 0 || !elect_one()) return;
         mbar_expect_tx(lbar[k & 1], 4 * kT * HD * 2);
         tma_tile(sm + b_ * kTileB, &tm.dyh, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k)) * HD));
         tma_tile(sm + (b_ + 1) * kTileB, &tm.dyl, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k)) * HD));
     };
     auto request_a2 = [&](int k, int a) {
-        if (c.tid != 0) return;
+        if (c.warp != 0 || !elect_one()) return;
         tma_tile(sm + a * kTileB, &tm.dyh, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k) + 1) * HD));
         tma_tile(sm + (a + 1) * kTileB, &tm.dyl, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k) + 1) * HD));
     };
@@ -308,7 +313,7 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
         if (!version_step(is_key, ch, l2, p.N, l1, b, src)) continue;
         const long mat = p.lv.dy_off[l1] / (HD * HD) + (long)s * p.lv.dy_cnt[l1] + b;
         const long row_dst = is_key ? kver_row(p.vl, s, l2, ch) : qver_row(p.vl, s, l2, ch);
-        if (c.tid == 0) {
+        if (c.warp == 0 && elect_one()) {
             mbar_expect_tx(&c.bars[0], (first ? 3 : 2) * kT * HD * 2);
             if (first) {
                 const long row_src = is_key ? kver_row(p.vl, s, l1, ch) : qver_row(p.vl, s, l1, ch);
@@ -319,12 +324,16 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
         }
         loads_wait(c);
         if (!first) publish();   // the left operand was written by this CTA's threads
-        if (c.tid == 0 && c.ok) {
+        if (leader(c)) {
             tc_fence_after_sync();
             const uint32_t a = smem_u32(sm);
-            const int bop = is_key ? OP_K : OP_MN;
-            mma(c.tmem, a, OP_K, a + kTileB, bop, HD / 16, HD, false);
-            mma(c.tmem, a, OP_K, a + 2 * kTileB, bop, HD / 16, HD, true);
+            if (is_key) {
+                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, a, a + kTileB, false);
+                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, true);
+            } else {
+                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + kTileB, false);
+                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, true);
+            }
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
@@ -407,7 +416,7 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
         tma_tile(base, gm, &c.bars[0], HD, (int)ver_row(l2, chx));
         tma_tile(base + kTileB, xm, &c.bars[0], HD, (int)ver_row(l1, chx));
     };
-    if (c.tid == 0) {   // first group: the run product itself, the operands of the level above, the first chunk
+    if (c.warp == 0 && elect_one()) {   // first group: the run product itself, the operands of the level above, the first chunk
         const uint32_t tile = kT * HD * 2;
         mbar_expect_tx(&c.bars[0], (ch >= 0 ? 3 : 0) * tile + (parent ? 2 : 0) * tile);
         if (ch >= 0) {
@@ -431,8 +440,8 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
         }
     };
     auto issue_parent = [&](uint32_t a) {
-        if (is_key) mma(c.tmem + colAcc, a + kTileB, OP_K, a + 2 * kTileB, OP_K, HD / 16, HD, false);      // dC B^T
-        else        mma(c.tmem + colAcc, a + 2 * kTileB, OP_MN, a + kTileB, OP_MN, HD / 16, HD, false);   // A^T dC
+        if (is_key) mma<OP_K, OP_K, HD / 16, HD>(c.tmem + colAcc, a + kTileB, a + 2 * kTileB, false);      // dC B^T
+        else        mma<OP_MN, OP_MN, HD / 16, HD>(c.tmem + colAcc, a + 2 * kTileB, a + kTileB, false);   // A^T dC
     };
     int buf = 0;
     bool first = true;
@@ -445,7 +454,7 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
         // every thread has read the previous chunk's carry out of tensor memory before the next product overwrites it
         tc_fence_before_sync();
         __syncthreads();
-        if (c.tid == 0 && c.ok) {
+        if (leader(c)) {
             if (nxt >= 0) {   // the other buffer's products retired before the previous mma_wait returned
                 mbar_expect_tx(&c.bars[0], 2 * kT * HD * 2);
                 chunk_loads(nxt, buf ^ 1);
@@ -455,11 +464,11 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
             if (first && parent) issue_parent(a);
             const bool acc = !first || parent;
             if (!is_key) {
-                mma(c.tmem + colCarry, g, OP_K, a, OP_K, HD / 16, HD, false);     // g Dy^T
-                mma(c.tmem + colAcc, x, OP_MN, g, OP_MN, 8, HD, acc);             // Xv^T g
+                mma<OP_K, OP_K, HD / 16, HD>(c.tmem + colCarry, g, a, false);     // g Dy^T
+                mma<OP_MN, OP_MN, 8, HD>(c.tmem + colAcc, x, g, acc);             // Xv^T g
             } else {
-                mma(c.tmem + colCarry, g, OP_K, a, OP_MN, HD / 16, HD, false);    // g Dy
-                mma(c.tmem + colAcc, g, OP_MN, x, OP_MN, 8, HD, acc);             // g^T Xv
+                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + colCarry, g, a, false);    // g Dy
+                mma<OP_MN, OP_MN, 8, HD>(c.tmem + colAcc, g, x, acc);             // g^T Xv
             }
             umma_commit(&c.bars[1]);
         }
@@ -487,7 +496,7 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
     }
     if (first && c.ok) {   // no version step: the level above is the only contribution
         loads_wait(c);
-        if (c.tid == 0 && c.ok) {
+        if (leader(c)) {
             tc_fence_after_sync();
             issue_parent(smem_u32(sm));
             umma_commit(&c.bars[1]);
@@ -549,7 +558,7 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
     const int c_hi = p.nseg > 1 ? min(p.N, c_lo + p.seg_chunks) : p.N, cnt = c_hi - c_lo;
     const int first = QUERY ? c_lo : c_hi - 1, step = QUERY ? 1 : -1;
     if (cnt <= 0) { teardown<256>(c, p.status); return; }
-    if (c.tid == 0) issue(first);
+    if (c.warp == 0 && elect_one()) issue(first);
 #pragma unroll 1
     for (int n = 0, J = first; n < cnt && c.ok; ++n, J += step) {
         const bool more = n + 1 < cnt;
@@ -557,22 +566,22 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
         const bool update = QUERY || more || (p.nseg > 1 && blockIdx.z > 0);
         loads_wait(c);
         publish();
-        if (c.tid == 0 && c.ok) {
+        if (leader(c)) {
             tc_fence_after_sync();
             const uint32_t a = smem_u32(sm);
-            mma(c.tmem, a, OP_K, a + 3 * kTileB, OP_MN, HD / 16, NC, false);                       // X R
-            mma(c.tmem, a, OP_K, a + 4 * kTileB, OP_MN, HD / 16, NC, true);
+            mma<OP_K, OP_MN, HD / 16, NC>(c.tmem, a, a + 3 * kTileB, false);                       // X R
+            mma<OP_K, OP_MN, HD / 16, NC>(c.tmem, a, a + 4 * kTileB, true);
             if (update) {
                 constexpr int pop = QUERY ? OP_K : OP_MN;                                          // P R  /  P^T R
-                mma(c.tmem + 128, a + 1 * kTileB, pop, a + 3 * kTileB, OP_MN, HD / 16, NC, false);
-                mma(c.tmem + 128, a + 2 * kTileB, pop, a + 3 * kTileB, OP_MN, HD / 16, NC, true);
-                mma(c.tmem + 128, a + 1 * kTileB, pop, a + 4 * kTileB, OP_MN, HD / 16, NC, true);
+                mma<pop, OP_MN, HD / 16, NC>(c.tmem + 128, a + 1 * kTileB, a + 3 * kTileB, false);
+                mma<pop, OP_MN, HD / 16, NC>(c.tmem + 128, a + 2 * kTileB, a + 3 * kTileB, true);
+                mma<pop, OP_MN, HD / 16, NC>(c.tmem + 128, a + 1 * kTileB, a + 4 * kTileB, true);
             }
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
         if (!c.ok) break;
-        if (c.tid == 0 && more) issue(J + step);   // every product has retired: the operand slots are free again
+        if (more && c.warp == 0 && elect_one()) issue(J + step);   // every product has retired: the operand slots are free again
         const int pos = J * kT + c.row, c0 = c.half * 32;
         float v[32];
         uint32_t hi[16], lo[16];
@@ -633,7 +642,7 @@ __global__ void __launch_bounds__(256, 1) suffix_kernel(const __grid_constant__ 
     __syncthreads();
 #pragma unroll 1
     for (int g = p.nseg - 1; g >= 1 && c.ok; --g) {
-        if (c.tid == 0) {
+        if (c.warp == 0 && elect_one()) {
             const long mrow = ((long)s * p.nseg + g) * 2 * HD;
             mbar_expect_tx(&c.bars[0], 2 * kT * HD * 2);
             tma_tile(sm, &tm.dyh, &c.bars[0], HD, (int)mrow);
@@ -641,12 +650,12 @@ __global__ void __launch_bounds__(256, 1) suffix_kernel(const __grid_constant__ 
         }
         loads_wait(c);
         publish();
-        if (c.tid == 0 && c.ok) {
+        if (leader(c)) {
             tc_fence_after_sync();
             const uint32_t a = smem_u32(sm);
-            mma(c.tmem, a, OP_K, a + 2 * kTileB, OP_MN, HD / 16, NC, false);       // M R
-            mma(c.tmem, a + kTileB, OP_K, a + 2 * kTileB, OP_MN, HD / 16, NC, true);
-            mma(c.tmem, a, OP_K, a + 3 * kTileB, OP_MN, HD / 16, NC, true);
+            mma<OP_K, OP_MN, HD / 16, NC>(c.tmem, a, a + 2 * kTileB, false);       // M R
+            mma<OP_K, OP_MN, HD / 16, NC>(c.tmem, a + kTileB, a + 2 * kTileB, true);
+            mma<OP_K, OP_MN, HD / 16, NC>(c.tmem, a, a + 3 * kTileB, true);
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
@@ -679,7 +688,7 @@ __global__ void __launch_bounds__(256, 2) apply_product_kernel(const __grid_cons
     uint8_t* sm = c.smem;   // slots: 0 x tile, 1 M hi, 2 M lo
     const long row0 = (long)s * p.Lp + (long)ch * kT;
     const long mi = p.nseg > 1 ? (long)s * p.nseg + ch / p.seg_chunks : (long)s;
-    if (c.tid == 0) {
+    if (c.warp == 0 && elect_one()) {
         mbar_expect_tx(&c.bars[0], 3 * kT * HD * 2);
         tma_tile(sm, &tm.qv, &c.bars[0], HD, (int)row0);
         tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(2 * mi * HD));
@@ -687,11 +696,11 @@ __global__ void __launch_bounds__(256, 2) apply_product_kernel(const __grid_cons
     }
     if (p.gq && c.tid < kT) p.gq[row0 + c.tid] += p.gtot[s];
     loads_wait(c);
-    if (c.tid == 0 && c.ok) {
+    if (leader(c)) {
         tc_fence_after_sync();
         const uint32_t a = smem_u32(sm);
-        mma(c.tmem, a, OP_K, a + kTileB, OP_MN, HD / 16, HD, false);
-        mma(c.tmem, a, OP_K, a + 2 * kTileB, OP_MN, HD / 16, HD, true);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + kTileB, false);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, true);
         umma_commit(&c.bars[1]);
     }
     mma_wait(c);
