@@ -23,6 +23,7 @@ enum : uint32_t {
 
 // What a forward that ran on a backward-sized workspace leaves at byte kStateRecordOffset of the status block: which
 // problem the chunk preparation in the workspace belongs to.  path_attn_bwd_reuse compares it on the device.
+constexpr size_t kNextItemOffset = 8;   // work-item counters of the persistent sweeps: 8 forward
 constexpr size_t kStateRecordOffset = 64;
 constexpr unsigned long long kStateMagic = 0x50615448537461ull;
 struct StateRecord {
@@ -121,6 +122,8 @@ struct FwdParams {
     // length and chunk count, and its gate terms [S, Lkp] (G then holds the query rows' terms; logit += G_i - Gk_j)
     const float* Gk;
     int Lkp, Nk;
+    int* next_item;     // work-item counter in the status block (zero on entry)
+    int group;          // slices per group of the work-item list (set by the launcher)
 };
 
 // Placement of the dyadic run products: level l holds dy_cnt[l] = N >> l matrices per slice, starting

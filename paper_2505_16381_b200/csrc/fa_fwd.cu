@@ -1,30 +1,30 @@
 // Fused forward sweep of PaTH attention (paper Sec. 3.3, the FlashAttention-style loop).
 //
-// A work item is one 128-row query chunk I of one (batch, head) slice; it walks the key chunks
-// J = I, I-1, ..., 0.  The diagonal chunk uses the raw q, k plus the in-chunk Householder
-// correction as a second contraction (Sec. 3.3, case i = j):
+// Query chunk I of one (batch, head) slice walks the key chunks J = I, I-1, ..., 0.  The diagonal chunk uses the raw q, k
+// plus the in-chunk Householder correction as a second contraction (Sec. 3.3, case i = j):
 //     S = Q K^T + (-lower(Q W^T)) (T^-1 strictLower(W K^T))           [operands q_raw,k_raw,xqn,yt]
-// Every earlier chunk J < I is an ordinary tile product of a query version and a key
-// version that meet at the dyadic boundary of (I, J):  S = Qv[l][I] Kv[l][J]^T, l = msb(I xor J).
-// The versions are prepared beforehand, so this loop contains no query update.
+// Every earlier chunk J < I is an ordinary tile product of a query version and a key version that meet at the dyadic
+// boundary of (I, J):  S = Qv[l][I] Kv[l][J]^T, l = msb(I xor J).  The versions are prepared beforehand, so this loop
+// contains no query update.
 //
-// The kernel is persistent: the work items are listed slice after slice, each slice as pairs (longest, shortest),
-// (second longest, second shortest), ..., and CTA c takes the pairs c, c + gridDim.x, ...  Every pair has the same
-// number of key chunks, CTAs that run together work on a few slices whose keys and values stay in L2, and the
-// loads and the first logit tile of the next item are produced while the current item's result is written out.
+// Two kernels.  fa_fwd_kernel: a work item is a PAIR of neighbouring query chunks (2k, 2k+1), one stream each: both meet
+// every key chunk J < 2k at the same level (the indices differ in bit 0 only), so one load of a key and a value tile
+// serves both.  fa_split_kernel: a work item is one query chunk whose key chunks are dealt alternately to the two streams
+// and whose two partial results are merged at the end; half the latency per chunk, twice the tile traffic: for problems
+// whose pairs do not fill the GPU.  The rule is at launch_fa_fwd.
 //
-// The key chunks are dealt alternately to two streams (n = I - J even / odd).  Each stream has its own
-// softmax warpgroup (one query row per thread, the whole 128-wide logit row held in registers), its own S tile
-// and O accumulator in tensor memory and its own running (max, sum); the two partial results are merged at
-// the end like a split-KV attention.  While one warpgroup does its exponentials the tensor pipe works for the
-// other stream.  P never touches shared memory: it overwrites the first half of its S tile as packed bf16 and
-// enters O += P V as the tensor-memory A operand.
+// A stream has its own softmax warpgroup (one query row per thread, the whole 128-wide logit row held in registers), its
+// own S tile and O accumulator in tensor memory and its own running (max, sum).  While one warpgroup does its
+// exponentials the tensor pipe works for the other stream.  P never touches shared memory: it is written to tensor memory
+// as packed bf16 and enters O += P V as the tensor-memory A operand.  It is handed over in two parts, so that
+// the P V of the first three quarters runs underneath the last quarter's exponentials.
 //
-// Warps: 0 = TMA producer, 1 = tcgen05 MMA issuer, 2-3 idle (they give their registers to the softmax
+// Warps of both kernels: 0 = TMA producer, 1 = tcgen05 MMA issuer, 2-3 idle (they give their registers to the softmax
 // warps), 4-7 = softmax of stream 0, 8-11 = softmax of stream 1.
 #include <type_traits>
 #include "common.cuh"
 #include "tc5.cuh"
+#include "tileops.cuh"
 
 namespace path {
 using namespace tc5;
@@ -63,6 +63,13 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return d;
 }
 
+// Plain (untiled) bulk copy global -> shared, completion counted in bytes on `bar`; 16-byte aligned, size % 16 == 0.
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
 // D[tmem] (+)= A[tmem, packed bf16, 8 columns per 16 elements of the contraction] * B[smem]
 __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                         uint32_t accumulate) {
@@ -74,13 +81,129 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
         : "memory");
 }
 
-struct FwdSmem {
+// One logit tile of one stream, one query row per thread: S (tensor memory) -> P (packed bf16, tensor memory), running
+// maximum m (log2 units) and sum l.  `tS`, `tP`, `tO`: tensor-memory addresses of the thread's lanes; `gk`: gate prefix of
+// the tile's key chunk (shared memory), `gi2` that of the row in log2 units; `have_o`: O holds an earlier result.
+//   SEP: P has columns of its own (d = 64, where the accumulators leave room) and S is handed back (`sfree`) as soon as it
+//   is in registers.  Otherwise P overwrites the first half of S.
+// The stream's previous P V has retired before the call: P may be overwritten and O is stable.
+// P is handed over in two parts (`pa`: the first 96 keys, `pb`).  Every hand-over is one arrival per warp.
+template <int HD, bool GATE, bool DIAG, bool SEP>
+__device__ __forceinline__ bool softmax_tile(uint32_t tS, uint32_t tP, uint32_t tO, int row, const uint64_t sl2x2, float sl2,
+                                             float gi2, const float* gk, bool have_o, float& m, float& l, uint64_t* sfree,
+                                             uint64_t* pa, uint64_t* pb, bool ok) {
+    constexpr bool PRE = DIAG || GATE;                 // logits are scaled (and gated, masked) in place first
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    if (ok) {
+        uint32_t r[4][32];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, r[c]);
+        tmem_ld_wait();
+        if (SEP) {
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane0) mbar_arrive(sfree);
+        }
+        float m_new = m;
+        if (PRE) {
+            const uint64_t gi22 = pack2(gi2, gi2), nlog2 = pack2(-1.4426950408889634f, -1.4426950408889634f);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int e = 0; e < 32; e += 4) {
+                    uint64_t v[2];
+#pragma unroll
+                    for (int y = 0; y < 2; ++y)
+                        v[y] = fma2(pack2(__uint_as_float(r[c][e + 2 * y]), __uint_as_float(r[c][e + 2 * y + 1])), sl2x2, gi22);
+                    if (GATE) {
+                        const float4 g4 = *reinterpret_cast<const float4*>(gk + c * 32 + e);
+                        v[0] = fma2(pack2(g4.x, g4.y), nlog2, v[0]);
+                        v[1] = fma2(pack2(g4.z, g4.w), nlog2, v[1]);
+                    }
+                    float a[4];
+                    unpack2(v[0], a[0], a[1]);
+                    unpack2(v[1], a[2], a[3]);
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) {
+                        if (DIAG && c * 32 + e + y > row) a[y] = -INFINITY;
+                        r[c][e + y] = __float_as_uint(a[y]);
+                    }
+                }
+        }
+        // row maximum of the scaled logits (log2 units)
+        float a4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int e = 0; e < 32; e += 2)
+                a4[(e >> 1) & 3] = max3(a4[(e >> 1) & 3], __uint_as_float(r[c][e]), __uint_as_float(r[c][e + 1]));
+        float mx = fmaxf(fmaxf(a4[0], a4[1]), fmaxf(a4[2], a4[3]));
+        if (!PRE) mx *= sl2;
+        const bool grow = mx > m + 8.f;       // lazy rescaling: a stale maximum is tolerated up to 2^8
+        if (grow) m_new = mx;
+        if (__any_sync(0xffffffffu, grow)) {
+            const float alpha = ex2(m - m_new);
+            l *= alpha;
+            if (have_o) {
+#pragma unroll 1
+                for (int c = 0; c < HD / 16; ++c) {
+                    uint32_t o[16];
+                    tmem_ld16(tO + c * 16, o);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                    tmem_st16(tO + c * 16, o);
+                }
+            }
+        }
+        m = m_new;
+        const uint64_t nm2 = pack2(-m, -m);
+        const uint64_t mul2 = PRE ? pack2(1.f, 1.f) : sl2x2;
+        uint64_t lacc[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            uint32_t pk[16];
+#pragma unroll
+            for (int e = 0; e < 32; e += 2) {
+                const uint64_t v = fma2(pack2(__uint_as_float(r[c][e]), __uint_as_float(r[c][e + 1])), mul2, nm2);
+                float a, b;
+                unpack2(v, a, b);
+                a = ex2(a);
+                b = ex2(b);
+                lacc[(e >> 1) & 1] = add2(lacc[(e >> 1) & 1], pack2(a, b));
+                pk[e >> 1] = pack_bf16(a, b);
+            }
+            tmem_st16(tP + c * 16, pk);
+            if (c == 2) {
+                tmem_st_wait();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane0) mbar_arrive(pa);
+            }
+        }
+        float la, lb;
+        unpack2(add2(lacc[0], lacc[1]), la, lb);
+        l += la + lb;
+        tmem_st_wait();
+    }
+    tc_fence_before_sync();
+    __syncwarp();
+    if (lane0) {
+        if (!ok) mbar_arrive(pa);
+        if (SEP && !ok) mbar_arrive(sfree);
+        mbar_arrive(pb);
+    }
+    return ok;
+}
+
+// ------------------------------------------------------------------------------------------------ one chunk, two streams
+struct SplitSmem {
     static constexpr uint32_t offQ = 0;                       // 3 slots: ring of query operands
     static constexpr uint32_t offK = offQ + 3 * kSlotBytes;   // 2 slots: one per stream
     static constexpr uint32_t offV = offK + 2 * kSlotBytes;   // 2 slots: one per stream
     static constexpr uint32_t offBar = offV + 2 * kSlotBytes;
-    // [2 streams][128] pairs: .x = gate prefix of the stream's current key chunk during the sweep; at the end of
-    // a work item the pair is the stream's (running max, running sum)
+    // [2 streams][128] pairs: at the end of a work item the stream's (running max, running sum) per row; before that the
+    // first half of a stream's part holds the gate prefix of its current key chunk
     static constexpr uint32_t offStat = offBar + 256;
     static constexpr uint32_t total = offStat + 2 * kTile * 8;
     static constexpr uint32_t alloc = 232448;                 // everything an SM offers one CTA
@@ -88,36 +211,31 @@ struct FwdSmem {
 };
 
 enum { B_QFULL = 0, B_QEMPTY = 3, B_KFULL = 6, B_KEMPTY = 8, B_VFULL = 10, B_VEMPTY = 12,
-       B_SFULL = 14, B_PFULL = 16, B_OFULL = 18, B_OFREE = 20, B_COUNT = 21 };
+       B_SFULL = 14, B_PA = 16, B_PB = 18, B_OFULL = 20, B_OFREE = 22, B_COUNT = 23 };
 
-// CROSS = true is the segment-against-segment variant used by the context-parallel path (paper Sec. 3.5): a work item is a
-// query chunk of one segment, it visits EVERY key chunk of another (earlier) segment, there is no diagonal chunk and no
-// causal mask, queries and keys come as one prepared tile each (tm.qv / tm.kv, no levels), the key-side gate terms are
-// their own array (whose padded tail holds a huge value, which masks the padded keys), and the result is written
-// normalised in float32 together with its LSE so that the caller can merge it into a running state.
-template <int HD, bool GATE, bool CROSS = false>
+template <int HD, bool GATE>
 __global__ void __launch_bounds__(384, 1)
-fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
+fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    if ((uint32_t)(smem - smem_raw) + FwdSmem::total > FwdSmem::alloc) {   // uniform over the CTA
+    if ((uint32_t)(smem - smem_raw) + SplitSmem::total > SplitSmem::alloc) {   // uniform over the CTA
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_FWD_PRODUCER);
         return;
     }
-    uint8_t* sQ = smem + FwdSmem::offQ;
-    uint8_t* sK = smem + FwdSmem::offK;
-    uint8_t* sV = smem + FwdSmem::offV;
-    uint64_t* bars = (uint64_t*)(smem + FwdSmem::offBar);
+    uint8_t* sQ = smem + SplitSmem::offQ;
+    uint8_t* sK = smem + SplitSmem::offK;
+    uint8_t* sV = smem + SplitSmem::offV;
+    uint64_t* bars = (uint64_t*)(smem + SplitSmem::offBar);
     uint32_t* tmem_slot = (uint32_t*)(bars + B_COUNT);
     volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);
-    float2* stat = (float2*)(smem + FwdSmem::offStat);
+    float2* stat = (float2*)(smem + SplitSmem::offStat);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int items = p.N * p.S;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < B_COUNT; ++i)
-            mbar_init(&bars[i], (i == B_PFULL || i == B_PFULL + 1) ? 128u : (i == B_OFREE ? 256u : 1u));
+            mbar_init(&bars[i], (i >= B_PA && i < B_OFULL) ? 4u : (i == B_OFREE ? 256u : 1u));
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -130,9 +248,10 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     // tensor memory columns: S of stream x at x*128 (P aliases its first 64 columns), O of stream x at 256 + x*128
-    // k-th work item of this CTA: pairs (long, short) of one slice, slice after slice (keeps a slice's keys in L2)
+    // k-th work item of this CTA: one if there are CTAs enough, otherwise pairs (long, short) of one slice, slice after slice
+    const bool single = (int)gridDim.x >= items;
     auto item_of = [&](int k, int& I, int& s) {
-        const int w = 2 * ((int)blockIdx.x + (k >> 1) * (int)gridDim.x) + (k & 1);
+        const int w = single ? (k == 0 ? (int)blockIdx.x : items) : 2 * ((int)blockIdx.x + (k >> 1) * (int)gridDim.x) + (k & 1);
         if (w >= items) return false;
         s = w / p.N;
         const int j = w % p.N;
@@ -142,7 +261,6 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
     // key chunks a work item visits, counted from the diagonal: all I + 1 of them, or fewer when the gate has made the
     // far ones negligible (every warp role reads the same precomputed number)
     auto steps_of = [&](int I, int s) {
-        if (CROSS) return p.Nk;
         return p.nkeep ? min(I + 1, p.nkeep[s * p.N + I]) : I + 1;
     };
 
@@ -179,15 +297,6 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
             for (int it = 0; ok && item_of(it, I, s); ++it) {
                 const int NS = steps_of(I, s);
                 const int rowRaw = s * p.Lp + I * kTile;
-                if (CROSS) {   // one query tile, then every key chunk of the other segment, last chunk first
-                    load_q(&tm.qv, HD, rowRaw);
-                    for (int n = 0; n < NS && ok; ++n) {
-                        const int x = n & 1, rowK = s * p.Lkp + (NS - 1 - n) * kTile;
-                        load_kv(sK, B_KFULL, B_KEMPTY, x, kf, &tm.kv, HD, rowK);
-                        load_kv(sV, B_VFULL, B_VEMPTY, x, vf, &tm.v, HD, rowK);
-                    }
-                    continue;
-                }
                 // diagonal chunk: raw q, k and the correction operands (both K slots), V of chunk I
                 load_q(&tm.q_raw, HD, rowRaw);
                 load_kv(sK, B_KFULL, B_KEMPTY, 0, kf, &tm.k_raw, HD, rowRaw);
@@ -244,24 +353,13 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                 int cur_level = -1;
                 int q_of0, q_of1;              // operand index used by each stream's most recent S product
                 auto advance_q = [&](int n) {  // operand index of step n >= 1 (waits for a newly needed one)
-                    const int l = CROSS ? 0 : msb32((unsigned)(I ^ (I - n)));
+                    const int l = msb32((unsigned)(I ^ (I - n)));
                     if (l != cur_level) {
                         cur_level = l;
                         take_q();
                     }
                     return qi_next - 1;
                 };
-                if (CROSS) {   // S of step 0 (stream 0): an ordinary tile product; the one query operand serves every step
-                    cur_level = 0;
-                    const int q0 = take_q();
-                    take_k(0);
-                    tc_fence_after_sync();
-                    if (!ok) break;
-                    issue_s(0, q0 % 3, 0, HD, false);
-                    umma_commit(&bars[B_SFULL + 0]);
-                    umma_commit(&bars[B_KEMPTY + 0]);
-                    q_of0 = q_of1 = q0;
-                } else {
                 // S of step 0 (diagonal, stream 0): two contractions
                 const int q0 = take_q();
                 take_k(0);
@@ -277,7 +375,6 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                 umma_commit(&bars[B_VEMPTY + 1]);
                 release_q(q1 + 1);             // rawQ and Xqn go back once the diagonal products retire
                 q_of0 = q_of1 = q1 + 1;
-                }
                 // S of step 1 (stream 1)
                 if (NS > 1) {
                     q_of1 = advance_q(1);
@@ -293,19 +390,26 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                     const int x = n & 1, t = n >> 1;
                     // O_x += P_x V_n; the first product of a work item overwrites O_x, which the previous item's
                     // epilogue must have read
-                    wait(B_PFULL + x, (int)((pc >> x) & 1u)); pc ^= 1u << x;
+                    const uint32_t pp = (pc >> x) & 1u;
+                    pc ^= 1u << x;
                     wait(B_VFULL + x, (int)((vc >> x) & 1u)); vc ^= 1u << x;
                     if (t == 0 && item > 0) wait(B_OFREE, item - 1);
+                    wait(B_PA + x, (int)pp);
                     tc_fence_after_sync();
                     if (!ok) break;
                     {
-                        uint32_t b_lo = umma_desc_lo(smem_u32(sV + x * kSlotBytes), kPanelBytes);
+                        const uint32_t b_lo = umma_desc_lo(smem_u32(sV + x * kSlotBytes), kPanelBytes);
 #pragma unroll
                         for (int kk = 0; kk < kTile / 16; ++kk) {
-                            umma_ts(tmem + 256 + x * 128, tmem + x * 128 + kk * 8, umma_desc_join(b_lo), idescO,
+                            if (kk == 6) {
+                                wait(B_PB + x, (int)pp);
+                                tc_fence_after_sync();
+                                if (!ok) break;
+                            }
+                            umma_ts(tmem + 256 + x * 128, tmem + x * 128 + kk * 8, umma_desc_join(b_lo + kk * 128u), idescO,
                                     (t > 0 || kk > 0) ? 1u : 0u);
-                            b_lo += 128u;
                         }
+                        if (!ok) break;
                         umma_commit(&bars[B_VEMPTY + x]);
                     }
                     // the stream's next S overwrites P; products issued by one thread execute in order, so it lands
@@ -344,6 +448,7 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
         int o1 = 0;                             // work items so far in which stream 1 had steps
         int item = 0;
         float2* statx = stat + x * kTile;
+        float* gkx = reinterpret_cast<float*>(statx);
         auto wg_sync = [&]() {
             __syncwarp();   // bar.sync is warp-aligned: reconverge first
             if (x == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -363,102 +468,23 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
 
             auto softmax_step = [&](auto diag_tag, const int t) {
                 constexpr bool DIAG = decltype(diag_tag)::value;   // the diagonal chunk (step 0): causal mask
-                constexpr bool PRE = DIAG || GATE;                 // logits are scaled (and gated, masked) in place first
-                const int n = 2 * t + x, J = CROSS ? NS - 1 - n : I - n;
+                const int J = I - (2 * t + x);
                 if (GATE) {
                     wg_sync();   // everyone is done with the previous chunk's values
-                    statx[row].x = CROSS ? p.Gk[(size_t)s * p.Lkp + J * kTile + row] * kLog2e
-                                         : p.G[(size_t)s * p.Lp + J * kTile + row] * kLog2e;
+                    gkx[row] = p.G[(size_t)s * p.Lp + J * kTile + row];
                     wg_sync();
                 }
                 if (ok && !mbar_wait(&bars[B_SFULL + x], sc & 1, abort_flag, ST_FWD_SOFTMAX)) ok = false;
                 ++sc;
                 ok = __all_sync(0xffffffffu, ok);  // keep the warp-collective TMEM accesses convergent
                 tc_fence_after_sync();
-                if (ok) {
-                    uint32_t r[4][32];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) tmem_ld32(tlane + colS + c * 32, r[c]);
-                    tmem_ld_wait();
-                    if (PRE) {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-#pragma unroll
-                            for (int e = 0; e < 32; e += 2) {
-                                float g0 = 0.f, g1 = 0.f;
-                                if (GATE) { g0 = gi2 - statx[c * 32 + e].x; g1 = gi2 - statx[c * 32 + e + 1].x; }
-                                const uint64_t v = fma2(pack2(__uint_as_float(r[c][e]), __uint_as_float(r[c][e + 1])), sl2x2,
-                                                        pack2(g0, g1));
-                                float a, b;
-                                unpack2(v, a, b);
-                                if (DIAG) {
-                                    if (c * 32 + e > row) a = -INFINITY;
-                                    if (c * 32 + e + 1 > row) b = -INFINITY;
-                                }
-                                r[c][e] = __float_as_uint(a);
-                                r[c][e + 1] = __float_as_uint(b);
-                            }
-                    }
-                    // row maximum of the scaled logits (log2 units)
-                    float a4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-#pragma unroll
-                        for (int e = 0; e < 32; e += 2)
-                            a4[(e >> 1) & 3] = max3(a4[(e >> 1) & 3], __uint_as_float(r[c][e]), __uint_as_float(r[c][e + 1]));
-                    float mx = fmaxf(fmaxf(a4[0], a4[1]), fmaxf(a4[2], a4[3]));
-                    if (!PRE) mx *= sl2;
-                    // lazy rescaling: tolerate a stale maximum up to 2^8.  O of this stream is stable here: its S
-                    // tile only becomes ready after the stream's previous P V has retired
-                    float m_new = m;
-                    const bool grow = mx > m + 8.f;
-                    if (grow) m_new = mx;
-                    if (__any_sync(0xffffffffu, grow)) {
-                        const float alpha = ex2(m - m_new);
-                        l *= alpha;
-                        if (t > 0) {
-#pragma unroll 1
-                            for (int c = 0; c < HD / 16; ++c) {
-                                uint32_t o[16];
-                                tmem_ld16(tlane + colO + c * 16, o);
-                                tmem_ld_wait();
-#pragma unroll
-                                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                                tmem_st16(tlane + colO + c * 16, o);
-                            }
-                        }
-                    }
-                    m = m_new;
-                    // probabilities -> packed bf16 over the first 64 columns of the S tile
-                    const uint64_t nm2 = pack2(-m, -m);
-                    const uint64_t mul2 = PRE ? pack2(1.f, 1.f) : sl2x2;
-                    uint64_t lacc = pack2(0.f, 0.f);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t pk[16];
-#pragma unroll
-                        for (int e = 0; e < 32; e += 2) {
-                            const uint64_t v = fma2(pack2(__uint_as_float(r[c][e]), __uint_as_float(r[c][e + 1])), mul2, nm2);
-                            float a, b;
-                            unpack2(v, a, b);
-                            a = ex2(a);
-                            b = ex2(b);
-                            lacc = add2(lacc, pack2(a, b));
-                            pk[e >> 1] = pack_bf16(a, b);
-                        }
-                        tmem_st16(tlane + colS + c * 16, pk);
-                    }
-                    float la, lb;
-                    unpack2(lacc, la, lb);
-                    l += la + lb;
-                    tmem_st_wait();
-                }
-                tc_fence_before_sync();
-                mbar_arrive(&bars[B_PFULL + x]);
+                // O of this stream is stable here: its S tile only becomes ready after the stream's previous P V has retired
+                ok = softmax_tile<HD, GATE, DIAG, false>(tlane + colS, tlane + colS, tlane + colO, row, sl2x2, sl2, gi2, gkx, t > 0, m,
+                                                         l, nullptr, &bars[B_PA + x], &bars[B_PB + x], ok);
             };
             {
                 int t = 0;
-                if (!CROSS && x == 0 && TX > 0) {
+                if (x == 0 && TX > 0) {
                     softmax_step(std::true_type{}, 0);
                     t = 1;
                 }
@@ -547,26 +573,483 @@ fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
     }
 }
 
-// Host-side launcher (called from the C-ABI translation unit).
-template <int HD>
-static cudaError_t launch_hd(const FwdTensorMaps& tm, const FwdParams& p, cudaStream_t st) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int pairs = (p.N * p.S + 1) / 2;
-    dim3 grid(pairs < sms ? pairs : sms), block(384);
-    if (p.G) {
-        e = cudaFuncSetAttribute(fa_fwd_kernel<HD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem::alloc);
-        if (e != cudaSuccess) return e;
-        fa_fwd_kernel<HD, true><<<grid, block, FwdSmem::alloc, st>>>(tm, p);
-    } else {
-        e = cudaFuncSetAttribute(fa_fwd_kernel<HD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem::alloc);
-        if (e != cudaSuccess) return e;
-        fa_fwd_kernel<HD, false><<<grid, block, FwdSmem::alloc, st>>>(tm, p);
+// ------------------------------------------------------------------------------------------------ pairs of query chunks
+// Work items come from a counter (p.next_item, zero on entry): CTA c starts with item c, every further one is the next
+// unclaimed.  The list goes through groups of slices whose keys and values stay in L2 together (p.group slices), inside a
+// group longest pairs first, so that the CTAs end together without the items having to be cut alike.
+//
+// Per item, with I1 = 2k+1 (stream 1) and I0 = 2k (stream 0): stream 1's step n meets key chunk J = I1 - n, stream 0's
+// step n - 1 the same chunk.  The loop runs over n; n = 0 is stream 1's diagonal chunk alone, n = 1 stream 0's diagonal
+// and stream 1's first earlier chunk (level 0), from n = 2 on both streams use the same key tile.  The products are issued
+// in the order  PV0(n), S0(n+1), PV1(n), S1(n+1)  (d = 128: P lies over S) or  S0(n+1), PV0(n), S1(n+1), PV1(n)  (d = 64:
+// P has its own columns and S(n+1) only waits until S(n) is in registers).
+//
+// What bounds it: at d = 128 a tile pair is two products of 512 cycles and 16384 exponentials at 16 per cycle (1024
+// cycles); shared memory moves 64 cycles' worth of operands per 64-cycle step of S and half of that for P V, plus the
+// arriving tiles, which is why one key and value tile serves two query chunks here.  Measured, against one chunk over two
+// streams with P handed over whole: 32 slices x 32768 tokens x d = 128: 8.33 -> 7.85 ms (1120 TFLOP/s; the board is at its
+// power cap there); 128 x 2048 x 64: 158 -> 148 us; 128 x 4096 x 64: 517 -> 482 us; 64 x 4096 x 128: 312 -> 308 us; gated
+// 32 x 8192 x 128: 187 -> 169 us.  A stream's cycle of about 3400 clocks is 1450 of exponentials (1120 for a warpgroup that
+// has the unit to itself), 300 for the maximum, 300 for tensor-memory transfers and 1200 waiting for P V and the next S.
+//
+// CROSS = true is the segment-against-segment variant of the context-parallel path (paper Sec. 3.5): every query chunk of
+// one segment visits EVERY key chunk of another (earlier) one, no diagonal chunk, no causal mask, queries and keys come as
+// one prepared tile each (tm.qv / tm.kv, no levels), the key-side gate terms are their own array (whose padded tail holds a
+// huge value, which masks the padded keys), and the result is written normalised in float32 together with its LSE so
+// that the caller can merge it into a running state.
+struct FwdSmem {
+    static constexpr uint32_t offQ = 0;                        // ring of 3 query operands
+    static constexpr uint32_t offKV = offQ + 3 * kSlotBytes;   // ring of 4 key / value operands, in the order of their use
+    static constexpr uint32_t offBar = offKV + 4 * kSlotBytes;
+    static constexpr uint32_t offGk = offBar + 512;            // [2 streams][2][128] gate prefix of a key chunk
+    static constexpr uint32_t total = offGk + 2 * 2 * kTile * 4;
+    static constexpr uint32_t alloc = 232448;                  // everything an SM offers one CTA
+    static_assert(total + 512 <= alloc, "no room left to align the base");
+};
+enum { F_QFULL = 0, F_QEMPTY = F_QFULL + 3, F_KVFULL = F_QEMPTY + 3, F_KVEMPTY = F_KVFULL + 4, F_SFULL = F_KVEMPTY + 4,
+       F_SFREE = F_SFULL + 2, F_PA = F_SFREE + 2, F_PB = F_PA + 2, F_PFREE = F_PB + 2, F_OFULL = F_PFREE + 2,
+       F_OFREE = F_OFULL + 2, F_GKFULL = F_OFREE + 2, F_GKEMPTY = F_GKFULL + 4, F_ITFULL = F_GKEMPTY + 4,
+       F_ITEMPTY = F_ITFULL + 2, F_COUNT = F_ITEMPTY + 2 };
+
+template <int HD, bool GATE, bool CROSS>
+__global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
+    constexpr bool SEP = HD == 64;
+    constexpr int kOff = CROSS ? 0 : 1;                        // stream 0's step index is n - kOff
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    if ((uint32_t)(smem - smem_raw) + FwdSmem::total > FwdSmem::alloc) {   // uniform over the CTA
+        if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_FWD_PRODUCER);
+        return;
     }
+    uint8_t* sQ = smem + FwdSmem::offQ;
+    uint8_t* sKV = smem + FwdSmem::offKV;
+    uint64_t* bars = (uint64_t*)(smem + FwdSmem::offBar);
+    uint32_t* tmem_slot = (uint32_t*)(bars + F_COUNT);
+    volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);
+    volatile int* item_ring = (volatile int*)(tmem_slot + 2);  // [2]
+    static_assert(F_COUNT * 8 + 16 <= 512, "barriers and words must fit");
+    float* sGk = (float*)(smem + FwdSmem::offGk);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int NP = (p.N + 1) >> 1, items = NP * p.S;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < F_COUNT; ++i) {
+            uint32_t n = 1;
+            if ((i >= F_SFREE && i < F_PFREE) || (i >= F_OFREE && i < F_GKFULL) || (i >= F_GKEMPTY && i < F_ITFULL)) n = 4;   // one per softmax warp
+            if (i >= F_ITEMPTY) n = 9;                         // eight softmax warps and the issuer
+            mbar_init(&bars[i], n);
+        }
+        *abort_flag = 0;
+        mbar_fence_init();
+    }
+    if (warp == 2 && lane < 7) tma_prefetch_desc(reinterpret_cast<const CUtensorMap*>(&tm) + lane);   // the seven maps are contiguous
+    if (warp == 1) tmem_alloc(tmem_slot, 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+    // tensor-memory columns of stream x: S at x * 128, O at 256 + x * HD, P over S or (d = 64) at 384 + x * 64
+    auto colP = [](int x) { return SEP ? 384u + (uint32_t)x * 64u : (uint32_t)x * 128u; };
+    auto decode = [&](int idx, int& k, int& s) {
+        const int per = p.group * NP, g = idx / per, w = idx - g * per;
+        const int gl = min(p.group, p.S - g * p.group);
+        k = NP - 1 - w / gl;
+        s = g * p.group + w % gl;
+    };
+    // key chunks query chunk I visits, counted from the diagonal: all I + 1 of them, or fewer when the gate has made the
+    // far ones negligible (every warp role reads the same precomputed number); none if the chunk does not exist
+    auto steps_of = [&](int I, int s) {
+        if (I >= p.N) return 0;
+        if (CROSS) return p.Nk;
+        return p.nkeep ? min(I + 1, p.nkeep[s * p.N + I]) : I + 1;
+    };
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        if (warp == 0 && elect_one()) {
+            // ------------------------------------------------------------ TMA producer (and item scheduler)
+            bool ok = true;
+            int nq = 0, nkv = 0, it = 0;      // query operands, key / value operands, items handed out so far
+            int ng[2] = {0, 0};               // gate vectors so far, per stream
+            auto wait_empty = [&](int bar, int use) {
+                if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_FWD_PRODUCER)) ok = false;
+            };
+            auto load_q = [&](const CUtensorMap* m, int kdim, int row0) {
+                const int slot = nq % 3;
+                wait_empty(F_QEMPTY + slot, nq / 3);
+                if (!ok) return;
+                mbar_expect_tx(&bars[F_QFULL + slot], (uint32_t)(kTile * kdim * 2));
+                for (int h = 0; h < kdim / 64; ++h)
+                    tma_load_2d(sQ + slot * kSlotBytes + h * kPanelBytes, m, &bars[F_QFULL + slot], h * 64, row0);
+                ++nq;
+            };
+            auto load_kv = [&](const CUtensorMap* m, int kdim, int row0) {
+                const int slot = nkv & 3;
+                wait_empty(F_KVEMPTY + slot, nkv >> 2);
+                if (!ok) return;
+                mbar_expect_tx(&bars[F_KVFULL + slot], (uint32_t)(kTile * kdim * 2));
+                for (int h = 0; h < kdim / 64; ++h)
+                    tma_load_2d(sKV + slot * kSlotBytes + h * kPanelBytes, m, &bars[F_KVFULL + slot], h * 64, row0);
+                ++nkv;
+            };
+            auto load_gk = [&](int x, const float* src) {
+                const int b = x * 2 + (ng[x] & 1);
+                wait_empty(F_GKEMPTY + b, ng[x] >> 1);
+                if (!ok) return;
+                mbar_expect_tx(&bars[F_GKFULL + b], kTile * 4);
+                bulk_load(sGk + b * kTile, src, kTile * 4, &bars[F_GKFULL + b]);
+                ++ng[x];
+            };
+            int idx = blockIdx.x;
+            for (; ok; ++it) {
+                // hand the item to the other roles (-1: no more)
+                wait_empty(F_ITEMPTY + (it & 1), it >> 1);
+                if (!ok) break;
+                item_ring[it & 1] = idx < items ? idx : -1;
+                mbar_arrive(&bars[F_ITFULL + (it & 1)]);
+                if (idx >= items) break;
+                const int next = (int)gridDim.x + atomicAdd(p.next_item, 1);   // (its latency hides under this item's loads)
+                int k, s;
+                decode(idx, k, s);
+                const int I0 = 2 * k, I1 = 2 * k + 1;
+                const int NS0 = steps_of(I0, s), NS1 = steps_of(I1, s), NV = max(NS1, NS0 + kOff);
+                const int rowS = s * p.Lp;
+                auto chunk_at = [&](int n) { return CROSS ? p.Nk - 1 - n : I1 - n; };
+                auto level_at = [&](int n) { return n == 1 ? 0 : msb32((unsigned)(I0 ^ (I1 - n))); };
+                auto load_step = [&](int n) {   // operands of the logit tiles of step n (n >= 1; CROSS: n >= 0)
+                    const bool u0 = n >= 1 + kOff && n - kOff < NS0, u1 = n >= 1 && n < NS1;
+                    if (CROSS) {
+                        if (u0 || u1) load_kv(&tm.kv, HD, s * p.Lkp + chunk_at(n) * kTile);
+                        return;
+                    }
+                    if (!u0 && !u1) return;
+                    const int l = level_at(n);
+                    const bool fresh = n <= 2 || l != level_at(n - 1);
+                    // (query tiles first: both are ahead of the key tile in the order of use only when they are new)
+                    if (u0 && fresh) load_q(&tm.qv, HD, (int)qver_row(p.vl, s, l, I0));
+                    load_kv(&tm.kv, HD, (int)kver_row(p.vl, s, l, I1 - n));
+                    if (u1 && fresh) load_q(&tm.qv, HD, (int)qver_row(p.vl, s, l, I1));
+                };
+                if (CROSS) {
+                    load_q(&tm.qv, HD, rowS + I0 * kTile);
+                    load_kv(&tm.kv, HD, s * p.Lkp + chunk_at(0) * kTile);
+                    if (NS1 > 0) load_q(&tm.qv, HD, rowS + I1 * kTile);
+                } else {
+                    if (NS1 > 0) {   // stream 1's diagonal chunk: raw q, k and the correction operands
+                        load_q(&tm.q_raw, HD, rowS + I1 * kTile);
+                        load_kv(&tm.k_raw, HD, rowS + I1 * kTile);
+                        load_q(&tm.xqn, kTile, rowS + I1 * kTile);
+                        load_kv(&tm.yt, kTile, rowS + I1 * kTile);
+                    }
+                    load_q(&tm.q_raw, HD, rowS + I0 * kTile);
+                    load_kv(&tm.k_raw, HD, rowS + I0 * kTile);
+                    load_q(&tm.xqn, kTile, rowS + I0 * kTile);
+                    load_kv(&tm.yt, kTile, rowS + I0 * kTile);
+                }
+                for (int n = 0; n < NV && ok; ++n) {
+                    const bool u0 = n >= kOff && n - kOff < NS0, u1 = n < NS1;
+                    if (SEP) load_step(n + 1);
+                    if (u0 || u1) {
+                        const int J = chunk_at(n);
+                        if (GATE) {
+                            const float* g = CROSS ? p.Gk + (size_t)s * p.Lkp + J * kTile : p.G + (size_t)s * p.Lp + J * kTile;
+                            if (u0) load_gk(0, g);
+                            if (u1) load_gk(1, g);
+                        }
+                        load_kv(&tm.v, HD, (CROSS ? s * p.Lkp : rowS) + J * kTile);
+                    }
+                    if (!SEP) load_step(n + 1);
+                }
+                idx = next;
+            }
+        } else if (warp == 1 && elect_one()) {
+            // ------------------------------------------------------------ MMA issuer
+            // a negative scale is applied as a sign flip of the logits here (negate-A bit), its magnitude in the softmax
+            const uint32_t idescS = umma_idesc(128, 128, 0, 0) | (p.scale < 0.f ? (1u << 13) : 0u);
+            constexpr uint32_t idescO = umma_idesc(128, HD, 0, 1);
+            bool ok = true;
+            int nq = 0, nkv = 0;              // query and key / value operands used so far
+            int ns[2] = {0, 0}, np[2] = {0, 0}, no[2] = {0, 0};   // logit tiles, P tiles, finished results per stream so far
+            int curq[2] = {0, 0};             // ring index of the query tile a stream uses
+            auto wait = [&](int bar, int parity) {
+                if (ok && !mbar_wait(&bars[bar], parity & 1, abort_flag, ST_FWD_MMA)) ok = false;
+            };
+            auto q_wait = [&](int i) { wait(F_QFULL + i % 3, i / 3); };
+            auto kv_wait = [&](int i) { wait(F_KVFULL + (i & 3), i >> 2); };
+            auto q_free = [&](int i) { umma_commit(&bars[F_QEMPTY + i % 3]); };
+            auto kv_free = [&](int i) { umma_commit(&bars[F_KVEMPTY + (i & 3)]); };
+            auto issue_s = [&](int x, int qi, int ki, auto kdim_tag, bool acc) {
+                constexpr int KD = decltype(kdim_tag)::value;
+                // (descriptors advance by their low word only: 32 bytes per step, the next panel after four steps)
+                const uint32_t a_lo = umma_desc_lo(smem_u32(sQ + (qi % 3) * kSlotBytes), 16), b_lo = umma_desc_lo(smem_u32(sKV + (ki & 3) * kSlotBytes), 16);
+#pragma unroll
+                for (int kk = 0; kk < KD / 16; ++kk) {
+                    const uint32_t o = (uint32_t)(kk >> 2) * (kPanelBytes >> 4) + (uint32_t)(kk & 3) * 2u;
+                    umma_ss(tmem + x * 128, umma_desc_join(a_lo + o), umma_desc_join(b_lo + o), idescS, (acc || kk > 0) ? 1u : 0u);
+                }
+            };
+            auto s_ready = [&](int x) {       // the stream's S tile may be overwritten
+                if (SEP && ns[x] > 0) wait(F_SFREE + x, ns[x] - 1);
+                ++ns[x];
+            };
+            std::integral_constant<int, HD> kHD;
+            std::integral_constant<int, kTile> kT128;
+#pragma unroll 1
+            for (int it = 0; ok; ++it) {
+                wait(F_ITFULL + (it & 1), it >> 1);
+                if (!ok) break;
+                const int idx = item_ring[it & 1];
+                mbar_arrive(&bars[F_ITEMPTY + (it & 1)]);
+                if (idx < 0) break;
+                int k, s;
+                decode(idx, k, s);
+                const int I0 = 2 * k, I1 = 2 * k + 1;
+                const int NS[2] = {steps_of(I0, s), steps_of(I1, s)}, NV = max(NS[1], NS[0] + kOff);
+                auto level_at = [&](int n) { return CROSS ? 0 : (n == 1 ? 0 : msb32((unsigned)(I0 ^ (I1 - n)))); };
+                // first logit tile of either stream
+                if (CROSS) {
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        if (NS[x] == 0) continue;
+                        curq[x] = nq++;
+                        q_wait(curq[x]);
+                        kv_wait(nkv);
+                        s_ready(x);
+                        tc_fence_after_sync();
+                        if (!ok) break;
+                        issue_s(x, curq[x], nkv, kHD, false);
+                        umma_commit(&bars[F_SFULL + x]);
+                        if (NS[x] == 1) q_free(curq[x]);
+                    }
+                    if (ok) kv_free(nkv);
+                    ++nkv;
+                } else {
+#pragma unroll
+                    for (int x = 1; x >= 0; --x) {   // two contractions
+                        if (NS[x] == 0) continue;
+                        q_wait(nq);
+                        kv_wait(nkv);
+                        s_ready(x);
+                        tc_fence_after_sync();
+                        if (!ok) break;
+                        issue_s(x, nq, nkv, kHD, false);
+                        q_wait(nq + 1);
+                        kv_wait(nkv + 1);
+                        tc_fence_after_sync();
+                        if (!ok) break;
+                        issue_s(x, nq + 1, nkv + 1, kT128, true);
+                        umma_commit(&bars[F_SFULL + x]);
+                        q_free(nq);
+                        q_free(nq + 1);
+                        kv_free(nkv);
+                        kv_free(nkv + 1);
+                        nq += 2;
+                        nkv += 2;
+                    }
+                }
+#pragma unroll 1
+                for (int n = 0; n < NV && ok; ++n) {
+                    const bool u[2] = {n >= kOff && n - kOff < NS[0], n < NS[1]};
+                    const bool nx[2] = {u[0] && n - kOff + 1 < NS[0], n + 1 < NS[1]};
+                    const int has_v = (u[0] || u[1]) ? 1 : 0, has_k = (nx[0] || nx[1]) ? 1 : 0;
+                    const int vi = nkv + (SEP ? has_k : 0), ki = nkv + (SEP ? 0 : has_v);
+                    nkv += has_v + has_k;
+                    const bool fresh = !CROSS && (n <= 1 || level_at(n + 1) != level_at(n));
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        if (!u[x]) continue;
+                        const int t = n - (x == 0 ? kOff : 0);
+                        auto next_s = [&]() {
+                            if (!nx[x]) return;
+                            if (fresh) {
+                                curq[x] = nq++;
+                                q_wait(curq[x]);
+                            }
+                            kv_wait(ki);
+                            s_ready(x);
+                            tc_fence_after_sync();
+                            if (!ok) return;
+                            issue_s(x, curq[x], ki, kHD, false);
+                            umma_commit(&bars[F_SFULL + x]);
+                            if (t + 2 >= NS[x] || level_at(n + 2) != level_at(n + 1)) q_free(curq[x]);
+                            if (x == 1 || !nx[1]) kv_free(ki);
+                        };
+                        if (SEP) next_s();
+                        // O_x += P_x V_n; the first product of a work item overwrites O_x, which the previous item's
+                        // epilogue must have read
+                        kv_wait(vi);
+                        if (t == 0 && no[x] > 0) wait(F_OFREE + x, no[x] - 1);
+                        wait(F_PA + x, np[x]);
+                        tc_fence_after_sync();
+                        if (!ok) break;
+                        const uint32_t b_lo = umma_desc_lo(smem_u32(sKV + (vi & 3) * kSlotBytes), kPanelBytes);
+                        const uint32_t tO = tmem + 256 + x * HD, tP = tmem + colP(x);
+#pragma unroll
+                        for (int kk = 0; kk < 6; ++kk)
+                            umma_ts(tO, tP + kk * 8, umma_desc_join(b_lo + kk * 128u), idescO, (t > 0 || kk > 0) ? 1u : 0u);
+                        wait(F_PB + x, np[x]);
+                        tc_fence_after_sync();
+                        if (!ok) break;
+#pragma unroll
+                        for (int kk = 6; kk < 8; ++kk) umma_ts(tO, tP + kk * 8, umma_desc_join(b_lo + kk * 128u), idescO, 1u);
+                        ++np[x];
+                        if (SEP) umma_commit(&bars[F_PFREE + x]);
+                        if (x == 1 || !u[1]) kv_free(vi);
+                        if (t + 1 == NS[x]) {
+                            umma_commit(&bars[F_OFULL + x]);
+                            ++no[x];
+                        }
+                        if (!SEP) next_s();   // overwrites P: in-order execution puts it after the product above
+                        if (!ok) break;
+                    }
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        // ------------------------------------------------------------ softmax warpgroups, one row per thread
+        const int x = (warp - 4) >> 2;          // stream
+        const int q4 = warp & 3;                // TMEM lane quadrant this warp may touch
+        const int row = q4 * 32 + lane;
+        const uint32_t tlane = tmem + ((uint32_t)(q4 * 32) << 16);
+        const uint32_t tS = tlane + x * 128, tO = tlane + 256 + x * HD, tP = tlane + colP(x);
+        const float kLog2e = 1.4426950408889634f;
+        const float sl2 = fabsf(p.scale) * kLog2e;
+        const uint64_t sl2x2 = pack2(sl2, sl2);
+        bool ok = true;
+        int sc = 0, no = 0;                     // tiles and results of this stream so far
+#pragma unroll 1
+        for (int it = 0; ok; ++it) {
+            if (!mbar_wait(&bars[F_ITFULL + (it & 1)], (it >> 1) & 1, abort_flag, ST_FWD_SOFTMAX)) ok = false;
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            const int idx = item_ring[it & 1];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars[F_ITEMPTY + (it & 1)]);
+            if (idx < 0) break;
+            int k, s;
+            decode(idx, k, s);
+            const int I = 2 * k + x, T = steps_of(I, s);
+            if (T == 0) continue;
+            const int qi = I * kTile + row;     // position within the slice (may be >= L in the ragged tail)
+            float gi2 = 0.f;
+            if (GATE) gi2 = p.G[(size_t)s * p.Lp + qi] * kLog2e;
+            float m = -INFINITY, l = 0.f;
+            auto step = [&](auto diag_tag, const int t) {
+                constexpr bool DIAG = decltype(diag_tag)::value;
+                const int gb = x * 2 + (sc & 1);
+                if (GATE && ok && !mbar_wait(&bars[F_GKFULL + gb], (sc >> 1) & 1, abort_flag, ST_FWD_SOFTMAX)) ok = false;
+                if (SEP && sc > 0 && ok && !mbar_wait(&bars[F_PFREE + x], (sc - 1) & 1, abort_flag, ST_FWD_SOFTMAX)) ok = false;
+                if (ok && !mbar_wait(&bars[F_SFULL + x], sc & 1, abort_flag, ST_FWD_SOFTMAX)) ok = false;
+                ok = __all_sync(0xffffffffu, ok);  // keep the warp-collective TMEM accesses convergent
+                tc_fence_after_sync();
+                ok = softmax_tile<HD, GATE, DIAG, SEP>(tS, tP, tO, row, sl2x2, sl2, gi2, sGk + gb * kTile, t > 0, m, l,
+                                                       &bars[F_SFREE + x], &bars[F_PA + x], &bars[F_PB + x], ok);
+                if (GATE && lane == 0) mbar_arrive(&bars[F_GKEMPTY + gb]);
+                ++sc;
+            };
+            int t = 0;
+            if (!CROSS) {
+                step(std::true_type{}, 0);
+                t = 1;
+            }
+#pragma unroll 1
+            for (; t < T; ++t) step(std::false_type{}, t);
+            // ---- write O, LSE
+            if (ok && !mbar_wait(&bars[F_OFULL + x], no & 1, abort_flag, ST_FWD_SOFTMAX)) ok = false;
+            ++no;
+            ok = __all_sync(0xffffffffu, ok);
+            tc_fence_after_sync();
+            if (!ok) break;
+            const float inv = 1.f / l;
+            const bool live = qi < p.L;
+            const int row0 = I * kTile + q4 * 32;
+#pragma unroll
+            for (int h = 0; h < HD / 64; ++h) {   // 64 columns at a time: one 128-byte line per row
+                uint32_t o[2][32];
+                tmem_ld32(tO + h * 64, o[0]);
+                tmem_ld32(tO + h * 64 + 32, o[1]);
+                tmem_ld_wait();
+                if (h == HD / 64 - 1) {
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bars[F_OFREE + x]);   // O may be overwritten
+                }
+                if (p.out_fp32) {
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        float v[32];
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(o[c][e]) * inv;
+                        tile::gstore_f32x32((float*)p.o + ((size_t)s * p.L + (live ? qi : 0)) * HD + h * 64 + c * 32, v, live);
+                    }
+                } else {
+                    uint32_t w[32];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int e = 0; e < 16; ++e)
+                            w[c * 16 + e] = pack_bf16(__uint_as_float(o[c][2 * e]) * inv, __uint_as_float(o[c][2 * e + 1]) * inv);
+                    warp_store_rows128((__nv_bfloat16*)p.o + ((size_t)s * p.L + row0) * HD + h * 64, (size_t)HD * 2, w, p.L - row0);
+                }
+            }
+            if (live) p.lse[(size_t)s * p.L + qi] = (m + log2f(l)) * 0.6931471805599453f;
+        }
+    }
+
+    tc_fence_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    if (warp == 1) {
+        tc_fence_after_sync();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
+static cudaError_t sm_count(int& sms) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
+template <class K>
+static cudaError_t launch_one(K kern, int grid, uint32_t smem, const FwdTensorMaps& tm, const FwdParams& p, cudaStream_t st) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, 384, smem, st>>>(tm, p);
     return cudaGetLastError();
+}
+
+// Slices per group of the item list: what about 64 MB of keys, values and versions (half of L2) come from, but enough that
+// a group's items fill the GPU twice.
+static int slices_per_group(const FwdParams& p, int hd, int sms, int key_rows) {
+    const int np = (p.N + 1) / 2;
+    const long per_slice = (long)key_rows * hd * 2;
+    const int fit = (int)((64L << 20) / (per_slice > 0 ? per_slice : 1)), fill = (2 * sms + np - 1) / np;
+    const int g = fit > fill ? fit : fill;
+    return g < 1 ? 1 : (g > p.S ? p.S : g);
+}
+
+template <int HD>
+static cudaError_t launch_hd(const FwdTensorMaps& tm, FwdParams p, cudaStream_t st) {
+    int sms = 0;
+    cudaError_t e = sm_count(sms);
+    if (e != cudaSuccess) return e;
+    const int chunks = p.N * p.S, pairs = (p.N + 1) / 2 * p.S;
+    // Pairs that do not fill the GPU leave the time to the longest of them: then one chunk per item, dealt over both streams
+    // (S = 8 slices, L = 4096, d = 128: 52 us against 74; S = 1, L = 32768: 269 against 466).  From one pair per SM on the
+    // pairs are faster (S = 10, L = 4096: 82 against 93 us; S = 2, L = 20000: 304 against 328), and also below that where
+    // items are short and there are more chunks than SMs (S = 64, L = 512: 19 against 23 us).
+    if (pairs < sms && (chunks <= sms || p.N >= 8)) {
+        const int grid = chunks <= sms ? chunks : ((chunks + 1) / 2 < sms ? (chunks + 1) / 2 : sms);
+        return p.G ? launch_one(fa_split_kernel<HD, true>, grid, SplitSmem::alloc, tm, p, st)
+                   : launch_one(fa_split_kernel<HD, false>, grid, SplitSmem::alloc, tm, p, st);
+    }
+    p.group = slices_per_group(p, HD, sms, 2 * p.Lp + p.vl.ek * CHUNK);
+    const int grid = pairs < sms ? pairs : sms;
+    return p.G ? launch_one(fa_fwd_kernel<HD, true, false>, grid, FwdSmem::alloc, tm, p, st)
+               : launch_one(fa_fwd_kernel<HD, false, false>, grid, FwdSmem::alloc, tm, p, st);
 }
 
 cudaError_t launch_fa_fwd(const FwdTensorMaps& tm, const FwdParams& p, int hd, cudaStream_t st) {
@@ -574,18 +1057,14 @@ cudaError_t launch_fa_fwd(const FwdTensorMaps& tm, const FwdParams& p, int hd, c
 }
 
 template <int HD>
-static cudaError_t launch_cross_hd(const FwdTensorMaps& tm, const FwdParams& p, cudaStream_t st) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+static cudaError_t launch_cross_hd(const FwdTensorMaps& tm, FwdParams p, cudaStream_t st) {
+    int sms = 0;
+    const cudaError_t e = sm_count(sms);
     if (e != cudaSuccess) return e;
     if (!p.G || !p.Gk || p.Nk < 1) return cudaErrorInvalidValue;
-    const int pairs = (p.N * p.S + 1) / 2;
-    e = cudaFuncSetAttribute(fa_fwd_kernel<HD, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem::alloc);
-    if (e != cudaSuccess) return e;
-    fa_fwd_kernel<HD, true, true><<<dim3(pairs < sms ? pairs : sms), 384, FwdSmem::alloc, st>>>(tm, p);
-    return cudaGetLastError();
+    const int pairs = (p.N + 1) / 2 * p.S;
+    p.group = slices_per_group(p, HD, sms, 2 * p.Lkp);
+    return launch_one(fa_fwd_kernel<HD, true, true>, pairs < sms ? pairs : sms, FwdSmem::alloc, tm, p, st);
 }
 
 cudaError_t launch_fa_fwd_cross(const FwdTensorMaps& tm, const FwdParams& p, int hd, cudaStream_t st) {

@@ -487,6 +487,7 @@ int path_attn_fwd(const void* q, const void* k, const void* v, const void* w, co
     FwdParams fp{};
     fp.o = o; fp.lse = lse; fp.G = log_f ? at<float>(workspace, p.G) : nullptr;
     fp.status = at<uint32_t>(workspace, p.status);
+    fp.next_item = at<int>(workspace, p.status + kNextItemOffset);
     fp.S = p.S; fp.L = L; fp.Lp = p.Lp; fp.N = p.N; fp.scale = scale; fp.out_fp32 = 0; fp.vl = p.vl;
     prof_mark(STG_FA_FWD, 0, st);
     if (log_f) fp.nkeep = at<int>(workspace, p.nkeep);   // block skipping: see run_gate_skip
@@ -698,6 +699,7 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
         FwdParams fp{};
         fp.o = at<float>(state, c.o_acc); fp.lse = at<float>(state, c.lse_acc); fp.G = log_f ? at<float>(workspace, p.G) : nullptr;
         fp.status = at<uint32_t>(workspace, p.status);
+    fp.next_item = at<int>(workspace, p.status + kNextItemOffset);
         fp.S = p.S; fp.L = L; fp.Lp = p.Lp; fp.N = p.N; fp.scale = scale; fp.out_fp32 = 1; fp.vl = p.vl;
         if (log_f) fp.nkeep = at<int>(workspace, p.nkeep);
         LAUNCH(launch_fa_fwd(tm, fp, d, st));
@@ -745,6 +747,7 @@ int path_attn_cp_step(void* state, const void* message, int B, int H, int Lq, in
         fp.o = at<float>(workspace, cq.o_t); fp.lse = at<float>(workspace, cq.lse_t);
         fp.G = at<float>(state, cq.gq); fp.Gk = at<float>(msg, ck.gk);
         fp.status = (uint32_t*)workspace;
+        fp.next_item = at<int>(workspace, kNextItemOffset);
         fp.S = cq.S; fp.L = Lq; fp.Lp = cq.Lp; fp.N = cq.N; fp.Nk = ck.N; fp.Lkp = ck.Lp; fp.scale = scale; fp.out_fp32 = 1;
         LAUNCH(launch_fa_fwd_cross(tm, fp, d, st));
     }

@@ -152,6 +152,20 @@ def test_persistent_scheduling_shapes(binding, oracle, B, H, L, d, gate):
     compare_all(binding, oracle, inp)
 
 
+@pytest.mark.parametrize("B,H,L,d,gate,scale", [
+    (37, 4, 100, 64, False, 1.0),     # 148 slices of one chunk: items without a second stream
+    (37, 2, 300, 128, True, 1.0),     # 3 chunks: the last item of a slice has no second stream; gate and ragged tail
+    (10, 15, 256, 128, False, -0.5),  # 2 chunks: stream 1's level-0 step only; negative scale
+    (9, 5, 1000, 64, True, 1.0),      # 8 chunks, ragged: levels 0 .. 2, several items per CTA
+    (1, 40, 1152, 128, False, 1.0),   # 9 chunks: odd count, level 3
+])
+def test_forward_pairs_of_query_chunks(binding, oracle, B, H, L, d, gate, scale):
+    """Problems with at least as many pairs of query chunks as SMs: the sweep that takes two query chunks at a time."""
+    inp = synth.make_inputs(B, H, L, d, "bf16", gate=gate, seed=800 + L)
+    idx = [0, 1, B * H // 2, B * H - 1]
+    compare_all(binding, oracle, inp, scale=scale, idx=idx, backward=False)
+
+
 def _random_cases(n, seed=20250516):
     """Seeded list of small problems: lengths below, at and across chunk boundaries, both head sizes, gate, scale sign."""
     import random
