@@ -4,7 +4,7 @@
 // T~ = Ainv D, Ainv = (I + strictLower(D W W^T))^-1 and s = scale:
 //   dXq = lower(-dQl U^T - s dSd Y^T)            dY  = -W dKr^T - s Xq^T dSd           dU = -Xq^T dQl - W dP
 //   dT  = lower(dY Xk^T + dU W^T)                dXk = strictLower(T~^T dY)
-//   M   = Ainv^T dT,   dbeta_c  = M_cc,          dA  = strictLower(-(M D) Ainv^T)
+//   M   = Ainv^T dT,   dbeta_c  = M_cc,          dA  = strictLower(-M T~^T)       (Ainv^T = D^-1 T~^T: beta is never exactly 0 here)
 //   dbeta_r += sum_c dA_rc (W W^T)_rc,           dGm = D dA
 //   dq = dQl + s dSd K + dXq W                   dk = dKr + s dSd^T Q + dXk^T W
 //   dw = -Y dKr - U dP^T + T~^T dU + dXq^T Q + dXk K + (dGm + dGm^T) W
@@ -14,7 +14,7 @@
 // through mbarriers: the workers hand tiles over and go on (they wait for products, never for the issuer), the issuer
 // sends out first whatever does not depend on the read-out in progress, starts the next chunk's first products while
 // the current chunk's results are still leaving, and requests tiles the moment their slots are free.  dQl and dKr
-// arrive as bf16 tiles.  T~ and Ainv enter as bf16 hi + lo pairs, and so do the in-kernel intermediates dT, M D and dGm;
+// arrive as bf16 tiles.  T~ enters as a bf16 hi + lo pair, and so do the in-kernel intermediates dT, M and dGm;
 // everything else is rounded to bf16 once.  dw accumulates in tensor memory across all phases.
 #include "tileops.cuh"
 
@@ -71,8 +71,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tc_fence_after_sync();
         return ok;
     };
-    // slots: 0 U->dXq   1 dQl->T~ hi->Ainv hi->K   2 Y^T->-Xq->Xk->dT hi->tmp hi->dGm hi   3 dSd->T~ lo->dT lo->tmp lo->dSd
-    //        4 W   5 dKr->dY->dXk->dGm lo   6 dP->dU->Ainv lo->Q
+    // slots: 0 U->dXq   1 dQl->T~ hi->K   2 Y->Xq->Xk->dT hi->M hi->dGm hi   3 dSd->T~ lo->dSd
+    //        4 W   5 dKr->dY->dXk->dGm lo   6 dP->dU->dT lo->M lo->Q
     // First tiles of a chunk, in two parts: five of the seven slots are free as soon as the products that finish dq and dk
     // have retired, and these five tiles are all that the chunk's first two products read; the other two slots feed the
     // previous chunk's very last products.
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tma_tile(slot(1), &tm.dql, &bars[B_LOAD], HD, ch * kT);
         tma_tile(slot(0), &tm.u, &bars[B_LOAD], HD, ch * kT);
         tma_tile(slot(3), &tm.dsdt, &bars[B_LOAD], kT, ch * kT);   // (s dSd)^T: every use takes the transposed view
-        tma_tile(slot(2), &tm.yt, &bars[B_LOAD], kT, ch * kT);
+        tma_tile(slot(2), &tm.y, &bars[B_LOAD], kT, ch * kT);
         tma_tile(slot(6), &tm.dp, &bars[B_LOAD], HD, ch * HD);
     };
     auto first_loads_b = [&](int ch) {
@@ -100,27 +100,27 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         // the other columns; then dw = -Y dKr - U dP^T
         if (!wait(B_LOAD)) break;
         mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(1), sa(0), false);
-        mma<OP_MN, OP_MN, K8, 128>(tmem + cA, sa(3), sa(2), true);          // slot 2 holds Y^T
+        mma<OP_MN, OP_K, K8, 128>(tmem + cA, sa(3), sa(2), true);
         if (chunk != (int)blockIdx.x && !wait(B_R1)) break;                      // the previous chunk's dw has left cDW
         if (!wait(B_LOAD2)) break;
-        mma<OP_MN, OP_MN, K8, HD, true>(tmem + cDW, sa(2), sa(5), false);
+        mma<OP_K, OP_MN, K8, HD, true>(tmem + cDW, sa(2), sa(5), false);
         mma<OP_K, OP_K, KD, HD, true>(tmem + cDW, sa(0), sa(6), true);
         umma_commit(&bars[B_MMA]);
         // ---- phase 1: dY = -(W dKr^T + Xq^T s dSd) -> cA,  dU = -(Xq^T dQl + W dP) -> cB.  dU's products read no tile
         // that the workers are writing and go to their own columns: they run underneath the read-out of dXq.
         if (!wait(B_MMA)) break;
         mbar_expect_tx(&bars[B_LOAD], kTileB);
-        tma_tile(slot(2), &tm.xqn, &bars[B_LOAD], kT, r0);
+        tma_tile(slot(2), &tm.xq, &bars[B_LOAD], kT, r0);
         mma<OP_K, OP_MN, KD, HD>(tmem + cB, sa(4), sa(6), false);           // W dP needs no new tile
         if (!wait(B_LOAD)) break;
-        mma<OP_MN, OP_MN, K8, HD, true>(tmem + cB, sa(2), sa(1), true);     // slot 2 holds -Xq: negated back
+        mma<OP_MN, OP_MN, K8, HD>(tmem + cB, sa(2), sa(1), true);
         if (!wait(B_R0)) break;                                                  // dXq has left cA
         mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(4), sa(5), false);
-        mma<OP_MN, OP_K, K8, 128, true>(tmem + cA, sa(2), sa(3), true);
+        mma<OP_MN, OP_K, K8, 128>(tmem + cA, sa(2), sa(3), true);
         umma_commit(&bars[B_MMA]);
         // ---- phase 2: dT = lower(dY Xk^T + dU W^T) -> cA, and phase 3 right behind it (the same dY and dU tiles and T~):
         // dXk = strictLower(T~^T dY) -> cB,  dw += T~^T dU.  (s dSd)^T is not needed again before phase 5, where it is
-        // loaded once more: until then its slot (3) takes the lo parts of the bf16 pairs.
+        // loaded once more: until then its slot (3) holds T~ lo.
         if (!wait(B_MMA)) break;
         mbar_expect_tx(&bars[B_LOAD], 3 * kTileB);
         tma_tile(slot(2), &tm.xk, &bars[B_LOAD], kT, r0);
@@ -136,27 +136,23 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(1), sa(6), true);
         mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(3), sa(6), true);
         umma_commit(&bars[B_MMA2]);
-        // ---- phase 4: M = Ainv^T dT -> cG;  tmp = M D;  dA = strictLower(-tmp Ainv^T) -> cA;  W W^T -> cB (for dbeta)
+        // ---- phase 4: D M = T~^T dT -> cG;  dA = strictLower(-M T~^T) -> cA;  W W^T -> cB (for dbeta).  T~ is still there.
         if (!wait(B_MMA) || !wait(B_MMA2)) break;
-        mbar_expect_tx(&bars[B_LOAD], 2 * kTileB);
-        tma_tile(slot(1), &tm.ah, &bars[B_LOAD], kT, r0);
-        tma_tile(slot(6), &tm.al, &bars[B_LOAD], kT, r0);
-        if (!wait(B_LOAD)) break;
         if (!wait(B_R0)) break;                                                  // dT hi, lo tiles
         mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(1), sa(2), false);
-        mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(6), sa(2), true);
-        mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(1), sa(3), true);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(3), sa(2), true);
+        mma<OP_MN, OP_MN, K8, 128>(tmem + cG, sa(1), sa(6), true);
         umma_commit(&bars[B_MMA]);
         if (!wait(B_R1)) break;                                                  // dXk has left cB
         mma<OP_K, OP_K, KD, 128>(tmem + cB, sa(4), sa(4), false);          // retires with the next group
         if (!wait(B_MMA)) break;
-        if (!wait(B_R0)) break;                                                  // tmp hi, lo tiles
+        if (!wait(B_R0)) break;                                                  // M hi, lo tiles
         mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(2), sa(1), false);
-        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(2), sa(6), true);
-        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(3), sa(1), true);
+        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(2), sa(3), true);
+        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(6), sa(1), true);
         umma_commit(&bars[B_MMA]);
-        // ---- phase 5: dq -> cB, dk -> cG and the rest of dw, in three groups.  K and Q replace Ainv hi / lo, (s dSd)^T
-        // returns.  First the products that need neither dGm nor the columns that dbeta still reads; when they have
+        // ---- phase 5: dq -> cB, dk -> cG and the rest of dw, in three groups.  K, (s dSd)^T and Q replace T~ and M
+        // lo.  First the products that need neither dGm nor the columns that dbeta still reads; when they have
         // retired, dXk's slot is free for dGm lo.  The second group finishes dq and dk, the third (dGm lo) only dw.
         if (!wait(B_MMA)) break;
         mbar_expect_tx(&bars[B_LOAD], 2 * kT * HD * 2 + kTileB);
@@ -270,7 +266,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         }
     };
     auto f_dT = [&](float x, int col) { return col <= row ? x : 0.f; };
-    auto f_tmp = [&](float x, int col) { return x * bt[col]; };
+    float inv_b = 0.f;   // 1 / beta of this thread's row
+    auto f_M = [&](float x, int col) { return x * inv_b; };
     auto f_dGm = [&](float x, int col) { return col < row ? -bt[row] * x : 0.f; };
 
 #pragma unroll 1
@@ -278,7 +275,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         const int s_idx = chunk / p.N, pos = (chunk % p.N) * kT + row;   // slice and position of this thread's row
         const bool row_valid = pos < p.L;
         const size_t urow = (size_t)s_idx * p.L + pos;                   // row in the caller's [S][L][.] tensors
-        if (tid < kT) bt[tid] = p.beta[(size_t)chunk * kT + tid];   // first read after several barriers (phase 4)
+        if (tid < kT) bt[tid] = beta_floor(p.beta[(size_t)chunk * kT + tid]);   // first read after several barriers (phase 4)
         mma_wait();                                                 // phase 0
         if (!ok) break;
         acc_to_tile(cA, kT, slot(0), -1.f, M_LOWER);                // dXq (over U)
@@ -290,27 +287,28 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         publish(B_R1);
         mma_wait();                                                 // phase 2
         if (!ok) break;
-        // dT stays in tensor memory (cA); its bf16 hi part goes over Xk now, the lo part follows once T~ lo has been read
+        // dT stays in tensor memory (cA); its bf16 hi part goes over Xk now, the lo part follows once dU has been read
         split_to_tile(cA, slot(2), false, f_dT);
         mma_wait(B_MMA2);                                           // phase 3
         if (!ok) break;
-        split_to_tile(cA, slot(3), true, f_dT);                     // dT lo (over T~ lo)
+        split_to_tile(cA, slot(6), true, f_dT);                     // dT lo (over dU)
         publish(B_R0);
         // dXk leaves its columns while M is being computed; W W^T takes them over as soon as it has
         acc_to_tile(cB, kT, slot(5), 1.f, M_STRICT);                // dXk (over dY)
         publish(B_R1);
-        mma_wait();                                                 // M
+        mma_wait();                                                 // D M
         if (!ok) break;
+        inv_b = 1.f / bt[row];
         {   // diagonal of M -> t1 (dbeta's column part)
             const int c0 = (row >> 5) << 5;
             if ((c0 >> 6) == half) {
                 tmem_row32(tl + cG + c0, v);
 #pragma unroll
                 for (int x = 0; x < 32; ++x)
-                    if (c0 + x == row) t1[row] = v[x];
+                    if (c0 + x == row) t1[row] = v[x] * inv_b;
             }
         }
-        split_both(cG, slot(2), slot(3), f_tmp);                    // tmp = M D, hi (over dT hi) and lo (over dT lo)
+        split_both(cG, slot(2), slot(6), f_M);                      // M, hi (over dT hi) and lo (over dT lo)
         publish(B_R0);
         mma_wait();                                                 // dA and W W^T
         if (!ok) break;

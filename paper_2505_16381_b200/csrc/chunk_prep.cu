@@ -3,23 +3,29 @@
 //
 // With W, Q, K the rows of one 128-token chunk and D = diag(beta):
 //   Gm = W W^T,  Xq = lower(Q W^T),  Xk = strictLower(W K^T)
-//   T~ = (I + strictLower(D Gm))^-1 D        (float32 blocked substitution up to 64-row blocks; the last merge level is two
-//                                             64 x 64 x 64 products of bf16 pairs on the tensor cores)
+//   T~ = (I + strictLower(D Gm))^-1 D        (16 x 16 blocks by float32 substitution, merged by warp-level products: tri_inverse)
 //   U = T~ W,  Y = T~ Xk
 //   Qleft = Q - Xq U,  Kright = K - Y^T W,  P = I - W^T U
-// and the bf16 operands of the diagonal-chunk correction of the attention sweep, Xqn = -Xq and Yt = Y^T.
+// Xq and Y are also the bf16 operands of the diagonal-chunk correction -Xq Y of the attention sweep.
 //
-// Every product is a 128 x 128 x {64,128} tcgen05 MMA whose operands sit in shared memory as row-major
+// The products are 128 x 128 x {64,128} tcgen05 MMAs whose operands sit in shared memory as row-major
 // 128-byte-swizzled tiles; whether a tile enters as X, X^T, on the left or on the right is only a matter of
 // the descriptor's major-ness, so nothing is ever transposed in memory.  Accumulators live in tensor memory and
 // are read back one row per thread.  T~ is kept as a bf16 pair (hi + lo) because everything downstream
 // depends on it; the other intermediates are rounded to bf16 once, like the tiles the attention sweep consumes.
 //
 // The kernel is persistent: one CTA per SM walks over chunks.  Eight worker warps do the element-wise work (the
-// triangular inverse, accumulator read-outs, conversions, global stores); a ninth warp's first lane issues the TMA
-// loads and every product as soon as its operands are published, so the products run underneath the workers'
-// next phase and the first product of the next chunk is already finished when the workers get there.
-#include <type_traits>
+// triangular inverse, accumulator read-outs, conversions); one lane of a ninth warp issues the TMA loads and stores and
+// every product as soon as its operands are published, so the products run underneath the workers' next phase and the
+// first product of the next chunk is already finished when the workers get there.  Every result leaves by a TMA store from
+// the tile that the workers have written anyway (or write for that): no worker touches global memory but for beta.
+//
+// What bounds it: the chain of dependent phases of one chunk (its seven tiles and four accumulators fill the SM, so there is
+// one chunk per SM at a time) and, in the backward's instance, bursts of stores: 416 KB per chunk against about 23 bytes per
+// cycle and SM of memory bandwidth.  Cycles per chunk at B=4, H=16, L=4096, d=128 (backward's instance) / 32 x 32768 x 128
+// (forward's): 27.2 k / 23.6 k, of which the inverse 8 k, 116 product steps 7.5 k (mostly underneath), E1 1.9 k, Xk and Xq
+// 3 k, U and Y 1.8 k, P, Q<- and K-> 3.9 k, the rest waits.  With the inverse in float32 loops plus one tcgen05 level and
+// rows stored and fetched by the workers: 43.5 k / 33.9 k.  Time 352 -> 225 us and 1240 -> 870 us; 128 x 2048 x 64: 278 -> 187.
 #include "tileops.cuh"
 
 namespace path {
@@ -28,26 +34,21 @@ using namespace tc5;
 namespace {
 
 using namespace tile;
-constexpr int kLd = kT + 4;  // row stride of the float32 triangular buffer (rows stay 16-byte aligned)
-constexpr uint32_t kInvTileB = 8192;   // a [64 x 64] bf16 operand tile of the inverse's last merge level
 
-// Seven 32 KB tile slots.  0: W.  1, 2: Q, K -> operands of the inverse's last merge level -> T~ hi, lo -> U hi, lo.  3..6: float32 triangular buffer and its
-// scratch -> Xq hi, lo, Xk hi, lo -> (5, 6) Y hi, lo.
+// Seven 32 KB tile slots.  0: W.  1, 2: N hi, lo -> (I + N)^-1 -> T~ -> U -> Q, K once more.  3: K -> Xq hi -> P lo.
+// 4: Q -> Xq lo -> P hi.  5: Xk hi -> Y hi -> Q<-.  6: Xk lo -> Y lo -> K->.  The four results of a chunk wait in slots 3 - 6
+// for their TMA stores to read them while the next chunk's triangular inverse runs in slots 1, 2 and in registers; its Q and K
+// arrive meanwhile.
 struct PrepSmem {
-    static constexpr uint32_t offW = 0;
-    static constexpr uint32_t offQK = kTileB;
-    static constexpr uint32_t offBig = 3 * kTileB;
-    static constexpr uint32_t offDiag = offBig + ((kT * kLd * 4 + 1023) / 1024) * 1024;   // [64][64] float scratch
     static constexpr uint32_t offBar = 7 * kTileB;
     static constexpr uint32_t offBeta = offBar + 256;                                      // [128] float
     static constexpr uint32_t total = offBeta + kT * 4;
     static constexpr uint32_t alloc = total + 1024;
-    static_assert(offDiag + 64 * 64 * 4 <= offBar, "scratch must fit in the tile slots it aliases");
 };
 
 // mbarriers.  Issuer -> workers: one per group of products (and the TMA load, which only the issuer waits for).
 // Workers -> issuer (256 arrivals): operands published / accumulators drained.  Each completes once per chunk.
-enum { B_LOAD = 0, B_GM, B_XQK, B_M1, B_M2, B_U, B_Y, B_G3A, B_G3B, R_TT, R_M1, R_M2, R_XK, R_U, R_Y, R_E3, B_COUNT };
+enum { B_LOAD = 0, B_LOADQK, B_GM, B_XQK, B_U, B_Y, B_G3A, B_G3B, B_ST, B_LOADR, R_TT, R_XK, R_XQ, R_U, R_Y, R_P, R_E3, B_COUNT };
 constexpr int kWorkers = 256, kThreads = 384;   // warps 8..11: the issuer's warpgroup (one active lane)
 
 // Barriers over the eight worker warps.  bar.sync / bar.red are warp-aligned instructions: a warp whose lanes left a
@@ -70,6 +71,190 @@ __device__ __forceinline__ bool wsync_and(bool ok) {   // barrier over the worke
     return r != 0;
 }
 
+// ------------------------------------------------------------------------------------------------ triangular inverse
+// In place on a [128 x 128] matrix held as a bf16 pair of swizzled tiles (aH, aL):  N strictly lower -> T~ = (I + N)^-1 D.
+// 16 x 16 diagonal blocks by float32 forward substitution (`dblk`: the blocks [8][16][16] in float32), then three merge
+// levels  [[A,0],[C,B]]^-1 = [[A^-1,0],[-B^-1 C A^-1, B^-1]]  of 16-, 32- and 64-row blocks as warp-level products
+// (mma.sync m16n8k16, bf16 pairs, lo x lo left out: the precision T~ is kept in afterwards).  A warp owns a 16-row strip of
+// B^-1 C: its accumulators are the A fragments of the second product, so nothing goes through memory in between.
+// Why not tcgen05: its smallest tile has 64 rows and every product costs a round trip through tensor memory, a shared
+// memory tile and two hand-overs (about 1500 cycles each, measured); here the blocks are 16 to 64 rows and dependent.
+// 8 thousand cycles for the whole inverse (substitution 2.0, merges 0.6, 1.2, 2.9, scaling 1.0); float32 loops up to 64 rows
+// plus one tcgen05 level took 14 thousand.
+__device__ __forceinline__ uint32_t frag_addr(uint32_t tile_, int r0, int c0, int lane) {
+    const int rr = r0 + (lane & 15), c = c0 + (lane >> 4) * 8;
+    return tile_ + (uint32_t)(c >> 6) * kPanelB + sw128_off((uint32_t)rr, (uint32_t)((c & 63) >> 3));
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&f)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&f)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// d[16 x 16] += (ah + al) (bh + bl) without al bl
+__device__ __forceinline__ void mma_pair(float (&d)[2][4], const uint32_t (&ah)[4], const uint32_t (&al)[4], const uint32_t (&bh)[4],
+                                         const uint32_t (&bl)[4]) {
+#pragma unroll
+    for (int n = 0; n < 2; ++n) mma16816(d[n], ah, bh[2 * n], bh[2 * n + 1]);
+#pragma unroll
+    for (int n = 0; n < 2; ++n) mma16816(d[n], ah, bl[2 * n], bl[2 * n + 1]);
+#pragma unroll
+    for (int n = 0; n < 2; ++n) mma16816(d[n], al, bh[2 * n], bh[2 * n + 1]);
+}
+__device__ __forceinline__ uint32_t split_pair(float a, float b, uint32_t& l) {   // packed hi, l = packed lo
+    const uint32_t h = pack_bf16(a, b);
+    l = pack_bf16(a - __uint_as_float(h << 16), b - __uint_as_float(h & 0xffff0000u));
+    return h;
+}
+// One merge level of blocks of NBK 16-row strips.  The two warps that share a scheduler (w, w + 4) take a long and a short
+// strip (B^-1 is lower triangular: strip rb needs its first rb + 1 blocks).  The last level's result is scaled by D.
+template <int NBK>
+__device__ __forceinline__ void merge_level(uint8_t* aH, uint8_t* aL, const float* bt, int warp, int lane) {
+    constexpr int CBN = NBK == 4 ? 2 : 1;   // 16-column blocks of the result per warp
+    const uint32_t tH = smem_u32(aH), tL = smem_u32(aL);
+    const int hw = warp >> 2, w4 = warp & 3;
+    const int pair = NBK == 1 ? w4 : (NBK == 2 ? (w4 & 1) : 0);
+    const int rb = NBK == 1 ? 0 : (NBK == 2 ? ((w4 >> 1) ^ hw) : (hw ? 3 - w4 : w4));
+    const int cb0 = NBK == 1 ? 0 : hw * CBN;
+    const int base_a = pair * 2 * NBK * 16, base_b = base_a + NBK * 16, row0 = base_b + rb * 16;
+    const bool active = NBK > 1 || hw == 0;
+    float m[CBN][2][4];
+    if (active) {
+        float p1[NBK][2][4];
+#pragma unroll
+        for (int k = 0; k < NBK; ++k)
+#pragma unroll
+            for (int x = 0; x < 8; ++x) p1[k][x >> 2][x & 3] = 0.f;
+#pragma unroll
+        for (int k = 0; k < CBN; ++k)
+#pragma unroll
+            for (int x = 0; x < 8; ++x) m[k][x >> 2][x & 3] = 0.f;
+#pragma unroll 1
+        for (int j = 0; j <= rb; ++j) {
+            uint32_t ah[4], al[4];
+            ldsm4(ah, frag_addr(tH, row0, base_b + j * 16, lane));
+            ldsm4(al, frag_addr(tL, row0, base_b + j * 16, lane));
+#pragma unroll
+            for (int kb = 0; kb < NBK; ++kb) {
+                if (kb < cb0) continue;       // A^-1 is lower triangular: columns cb0.. need no earlier block
+                uint32_t bh[4], bl[4];
+                ldsm4t(bh, frag_addr(tH, base_b + j * 16, base_a + kb * 16, lane));
+                ldsm4t(bl, frag_addr(tL, base_b + j * 16, base_a + kb * 16, lane));
+                mma_pair(p1[kb], ah, al, bh, bl);
+            }
+        }
+#pragma unroll
+        for (int kb = 0; kb < NBK; ++kb) {
+            if (kb < cb0) continue;
+            uint32_t ah[4], al[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) ah[x] = split_pair(p1[kb][x >> 1][(x & 1) * 2], p1[kb][x >> 1][(x & 1) * 2 + 1], al[x]);
+#pragma unroll
+            for (int i = 0; i < CBN; ++i) {
+                if (kb < cb0 + i) continue;
+                uint32_t bh[4], bl[4];
+                ldsm4t(bh, frag_addr(tH, base_a + kb * 16, base_a + (cb0 + i) * 16, lane));
+                ldsm4t(bl, frag_addr(tL, base_a + kb * 16, base_a + (cb0 + i) * 16, lane));
+                mma_pair(m[i], ah, al, bh, bl);
+            }
+        }
+    }
+    if (NBK > 1) wsync();   // the other strips of the pair read C as well
+    else __syncwarp();
+    if (active) {
+#pragma unroll
+        for (int i = 0; i < CBN; ++i)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const int col = base_a + (cb0 + i) * 16 + n * 8 + 2 * (lane & 3);
+                const float s0 = NBK == 4 ? -bt[col] : -1.f, s1 = NBK == 4 ? -bt[col + 1] : -1.f;
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const int rr = row0 + (lane >> 2) + 8 * y;
+                    uint32_t l;
+                    const uint32_t h = split_pair(s0 * m[i][n][2 * y], s1 * m[i][n][2 * y + 1], l);
+                    const uint32_t off = (uint32_t)(col >> 6) * kPanelB + sw128_off((uint32_t)rr, (uint32_t)((col & 63) >> 3)) + (col & 7) * 2;
+                    *reinterpret_cast<uint32_t*>(aH + off) = h;
+                    *reinterpret_cast<uint32_t*>(aL + off) = l;
+                }
+            }
+    }
+}
+__device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const float* dblk, const float* bt, int warp, int lane, int row,
+                                            int half) {
+    {   // diagonal block `warp`: lane j (and its copy j + 16, which stores the lo parts) keeps column j in registers
+        const float* Lb = dblk + warp * 256;
+        const int o = warp * 16, j = lane & 15;
+        float x[16];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {   // four rows at a time: their loads are issued together, ahead of the dependent sums
+            float4 f[4][4];
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+#pragma unroll
+                for (int c = 0; c <= g; ++c) f[y][c] = *reinterpret_cast<const float4*>(Lb + (4 * g + y) * 16 + 4 * c);
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int rr = 4 * g + y;
+                float acc[4] = {rr == j ? 1.f : 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int c = 0; c < g; ++c) {
+                    acc[0] -= f[y][c].x * x[4 * c];
+                    acc[1] -= f[y][c].y * x[4 * c + 1];
+                    acc[2] -= f[y][c].z * x[4 * c + 2];
+                    acc[3] -= f[y][c].w * x[4 * c + 3];
+                }
+                float a = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                if (y > 0) a -= f[y][g].x * x[4 * g];
+                if (y > 1) a -= f[y][g].y * x[4 * g + 1];
+                if (y > 2) a -= f[y][g].z * x[4 * g + 2];
+                x[rr] = rr >= j ? a : 0.f;
+            }
+        }
+        uint8_t* t_ = (lane < 16 ? aH : aL) + (o >> 6) * kPanelB + ((o + j) & 7) * 2;
+#pragma unroll
+        for (int rr = 0; rr < 16; ++rr) {
+            const __nv_bfloat16 h = __float2bfloat16_rn(x[rr]);
+            *reinterpret_cast<__nv_bfloat16*>(t_ + sw128_off((uint32_t)(o + rr), (uint32_t)(((o + j) & 63) >> 3))) =
+                lane < 16 ? h : __float2bfloat16_rn(x[rr] - __bfloat162float(h));
+        }
+    }
+    wsync();
+    merge_level<1>(aH, aL, bt, warp, lane);
+    wsync();
+    merge_level<2>(aH, aL, bt, warp, lane);
+    wsync();
+    merge_level<4>(aH, aL, bt, warp, lane);   // (from its barrier on nobody reads the diagonal blocks any more)
+    {   // the 64 x 64 diagonal blocks are scaled by D; the corner that held the float32 blocks becomes zero
+        const int cb = row & 64;
+        uint8_t* ph = aH + (cb >> 6) * kPanelB;
+        uint8_t* pl = aL + (cb >> 6) * kPanelB;
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+            const uint32_t off = sw128_off((uint32_t)row, (uint32_t)(half * 4 + ch));
+            const uint4 h4 = *reinterpret_cast<const uint4*>(ph + off), l4 = *reinterpret_cast<const uint4*>(pl + off);
+            const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
+            uint32_t ho[4], lo[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const float2 b2 = *reinterpret_cast<const float2*>(bt + cb + half * 32 + ch * 8 + 2 * x);
+                ho[x] = split_pair((__uint_as_float(hw[x] << 16) + __uint_as_float(lw[x] << 16)) * b2.x,
+                                   (__uint_as_float(hw[x] & 0xffff0000u) + __uint_as_float(lw[x] & 0xffff0000u)) * b2.y, lo[x]);
+            }
+            *reinterpret_cast<uint4*>(ph + off) = make_uint4(ho[0], ho[1], ho[2], ho[3]);
+            *reinterpret_cast<uint4*>(pl + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            if (row < 64) *reinterpret_cast<uint4*>(aH + kPanelB + off) = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+}
+
 // MODE: PREP_FWD = everything the forward needs; PREP_SAVE = also keeps the tiles of the chain rule (the backward's instance);
 // PREP_KEYS = the key side only (prompt key cache: Kright and the chunk products; no query is involved, so Xq, Xq U,
 // Qleft and the diagonal-correction operands are left out and q is not even loaded).
@@ -79,11 +264,8 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
     constexpr bool SAVE = MODE == PREP_SAVE, KEYS = MODE == PREP_KEYS;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* sW = smem + PrepSmem::offW;
-    uint8_t* sQK = smem + PrepSmem::offQK;
-    uint8_t* sBig = smem + PrepSmem::offBig;
-    float* Xb = (float*)sBig;
-    float* diagX = (float*)(smem + PrepSmem::offDiag);
+    auto slot = [&](int i) { return smem + i * kTileB; };
+    uint8_t* sW = slot(0);
     float* bt = (float*)(smem + PrepSmem::offBeta);
     uint64_t* bars = (uint64_t*)(smem + PrepSmem::offBar);
     uint32_t* tmem_slot = (uint32_t*)(bars + B_COUNT);
@@ -99,7 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, 512);
-    if (tid < kT && (int)blockIdx.x < nchunks) bt[tid] = p.beta[(size_t)blockIdx.x * kT + tid];
+    if (tid < kT && (int)blockIdx.x < nchunks) bt[tid] = beta_floor(p.beta[(size_t)blockIdx.x * kT + tid]);
     if (HD == 64) {  // second panel of W must read as zeros when W^T is used with M = 128
         for (int i = tid; i < (int)(kPanelB / 16); i += kThreads) reinterpret_cast<uint4*>(sW + kPanelB)[i] = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
@@ -109,121 +291,144 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t aW_ = smem_u32(sW), aQ_ = smem_u32(sQK), aK_ = smem_u32(sQK + kTileB), aBig_ = smem_u32(sBig);
+    const uint32_t base_ = smem_u32(smem);
     constexpr int KS = HD / 16;  // k-steps over the head dimension
-    // tensor-memory columns:  0: Gm -> the inverse's last merge level (0: C A^-1, 64: B^-1 C A^-1) -> U   128: Xq -> W^T U
-    //                         256: Xk -> Xq U   384: Y -> Y^T W
+    // tensor-memory columns:  0: Gm -> U   128: Xq -> W^T U   256: Xk -> Xq U   384: Y -> Y^T W
 
     if (warp >= kWorkers / 32) {
         // ------------------------------------------------------------------ issuer
         asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
         if (warp == kWorkers / 32 && elect_one()) {
             auto wait = [&](int b, uint32_t par) { return mbar_wait(&bars[b], par, abort_flag, ST_PREP); };
-            auto load = [&](int chunk) {
-                mbar_expect_tx(&bars[B_LOAD], (KEYS ? 2 : 3) * kT * HD * 2);
-                for (int h = 0; h < HD / 64; ++h) {
-                    tma_load_2d(sW + h * kPanelB, &tm.w, &bars[B_LOAD], h * 64, chunk * kT);
-                    if (!KEYS) tma_load_2d(sQK + h * kPanelB, &tm.q, &bars[B_LOAD], h * 64, chunk * kT);
-                    tma_load_2d(sQK + kTileB + h * kPanelB, &tm.k, &bars[B_LOAD], h * 64, chunk * kT);
-                }
+            auto fetch = [&](const CUtensorMap* m, int i, int b, int chunk_) {
+                for (int h = 0; h < HD / 64; ++h) tma_load_2d(slot(i) + h * kPanelB, m, &bars[b], h * 64, chunk_ * kT);
             };
-            auto store = [&](const CUtensorMap* m, const uint8_t* tile_, int ncols, int chunk_) {
-                for (int h = 0; h < ncols / 64; ++h) tma_store_2d(m, tile_ + h * kPanelB, h * 64, chunk_ * kT);
+            auto load_w = [&](int chunk_) {
+                mbar_expect_tx(&bars[B_LOAD], kT * HD * 2);
+                fetch(&tm.w, 0, B_LOAD, chunk_);
+            };
+            auto load_qk = [&](int chunk_) {
+                mbar_expect_tx(&bars[B_LOADQK], (KEYS ? 1 : 2) * kT * HD * 2);
+                if (!KEYS) fetch(&tm.q, 4, B_LOADQK, chunk_);
+                fetch(&tm.k, 3, B_LOADQK, chunk_);
+            };
+            auto store = [&](const CUtensorMap* m, int i, int ncols, int row0) {
+                for (int h = 0; h < ncols / 64; ++h) tma_store_2d(m, slot(i) + h * kPanelB, h * 64, row0);
             };
             int chunk = blockIdx.x;
             bool ok = chunk < nchunks;
             if (ok) {
-                load(chunk);
+                load_w(chunk);
+                load_qk(chunk);
                 ok = wait(B_LOAD, 0);
                 if (ok) {
                     tc_fence_after_sync();
-                    mma<OP_K, OP_K, KS, 128>(tmem + 0, aW_, aW_, false);
+                    mma<OP_K, OP_K, KS, 128>(tmem + 0, base_, base_, false);
                     umma_commit(&bars[B_GM]);
                 }
             }
             for (uint32_t it = 0; ok && chunk < nchunks; ++it, chunk += gridDim.x) {
                 const uint32_t par = it & 1;
-                // (the tile addresses are made opaque once per chunk: otherwise every descriptor of every product is
+                const int r0 = chunk * kT, next = chunk + (int)gridDim.x;
+                // (the tiles' address is made opaque once per chunk: otherwise every descriptor of every product is
                 // hoisted out of this loop and the thread's small register allotment spills)
-                uint32_t aW = aW_, aQ = aQ_, aK = aK_, aBig = aBig_;
-                asm volatile("" : "+r"(aW), "+r"(aQ), "+r"(aK), "+r"(aBig));
-                // Xq, Xk: their columns held the previous chunk's W^T U and Xq U
-                if (it > 0 && !wait(R_E3, par ^ 1)) break;
+                uint32_t a0 = base_;
+                asm volatile("" : "+r"(a0));
+                auto t = [&](int i) { return a0 + i * kTileB; };
+                // Xq, Xk: their columns' previous contents have been read (R_P, R_E3 at the end of the previous chunk)
+                if (!(ok = wait(B_LOADQK, par))) break;
                 tc_fence_after_sync();
-                if (!KEYS) mma<OP_K, OP_K, KS, 128>(tmem + 128, aQ, aW, false);
-                mma<OP_K, OP_K, KS, 128>(tmem + 256, aW, aK, false);
+                if (!KEYS) mma<OP_K, OP_K, KS, 128>(tmem + 128, t(4), t(0), false);
+                mma<OP_K, OP_K, KS, 128>(tmem + 256, t(0), t(3), false);
+                tma_store_wait_read();   // the previous chunk's Q<- and K-> tiles: Xk goes over them
                 umma_commit(&bars[B_XQK]);
-                // last merge level of the triangular inverse: T = C A^-1, then B^-1 T, as bf16 pairs (64 x 64 x 64 each; the
-                // eight 8 KB operand tiles sit in the Q / K slots, whose products have retired by then)
-                if (!wait(R_M1, par)) break;
+                // U = T~ W  (lo x lo terms are dropped everywhere).  In the backward's instance the tiles kept for the chain
+                // rule leave through TMA stores, straight from the operand slots.
+                if (!(ok = wait(R_TT, par))) break;
                 tc_fence_after_sync();
-                mma<OP_K, OP_MN, 4, 64>(tmem + 0, aQ, aQ + 2 * kInvTileB, false);
-                mma<OP_K, OP_MN, 4, 64>(tmem + 0, aQ, aQ + 3 * kInvTileB, true);
-                mma<OP_K, OP_MN, 4, 64>(tmem + 0, aQ + kInvTileB, aQ + 2 * kInvTileB, true);
-                umma_commit(&bars[B_M1]);
-                if (!wait(R_M2, par)) break;
-                tc_fence_after_sync();
-                mma<OP_K, OP_MN, 4, 64>(tmem + 64, aQ + 4 * kInvTileB, aQ + 6 * kInvTileB, false);
-                mma<OP_K, OP_MN, 4, 64>(tmem + 64, aQ + 4 * kInvTileB, aQ + 7 * kInvTileB, true);
-                mma<OP_K, OP_MN, 4, 64>(tmem + 64, aQ + 5 * kInvTileB, aQ + 6 * kInvTileB, true);
-                umma_commit(&bars[B_M2]);
-                // U = T~ W  (lo x lo terms are dropped everywhere)
-                if (!wait(R_TT, par)) break;
-                tc_fence_after_sync();
-                mma<OP_K, OP_MN, 8, HD>(tmem + 0, aQ, aW, false);
-                mma<OP_K, OP_MN, 8, HD>(tmem + 0, aK, aW, true);
-                umma_commit(&bars[B_U]);
-                if (SAVE) {   // the tiles kept for the chain rule leave through TMA stores, straight from the operand slots
-                    store(&tm.th, sQK, kT, chunk);
-                    store(&tm.tl, sQK + kTileB, kT, chunk);
-                }
-                // Y = T~ Xk
-                if (!wait(R_XK, par)) break;
-                tc_fence_after_sync();
-                if (SAVE) {   // (requested before the products are issued: the issue takes as long as the store's reads)
-                    store(&tm.xk, sBig + 2 * kTileB, kT, chunk);
+                if (SAVE) {
+                    store(&tm.th, 1, kT, r0);
+                    store(&tm.tl, 2, kT, r0);
                     tma_store_commit();
                 }
-                mma<OP_K, OP_MN, 8, 128>(tmem + 384, aQ, aBig + 2 * kTileB, false);
-                mma<OP_K, OP_MN, 8, 128>(tmem + 384, aK, aBig + 2 * kTileB, true);
-                mma<OP_K, OP_MN, 8, 128>(tmem + 384, aQ, aBig + 3 * kTileB, true);
+                mma<OP_K, OP_MN, 8, HD>(tmem + 0, t(1), t(0), false);
+                mma<OP_K, OP_MN, 8, HD>(tmem + 0, t(2), t(0), true);
+                umma_commit(&bars[B_U]);
+                // Y = T~ Xk
+                if (!(ok = wait(R_XK, par))) break;
+                tc_fence_after_sync();
+                if (SAVE) {
+                    store(&tm.xk, 5, kT, r0);
+                    tma_store_commit();
+                }
+                mma<OP_K, OP_MN, 8, 128>(tmem + 384, t(1), t(5), false);
+                mma<OP_K, OP_MN, 8, 128>(tmem + 384, t(2), t(5), true);
+                mma<OP_K, OP_MN, 8, 128>(tmem + 384, t(1), t(6), true);
                 // B_Y lets the workers overwrite T~ (with U) and Xk (with Y): the stores must have read them
                 if (SAVE) tma_store_wait_read();
                 umma_commit(&bars[B_Y]);
-                // Xq U and W^T U
-                if (!wait(R_U, par)) break;
-                tc_fence_after_sync();
                 if (!KEYS) {
-                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, aBig, aQ, false);
-                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, aBig + kTileB, aQ, true);
-                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, aBig, aK, true);
-                }
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, aW, aQ, false);
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, aW, aK, true);
-                umma_commit(&bars[B_G3A]);
-                if (SAVE) {
-                    store(&tm.u, sQK, HD, chunk);
+                    if (!(ok = wait(R_XQ, par))) break;
+                    store(&tm.xq, 3, kT, r0);
                     tma_store_commit();
                 }
-                // Y^T W
-                if (!wait(R_Y, par)) break;
+                // Xq U and W^T U
+                if (!(ok = wait(R_U, par))) break;
                 tc_fence_after_sync();
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, aBig + 2 * kTileB, aW, false);
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, aBig + 3 * kTileB, aW, true);
-                umma_commit(&bars[B_G3B]);
-                // next chunk: once this chunk's last product has retired every tile slot is free
-                const int next = chunk + (int)gridDim.x;
-                if (next < nchunks) {
-                    if (!wait(B_G3B, par)) break;
-                    if (SAVE) tma_store_wait_read();   // the U tile: the loads overwrite it
-                    load(next);
-                    if (!wait(B_LOAD, par ^ 1)) break;
-                    tc_fence_after_sync();
-                    mma<OP_K, OP_K, KS, 128>(tmem + 0, aW, aW, false);
-                    umma_commit(&bars[B_GM]);
+                tma_store_wait_read();   // Xq: the workers' next tile goes over it when this group has retired
+                if (SAVE) {
+                    store(&tm.u, 1, HD, r0);
+                    tma_store_commit();
                 }
+                if (!KEYS) {
+                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, t(3), t(1), false);
+                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, t(4), t(1), true);
+                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, t(3), t(2), true);
+                }
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, t(0), t(1), false);
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, t(0), t(2), true);
+                umma_commit(&bars[B_G3A]);
+                // Y^T W
+                if (!(ok = wait(R_Y, par))) break;
+                tc_fence_after_sync();
+                if (!KEYS) {
+                    store(&tm.y, 5, kT, r0);
+                    tma_store_commit();
+                }
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, t(5), t(0), false);
+                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, t(6), t(0), true);
+                umma_commit(&bars[B_G3B]);
+                // U's slots take the Q and K rows once more (from L2), for the sums that finish Q<- and K->
+                if (!(ok = wait(B_G3A, par))) break;
+                mbar_expect_tx(&bars[B_LOADR], (KEYS ? 1 : 2) * kT * HD * 2);
+                fetch(&tm.k, 2, B_LOADR, chunk);
+                tma_store_wait_read();
+                mbar_arrive(&bars[B_ST]);
+                if (!KEYS) fetch(&tm.q, 1, B_LOADR, chunk);
+                // W's slot is free once this chunk's last product has retired: the next chunk's Gram matrix is ready before
+                // the workers have written the last results of this one
+                if (next < nchunks) {
+                    if (!(ok = wait(B_G3B, par))) break;
+                    load_w(next);
+                }
+                if (!(ok = wait(R_P, par))) break;
+                store(&tm.ph, 4, HD, chunk * HD);
+                store(&tm.pl, 3, HD, chunk * HD);
+                tma_store_commit();
+                if (next < nchunks) {
+                    if (!(ok = wait(B_LOAD, par ^ 1))) break;
+                    tc_fence_after_sync();
+                    mma<OP_K, OP_K, KS, 128>(tmem + 0, t(0), t(0), false);
+                    umma_commit(&bars[B_GM]);
+                    tma_store_wait_read();
+                    load_qk(next);
+                }
+                if (!(ok = wait(R_E3, par))) break;
+                if (!KEYS) store(&tm.ql, 5, HD, r0);
+                store(&tm.kr, 6, HD, r0);
+                tma_store_commit();
             }
-            if (SAVE) tma_store_wait_all();
+            tma_store_wait_all();
         }
         __syncwarp();
     } else {
@@ -235,8 +440,8 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         uint32_t hi[16], lo[16];
         // lane 0 of every warp waits; the vote that follows is also the barrier that releases the other lanes
         auto wwait = [&](int b, uint32_t par) {
-            bool good = true;
-            if (lane == 0) good = mbar_wait(&bars[b], par, abort_flag, ST_PREP);
+            bool good = ok;
+            if (lane == 0 && good) good = mbar_wait(&bars[b], par, abort_flag, ST_PREP);
             good = wsync_and(good);
             tc_fence_after_sync();
             return good;
@@ -244,10 +449,13 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         int chunk = blockIdx.x;
         for (uint32_t it = 0; chunk < nchunks; ++it, chunk += gridDim.x) {
             const uint32_t par = it & 1;
-            const size_t grow = (size_t)chunk * kT + row;   // global row
             if (!(ok = wwait(B_GM, par))) break;
 
-            // ---- E1: Gm -> strictLower(D Gm) in the float32 buffer
+            // ---- E1: N = strictLower(D Gm) as a bf16 pair into slots 1, 2, its 16 x 16 diagonal blocks also in float32.  The
+            // blocks borrow 8 KB of the tile's zero corner (rows 0 - 63 of its second panel).
+            uint8_t* aH = slot(1);
+            uint8_t* aL = slot(2);
+            float* dblk = (float*)(aH + kPanelB);
             for (int c = 0; c < 2; ++c) {
                 const int c0 = half * 64 + c * 32;
                 tmem_ld32(tl + 0 + c0, r);
@@ -255,172 +463,26 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                 const float b = bt[row];
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = (c0 + x < row) ? b * __uint_as_float(r[x]) : 0.f;
+                split32(v, hi, lo);
+                if (c0 < 64 || row >= 64) tile_store_w16(aH, row, c0, hi);
+                tile_store_w16(aL, row, c0, lo);
+                if ((row >> 5) == (c0 >> 5)) {
+                    float4* d = reinterpret_cast<float4*>(dblk + row * 16);
+                    const bool up = lane >= 16;
 #pragma unroll
-                for (int x = 0; x < 8; ++x)
-                    *reinterpret_cast<float4*>(Xb + row * kLd + c0 + 4 * x) = make_float4(v[4 * x], v[4 * x + 1], v[4 * x + 2], v[4 * x + 3]);
-            }
-            wsync();
-
-            // ---- (I + Nl)^-1 in place, 16-row panels
-            if (lane < 16) {   // diagonal blocks: warp w inverts block w by forward substitution, lane j keeps column j in registers
-                const int o = warp * 16, j = lane;
-                float* dx = diagX + warp * 16 * 17;
-                float x[16];
-#pragma unroll
-                for (int rr = 0; rr < 16; ++rr) {
-                    float acc = (rr == j) ? 1.f : 0.f;
-#pragma unroll
-                    for (int c = 0; c < rr; ++c) acc -= Xb[(o + rr) * kLd + o + c] * x[c];
-                    x[rr] = (rr >= j) ? acc : 0.f;
-                    dx[rr * 17 + j] = x[rr];
+                    for (int x = 0; x < 4; ++x)
+                        d[x] = make_float4(up ? v[16 + 4 * x] : v[4 * x], up ? v[17 + 4 * x] : v[4 * x + 1],
+                                           up ? v[18 + 4 * x] : v[4 * x + 2], up ? v[19 + 4 * x] : v[4 * x + 3]);
                 }
             }
             wsync();
-            for (int bi = 0; bi < kT / 16; ++bi) {   // inverted diagonal blocks into place (their upper triangles are zero)
-                const int rr = tid >> 4, k = tid & 15;
-                Xb[(bi * 16 + rr) * kLd + bi * 16 + k] = diagX[bi * 16 * 17 + rr * 17 + k];
-            }
-            wsync();
-            // Three merge levels on blocks of NB = 16, 32, 64 rows:  [[A,0],[C,B]]^-1 = [[A^-1,0],[-B^-1 C A^-1, B^-1]].
-            // Every level has 64 x NB entries of C blocks in total; each thread owns an (NB/16) x 4 tile of them.
-            // T = C A^-1 goes through the scratch area (the diagonal-block buffer is dead by now), M = -B^-1 T replaces C.
-            {
-                float* T = diagX;   // [64][64]
-                auto merge = [&](auto nb_tag) {
-                    constexpr int NB = decltype(nb_tag)::value, RT = NB / 16;
-                    const int pr = tid / (4 * NB), u = tid % (4 * NB);
-                    const int i0 = (u / (NB / 4)) * RT, j0 = (u % (NB / 4)) * 4, base = pr * 2 * NB;
-                    const float* Cp = Xb + (base + NB + i0) * kLd + base;          // rows i0.. of C
-                    float acc[RT][4];
-#pragma unroll
-                    for (int r_ = 0; r_ < RT; ++r_)
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) acc[r_][x] = 0.f;
-                    // T[i][j] = sum_k C[i][k] A^-1[k][j].  A^-1 is lower triangular with its zeros stored, so the rows k < j0
-                    // could be skipped, but a loop that starts at the lane's own j0 puts every lane of a warp on a different
-                    // row at the same time (no broadcast, bank conflicts: measured 6x slower than the full loop)
-#pragma unroll 4
-                    for (int k = 0; k < NB; ++k) {
-                        const float4 a4 = *reinterpret_cast<const float4*>(Xb + (base + k) * kLd + base + j0);
-#pragma unroll
-                        for (int r_ = 0; r_ < RT; ++r_) {
-                            const float ck = Cp[r_ * kLd + k];
-                            acc[r_][0] += ck * a4.x; acc[r_][1] += ck * a4.y; acc[r_][2] += ck * a4.z; acc[r_][3] += ck * a4.w;
-                        }
-                    }
-#pragma unroll
-                    for (int r_ = 0; r_ < RT; ++r_)
-                        *reinterpret_cast<float4*>(T + (pr * NB + i0 + r_) * 64 + j0) =
-                            make_float4(acc[r_][0], acc[r_][1], acc[r_][2], acc[r_][3]);
-                    wsync();
-                    // M[i][j] = -sum_{k <= i} B^-1[i][k] T[k][j]
-#pragma unroll
-                    for (int r_ = 0; r_ < RT; ++r_)
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) acc[r_][x] = 0.f;
-                    const float* Bp = Xb + (base + NB + i0) * kLd + base + NB;     // rows i0.. of B^-1
-                    const float* Tp = T + (pr * NB) * 64 + j0;
-#pragma unroll 4
-                    for (int k = 0; k < i0 + RT; ++k) {                            // B^-1[i][k] = 0 for k > i
-                        const float4 t4 = *reinterpret_cast<const float4*>(Tp + k * 64);
-#pragma unroll
-                        for (int r_ = 0; r_ < RT; ++r_) {
-                            const float bk = Bp[r_ * kLd + k];
-                            acc[r_][0] -= bk * t4.x; acc[r_][1] -= bk * t4.y; acc[r_][2] -= bk * t4.z; acc[r_][3] -= bk * t4.w;
-                        }
-                    }
-#pragma unroll
-                    for (int r_ = 0; r_ < RT; ++r_)
-                        *reinterpret_cast<float4*>(Xb + (base + NB + i0 + r_) * kLd + base + j0) =
-                            make_float4(acc[r_][0], acc[r_][1], acc[r_][2], acc[r_][3]);
-                    wsync();
-                };
-                merge(std::integral_constant<int, 16>{});
-                merge(std::integral_constant<int, 32>{});
-            }
-            // Last level (64-row blocks) on the tensor cores: both products are 64 x 64 x 64, which the CUDA cores take
-            // ten thousand cycles for (the triangular second product keeps only the warps with the long rows busy).  The
-            // operands go as bf16 pairs (hi hi + hi lo + lo hi), the precision T~ itself is kept in afterwards.
-            if (!(ok = wwait(B_XQK, par))) break;   // the products that read the Q and K tiles have retired
-            {
-                const int r_ = tid >> 2, seg = tid & 3;   // this thread: 16 columns of one row of C, A^-1 and B^-1
-                const float* src[3] = {Xb + (64 + r_) * kLd + seg * 16, Xb + r_ * kLd + seg * 16, Xb + (64 + r_) * kLd + 64 + seg * 16};
-#pragma unroll
-                for (int m = 0; m < 3; ++m) {
-                    uint32_t h8[8], l8[8];
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const float4 f = *reinterpret_cast<const float4*>(src[m] + 4 * x);
-                        const uint32_t a = pack_bf16(f.x, f.y), b = pack_bf16(f.z, f.w);
-                        h8[2 * x] = a;
-                        h8[2 * x + 1] = b;
-                        l8[2 * x] = pack_bf16(f.x - __uint_as_float(a << 16), f.y - __uint_as_float(a & 0xffff0000u));
-                        l8[2 * x + 1] = pack_bf16(f.z - __uint_as_float(b << 16), f.w - __uint_as_float(b & 0xffff0000u));
-                    }
-                    uint8_t* th_ = sQK + (2 * m) * kInvTileB;
-                    uint8_t* tl_ = th_ + kInvTileB;
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const uint32_t off = sw128_off((uint32_t)r_, (uint32_t)(seg * 2 + c));
-                        *reinterpret_cast<uint4*>(th_ + off) = make_uint4(h8[4 * c], h8[4 * c + 1], h8[4 * c + 2], h8[4 * c + 3]);
-                        *reinterpret_cast<uint4*>(tl_ + off) = make_uint4(l8[4 * c], l8[4 * c + 1], l8[4 * c + 2], l8[4 * c + 3]);
-                    }
-                }
-                fence_proxy_async_smem();
-                tc_fence_before_sync();
-                mbar_arrive(&bars[R_M1]);
-                if (!(ok = wwait(B_M1, par))) break;
-                if (row < 64) {   // T: rows 0..63 of the accumulator -> bf16 pair, the right-hand operand of the second product
-                    tmem_ld32(tl + 0 + half * 32, r);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(r[x]);
-                    split32(v, hi, lo);
-                    tile_store_w16(sQK + 6 * kInvTileB, row, half * 32, hi);
-                    tile_store_w16(sQK + 7 * kInvTileB, row, half * 32, lo);
-                }
-                fence_proxy_async_smem();
-                tc_fence_before_sync();
-                mbar_arrive(&bars[R_M2]);
-                if (!(ok = wwait(B_M2, par))) break;
-                if (row < 64) {   // -B^-1 T replaces C
-                    tmem_ld32(tl + 64 + half * 32, r);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int x = 0; x < 8; ++x)
-                        *reinterpret_cast<float4*>(Xb + (64 + row) * kLd + half * 32 + 4 * x) =
-                            make_float4(-__uint_as_float(r[4 * x]), -__uint_as_float(r[4 * x + 1]), -__uint_as_float(r[4 * x + 2]),
-                                        -__uint_as_float(r[4 * x + 3]));
-                }
-                tc_fence_before_sync();
-                wsync();
-            }
-
-            // ---- T~ = X D as a bf16 pair into the Q / K tiles' space
-            for (int c = 0; c < 2; ++c) {
-                const int c0 = half * 64 + c * 32;
-                float t[32];
-#pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                    const float4 f = *reinterpret_cast<const float4*>(Xb + row * kLd + c0 + 4 * x);
-                    v[4 * x] = f.x; v[4 * x + 1] = f.y; v[4 * x + 2] = f.z; v[4 * x + 3] = f.w;
-                }
-#pragma unroll
-                for (int x = 0; x < 32; ++x) t[x] = v[x] * bt[c0 + x];
-                split32(t, hi, lo);
-                tile_store_w16(sQK, row, c0, hi);
-                tile_store_w16(sQK + kTileB, row, c0, lo);
-                if (SAVE) {
-                    split32(v, hi, lo);
-                    gstore_bf16_w16(p.sAh + grow * kT + c0, hi);
-                    gstore_bf16_w16(p.sAl + grow * kT + c0, lo);
-                }
-            }
+            tri_inverse(aH, aL, dblk, bt, warp, lane, row, half);   // -> T~ = (I + N)^-1 D
             fence_proxy_async_smem();
+            tc_fence_before_sync();
             mbar_arrive(&bars[R_TT]);
-            wsync();  // everyone has read the float32 buffer; it now becomes the Xq / Xk tiles
 
-            // ---- E1b: Xk = strictLower(.) -> bf16 hi / lo tiles (slots 5, 6), then Xq = lower(.) (slots 3, 4); Xqn = -Xq -> global
+            if (!(ok = wwait(B_XQK, par))) break;
+            // ---- E1b: Xk = strictLower(.) -> bf16 hi / lo tiles (slots 5, 6), then Xq = lower(.) (slots 3, 4)
             for (int c = 0; c < 2; ++c) {
                 const int c0 = half * 64 + c * 32;
                 tmem_ld32(tl + 256 + c0, r);
@@ -428,8 +490,8 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = (c0 + x < row) ? __uint_as_float(r[x]) : 0.f;
                 split32(v, hi, lo);
-                tile_store_w16(sBig + 2 * kTileB, row, c0, hi);
-                tile_store_w16(sBig + 3 * kTileB, row, c0, lo);
+                tile_store_w16(slot(5), row, c0, hi);
+                tile_store_w16(slot(6), row, c0, lo);
             }
             fence_proxy_async_smem();
             tc_fence_before_sync();
@@ -441,15 +503,17 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = (c0 + x <= row) ? __uint_as_float(r[x]) : 0.f;
                 split32(v, hi, lo);
-                tile_store_w16(sBig, row, c0, hi);
-                tile_store_w16(sBig + kTileB, row, c0, lo);
-#pragma unroll
-                for (int x = 0; x < 16; ++x) hi[x] ^= 0x80008000u;   // -Xq
-                gstore_bf16_w16(p.Xqn + grow * kT + c0, hi);
+                tile_store_w16(slot(3), row, c0, hi);
+                tile_store_w16(slot(4), row, c0, lo);
+            }
+            if (!KEYS) {
+                fence_proxy_async_smem();
+                tc_fence_before_sync();
+                mbar_arrive(&bars[R_XQ]);
             }
 
             // ---- E2: U -> hi / lo tiles over T~ (slots 1, 2) once Y = T~ Xk has retired; Y -> hi / lo tiles over Xk
-            // (slots 5, 6); Yt = Y^T -> global
+            // (slots 5, 6)
             if (!(ok = wwait(B_U, par))) break;
             uint32_t uh[HD / 64][16], ul[HD / 64][16];
 #pragma unroll
@@ -465,13 +529,12 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
 #pragma unroll
             for (int c = 0; c < HD / 64; ++c) {
                 const int c0 = half * (HD / 2) + c * 32;
-                tile_store_w16(sQK, row, c0, uh[c]);
-                tile_store_w16(sQK + kTileB, row, c0, ul[c]);
+                tile_store_w16(slot(1), row, c0, uh[c]);
+                tile_store_w16(slot(2), row, c0, ul[c]);
             }
-            fence_proxy_async_smem();   // also covers the Xq tiles written above
+            fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&bars[R_U]);
-            uint32_t yh[2][16];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int c0 = half * 64 + c * 32;
@@ -479,98 +542,62 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                 tmem_ld_wait();
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(r[x]);
-                split32(v, yh[c], lo);
-                tile_store_w16(sBig + 2 * kTileB, row, c0, yh[c]);
-                tile_store_w16(sBig + 3 * kTileB, row, c0, lo);
+                split32(v, hi, lo);
+                tile_store_w16(slot(5), row, c0, hi);
+                tile_store_w16(slot(6), row, c0, lo);
             }
             fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&bars[R_Y]);
-            if (!KEYS) {
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    unsigned short* yt = reinterpret_cast<unsigned short*>(p.Yt) + ((size_t)chunk * kT + half * 64 + c * 32) * kT + row;
-#pragma unroll
-                    for (int x = 0; x < 16; ++x) {
-                        yt[(size_t)(2 * x) * kT] = (unsigned short)(yh[c][x] & 0xffffu);
-                        yt[(size_t)(2 * x + 1) * kT] = (unsigned short)(yh[c][x] >> 16);
-                    }
-                }
-            }
 
-            // ---- E3: Qleft = Q - Xq U, P = I - W^T U, then Kright = K - Y^T W; the q / k rows are fetched while the
-            // products run
-            // At d = 128 a thread's half row is one 128-byte line: four lanes fetch four lines together, a quarter of each per
-            // instruction (whole lines per request instead of 32 scattered pieces, which also hold up the products' operand reads)
-            uint32_t rq[4][8], rk[4][8];
-            uint4 pre_q[4], pre_k[4];
-            {
-                const __nv_bfloat16* gq = p.q + grow * HD + half * (HD / 2);
-                const __nv_bfloat16* gk = p.k + grow * HD + half * (HD / 2);
-                if (HD == 128) {
-                    if (!KEYS) gload_f32x32_issue(reinterpret_cast<const float*>(gq), rq);
-                    gload_f32x32_issue(reinterpret_cast<const float*>(gk), rk);
-                } else {
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        if (!KEYS) pre_q[x] = reinterpret_cast<const uint4*>(gq)[x];
-                        pre_k[x] = reinterpret_cast<const uint4*>(gk)[x];
-                    }
-                }
-            }
-            // in[] <- columns c * 32 .. + 31 of a fetched half row (`words`: the whole half row at d = 128, two bf16 per word)
-            auto row_part = [&](const float (&words)[32], const uint4 (&pre)[4], int c, float (&in)[32]) {
-                if (HD == 128) {
-#pragma unroll
-                    for (int x = 0; x < 16; ++x) {
-                        const uint32_t u = __float_as_uint(words[16 * c + x]);
-                        in[2 * x] = __uint_as_float(u << 16);
-                        in[2 * x + 1] = __uint_as_float(u & 0xffff0000u);
-                    }
-                } else {
-                    unpack_bf16x32(pre, in);
-                }
-            };
+            // ---- E3: P = I - W^T U, Qleft = Q - Xq U, Kright = K - Y^T W; the Q and K rows arrive in U's slots meanwhile
             const int next = chunk + (int)gridDim.x;
             float next_beta = 0.f;
             if (tid < kT && next < nchunks) next_beta = p.beta[(size_t)next * kT + tid];
             if (!(ok = wwait(B_G3A, par))) break;
-            float words[32];
-            if (HD == 128 && !KEYS) gload_f32x32_finish(rq, words);
 #pragma unroll
-            for (int c = 0; c < HD / 64; ++c) {
+            for (int c = 0; c < HD / 64; ++c) {   // P: hi over Xq lo, lo over Xq hi
                 const int c0 = half * (HD / 2) + c * 32;
-                if (!KEYS) {
-                    float in[32];
-                    tmem_ld32(tl + 256 + c0, r);
-                    tmem_ld_wait();
-                    row_part(words, pre_q, c, in);
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) v[x] = in[x] - __uint_as_float(r[x]);
-                    gstore_bf16x32(p.ql + grow * HD + c0, v);
-                }
                 tmem_ld32(tl + 128 + c0, r);
                 tmem_ld_wait();
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = ((c0 + x == row) ? 1.f : 0.f) - __uint_as_float(r[x]);
                 split32(v, hi, lo);
-                gstore_bf16_w16(p.Ph + ((size_t)chunk * HD + row) * HD + c0, hi, row < HD);
-                gstore_bf16_w16(p.Pl + ((size_t)chunk * HD + row) * HD + c0, lo, row < HD);
+                tile_store_w16(slot(4), row, c0, hi);
+                tile_store_w16(slot(3), row, c0, lo);
             }
+            fence_proxy_async_smem();
+            tc_fence_before_sync();
+            mbar_arrive(&bars[R_P]);
             if (!(ok = wwait(B_G3B, par))) break;
-            if (HD == 128) gload_f32x32_finish(rk, words);
+            // (a wait that runs out here ends everyone's loop at the next worker barrier)
+            if (!mbar_wait(&bars[B_LOADR], par, abort_flag, ST_PREP) || !mbar_wait(&bars[B_ST], par, abort_flag, ST_PREP)) ok = false;
+            if (!KEYS) {   // Qleft, over Y hi, which has been stored
 #pragma unroll
-            for (int c = 0; c < HD / 64; ++c) {
+                for (int c = 0; c < HD / 64; ++c) {
+                    const int c0 = half * (HD / 2) + c * 32;
+                    float in[32];
+                    tmem_ld32(tl + 256 + c0, r);
+                    tmem_ld_wait();
+                    tile_load32(slot(1), row, c0, in);
+#pragma unroll
+                    for (int x = 0; x < 32; ++x) v[x] = in[x] - __uint_as_float(r[x]);
+                    tile_store32(slot(5), row, c0, v);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < HD / 64; ++c) {   // Kright, over Y lo
                 const int c0 = half * (HD / 2) + c * 32;
                 float in[32];
                 tmem_ld32(tl + 384 + c0, r);
                 tmem_ld_wait();
-                row_part(words, pre_k, c, in);
+                tile_load32(slot(2), row, c0, in);
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = in[x] - __uint_as_float(r[x]);
-                gstore_bf16x32(p.kr + grow * HD + c0, v);
+                tile_store32(slot(6), row, c0, v);
             }
-            if (tid < kT) bt[tid] = next_beta;   // read again only after the next chunk's first wait (a worker barrier)
+            fence_proxy_async_smem();
+            if (tid < kT) bt[tid] = beta_floor(next_beta);   // read again only after the next chunk's first wait (a worker barrier)
             tc_fence_before_sync();
             mbar_arrive(&bars[R_E3]);
         }

@@ -105,7 +105,7 @@ __host__ __device__ inline long kver_row(const VerLayout& v, int s, int level, i
 }
 
 struct FwdTensorMaps {
-    CUtensorMap q_raw, k_raw, v, qv, kv, xqn, yt;  // qv/kv also serve as the low parts' maps in split mode
+    CUtensorMap q_raw, k_raw, v, qv, kv, xq, y;
 };
 
 struct FwdParams {
@@ -168,22 +168,16 @@ cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const Leve
 
 struct PrepTensorMaps {
     CUtensorMap w, q, k;   // [S*Lp][d] bf16, box 128 rows x 64 columns, 128-byte swizzle
-    // stores of the tiles kept for the chain rule (backward's instance only): [S*Lp][128]; u is [S*Lp][d]
+    // what the kernel leaves, all through TMA stores of its operand tiles:
+    CUtensorMap ql, kr;    // [S*Lp][d]   boundary-adjusted queries / keys (version slot 0)
+    CUtensorMap xq, y;     // [S*Lp][128] lower(Q W^T) and T~ strictLower(W K^T): the diagonal chunk's correction is -Xq Y
+    CUtensorMap ph, pl;    // [S*N*d][d]  chunk products as a bf16 hi + lo pair (level 0 of the run products), box d rows
+    // tiles kept for the chain rule (backward's instance only): T~ hi + lo, Xk rounded once, [S*Lp][128]; U rounded once, [S*Lp][d]
     CUtensorMap th, tl, xk, u;
 };
 
 struct PrepParams {
     const float* beta;            // [S*Lp] (zero in the ragged tail)
-    const __nv_bfloat16* q;       // [S*Lp][d]
-    const __nv_bfloat16* k;
-    __nv_bfloat16* ql;            // [S*Lp][d]   boundary-adjusted queries (version slot 0)
-    __nv_bfloat16* kr;            // [S*Lp][d]   boundary-adjusted keys (version slot 0)
-    __nv_bfloat16* Xqn;           // [S*Lp][128] -lower(Q W^T)
-    __nv_bfloat16* Yt;            // [S*Lp][128] (T~ strictLower(W K^T))^T
-    __nv_bfloat16 *Ph, *Pl;       // [S*N][d][d] chunk products as a bf16 hi + lo pair (level 0 of the run products)
-    // (I + N)^-1 as a bf16 hi + lo pair for the chain rule, written only by the backward's instance ([S*Lp][128]);
-    // that instance also keeps T~ (hi + lo) and Xk, U rounded once, through the tensor maps
-    __nv_bfloat16 *sAh, *sAl;
     uint32_t* status;
 };
 
@@ -194,7 +188,7 @@ cudaError_t launch_chunk_prep(const PrepTensorMaps& tm, const PrepParams& p, int
 
 struct ChainTensorMaps {
     CUtensorMap w, q, k, u;                       // [S*Lp][d]
-    CUtensorMap yt, xqn, xk, th, tl, ah, al;      // [S*Lp][128]; yt = Y^T and xqn = -Xq are the attention sweep's operands
+    CUtensorMap y, xq, xk, th, tl;                // [S*Lp][128]; y and xq are the attention sweep's operands
     CUtensorMap dsdt;                             // [S*N*128][128] bf16: (scale * lower(dS))^T of the diagonal chunks
     CUtensorMap dql, dkr;                         // [S*Lp][d] bf16 gradients of the boundary-adjusted queries / keys
     CUtensorMap dp;                               // [S*N*d][d] bf16 gradients of the chunk products
@@ -214,7 +208,7 @@ struct ChainParams {
 cudaError_t launch_chunk_chain(const ChainTensorMaps& tm, const ChainParams& p, int hd, int nchunks, cudaStream_t st);
 
 struct BwdTensorMaps {
-    CUtensorMap q_raw, k_raw, v, qv, kv, xqn, yt, d_o;
+    CUtensorMap q_raw, k_raw, v, qv, kv, xq, y, d_o;
 };
 
 struct BwdParams {

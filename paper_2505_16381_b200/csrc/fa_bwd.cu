@@ -146,8 +146,8 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
     }
     uint8_t* sK = smem;
     uint8_t* sV = sK + kSlotBytes;
-    uint8_t* sQ = sV + kSlotBytes;          // ring of 3; per item: rawQ, Xqn, then Q of step t >= 1 (entry t + 1)
-    uint8_t* sDO = sQ + 3 * kSlotBytes;     // ring of 2; per item: Yt, then dO of step t (entry t + 1)
+    uint8_t* sQ = sV + kSlotBytes;          // ring of 3; per item: rawQ, Xq, then Q of step t >= 1 (entry t + 1)
+    uint8_t* sDO = sQ + 3 * kSlotBytes;     // ring of 2; per item: Y, then dO of step t (entry t + 1)
     uint64_t* bars = (uint64_t*)(smem + 7 * kSlotBytes);
     uint32_t* tmem_slot = (uint32_t*)(bars + K_COUNT);
     volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);
@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                     }
                     if (t == 0) {
                         load_q(&tm.q_raw, HD, rowJ);
-                        load_q(&tm.xqn, kTile, rowJ);
-                        load_do(&tm.yt, kTile, rowJ);
+                        load_q(&tm.xq, kTile, rowJ);
+                        load_do(&tm.y, kTile, rowJ);
                         wait_empty(K_VEMPTY, nv);
                         if (!ok) break;
                         mbar_expect_tx(&bars[K_VFULL], kTile * HD * 2);
@@ -274,7 +274,14 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                 tc_fence_after_sync();
                 if (!ok) break;
                 mma_kk(tmem + colS, smem_u32(sK), q_addr(qb), HD, idescT, false);
-                mma_kk(tmem + colS, do_addr(db), q_addr(qb + 1), kTile, idescT, true);
+                {   // S^T -= Y^T Xq^T: Y as stored ([contraction][keys], MN-major), Xq K-major
+                    const uint32_t a_lo = umma_desc_lo(do_addr(db), kPanelBytes), b_lo = umma_desc_lo(q_addr(qb + 1), 16);
+#pragma unroll
+                    for (int kk = 0; kk < kTile / 16; ++kk)
+                        umma_ss(tmem + colS, umma_desc_join(a_lo + kk * 128u),
+                                umma_desc_join(b_lo + (uint32_t)(kk >> 2) * (kPanelBytes >> 4) + (uint32_t)(kk & 3) * 2u),
+                                umma_idesc(128, 128, 1, 0) | (1u << 13), 1u);
+                }
                 umma_commit(&bars[K_SFULL]);
                 umma_commit(&bars[K_QEMPTY + qb % 3]);         // raw q and the two correction operands are only needed here
                 umma_commit(&bars[K_QEMPTY + (qb + 1) % 3]);

@@ -2,7 +2,7 @@
 //
 // Query chunk I of one (batch, head) slice walks the key chunks J = I, I-1, ..., 0.  The diagonal chunk uses the raw q, k
 // plus the in-chunk Householder correction as a second contraction (Sec. 3.3, case i = j):
-//     S = Q K^T + (-lower(Q W^T)) (T^-1 strictLower(W K^T))           [operands q_raw,k_raw,xqn,yt]
+//     S = Q K^T - lower(Q W^T) (T~ strictLower(W K^T))                [operands q_raw, k_raw, xq, y]
 // Every earlier chunk J < I is an ordinary tile product of a query version and a key version that meet at the dyadic
 // boundary of (I, J):  S = Qv[l][I] Kv[l][J]^T, l = msb(I xor J).  The versions are prepared beforehand, so this loop
 // contains no query update.
@@ -79,6 +79,26 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+
+// S[tmem] = A B^T, both operands K-major [128][HD] tiles (descriptors advance by their low word only: 32 bytes per step, the next
+// 64-column panel after four steps).
+template <int HD>
+__device__ __forceinline__ void mma_kk(uint32_t d_tmem, uint32_t a0, uint32_t b0, uint32_t idesc) {
+    const uint32_t a_lo = umma_desc_lo(a0, 16), b_lo = umma_desc_lo(b0, 16);
+#pragma unroll
+    for (int kk = 0; kk < HD / 16; ++kk) {
+        const uint32_t o = (uint32_t)(kk >> 2) * (kPanelBytes >> 4) + (uint32_t)(kk & 3) * 2u;
+        umma_ss(d_tmem, umma_desc_join(a_lo + o), umma_desc_join(b_lo + o), idesc, kk > 0 ? 1u : 0u);
+    }
+}
+// S[tmem] += (+-) Xq Y for the diagonal chunk: Xq K-major, Y as stored ([128 contraction rows][128 keys], MN-major).
+__device__ __forceinline__ void mma_correction(uint32_t d_tmem, uint32_t xq, uint32_t y, uint32_t idesc) {
+    const uint32_t a_lo = umma_desc_lo(xq, 16), b_lo = umma_desc_lo(y, kPanelBytes);
+#pragma unroll
+    for (int kk = 0; kk < kTile / 16; ++kk)
+        umma_ss(d_tmem, umma_desc_join(a_lo + (uint32_t)(kk >> 2) * (kPanelBytes >> 4) + (uint32_t)(kk & 3) * 2u),
+                umma_desc_join(b_lo + kk * 128u), idesc, 1u);
 }
 
 // One logit tile of one stream, one query row per thread: S (tensor memory) -> P (packed bf16, tensor memory), running
@@ -300,8 +320,8 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                 // diagonal chunk: raw q, k and the correction operands (both K slots), V of chunk I
                 load_q(&tm.q_raw, HD, rowRaw);
                 load_kv(sK, B_KFULL, B_KEMPTY, 0, kf, &tm.k_raw, HD, rowRaw);
-                load_q(&tm.xqn, kTile, rowRaw);
-                load_kv(sV, B_VFULL, B_VEMPTY, 1, vf, &tm.yt, kTile, rowRaw);   // Yt borrows stream 1's V slot
+                load_q(&tm.xq, kTile, rowRaw);
+                load_kv(sV, B_VFULL, B_VEMPTY, 1, vf, &tm.y, kTile, rowRaw);   // Y borrows stream 1's V slot
                 load_kv(sV, B_VFULL, B_VEMPTY, 0, vf, &tm.v, HD, rowRaw);
                 int cur = -1;
                 for (int n = 1; n < NS && ok; ++n) {
@@ -318,21 +338,14 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
             // ------------------------------------------------------------ MMA issuer
             // a negative scale is applied as a sign flip of the logits here (negate-A bit), its magnitude in the softmax
             const uint32_t idescS = umma_idesc(128, 128, 0, 0) | (p.scale < 0.f ? (1u << 13) : 0u);
+            const uint32_t idescC = umma_idesc(128, 128, 0, 1) | (p.scale < 0.f ? 0u : (1u << 13));   // the correction is subtracted
             constexpr uint32_t idescO = umma_idesc(128, HD, 0, 1);
             bool ok = true;
             auto wait = [&](int bar, int parity) {
                 if (ok && !mbar_wait(&bars[bar], parity & 1, abort_flag, ST_FWD_MMA)) ok = false;
             };
-            auto issue_s = [&](int x, int qs, int ks, int kdim, bool acc) {   // ks >= 2: a V slot
-                // (descriptors advance by their low word only: 32 bytes per step, the next panel after four steps)
-                uint32_t a_lo = umma_desc_lo(smem_u32(sQ + qs * kSlotBytes), 16), b_lo = umma_desc_lo(smem_u32(sK + ks * kSlotBytes), 16);
-#pragma unroll
-                for (int kk = 0; kk < kdim / 16; ++kk) {
-                    umma_ss(tmem + x * 128, umma_desc_join(a_lo), umma_desc_join(b_lo), idescS, (acc || kk > 0) ? 1u : 0u);
-                    const uint32_t step = (kk & 3) == 3 ? (kPanelBytes - 96u) >> 4 : 2u;
-                    a_lo += step;
-                    b_lo += step;
-                }
+            auto issue_s = [&](int x, int qs, int ks) {
+                mma_kk<HD>(tmem + x * 128, smem_u32(sQ + qs * kSlotBytes), smem_u32(sK + ks * kSlotBytes), idescS);
             };
             int qi_next = 0;                   // query operands waited for so far (all work items)
             int released = 0;                  // query operands [0, released) have been handed back to the producer
@@ -364,16 +377,16 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                 const int q0 = take_q();
                 take_k(0);
                 tc_fence_after_sync();
-                if (ok) issue_s(0, q0 % 3, 0, HD, false);
+                if (ok) issue_s(0, q0 % 3, 0);
                 const int q1 = take_q();
                 wait(B_VFULL + 1, (int)((vc >> 1) & 1u)); vc ^= 2u;
                 tc_fence_after_sync();
                 if (!ok) break;
-                issue_s(0, q1 % 3, 3, kTile, true);
+                mma_correction(tmem, smem_u32(sQ + (q1 % 3) * kSlotBytes), smem_u32(sV + kSlotBytes), idescC);
                 umma_commit(&bars[B_SFULL + 0]);
                 umma_commit(&bars[B_KEMPTY + 0]);
                 umma_commit(&bars[B_VEMPTY + 1]);
-                release_q(q1 + 1);             // rawQ and Xqn go back once the diagonal products retire
+                release_q(q1 + 1);             // rawQ and Xq go back once the diagonal products retire
                 q_of0 = q_of1 = q1 + 1;
                 // S of step 1 (stream 1)
                 if (NS > 1) {
@@ -381,7 +394,7 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                     take_k(1);
                     tc_fence_after_sync();
                     if (!ok) break;
-                    issue_s(1, q_of1 % 3, 1, HD, false);
+                    issue_s(1, q_of1 % 3, 1);
                     umma_commit(&bars[B_SFULL + 1]);
                     umma_commit(&bars[B_KEMPTY + 1]);
                 }
@@ -420,7 +433,7 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                         take_k(x);
                         tc_fence_after_sync();
                         if (!ok) break;
-                        issue_s(x, qi % 3, x, HD, false);
+                        issue_s(x, qi % 3, x);
                         umma_commit(&bars[B_SFULL + x]);
                         umma_commit(&bars[B_KEMPTY + x]);
                         // operands older than what either stream used last can go back to the producer
@@ -739,13 +752,13 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
                     if (NS1 > 0) {   // stream 1's diagonal chunk: raw q, k and the correction operands
                         load_q(&tm.q_raw, HD, rowS + I1 * kTile);
                         load_kv(&tm.k_raw, HD, rowS + I1 * kTile);
-                        load_q(&tm.xqn, kTile, rowS + I1 * kTile);
-                        load_kv(&tm.yt, kTile, rowS + I1 * kTile);
+                        load_q(&tm.xq, kTile, rowS + I1 * kTile);
+                        load_kv(&tm.y, kTile, rowS + I1 * kTile);
                     }
                     load_q(&tm.q_raw, HD, rowS + I0 * kTile);
                     load_kv(&tm.k_raw, HD, rowS + I0 * kTile);
-                    load_q(&tm.xqn, kTile, rowS + I0 * kTile);
-                    load_kv(&tm.yt, kTile, rowS + I0 * kTile);
+                    load_q(&tm.xq, kTile, rowS + I0 * kTile);
+                    load_kv(&tm.y, kTile, rowS + I0 * kTile);
                 }
                 for (int n = 0; n < NV && ok; ++n) {
                     const bool u0 = n >= kOff && n - kOff < NS0, u1 = n < NS1;
@@ -767,6 +780,7 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
             // ------------------------------------------------------------ MMA issuer
             // a negative scale is applied as a sign flip of the logits here (negate-A bit), its magnitude in the softmax
             const uint32_t idescS = umma_idesc(128, 128, 0, 0) | (p.scale < 0.f ? (1u << 13) : 0u);
+            const uint32_t idescC = umma_idesc(128, 128, 0, 1) | (p.scale < 0.f ? 0u : (1u << 13));   // the correction is subtracted
             constexpr uint32_t idescO = umma_idesc(128, HD, 0, 1);
             bool ok = true;
             int nq = 0, nkv = 0;              // query and key / value operands used so far
@@ -779,22 +793,13 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
             auto kv_wait = [&](int i) { wait(F_KVFULL + (i & 3), i >> 2); };
             auto q_free = [&](int i) { umma_commit(&bars[F_QEMPTY + i % 3]); };
             auto kv_free = [&](int i) { umma_commit(&bars[F_KVEMPTY + (i & 3)]); };
-            auto issue_s = [&](int x, int qi, int ki, auto kdim_tag, bool acc) {
-                constexpr int KD = decltype(kdim_tag)::value;
-                // (descriptors advance by their low word only: 32 bytes per step, the next panel after four steps)
-                const uint32_t a_lo = umma_desc_lo(smem_u32(sQ + (qi % 3) * kSlotBytes), 16), b_lo = umma_desc_lo(smem_u32(sKV + (ki & 3) * kSlotBytes), 16);
-#pragma unroll
-                for (int kk = 0; kk < KD / 16; ++kk) {
-                    const uint32_t o = (uint32_t)(kk >> 2) * (kPanelBytes >> 4) + (uint32_t)(kk & 3) * 2u;
-                    umma_ss(tmem + x * 128, umma_desc_join(a_lo + o), umma_desc_join(b_lo + o), idescS, (acc || kk > 0) ? 1u : 0u);
-                }
-            };
+            auto q_addr = [&](int i) { return smem_u32(sQ + (i % 3) * kSlotBytes); };
+            auto kv_addr = [&](int i) { return smem_u32(sKV + (i & 3) * kSlotBytes); };
+            auto issue_s = [&](int x, int qi, int ki) { mma_kk<HD>(tmem + x * 128, q_addr(qi), kv_addr(ki), idescS); };
             auto s_ready = [&](int x) {       // the stream's S tile may be overwritten
                 if (SEP && ns[x] > 0) wait(F_SFREE + x, ns[x] - 1);
                 ++ns[x];
             };
-            std::integral_constant<int, HD> kHD;
-            std::integral_constant<int, kTile> kT128;
 #pragma unroll 1
             for (int it = 0; ok; ++it) {
                 wait(F_ITFULL + (it & 1), it >> 1);
@@ -818,7 +823,7 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
                         s_ready(x);
                         tc_fence_after_sync();
                         if (!ok) break;
-                        issue_s(x, curq[x], nkv, kHD, false);
+                        issue_s(x, curq[x], nkv);
                         umma_commit(&bars[F_SFULL + x]);
                         if (NS[x] == 1) q_free(curq[x]);
                     }
@@ -833,12 +838,12 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
                         s_ready(x);
                         tc_fence_after_sync();
                         if (!ok) break;
-                        issue_s(x, nq, nkv, kHD, false);
+                        issue_s(x, nq, nkv);
                         q_wait(nq + 1);
                         kv_wait(nkv + 1);
                         tc_fence_after_sync();
                         if (!ok) break;
-                        issue_s(x, nq + 1, nkv + 1, kT128, true);
+                        mma_correction(tmem + x * 128, q_addr(nq + 1), kv_addr(nkv + 1), idescC);
                         umma_commit(&bars[F_SFULL + x]);
                         q_free(nq);
                         q_free(nq + 1);
@@ -870,7 +875,7 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
                             s_ready(x);
                             tc_fence_after_sync();
                             if (!ok) return;
-                            issue_s(x, curq[x], ki, kHD, false);
+                            issue_s(x, curq[x], ki);
                             umma_commit(&bars[F_SFULL + x]);
                             if (t + 2 >= NS[x] || level_at(n + 2) != level_at(n + 1)) q_free(curq[x]);
                             if (x == 1 || !nx[1]) kv_free(ki);

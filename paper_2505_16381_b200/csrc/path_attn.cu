@@ -120,10 +120,10 @@ struct Plan {
     uint64_t rows_q, rows_k;   // rows (of d elements) of the query / key version buffers
     size_t total;
     // offsets (bytes)
-    size_t status, qp, kp, vp, wp, betap, G, tstats, nkeep, nvisit, Dyh, Dyl, Xqn, Yt, Qv16, Kv16;
+    size_t status, qp, kp, vp, wp, betap, G, tstats, nkeep, nvisit, Dyh, Dyl, Xq, Y, Qv16, Kv16;
     // backward only
     size_t dop, delta, lse2, dQv, dKv, dSd, dSdT, dG, dGrow, dGdiag, dDy;
-    size_t sTh, sTl, sAh, sAl, sXk, sU;   // bf16 tiles kept by the chunk preparation for the chain rule
+    size_t sTh, sTl, sXk, sU;   // bf16 tiles kept by the chunk preparation for the chain rule
     size_t dy_bytes, dy_mats;
 };
 
@@ -167,7 +167,6 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
     }
     const size_t keep = bwd ? 1 : 0;   // bf16 intermediates of the chunk preparation, kept for the chain rule
     p.sTh = bump(cur, keep * SNBB * 2); p.sTl = bump(cur, keep * SNBB * 2);
-    p.sAh = bump(cur, keep * SNBB * 2); p.sAl = bump(cur, keep * SNBB * 2);
     p.sXk = bump(cur, keep * SNBB * 2);
     p.sU = bump(cur, keep * SLd * 2);
     size_t dy_elems = 0;
@@ -179,8 +178,8 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
     p.Dyh = bump(cur, dy_elems * 2);
     p.Dyl = bump(cur, dy_elems * 2);
     p.dy_mats = dy_elems / ((size_t)d * d);
-    p.Xqn = bump(cur, SL * CHUNK * 2);
-    p.Yt = bump(cur, SL * CHUNK * 2);
+    p.Xq = bump(cur, SL * CHUNK * 2);
+    p.Y = bump(cur, SL * CHUNK * 2);
     p.Qv16 = bump(cur, p.rows_q * d * 2);
     p.Kv16 = bump(cur, p.rows_k * d * 2);
     p.dy_bytes = dy_elems * 2;
@@ -247,15 +246,16 @@ static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const
             g_last_cuda_error = (int)cudaErrorUnknown;
             return PATH_ERR_LAUNCH;
         }
-        typedef __nv_bfloat16 bf;
         PrepParams pp{};
         pp.beta = at<float>(ws, p.betap);
-        pp.q = (const bf*)q; pp.k = (const bf*)k;
-        pp.ql = at<bf>(ws, p.Qv16); pp.kr = at<bf>(ws, p.Kv16);
-        pp.Xqn = at<bf>(ws, p.Xqn); pp.Yt = at<bf>(ws, p.Yt);
-        pp.Ph = at<bf>(ws, p.Dyh); pp.Pl = at<bf>(ws, p.Dyl);
+        if (!(make_map(&tm.ql, at<void>(ws, p.Qv16), rows, d) && make_map(&tm.kr, at<void>(ws, p.Kv16), rows, d) &&
+              make_map(&tm.xq, at<void>(ws, p.Xq), rows, CHUNK) && make_map(&tm.y, at<void>(ws, p.Y), rows, CHUNK) &&
+              make_map_box(&tm.ph, at<void>(ws, p.Dyh), (uint64_t)nch * d, d, d) &&
+              make_map_box(&tm.pl, at<void>(ws, p.Dyl), (uint64_t)nch * d, d, d))) {
+            g_last_cuda_error = (int)cudaErrorUnknown;
+            return PATH_ERR_LAUNCH;
+        }
         if (p.bwd) {
-            pp.sAh = at<bf>(ws, p.sAh); pp.sAl = at<bf>(ws, p.sAl);
             if (!(make_map(&tm.th, at<void>(ws, p.sTh), rows, CHUNK) && make_map(&tm.tl, at<void>(ws, p.sTl), rows, CHUNK) &&
                   make_map(&tm.xk, at<void>(ws, p.sXk), rows, CHUNK) && make_map(&tm.u, at<void>(ws, p.sU), rows, d))) {
                 g_last_cuda_error = (int)cudaErrorUnknown;
@@ -326,10 +326,9 @@ static int run_chunk_chain(const Plan& p, void* ws, const void* q, const void* k
     const uint64_t rows = (uint64_t)p.S * p.Lp;
     ChainTensorMaps tm;
     bool ok = make_map(&tm.w, w, rows, d) && make_map(&tm.q, q, rows, d) && make_map(&tm.k, k, rows, d) &&
-              make_map(&tm.u, at<void>(ws, p.sU), rows, d) && make_map(&tm.yt, at<void>(ws, p.Yt), rows, CHUNK) &&
-              make_map(&tm.xqn, at<void>(ws, p.Xqn), rows, CHUNK) && make_map(&tm.xk, at<void>(ws, p.sXk), rows, CHUNK) &&
+              make_map(&tm.u, at<void>(ws, p.sU), rows, d) && make_map(&tm.y, at<void>(ws, p.Y), rows, CHUNK) &&
+              make_map(&tm.xq, at<void>(ws, p.Xq), rows, CHUNK) && make_map(&tm.xk, at<void>(ws, p.sXk), rows, CHUNK) &&
               make_map(&tm.th, at<void>(ws, p.sTh), rows, CHUNK) && make_map(&tm.tl, at<void>(ws, p.sTl), rows, CHUNK) &&
-              make_map(&tm.ah, at<void>(ws, p.sAh), rows, CHUNK) && make_map(&tm.al, at<void>(ws, p.sAl), rows, CHUNK) &&
               make_map(&tm.dsdt, at<void>(ws, p.dSdT), (uint64_t)p.S * p.N * CHUNK, CHUNK) &&
               make_map(&tm.dql, at<void>(ws, p.dQv), rows, d) && make_map(&tm.dkr, at<void>(ws, p.dKv), rows, d) &&
               make_map(&tm.dp, at<void>(ws, p.dDy), (uint64_t)p.S * p.N * d, d);   // level 0 of the run-product gradients
@@ -365,7 +364,7 @@ static int run_backward(const Plan& p, void* ws, const void* q, const void* k, c
     bool ok = make_map(&tm.q_raw, q, rows, d) && make_map(&tm.k_raw, k, rows, d) && make_map(&tm.v, v, rows, d) &&
               make_map(&tm.qv, at<void>(ws, p.Qv16), p.rows_q, d) &&
               make_map(&tm.kv, at<void>(ws, p.Kv16), p.rows_k, d) &&
-              make_map(&tm.xqn, at<void>(ws, p.Xqn), rows, CHUNK) && make_map(&tm.yt, at<void>(ws, p.Yt), rows, CHUNK) &&
+              make_map(&tm.xq, at<void>(ws, p.Xq), rows, CHUNK) && make_map(&tm.y, at<void>(ws, p.Y), rows, CHUNK) &&
               make_map(&tm.d_o, dop, rows, d);
     if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
     BwdParams bp{};
@@ -481,8 +480,8 @@ int path_attn_fwd(const void* q, const void* k, const void* v, const void* w, co
     bool ok = make_map(&tm.q_raw, q, rows, d) && make_map(&tm.k_raw, k, rows, d) && make_map(&tm.v, v, rows, d) &&
               make_map(&tm.qv, at<void>(workspace, p.Qv16), p.rows_q, d) &&
               make_map(&tm.kv, at<void>(workspace, p.Kv16), p.rows_k, d) &&
-              make_map(&tm.xqn, at<void>(workspace, p.Xqn), rows, CHUNK) &&
-              make_map(&tm.yt, at<void>(workspace, p.Yt), rows, CHUNK);
+              make_map(&tm.xq, at<void>(workspace, p.Xq), rows, CHUNK) &&
+              make_map(&tm.y, at<void>(workspace, p.Y), rows, CHUNK);
     if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
     FwdParams fp{};
     fp.o = o; fp.lse = lse; fp.G = log_f ? at<float>(workspace, p.G) : nullptr;
@@ -694,7 +693,7 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
         bool ok = make_map(&tm.q_raw, q, rows, d) && make_map(&tm.k_raw, k, rows, d) && make_map(&tm.v, v, rows, d) &&
                   make_map(&tm.qv, at<void>(workspace, p.Qv16), p.rows_q, d) &&
                   make_map(&tm.kv, at<void>(workspace, p.Kv16), p.rows_k, d) &&
-                  make_map(&tm.xqn, at<void>(workspace, p.Xqn), rows, CHUNK) && make_map(&tm.yt, at<void>(workspace, p.Yt), rows, CHUNK);
+                  make_map(&tm.xq, at<void>(workspace, p.Xq), rows, CHUNK) && make_map(&tm.y, at<void>(workspace, p.Y), rows, CHUNK);
         if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
         FwdParams fp{};
         fp.o = at<float>(state, c.o_acc); fp.lse = at<float>(state, c.lse_acc); fp.G = log_f ? at<float>(workspace, p.G) : nullptr;
@@ -742,7 +741,7 @@ int path_attn_cp_step(void* state, const void* message, int B, int H, int Lq, in
                   make_map(&tm.kv, at<void>(msg, ck.kend), (uint64_t)ck.S * ck.Lp, d) &&
                   make_map(&tm.v, at<void>(msg, ck.v), (uint64_t)ck.S * ck.Lp, d);
         if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
-        tm.q_raw = tm.k_raw = tm.xqn = tm.yt = tm.qv;   // unused by this sweep, but every descriptor gets prefetched
+        tm.q_raw = tm.k_raw = tm.xq = tm.y = tm.qv;   // unused by this sweep, but every descriptor gets prefetched
         FwdParams fp{};
         fp.o = at<float>(workspace, cq.o_t); fp.lse = at<float>(workspace, cq.lse_t);
         fp.G = at<float>(state, cq.gq); fp.Gk = at<float>(msg, ck.gk);
@@ -823,7 +822,7 @@ int path_attn_prefill_cache(const void* k, const void* v, const void* w, const f
         typedef __nv_bfloat16 bf;
         const size_t mats = (size_t)p.S * nseg * 2 * d * d;          // elements of one [S][nseg][2][d][d] buffer
         bf* edge = at<bf>(workspace, p.Qv16);
-        bf* pseg = at<bf>(workspace, p.Xqn);
+        bf* pseg = at<bf>(workspace, p.Xq);
         bf* sfx = pseg + mats;
         lp.nseg = nseg; lp.seg_chunks = (p.N + nseg - 1) / nseg;
         lp.edge16 = edge; lp.pseg = pseg; lp.sfx = sfx; lp.L = p.Lp;   // (whole padded chunks: padded rows are zero)

@@ -16,6 +16,10 @@ constexpr uint32_t kTileB = 32768, kPanelB = 16384;
 // K view: contraction over the tile's columns.  MN view: contraction over the tile's rows.
 enum { OP_K = 0, OP_MN = 1 };
 
+// beta as the per-chunk kernels use it: kept away from zero, so that the chain rule can divide by it (T~ = Ainv D is kept, and
+// Ainv is T~ with its columns divided by beta).  2^-80 of a unit transition is far below every rounding.
+__device__ __forceinline__ float beta_floor(float b) { return fabsf(b) < 0x1p-80f ? copysignf(0x1p-80f, b) : b; }
+
 // D[128 x N] (+)= (+-) op(A) op(B), KSTEPS steps of 16 along the contraction.  One thread issues all of them (elect_one), so
 // the instructions between two tcgen05.mma count: everything but the tiles' addresses is a compile-time constant, the loop is
 // unrolled, and only the low word of a descriptor changes from step to step (the start address; the strides and the swizzle
@@ -164,6 +168,15 @@ __device__ __forceinline__ void unpack_bf16x32(const uint4 (&u4)[4], float (&v)[
             v[8 * x + 2 * y + 1] = f.y;
         }
     }
+}
+// Columns c0 .. c0+31 of `row` of a swizzled bf16 tile.
+__device__ __forceinline__ void tile_load32(const uint8_t* t, int row, int c0, float (&v)[32]) {
+    const uint8_t* panel = t + (c0 >> 6) * kPanelB;
+    uint4 u[4];
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch)
+        u[ch] = *reinterpret_cast<const uint4*>(panel + sw128_off((uint32_t)row, (uint32_t)(((c0 & 63) >> 3) + ch)));
+    unpack_bf16x32(u, v);
 }
 __device__ __forceinline__ void tmem_row32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];

@@ -317,6 +317,19 @@ def test_explicit_scale(binding, oracle, scale):
     compare_all(binding, oracle, inp, scale=scale)
 
 
+@pytest.mark.parametrize("L,d", [(200, 64), (384, 128)])
+def test_zero_and_tiny_betas_between_ordinary_ones(binding, oracle, L, d):
+    """Tokens with beta = 0, -0 and 1e-30 (below the floor of the per-chunk kernels, which divide by beta in the chain rule),
+    negative betas and runs of nearly equal w (a triangular system whose inverse has large entries)."""
+    inp = synth.make_inputs(1, 2, L, d, "bf16", seed=31 + d)
+    inp["beta"][:, :, ::5] = 0.0
+    inp["beta"][:, :, 1::15] = -0.0
+    inp["beta"][:, :, 2::7] = 1e-30
+    inp["beta"][:, :, 3::11] *= -0.25
+    inp["w"][:, :, 40:72] = inp["w"][:, :, 40:41]
+    compare_all(binding, oracle, inp)
+
+
 @pytest.mark.parametrize("mode", ["beta0", "beta2", "beta1", "w0"])
 def test_degenerate_householders(binding, oracle, mode):
     """beta = 0 (plain causal attention), beta = 2 (exact reflections), beta = 1 (projections), some w = 0."""
