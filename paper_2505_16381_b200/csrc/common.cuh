@@ -241,9 +241,11 @@ size_t decode_partials_bytes(int S, int cap, int hd);
 cudaError_t launch_decode_step(const void* q_t, const void* k_t, const void* v_t, const void* w_t, const float* beta_t,
                                const float* log_f_t, float* kc, void* vc, float* gc, int t, int cap, void* o_t, float* lse_t,
                                int S, int hd, float scale, float* part, cudaStream_t st);
-// Float32 forward by the definition (PATH_FP32): q, k, v, w, o are [S][L][hd] float, G the gate prefix [S][ldG] or nullptr.
+// Float32 forward (PATH_FP32): q, k, v, w, o are [S][L][hd] float, G the gate prefix [S][ldG] or nullptr; `scratch` holds
+// fp32_scratch_bytes(S, L, hd), or is nullptr (slower).
+size_t fp32_scratch_bytes(int S, int L, int hd);
 cudaError_t launch_fp32_fwd(const float* q, const float* k, const float* v, const float* w, const float* beta, const float* G,
-                            float* o, float* lse, int S, int L, int ldG, int hd, float scale, cudaStream_t st);
+                            float* o, float* lse, int S, int L, int ldG, int hd, float scale, float* scratch, cudaStream_t st);
 // Layer front-end (paper Sec. 2.2 footnote, Sec. 2.4 gate): z [B][L][H*hd] bf16 and logits [B][L][H] -> w [B][H][L][hd] bf16,
 // beta / log f [B][H][L]; and the backward (dcw must be zero on entry: CTAs add into it).
 cudaError_t launch_frontend_fwd(const void* z, const float* cw, const float* bl, const float* gl, void* w, float* beta,

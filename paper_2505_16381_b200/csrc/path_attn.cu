@@ -123,7 +123,7 @@ struct Plan {
     size_t status, qp, kp, vp, wp, betap, G, tstats, nkeep, nvisit, Dyh, Dyl, Xq, Y, Qv16, Kv16;
     // backward only
     size_t dop, delta, lse2, dQv, dKv, dSd, dSdT, dG, dGrow, dGdiag, dDy;
-    size_t sTh, sTl, sXk, sU;   // bf16 tiles kept by the chunk preparation for the chain rule
+    size_t sTh, sTl, sXk, sU, f32;   // bf16 tiles kept by the chunk preparation for the chain rule
     size_t dy_bytes, dy_mats;
 };
 
@@ -149,9 +149,10 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
     size_t cur = 0;
     const size_t SLd = (size_t)S * Lp * d, SL = (size_t)S * Lp, SNBB = (size_t)S * p.N * CHUNK * CHUNK;
     p.status = bump(cur, 256);
-    if (dt == PATH_FP32) {   // float32 tensors: forward only, computed from the definition; needs the gate prefix alone
+    if (dt == PATH_FP32) {   // float32 tensors: forward only; the gate prefix and the per-block tiles of fp32_fwd.cu
         if (bwd) return false;
         p.G = bump(cur, gate ? SL * 4 : 0);
+        p.f32 = bump(cur, fp32_scratch_bytes(p.S, L, d));
         p.total = cur;
         return true;
     }
@@ -434,7 +435,8 @@ int path_attn_fwd(const void* q, const void* k, const void* v, const void* w, co
         if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(w) || !aligned16(beta) || !aligned16(o) ||
             !aligned16(lse) || (log_f && !aligned16(log_f)) || ((uintptr_t)workspace & 255))
             return PATH_ERR_ALIGN;
-        if (workspace_bytes < p.total) return PATH_ERR_WORKSPACE;
+        if (workspace_bytes < p.f32) return PATH_ERR_WORKSPACE;   // (the per-block tiles behind it are optional)
+        const bool tiles = workspace_bytes >= p.total;
         int rc32 = check_arch();
         if (rc32 != PATH_OK) return rc32;
         cudaStream_t st32 = (cudaStream_t)cuda_stream;
@@ -445,7 +447,8 @@ int path_attn_fwd(const void* q, const void* k, const void* v, const void* w, co
             LAUNCH(launch_gate_prefix(log_f, G, p.S, L, p.Lp, st32));
         }
         LAUNCH(launch_fp32_fwd((const float*)q, (const float*)k, (const float*)v, (const float*)w, beta, G, (float*)o, lse,
-                               p.S, L, p.Lp, d, scale, st32));
+                               p.S, L, p.Lp, d, scale, tiles ? at<float>(workspace, p.f32) : nullptr, st32));
+        if (tiles) ++g_launches;
         return PATH_OK;
     }
     // A workspace large enough for the backward gets the backward's layout: the chunk preparation then also keeps
@@ -605,8 +608,10 @@ int path_attn_fwd_static(const void* q, const void* k, const void* v, const void
                          const float* log_f, void* o, float* lse, int B, int H, int L, int d, float scale,
                          path_dtype_t dt, void* cuda_stream, void** scratch_out) {
     if (dt != PATH_BF16 && dt != PATH_FP32) return PATH_ERR_DTYPE;
-    const size_t need = path_attn_workspace_bytes(B, H, L, d, dt, log_f ? 1 : 0, 0);
-    if (need == 0) return PATH_ERR_SHAPE;
+    Plan p;
+    if (!make_plan(B, H, L, d, (int)dt, log_f ? 1 : 0, 0, p)) return PATH_ERR_SHAPE;
+    size_t need = p.total;
+    if (dt == PATH_FP32 && need > (size_t)PATH_ATTN_STATIC_SCRATCH_BYTES) need = p.f32;   // do without the per-block tiles
     if (need > (size_t)PATH_ATTN_STATIC_SCRATCH_BYTES) return PATH_ERR_STATIC_LIMIT;
     void* scratch = nullptr;
     int rc = static_scratch_address(&scratch);

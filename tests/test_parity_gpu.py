@@ -293,10 +293,26 @@ def test_c1_workload_float32(binding, oracle):
     (2, 3, 333, 128, True, 0.25),     # ragged length, gate, d = 128
     (1, 1, 1, 64, False, 1.0),
     (1, 2, 1100, 64, True, -0.125),
+    (3, 1, 32, 128, False, 1.0),      # exactly one block of 32 keys
+    (2, 5, 257, 64, True, 1.0),       # one key in the last block; more rows than one per warp of every SM
 ])
 def test_float32_shapes(binding, oracle, B, H, L, d, gate, scale):
     inp = synth.make_inputs(B, H, L, d, "fp32", gate=gate, seed=900 + L)
     compare_f32(binding, oracle, inp, scale=scale)
+
+
+def test_float32_without_room_for_the_block_tiles(binding, oracle):
+    """A workspace that holds the status block and the gate prefix only: the key-by-key kernel."""
+    inp = synth.make_inputs(1, 2, 300, 64, "fp32", gate=True, seed=77)
+    dev = to_dev(inp)
+    full = binding.workspace_bytes(1, 2, 300, 64, binding.PATH_FP32, True, False)
+    ws = torch.empty(256 + 2 * 384 * 4, dtype=torch.uint8, device="cuda")
+    assert ws.numel() < full
+    o, lse = binding.path_attn_fwd(dev["q"], dev["k"], dev["v"], dev["w"], dev["beta"], dev["log_f"], workspace=ws)
+    x = slices(inp, [0, 1])
+    o_ref, lse_ref = oracle.forward(x["q"], x["k"], x["v"], x["w"], x["beta"], x["log_f"])
+    check("o", o.reshape(2, 300, 64), o_ref, rel=F32_REL, mx=F32_ABS)
+    assert np.abs(lse.reshape(2, -1).cpu().double().numpy() - lse_ref).max() <= 2e-5 * max(1.0, np.abs(lse_ref).max())
 
 
 def test_float32_is_forward_only(binding):
