@@ -94,6 +94,28 @@ def test_decode_steps_match_oracle_rows(binding, oracle, B, H, L0, T, d, gate, s
     assert torch.equal(cache["vc"], dev["v"])
 
 
+@pytest.mark.parametrize("S,t,d", [(444, 1600, 64), (444, 1500, 64), (7, 63, 128), (7, 64, 128), (3, 6300, 128)])
+def test_decode_split_rule_does_not_change_the_step(binding, S, t, d):
+    """Many slices (few, long ranges per slice; from 1537 positions per range cut in four) against the same slice alone (many
+    short ranges), on both sides of the rule's steps.  Same float32 arithmetic in another order: o differs by bf16 rounding
+    of values that agree to 1e-5, the caches not at all."""
+    g = torch.Generator(device="cuda").manual_seed(S + t)
+    n = lambda *s_: torch.randn(*s_, generator=g, device="cuda")
+    kc, vc = n(1, 1, t, d) / d ** 0.5, n(1, 1, t, d).bfloat16()
+    tok = [n(1, 1, d).bfloat16() for _ in range(4)]
+    beta = torch.full((1, 1), 0.7, device="cuda")
+    def step(H):
+        cache = binding.alloc_cache(1, H, t + 1, d)
+        cache["kc"][:, :, :t], cache["vc"][:, :, :t] = kc, vc
+        o, lse = binding.path_attn_decode_step(*(x.expand(1, H, d).contiguous() for x in tok), beta.expand(1, H).contiguous(), cache, t)
+        return o, lse, cache
+    o1, l1, c1 = step(1)
+    o, l, c = step(S)
+    assert (o.float() - o1.float()).abs().max() <= 2 ** -8 * max(1.0, o1.float().abs().max().item())
+    assert (l - l1).abs().max() <= 1e-5 * max(1.0, l1.abs().max().item())
+    assert torch.equal(c["kc"], c1["kc"].expand_as(c["kc"])) and torch.equal(c["vc"], c1["vc"].expand_as(c["vc"]))
+
+
 def test_prefill_then_decode_end_to_end(binding, oracle):
     """Prompt through path_attn_prefill_cache, then decoding steps: outputs within the training path's bounds."""
     B, H, L0, T, d = 1, 2, 640, 6, 128
