@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     auto first_loads_b = [&](int ch) {
         mbar_expect_tx(&bars[B_LOAD2], 2 * kT * HD * 2);
         tma_tile(slot(5), &tm.dkr, &bars[B_LOAD2], HD, ch * kT);
-        tma_tile(slot(4), &tm.w, &bars[B_LOAD2], HD, ch * kT);
+        tma_rows(slot(4), &tm.w, &bars[B_LOAD2], HD, (ch % p.N) * kT, ch / p.N);
     };
     if ((int)blockIdx.x < nchunks) {
         first_loads_a(blockIdx.x);
@@ -157,8 +157,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         if (!wait(B_MMA)) break;
         mbar_expect_tx(&bars[B_LOAD], 2 * kT * HD * 2 + kTileB);
         tma_tile(slot(3), &tm.dsdt, &bars[B_LOAD], kT, r0);
-        tma_tile(slot(6), &tm.q, &bars[B_LOAD], HD, r0);
-        tma_tile(slot(1), &tm.k, &bars[B_LOAD], HD, r0);
+        tma_rows(slot(6), &tm.q, &bars[B_LOAD], HD, (chunk % p.N) * kT, chunk / p.N);
+        tma_rows(slot(1), &tm.k, &bars[B_LOAD], HD, (chunk % p.N) * kT, chunk / p.N);
         mma<OP_MN, OP_MN, K8, HD>(tmem + cG, sa(5), sa(4), false);          // dXk^T W needs no new tile
         if (!wait(B_LOAD)) break;
         mma<OP_K, OP_MN, K8, HD>(tmem + cG, sa(3), sa(6), true);            // s dSd^T Q
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         const int s_idx = chunk / p.N, pos = (chunk % p.N) * kT + row;   // slice and position of this thread's row
         const bool row_valid = pos < p.L;
         const size_t urow = (size_t)s_idx * p.L + pos;                   // row in the caller's [S][L][.] tensors
-        if (tid < kT) bt[tid] = beta_floor(p.beta[(size_t)chunk * kT + tid]);   // first read after several barriers (phase 4)
+        if (tid < kT) bt[tid] = beta_floor(row_valid ? p.beta[urow] : 0.f);   // first read after several barriers (phase 4)
         mma_wait();                                                 // phase 0
         if (!ok) break;
         acc_to_tile(cA, kT, slot(0), -1.f, M_LOWER);                // dXq (over U)

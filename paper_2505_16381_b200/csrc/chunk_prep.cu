@@ -281,7 +281,11 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, 512);
-    if (tid < kT && (int)blockIdx.x < nchunks) bt[tid] = beta_floor(p.beta[(size_t)blockIdx.x * kT + tid]);
+    auto beta_of = [&](int chunk_) {   // beta of this thread's row (tid < 128); 0 past the sequence's end
+        const int pos = (chunk_ % p.N) * kT + tid;
+        return pos < p.L ? p.beta[(size_t)(chunk_ / p.N) * p.L + pos] : 0.f;
+    };
+    if (tid < kT && (int)blockIdx.x < nchunks) bt[tid] = beta_floor(beta_of(blockIdx.x));
     if (HD == 64) {  // second panel of W must read as zeros when W^T is used with M = 128
         for (int i = tid; i < (int)(kPanelB / 16); i += kThreads) reinterpret_cast<uint4*>(sW + kPanelB)[i] = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
@@ -301,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         if (warp == kWorkers / 32 && elect_one()) {
             auto wait = [&](int b, uint32_t par) { return mbar_wait(&bars[b], par, abort_flag, ST_PREP); };
             auto fetch = [&](const CUtensorMap* m, int i, int b, int chunk_) {
-                for (int h = 0; h < HD / 64; ++h) tma_load_2d(slot(i) + h * kPanelB, m, &bars[b], h * 64, chunk_ * kT);
+                tma_rows(slot(i), m, &bars[b], HD, (chunk_ % p.N) * kT, chunk_ / p.N);
             };
             auto load_w = [&](int chunk_) {
                 mbar_expect_tx(&bars[B_LOAD], kT * HD * 2);
@@ -553,7 +557,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
             // ---- E3: P = I - W^T U, Qleft = Q - Xq U, Kright = K - Y^T W; the Q and K rows arrive in U's slots meanwhile
             const int next = chunk + (int)gridDim.x;
             float next_beta = 0.f;
-            if (tid < kT && next < nchunks) next_beta = p.beta[(size_t)next * kT + tid];
+            if (tid < kT && next < nchunks) next_beta = beta_of(next);
             if (!(ok = wwait(B_G3A, par))) break;
 #pragma unroll
             for (int c = 0; c < HD / 64; ++c) {   // P: hi over Xq lo, lo over Xq hi

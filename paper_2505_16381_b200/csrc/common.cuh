@@ -105,7 +105,7 @@ __host__ __device__ inline long kver_row(const VerLayout& v, int s, int level, i
 }
 
 struct FwdTensorMaps {
-    CUtensorMap q_raw, k_raw, v, qv, kv, xq, y;
+    CUtensorMap q_raw, k_raw, v, qv, kv, xq, y;   // q_raw, k_raw, v: the caller's [S][L][d] (v: [S*Lkp][d] in the segment sweep)
 };
 
 struct FwdParams {
@@ -167,7 +167,7 @@ enum { LEVEL_DYADIC_FWD = 0, LEVEL_DYADIC_FUSED, LEVEL_VERSION_FWD, LEVEL_BWD, L
 cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const LevelParams& p, int hd, cudaStream_t st);
 
 struct PrepTensorMaps {
-    CUtensorMap w, q, k;   // [S*Lp][d] bf16, box 128 rows x 64 columns, 128-byte swizzle
+    CUtensorMap w, q, k;   // the caller's [S][L][d] bf16, box 1 x 128 rows x 64 columns, 128-byte swizzle
     // what the kernel leaves, all through TMA stores of its operand tiles:
     CUtensorMap ql, kr;    // [S*Lp][d]   boundary-adjusted queries / keys (version slot 0)
     CUtensorMap xq, y;     // [S*Lp][128] lower(Q W^T) and T~ strictLower(W K^T): the diagonal chunk's correction is -Xq Y
@@ -177,8 +177,9 @@ struct PrepTensorMaps {
 };
 
 struct PrepParams {
-    const float* beta;            // [S*Lp] (zero in the ragged tail)
+    const float* beta;            // [S][L]
     uint32_t* status;
+    int N, L;                     // chunks per slice, positions per slice
 };
 
 // `mode`: what the kernel produces (see chunk_prep.cu).
@@ -187,7 +188,8 @@ cudaError_t launch_chunk_prep(const PrepTensorMaps& tm, const PrepParams& p, int
                               cudaStream_t st);
 
 struct ChainTensorMaps {
-    CUtensorMap w, q, k, u;                       // [S*Lp][d]
+    CUtensorMap w, q, k;                          // the caller's [S][L][d]
+    CUtensorMap u;                                // [S*Lp][d]
     CUtensorMap y, xq, xk, th, tl;                // [S*Lp][128]; y and xq are the attention sweep's operands
     CUtensorMap dsdt;                             // [S*N*128][128] bf16: (scale * lower(dS))^T of the diagonal chunks
     CUtensorMap dql, dkr;                         // [S*Lp][d] bf16 gradients of the boundary-adjusted queries / keys
@@ -197,7 +199,7 @@ struct ChainTensorMaps {
 struct ChainParams {
     const __nv_bfloat16* dql;   // [S*Lp][d]  gradient of the boundary-adjusted queries (version slot 0), bf16
     const __nv_bfloat16* dkr;   // [S*Lp][d]  gradient of the boundary-adjusted keys, bf16
-    const float* beta;    // [S*Lp]
+    const float* beta;    // [S][L]
     __nv_bfloat16 *dq, *dk, *dw;   // [S][L][d] outputs
     float* dbeta;         // [S][L]
     uint32_t* status;
@@ -208,7 +210,7 @@ struct ChainParams {
 cudaError_t launch_chunk_chain(const ChainTensorMaps& tm, const ChainParams& p, int hd, int nchunks, cudaStream_t st);
 
 struct BwdTensorMaps {
-    CUtensorMap q_raw, k_raw, v, qv, kv, xq, y, d_o;
+    CUtensorMap q_raw, k_raw, v, qv, kv, xq, y, d_o;   // q_raw, k_raw, v, d_o: the caller's [S][L][d]
 };
 
 struct BwdParams {

@@ -125,6 +125,8 @@ __device__ __forceinline__ void tma_tile(uint8_t* dst, const CUtensorMap* m, uin
     for (int h = 0; h < kdim / 64; ++h) tma_load_2d(dst + h * kPanelBytes, m, bar, h * 64, row0);
 }
 
+using tile::tma_rows;
+
 // ------------------------------------------------------------------------------------------------ dK, dV
 // Persistent: the work items (one key chunk of one slice each) are listed slice after slice as pairs (longest,
 // shortest), (second longest, second shortest), ...; CTA c takes the pairs c, c + gridDim.x, ...  Every ring and phase
@@ -197,20 +199,22 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
             auto wait_empty = [&](int bar, int use) {
                 if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_DKV_PRODUCER)) ok = false;
             };
-            auto load_q = [&](const CUtensorMap* m, int kdim, int row0) {
+            auto load_q = [&](const CUtensorMap* m, int kdim, int row0, int slice = -1) {   // slice >= 0: a caller's tensor
                 const int slot = qn % 3;
                 wait_empty(K_QEMPTY + slot, qn / 3);
                 if (!ok) return;
                 mbar_expect_tx(&bars[K_QFULL + slot], (uint32_t)(kTile * kdim * 2));
-                tma_tile(sQ + slot * kSlotBytes, m, &bars[K_QFULL + slot], kdim, row0);
+                if (slice >= 0) tma_rows(sQ + slot * kSlotBytes, m, &bars[K_QFULL + slot], kdim, row0, slice);
+                else tma_tile(sQ + slot * kSlotBytes, m, &bars[K_QFULL + slot], kdim, row0);
                 ++qn;
             };
-            auto load_do = [&](const CUtensorMap* m, int kdim, int row0) {
+            auto load_do = [&](const CUtensorMap* m, int kdim, int row0, int slice = -1) {
                 const int slot = dn & 1;
                 wait_empty(K_DOEMPTY + slot, dn >> 1);
                 if (!ok) return;
                 mbar_expect_tx(&bars[K_DOFULL + slot], (uint32_t)(kTile * kdim * 2));
-                tma_tile(sDO + slot * kSlotBytes, m, &bars[K_DOFULL + slot], kdim, row0);
+                if (slice >= 0) tma_rows(sDO + slot * kSlotBytes, m, &bars[K_DOFULL + slot], kdim, row0, slice);
+                else tma_tile(sDO + slot * kSlotBytes, m, &bars[K_DOFULL + slot], kdim, row0);
                 ++dn;
             };
 #pragma unroll 1
@@ -223,23 +227,23 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                         wait_empty(K_KEMPTY, nk);
                         if (!ok) break;
                         mbar_expect_tx(&bars[K_KFULL], kTile * HD * 2);
-                        if (t == 0) tma_tile(sK, &tm.k_raw, &bars[K_KFULL], HD, rowJ);
+                        if (t == 0) tma_rows(sK, &tm.k_raw, &bars[K_KFULL], HD, J * kTile, s);
                         else tma_tile(sK, &tm.kv, &bars[K_KFULL], HD, (int)krow(l, J));
                         ++nk;
                     }
                     if (t == 0) {
-                        load_q(&tm.q_raw, HD, rowJ);
+                        load_q(&tm.q_raw, HD, J * kTile, s);
                         load_q(&tm.xq, kTile, rowJ);
                         load_do(&tm.y, kTile, rowJ);
                         wait_empty(K_VEMPTY, nv);
                         if (!ok) break;
                         mbar_expect_tx(&bars[K_VFULL], kTile * HD * 2);
-                        tma_tile(sV, &tm.v, &bars[K_VFULL], HD, rowJ);
+                        tma_rows(sV, &tm.v, &bars[K_VFULL], HD, J * kTile, s);
                         ++nv;
-                        load_do(&tm.d_o, HD, rowJ);
+                        load_do(&tm.d_o, HD, J * kTile, s);
                     } else {
                         load_q(&tm.qv, HD, (int)qrow(l, I));
-                        load_do(&tm.d_o, HD, s * p.Lp + I * kTile);
+                        load_do(&tm.d_o, HD, I * kTile, s);
                     }
                     // per-query statistics of the step
                     wait_empty(K_STEMPTY + (sn & 1), sn >> 1);
@@ -599,7 +603,7 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
                 wait_empty(Q_DOEMPTY, nd);
                 if (!ok) break;
                 mbar_expect_tx(&bars[Q_DOFULL], kTile * HD * 2);
-                tma_tile(sDO, &tm.d_o, &bars[Q_DOFULL], HD, s * p.Lp + I * kTile);
+                tma_rows(sDO, &tm.d_o, &bars[Q_DOFULL], HD, I * kTile, s);
                 ++nd;
 #pragma unroll 1
                 for (int t = 0; t < T && ok; ++t) {
@@ -619,7 +623,7 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
                     wait_empty(Q_VEMPTY + (vn & 1), vn >> 1);
                     if (!ok) break;
                     mbar_expect_tx(&bars[Q_VFULL + (vn & 1)], kTile * HD * 2);
-                    tma_tile(sV + (vn & 1) * kSlotBytes, &tm.v, &bars[Q_VFULL + (vn & 1)], HD, s * p.Lp + J * kTile);
+                    tma_rows(sV + (vn & 1) * kSlotBytes, &tm.v, &bars[Q_VFULL + (vn & 1)], HD, J * kTile, s);
                     if (GATE) {   // gate prefix of the key chunk
                         wait_empty(Q_GKEMPTY + (vn & 1), vn >> 1);
                         if (!ok) break;
@@ -711,6 +715,7 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
             // chain rule starts at the highest level reached.
             if (T == 0) {
                 zero_dq(0);
+                if (GATE && h == 0) p.dGrow[(size_t)s * p.Lp + I * kTile + row] = 0.f;
                 continue;
             }
             const size_t qi = (size_t)s * p.Lp + I * kTile + row;

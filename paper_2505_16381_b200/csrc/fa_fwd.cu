@@ -295,22 +295,22 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
             auto wait_empty = [&](int bar, int use) {
                 if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_FWD_PRODUCER)) ok = false;
             };
-            auto load_q = [&](const CUtensorMap* m, int kdim, int row0) {
+            auto load_q = [&](const CUtensorMap* m, int kdim, int row0, int slice = -1) {   // slice >= 0: a caller's tensor
                 const int slot = nq % 3;
                 wait_empty(B_QEMPTY + slot, nq / 3);
                 if (!ok) return;
                 mbar_expect_tx(&bars[B_QFULL + slot], (uint32_t)(kTile * kdim * 2));
-                for (int h = 0; h < kdim / 64; ++h)
-                    tma_load_2d(sQ + slot * kSlotBytes + h * kPanelBytes, m, &bars[B_QFULL + slot], h * 64, row0);
+                if (slice >= 0) tile::tma_rows(sQ + slot * kSlotBytes, m, &bars[B_QFULL + slot], kdim, row0, slice);
+                else tile::tma_tile(sQ + slot * kSlotBytes, m, &bars[B_QFULL + slot], kdim, row0);
                 ++nq;
             };
             auto load_kv = [&](uint8_t* base, int bfull, int bempty, int slot, uint32_t& fills, const CUtensorMap* m,
-                               int kdim, int row0) {
+                               int kdim, int row0, int slice = -1) {
                 wait_empty(bempty + slot, (int)((fills >> slot) & 1u));
                 if (!ok) return;
                 mbar_expect_tx(&bars[bfull + slot], (uint32_t)(kTile * kdim * 2));
-                for (int h = 0; h < kdim / 64; ++h)
-                    tma_load_2d(base + slot * kSlotBytes + h * kPanelBytes, m, &bars[bfull + slot], h * 64, row0);
+                if (slice >= 0) tile::tma_rows(base + slot * kSlotBytes, m, &bars[bfull + slot], kdim, row0, slice);
+                else tile::tma_tile(base + slot * kSlotBytes, m, &bars[bfull + slot], kdim, row0);
                 fills ^= 1u << slot;
             };
             int I, s;
@@ -318,11 +318,11 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                 const int NS = steps_of(I, s);
                 const int rowRaw = s * p.Lp + I * kTile;
                 // diagonal chunk: raw q, k and the correction operands (both K slots), V of chunk I
-                load_q(&tm.q_raw, HD, rowRaw);
-                load_kv(sK, B_KFULL, B_KEMPTY, 0, kf, &tm.k_raw, HD, rowRaw);
+                load_q(&tm.q_raw, HD, I * kTile, s);
+                load_kv(sK, B_KFULL, B_KEMPTY, 0, kf, &tm.k_raw, HD, I * kTile, s);
                 load_q(&tm.xq, kTile, rowRaw);
                 load_kv(sV, B_VFULL, B_VEMPTY, 1, vf, &tm.y, kTile, rowRaw);   // Y borrows stream 1's V slot
-                load_kv(sV, B_VFULL, B_VEMPTY, 0, vf, &tm.v, HD, rowRaw);
+                load_kv(sV, B_VFULL, B_VEMPTY, 0, vf, &tm.v, HD, I * kTile, s);
                 int cur = -1;
                 for (int n = 1; n < NS && ok; ++n) {
                     const int J = I - n, x = n & 1, l = msb32((unsigned)(I ^ J));   // l is non-decreasing in n
@@ -331,7 +331,7 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
                         cur = l;
                     }
                     load_kv(sK, B_KFULL, B_KEMPTY, x, kf, &tm.kv, HD, (int)kver_row(p.vl, s, l, J));
-                    load_kv(sV, B_VFULL, B_VEMPTY, x, vf, &tm.v, HD, s * p.Lp + J * kTile);
+                    load_kv(sV, B_VFULL, B_VEMPTY, x, vf, &tm.v, HD, J * kTile, s);
                 }
             }
         } else if (warp == 1 && elect_one()) {
@@ -688,22 +688,22 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
             auto wait_empty = [&](int bar, int use) {
                 if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_FWD_PRODUCER)) ok = false;
             };
-            auto load_q = [&](const CUtensorMap* m, int kdim, int row0) {
+            auto load_q = [&](const CUtensorMap* m, int kdim, int row0, int slice = -1) {   // slice >= 0: a caller's tensor
                 const int slot = nq % 3;
                 wait_empty(F_QEMPTY + slot, nq / 3);
                 if (!ok) return;
                 mbar_expect_tx(&bars[F_QFULL + slot], (uint32_t)(kTile * kdim * 2));
-                for (int h = 0; h < kdim / 64; ++h)
-                    tma_load_2d(sQ + slot * kSlotBytes + h * kPanelBytes, m, &bars[F_QFULL + slot], h * 64, row0);
+                if (slice >= 0) tile::tma_rows(sQ + slot * kSlotBytes, m, &bars[F_QFULL + slot], kdim, row0, slice);
+                else tile::tma_tile(sQ + slot * kSlotBytes, m, &bars[F_QFULL + slot], kdim, row0);
                 ++nq;
             };
-            auto load_kv = [&](const CUtensorMap* m, int kdim, int row0) {
+            auto load_kv = [&](const CUtensorMap* m, int kdim, int row0, int slice = -1) {
                 const int slot = nkv & 3;
                 wait_empty(F_KVEMPTY + slot, nkv >> 2);
                 if (!ok) return;
                 mbar_expect_tx(&bars[F_KVFULL + slot], (uint32_t)(kTile * kdim * 2));
-                for (int h = 0; h < kdim / 64; ++h)
-                    tma_load_2d(sKV + slot * kSlotBytes + h * kPanelBytes, m, &bars[F_KVFULL + slot], h * 64, row0);
+                if (slice >= 0) tile::tma_rows(sKV + slot * kSlotBytes, m, &bars[F_KVFULL + slot], kdim, row0, slice);
+                else tile::tma_tile(sKV + slot * kSlotBytes, m, &bars[F_KVFULL + slot], kdim, row0);
                 ++nkv;
             };
             auto load_gk = [&](int x, const float* src) {
@@ -750,13 +750,13 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
                     if (NS1 > 0) load_q(&tm.qv, HD, rowS + I1 * kTile);
                 } else {
                     if (NS1 > 0) {   // stream 1's diagonal chunk: raw q, k and the correction operands
-                        load_q(&tm.q_raw, HD, rowS + I1 * kTile);
-                        load_kv(&tm.k_raw, HD, rowS + I1 * kTile);
+                        load_q(&tm.q_raw, HD, I1 * kTile, s);
+                        load_kv(&tm.k_raw, HD, I1 * kTile, s);
                         load_q(&tm.xq, kTile, rowS + I1 * kTile);
                         load_kv(&tm.y, kTile, rowS + I1 * kTile);
                     }
-                    load_q(&tm.q_raw, HD, rowS + I0 * kTile);
-                    load_kv(&tm.k_raw, HD, rowS + I0 * kTile);
+                    load_q(&tm.q_raw, HD, I0 * kTile, s);
+                    load_kv(&tm.k_raw, HD, I0 * kTile, s);
                     load_q(&tm.xq, kTile, rowS + I0 * kTile);
                     load_kv(&tm.y, kTile, rowS + I0 * kTile);
                 }
@@ -770,7 +770,8 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
                             if (u0) load_gk(0, g);
                             if (u1) load_gk(1, g);
                         }
-                        load_kv(&tm.v, HD, (CROSS ? s * p.Lkp : rowS) + J * kTile);
+                        if (CROSS) load_kv(&tm.v, HD, s * p.Lkp + J * kTile);
+                        else load_kv(&tm.v, HD, J * kTile, s);
                     }
                     if (!SEP) load_step(n + 1);
                 }

@@ -18,11 +18,6 @@ __global__ void pad_rows_kernel(const void* __restrict__ src, void* __restrict__
     ((uint4*)dst)[((long)blockIdx.y * Lp + row) * rowbytes16 + col] = v;
 }
 
-__global__ void pad_vec_kernel(const float* __restrict__ src, float* __restrict__ dst, int L, int Lp) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < Lp) dst[(size_t)blockIdx.y * Lp + i] = (i < L) ? src[(size_t)blockIdx.y * L + i] : 0.f;
-}
-
 // One CTA (1024 threads) per slice: each thread scans a contiguous segment, then a block scan of the segment sums.
 __global__ void __launch_bounds__(1024) gate_prefix_kernel(const float* __restrict__ g, float* __restrict__ G, int L,
                                                            int Lp) {
@@ -130,20 +125,23 @@ __global__ void __launch_bounds__(256) tile_stats_kernel(const __nv_bfloat16* __
     };
     for (int r = warp * rows_w + grp; r < CHUNK; r += 8 * rows_w) {
         const int t = c * CHUNK + r;
-        const size_t row = (size_t)sl * Lp + t;
-        const uint4 a = *reinterpret_cast<const uint4*>(q + row * hd + li * 8);
-        const uint4 b = *reinterpret_cast<const uint4*>(k + row * hd + li * 8);
-        const uint4 x = *reinterpret_cast<const uint4*>(w + row * hd + li * 8);
+        const size_t row = (size_t)sl * L + t;
+        uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a, x = a;
+        if (t < L) {
+            a = *reinterpret_cast<const uint4*>(q + row * hd + li * 8);
+            b = *reinterpret_cast<const uint4*>(k + row * hd + li * 8);
+            x = *reinterpret_cast<const uint4*>(w + row * hd + li * 8);
+        }
         float qq = dot8(a, a), kk = dot8(b, b), qk = dot8(a, b), ww = dot8(x, x);
         for (int off = lpr / 2; off >= 1; off >>= 1) {
             qq += __shfl_xor_sync(0xffffffffu, qq, off); kk += __shfl_xor_sync(0xffffffffu, kk, off);
             qk += __shfl_xor_sync(0xffffffffu, qk, off); ww += __shfl_xor_sync(0xffffffffu, ww, off);
         }
-        const float g = G[row];
+        const float g = G[(size_t)sl * Lp + t], bt = t < L ? beta[row] : 0.f;
         qn = fmaxf(qn, sqrtf(qq)); kn = fmaxf(kn, sqrtf(kk));
         gmax = fmaxf(gmax, g); gmin = fminf(gmin, g);
         if (t < L) mlo = fminf(mlo, scale * qk);
-        gam += logf(fmaxf(1.f, fabsf(1.f - beta[row] * ww)));
+        gam += logf(fmaxf(1.f, fabsf(1.f - bt * ww)));
     }
     // the lanes of a group hold the same values; combine the groups of the warp (the growth sum counts each group once)
     for (int off = lpr; off < 32; off <<= 1) {
@@ -327,12 +325,6 @@ cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, in
     const long total = (long)Lp * rowbytes16;
     dim3 grid((unsigned)((total + 255) / 256), S);
     pad_rows_kernel<<<grid, 256, 0, st>>>(src, dst, L, Lp, rowbytes16);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pad_vec(const float* src, float* dst, int S, int L, int Lp, cudaStream_t st) {
-    dim3 grid((Lp + 255) / 256, S);
-    pad_vec_kernel<<<grid, 256, 0, st>>>(src, dst, L, Lp);
     return cudaGetLastError();
 }
 

@@ -7,8 +7,6 @@ namespace path {
 
 // dst[S][Lp][d] <- src[S][L][d] (zero tail); bf16 elements when !f32.
 cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, int f32, cudaStream_t st);
-// dst[S][Lp] <- src[S][L] (zero tail), float.
-cudaError_t launch_pad_vec(const float* src, float* dst, int S, int L, int Lp, cudaStream_t st);
 // G[S][Lp] <- inclusive prefix sum of g[S][L] (tail repeats the last value).
 cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, cudaStream_t st);
 
@@ -21,7 +19,7 @@ cudaError_t launch_dsd_rowsum(const float* dsd, float* rs, int nchunks, cudaStre
 // Gated problems (PaTH-FoX): which key chunks a query chunk can skip because the accumulated gate has made every logit
 // of the pair negligible.  stats: [S*N][8] floats of scratch; nkeep: [S*N] key chunks each query chunk visits (counted
 // from the diagonal); nvisit: [S*N] query chunks each key chunk meets (the same pairs, key-major); counters: {kept pairs,
-// all pairs}, added to (zeroed by the caller).  q, k, w: [S][Lp][hd] bf16 (padded), beta, G: [S][Lp].
+// all pairs}, added to (zeroed by the caller).  q, k, w: [S][L][hd] bf16, beta: [S][L], G: [S][Lp].
 cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const float* beta, const float* G, float* stats,
                              int* nkeep, int* nvisit, unsigned long long* counters, int S, int L, int Lp, int hd, float scale,
                              cudaStream_t st);

@@ -114,15 +114,15 @@ static bool make_map_box(CUtensorMap* m, const void* base, uint64_t rows, uint64
 
 // ------------------------------------------------------------------------------------------- workspace plan
 struct Plan {
-    int S, L, Lp, N, d, nlev, gate, bwd, ragged;
+    int S, L, Lp, N, d, nlev, gate, bwd;
     LevelTable lv;
     VerLayout vl;
     uint64_t rows_q, rows_k;   // rows (of d elements) of the query / key version buffers
     size_t total;
     // offsets (bytes)
-    size_t status, qp, kp, vp, wp, betap, G, tstats, nkeep, nvisit, Dyh, Dyl, Xq, Y, Qv16, Kv16;
+    size_t status, G, tstats, nkeep, nvisit, Dyh, Dyl, Xq, Y, Qv16, Kv16;
     // backward only
-    size_t dop, delta, lse2, dQv, dKv, dSd, dSdT, dG, dGrow, dGdiag, dDy;
+    size_t delta, lse2, dQv, dKv, dSd, dSdT, dG, dGrow, dGdiag, dDy;
     size_t sTh, sTl, sXk, sU, f32;   // bf16 tiles kept by the chunk preparation for the chain rule
     size_t dy_bytes, dy_mats;
 };
@@ -145,7 +145,6 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
     p.vl = make_ver_layout(p.S, p.N, p.Lp, p.nlev);
     p.rows_q = (uint64_t)S * Lp + (uint64_t)S * p.vl.eq * CHUNK;
     p.rows_k = (uint64_t)S * Lp + (uint64_t)S * p.vl.ek * CHUNK;
-    p.ragged = (L != p.Lp);
     size_t cur = 0;
     const size_t SLd = (size_t)S * Lp * d, SL = (size_t)S * Lp, SNBB = (size_t)S * p.N * CHUNK * CHUNK;
     p.status = bump(cur, 256);
@@ -156,10 +155,6 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
         p.total = cur;
         return true;
     }
-    if (p.ragged) {
-        p.qp = bump(cur, SLd * 2); p.kp = bump(cur, SLd * 2); p.vp = bump(cur, SLd * 2); p.wp = bump(cur, SLd * 2);
-    }
-    p.betap = bump(cur, SL * 4);
     if (gate) {
         p.G = bump(cur, SL * 4);
         p.tstats = bump(cur, (size_t)S * p.N * 8 * 4);   // per-chunk bounds and the resulting key-chunk counts: block skipping
@@ -185,7 +180,6 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
     p.Kv16 = bump(cur, p.rows_k * d * 2);
     p.dy_bytes = dy_elems * 2;
     if (bwd) {
-        if (p.ragged) p.dop = bump(cur, SLd * 2);
         p.delta = bump(cur, SL * 4); p.lse2 = bump(cur, SL * 4);
         p.dQv = bump(cur, p.rows_q * d * 2); p.dKv = bump(cur, p.rows_k * d * 2);   // bf16
         p.dSd = bump(cur, gate ? SNBB * 4 : 0); p.dSdT = bump(cur, SNBB * 2); p.dG = bump(cur, SL * 4);
@@ -196,6 +190,20 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
     }
     p.total = cur;
     return true;
+}
+
+// A caller's bf16 tensor [S][L][d], box = one slice x 128 rows x 64 columns, 128-byte swizzle: rows past a slice's end read as
+// zeros, so a length that is no multiple of the chunk needs no padded copy (four copies of 6 us each at 64 x 1500 x 64).
+static bool make_map_rows(CUtensorMap* m, const void* base, const Plan& p) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)p.d, (cuuint64_t)p.L, (cuuint64_t)p.S};
+    cuuint64_t strides[2] = {(cuuint64_t)p.d * 2, (cuuint64_t)p.L * p.d * 2};
+    cuuint32_t box[3] = {64, 128, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <class T>
@@ -224,10 +232,10 @@ static LevelParams level_params(const Plan& p, void* ws) {
 }
 
 // Gated problems: which chunk pairs the sweeps can leave out (counts per query chunk and per key chunk, three small
-// kernels).  Runs before the chunk preparation: the version chains stop at the highest level a kept pair uses.
-static int run_gate_skip(const Plan& p, void* ws, const void* q, const void* k, const void* w, float scale, cudaStream_t st) {
-    CK(cudaMemsetAsync(at<uint8_t>(ws, p.status + kSkipCounterOffset), 0, 16, st));
-    LAUNCH(launch_gate_skip(q, k, w, at<float>(ws, p.betap), at<float>(ws, p.G), at<float>(ws, p.tstats), at<int>(ws, p.nkeep),
+// kernels; the status block's pair counters are zero on entry).  Runs before the chunk preparation: the version chains stop at the highest level a kept pair uses.
+static int run_gate_skip(const Plan& p, void* ws, const void* q, const void* k, const void* w, const float* beta, float scale,
+                         cudaStream_t st) {
+    LAUNCH(launch_gate_skip(q, k, w, beta, at<float>(ws, p.G), at<float>(ws, p.tstats), at<int>(ws, p.nkeep),
                             at<int>(ws, p.nvisit), at<unsigned long long>(ws, p.status + kSkipCounterOffset), p.S, p.L, p.Lp,
                             p.d, scale, st));
     g_launches += 2;
@@ -235,7 +243,7 @@ static int run_gate_skip(const Plan& p, void* ws, const void* q, const void* k, 
 }
 
 // Chunk preparation + dyadic run products + version chains (paper Sec. 3.1, 3.3).  Shared by forward and backward.
-static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const void* w, bool in_backward,
+static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const void* w, const float* beta, bool in_backward,
                     cudaStream_t st, bool with_levels = true, bool keys_only = false) {
     const int d = p.d, nch = p.S * p.N;
     const int stg_prep = in_backward ? STG_PREP_BWD : STG_PREP, stg_lev = in_backward ? STG_LEVELS_BWDPREP : STG_LEVELS;
@@ -243,12 +251,12 @@ static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const
     {
         PrepTensorMaps tm{};
         const uint64_t rows = (uint64_t)p.S * p.Lp;
-        if (!(make_map(&tm.w, w, rows, d) && make_map(&tm.q, q, rows, d) && make_map(&tm.k, k, rows, d))) {
+        if (!(make_map_rows(&tm.w, w, p) && make_map_rows(&tm.q, q, p) && make_map_rows(&tm.k, k, p))) {
             g_last_cuda_error = (int)cudaErrorUnknown;
             return PATH_ERR_LAUNCH;
         }
         PrepParams pp{};
-        pp.beta = at<float>(ws, p.betap);
+        pp.beta = beta; pp.N = p.N; pp.L = p.L;
         if (!(make_map(&tm.ql, at<void>(ws, p.Qv16), rows, d) && make_map(&tm.kr, at<void>(ws, p.Kv16), rows, d) &&
               make_map(&tm.xq, at<void>(ws, p.Xq), rows, CHUNK) && make_map(&tm.y, at<void>(ws, p.Y), rows, CHUNK) &&
               make_map_box(&tm.ph, at<void>(ws, p.Dyh), (uint64_t)nch * d, d, d) &&
@@ -296,37 +304,17 @@ static int check_arch() {
 
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
-// Pads q, k, v, w (ragged L) and beta into the workspace; returns the pointers the kernels should read.
-// With run = false only the pointers are redirected (the padded copies are already in the workspace).
-static int stage_inputs(const Plan& p, void* ws, const void*& q, const void*& k, const void*& v, const void*& w,
-                        const float* beta, const float* log_f, bool run, cudaStream_t st) {
-    if (p.ragged) {
-        if (run) {
-            LAUNCH(launch_pad_rows(q, at<void>(ws, p.qp), p.S, p.L, p.Lp, p.d, 0, st));
-            LAUNCH(launch_pad_rows(k, at<void>(ws, p.kp), p.S, p.L, p.Lp, p.d, 0, st));
-            LAUNCH(launch_pad_rows(v, at<void>(ws, p.vp), p.S, p.L, p.Lp, p.d, 0, st));
-            LAUNCH(launch_pad_rows(w, at<void>(ws, p.wp), p.S, p.L, p.Lp, p.d, 0, st));
-        }
-        q = at<void>(ws, p.qp); k = at<void>(ws, p.kp); v = at<void>(ws, p.vp); w = at<void>(ws, p.wp);
-    }
-    if (run) {
-        LAUNCH(launch_pad_vec(beta, at<float>(ws, p.betap), p.S, p.L, p.Lp, st));
-        if (log_f) LAUNCH(launch_gate_prefix(log_f, at<float>(ws, p.G), p.S, p.L, p.Lp, st));
-    }
-    return PATH_OK;
-}
-
 }  // namespace path
 
 namespace path {
 
 // Per-chunk chain rule through the UT transform and the boundary-adjusted tiles: one fused kernel.
-static int run_chunk_chain(const Plan& p, void* ws, const void* q, const void* k, const void* w, void* dq, void* dk,
-                           void* dw, float* dbeta, float scale, cudaStream_t st) {
+static int run_chunk_chain(const Plan& p, void* ws, const void* q, const void* k, const void* w, const float* beta, void* dq,
+                           void* dk, void* dw, float* dbeta, float scale, cudaStream_t st) {
     const int d = p.d;
     const uint64_t rows = (uint64_t)p.S * p.Lp;
     ChainTensorMaps tm;
-    bool ok = make_map(&tm.w, w, rows, d) && make_map(&tm.q, q, rows, d) && make_map(&tm.k, k, rows, d) &&
+    bool ok = make_map_rows(&tm.w, w, p) && make_map_rows(&tm.q, q, p) && make_map_rows(&tm.k, k, p) &&
               make_map(&tm.u, at<void>(ws, p.sU), rows, d) && make_map(&tm.y, at<void>(ws, p.Y), rows, CHUNK) &&
               make_map(&tm.xq, at<void>(ws, p.Xq), rows, CHUNK) && make_map(&tm.xk, at<void>(ws, p.sXk), rows, CHUNK) &&
               make_map(&tm.th, at<void>(ws, p.sTh), rows, CHUNK) && make_map(&tm.tl, at<void>(ws, p.sTl), rows, CHUNK) &&
@@ -336,7 +324,7 @@ static int run_chunk_chain(const Plan& p, void* ws, const void* q, const void* k
     if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
     ChainParams cp{};
     cp.dql = at<__nv_bfloat16>(ws, p.dQv); cp.dkr = at<__nv_bfloat16>(ws, p.dKv);   // slot 0 of the version gradients: the final sums
-    cp.beta = at<float>(ws, p.betap);
+    cp.beta = beta;
     cp.dq = (__nv_bfloat16*)dq; cp.dk = (__nv_bfloat16*)dk; cp.dw = (__nv_bfloat16*)dw; cp.dbeta = dbeta;
     cp.status = at<uint32_t>(ws, p.status);
     cp.N = p.N; cp.L = p.L; cp.scale = scale;
@@ -344,7 +332,7 @@ static int run_chunk_chain(const Plan& p, void* ws, const void* q, const void* k
     return PATH_OK;
 }
 
-static int run_backward(const Plan& p, void* ws, const void* q, const void* k, const void* v, const void* w,
+static int run_backward(const Plan& p, void* ws, const void* q, const void* k, const void* v, const void* w, const float* beta,
                         const void* o, const float* lse, const void* d_o, void* dq, void* dk, void* dv, void* dw,
                         float* dbeta, float* dlog_f, float scale, cudaStream_t st) {
     const int d = p.d;
@@ -353,20 +341,13 @@ static int run_backward(const Plan& p, void* ws, const void* q, const void* k, c
     prof_mark(STG_ROWSTATS, 0, st);
     LAUNCH(launch_rowstats(o, d_o, lse, p.gate ? at<float>(ws, p.G) : nullptr, at<float>(ws, p.delta), at<float>(ws, p.lse2),
                            p.S, p.L, p.Lp, d, st));
-    const void* dop = d_o;
-    if (p.ragged) {
-        LAUNCH(launch_pad_rows(d_o, at<void>(ws, p.dop), p.S, p.L, p.Lp, d, 0, st));
-        dop = at<void>(ws, p.dop);
-    }
-    if (p.gate) CK(cudaMemsetAsync(at<float>(ws, p.dGrow), 0, (size_t)p.S * p.Lp * 4, st));
-
     BwdTensorMaps tm;
     const uint64_t rows = (uint64_t)p.S * p.Lp;
-    bool ok = make_map(&tm.q_raw, q, rows, d) && make_map(&tm.k_raw, k, rows, d) && make_map(&tm.v, v, rows, d) &&
+    bool ok = make_map_rows(&tm.q_raw, q, p) && make_map_rows(&tm.k_raw, k, p) && make_map_rows(&tm.v, v, p) &&
               make_map(&tm.qv, at<void>(ws, p.Qv16), p.rows_q, d) &&
               make_map(&tm.kv, at<void>(ws, p.Kv16), p.rows_k, d) &&
               make_map(&tm.xq, at<void>(ws, p.Xq), rows, CHUNK) && make_map(&tm.y, at<void>(ws, p.Y), rows, CHUNK) &&
-              make_map(&tm.d_o, dop, rows, d);
+              make_map_rows(&tm.d_o, d_o, p);
     if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
     BwdParams bp{};
     bp.dqv = dQv; bp.dkv = dKv; bp.dv = dv; bp.dsd = p.gate ? at<float>(ws, p.dSd) : nullptr; bp.dsdt = at<__nv_bfloat16>(ws, p.dSdT); bp.dG = at<float>(ws, p.dG); bp.dGrow = at<float>(ws, p.dGrow);
@@ -398,7 +379,7 @@ static int run_backward(const Plan& p, void* ws, const void* q, const void* k, c
     }
     prof_mark(STG_LEVELS_BWD, 1, st);
     prof_mark(STG_CHAIN, 0, st);
-    int rc = run_chunk_chain(p, ws, q, k, w, dq, dk, dw, dbeta, scale, st);
+    int rc = run_chunk_chain(p, ws, q, k, w, beta, dq, dk, dw, dbeta, scale, st);
     if (rc != PATH_OK) return rc;
     prof_mark(STG_CHAIN, 1, st);
     prof_mark(STG_GATE, 0, st);
@@ -469,18 +450,17 @@ int path_attn_fwd(const void* q, const void* k, const void* v, const void* w, co
     CK(cudaMemsetAsync(workspace, 0, 256, st));
 
     prof_reset(STG_PREP, STG_PREP_BWD);
-    rc = stage_inputs(p, workspace, q, k, v, w, beta, log_f, true, st);
-    if (rc != PATH_OK) return rc;
     if (log_f) {
-        rc = run_gate_skip(p, workspace, q, k, w, scale, st);
+        LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
+        rc = run_gate_skip(p, workspace, q, k, w, beta, scale, st);
         if (rc != PATH_OK) return rc;
     }
-    rc = run_prep(p, workspace, q, k, w, false, st);
+    rc = run_prep(p, workspace, q, k, w, beta, false, st);
     if (rc != PATH_OK) return rc;
 
     FwdTensorMaps tm;
     const uint64_t rows = (uint64_t)p.S * p.Lp;
-    bool ok = make_map(&tm.q_raw, q, rows, d) && make_map(&tm.k_raw, k, rows, d) && make_map(&tm.v, v, rows, d) &&
+    bool ok = make_map_rows(&tm.q_raw, q, p) && make_map_rows(&tm.k_raw, k, p) && make_map_rows(&tm.v, v, p) &&
               make_map(&tm.qv, at<void>(workspace, p.Qv16), p.rows_q, d) &&
               make_map(&tm.kv, at<void>(workspace, p.Kv16), p.rows_k, d) &&
               make_map(&tm.xq, at<void>(workspace, p.Xq), rows, CHUNK) &&
@@ -519,27 +499,25 @@ static int backward_entry(const void* q, const void* k, const void* v, const voi
     int rc = check_arch();
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    CK(cudaMemsetAsync(workspace, 0, kSkipCounterOffset, st));   // the status word; the block-skipping counters may be reused
+    // the status word, and what a reused forward left only if it is not reused: the block-skipping counters and the record
+    CK(cudaMemsetAsync(workspace, 0, reuse ? kSkipCounterOffset : 256, st));
     prof_reset(STG_PREP_BWD, STG_COUNT);
     if (reuse) {
         // the record the forward left must describe this very problem (for a gated one the scale too: the block-skipping
         // counts, and with them the levels the version chains were built up to, depend on it)
         LAUNCH(launch_state_check(at<void>(workspace, p.status + kStateRecordOffset),
                                   make_record(q, k, v, w, beta, log_f, B, H, L, d, scale), at<uint32_t>(workspace, p.status), st));
-    } else {
-        CK(cudaMemsetAsync(at<uint8_t>(workspace, p.status + kStateRecordOffset), 0, sizeof(StateRecord), st));
     }
-    rc = stage_inputs(p, workspace, q, k, v, w, beta, log_f, !reuse, st);
-    if (rc != PATH_OK) return rc;
     if (!reuse) {
         if (log_f) {
-            rc = run_gate_skip(p, workspace, q, k, w, scale, st);
+            LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
+            rc = run_gate_skip(p, workspace, q, k, w, beta, scale, st);
             if (rc != PATH_OK) return rc;
         }
-        rc = run_prep(p, workspace, q, k, w, true, st);
+        rc = run_prep(p, workspace, q, k, w, beta, true, st);
         if (rc != PATH_OK) return rc;
     }
-    return run_backward(p, workspace, q, k, v, w, o, lse, d_o, dq, dk, dv, dw, dbeta, dlog_f, scale, st);
+    return run_backward(p, workspace, q, k, v, w, beta, o, lse, d_o, dq, dk, dv, dw, dbeta, dlog_f, scale, st);
 }
 
 int path_attn_bwd(const void* q, const void* k, const void* v, const void* w, const float* beta, const float* log_f,
@@ -683,19 +661,18 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     CK(cudaMemsetAsync(workspace, 0, 256, st));
-    rc = stage_inputs(p, workspace, q, k, v, w, beta, log_f, true, st);
-    if (rc != PATH_OK) return rc;
     if (log_f) {
-        rc = run_gate_skip(p, workspace, q, k, w, scale, st);
+        LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
+        rc = run_gate_skip(p, workspace, q, k, w, beta, scale, st);
         if (rc != PATH_OK) return rc;
     }
-    rc = run_prep(p, workspace, q, k, w, false, st);
+    rc = run_prep(p, workspace, q, k, w, beta, false, st);
     if (rc != PATH_OK) return rc;
     // the segment's own (causal) attention, as a float32 running result
     {
         FwdTensorMaps tm;
         const uint64_t rows = (uint64_t)p.S * p.Lp;
-        bool ok = make_map(&tm.q_raw, q, rows, d) && make_map(&tm.k_raw, k, rows, d) && make_map(&tm.v, v, rows, d) &&
+        bool ok = make_map_rows(&tm.q_raw, q, p) && make_map_rows(&tm.k_raw, k, p) && make_map_rows(&tm.v, v, p) &&
                   make_map(&tm.qv, at<void>(workspace, p.Qv16), p.rows_q, d) &&
                   make_map(&tm.kv, at<void>(workspace, p.Kv16), p.rows_k, d) &&
                   make_map(&tm.xq, at<void>(workspace, p.Xq), rows, CHUNK) && make_map(&tm.y, at<void>(workspace, p.Y), rows, CHUNK);
@@ -720,7 +697,9 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
         lp.pseg = at<__nv_bfloat16>(message, c.pseg);
         LAUNCH(launch_level_kernel(LEVEL_QUERY_EDGE, tm, lp, d, st));
     }
-    CK(cudaMemcpyAsync(at<void>(message, c.v), v, (size_t)p.S * p.Lp * d * 2, cudaMemcpyDeviceToDevice, st));
+    // (a sweep reads the message's values in whole chunks)
+    if (p.L == p.Lp) CK(cudaMemcpyAsync(at<void>(message, c.v), v, (size_t)p.S * p.Lp * d * 2, cudaMemcpyDeviceToDevice, st));
+    else LAUNCH(launch_pad_rows(v, at<void>(message, c.v), p.S, p.L, p.Lp, d, 0, st));
     LAUNCH(launch_cp_gate(log_f ? at<float>(workspace, p.G) : nullptr, at<float>(state, c.gq), at<float>(message, c.gk),
                           at<float>(message, c.gtot), p.S, L, p.Lp, st));
     return PATH_OK;
@@ -805,11 +784,9 @@ int path_attn_prefill_cache(const void* k, const void* v, const void* w, const f
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     CK(cudaMemsetAsync(workspace, 0, 256, st));
+    if (log_f) LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
     // the chunk preparation needs no queries for the key side: the keys stand in for them
-    const void* qd = k; const void* kd = k; const void* vd = v; const void* wd = w;
-    rc = stage_inputs(p, workspace, qd, kd, vd, wd, beta, log_f, true, st);
-    if (rc != PATH_OK) return rc;
-    rc = run_prep(p, workspace, qd, kd, wd, false, st, false, true);
+    rc = run_prep(p, workspace, k, k, w, beta, false, st, false, true);
     if (rc != PATH_OK) return rc;
     LevelTensorMaps tm;
     if (!make_level_maps(p, workspace, tm)) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }

@@ -185,6 +185,10 @@ __device__ __forceinline__ void tmem_row32(uint32_t taddr, float (&v)[32]) {
 #pragma unroll
     for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(r[x]);
 }
+// The same from a caller's tensor [slices][L][ncols]: rows row .. row + 127 of a slice, zeros past its end.
+__device__ __forceinline__ void tma_rows(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int ncols, int row, int slice) {
+    for (int h = 0; h < ncols / 64; ++h) tma_load_3d(dst + h * kPanelB, m, bar, h * 64, row, slice);
+}
 // TMA load of a [128 x ncols] bf16 tile (ncols = 64 or 128) whose first row is `row0` of the mapped matrix.
 __device__ __forceinline__ void tma_tile(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int ncols, int row0) {
     for (int h = 0; h < ncols / 64; ++h) tma_load_2d(dst + h * kPanelB, m, bar, h * 64, row0);
