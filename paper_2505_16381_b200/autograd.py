@@ -30,10 +30,13 @@ class _PathAttention(torch.autograd.Function):
         ctx.save_for_backward(q, k, v, w, beta, log_f, o, lse)
         ctx.scale, ctx.ws = scale, (ws if keep else None)
         ctx.mark_non_differentiable(lse)
+        ctx.set_materialize_grads(False)   # (no tensor of zeros for lse in every backward)
         return o, lse
 
     @staticmethod
     def backward(ctx, d_o, _d_lse):
+        if d_o is None:
+            return (None,) * 8
         q, k, v, w, beta, log_f, o, lse = ctx.saved_tensors
         g = binding.path_attn_bwd(q, k, v, w, beta, o, lse, d_o.contiguous(), log_f, scale=ctx.scale, workspace=ctx.ws,
                                   reuse=ctx.ws is not None)
