@@ -52,6 +52,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();
+    grid_launch();
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     auto slot = [&](int i) { return smem + i * kTileB; };
     auto sa = [&](int i) { return smem_u32(smem + i * kTileB); };
@@ -417,19 +419,12 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
 }  // namespace
 
 cudaError_t launch_chunk_chain(const ChainTensorMaps& tm, const ChainParams& p, int hd, int nchunks, cudaStream_t st) {
-    int dev = 0, sms = 0;
-    cudaError_t e0 = cudaGetDevice(&dev);
-    if (e0 != cudaSuccess) return e0;
-    e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e0 != cudaSuccess) return e0;
+    int sms = 0;
+    const cudaError_t e = sm_count(sms);
+    if (e != cudaSuccess) return e;
     const int grid = nchunks < sms ? nchunks : sms;
-    auto go = [&](auto kern) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem);
-        if (e != cudaSuccess) return e;
-        kern<<<grid, kChainThreads, kChainSmem, st>>>(tm, p, nchunks);
-        return cudaGetLastError();
-    };
-    return hd == 64 ? go(chunk_chain_kernel<64>) : go(chunk_chain_kernel<128>);
+    return hd == 64 ? launch<chunk_chain_kernel<64>>(grid, kChainThreads, kChainSmem, st, tm, p, nchunks)
+                    : launch<chunk_chain_kernel<128>>(grid, kChainThreads, kChainSmem, st, tm, p, nchunks);
 }
 
 }  // namespace path

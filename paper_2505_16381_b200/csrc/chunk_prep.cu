@@ -26,6 +26,7 @@
 // (forward's): 27.2 k / 23.6 k, of which the inverse 8 k, 116 product steps 7.5 k (mostly underneath), E1 1.9 k, Xk and Xq
 // 3 k, U and Y 1.8 k, P, Q<- and K-> 3.9 k, the rest waits.  With the inverse in float32 loops plus one tcgen05 level and
 // rows stored and fetched by the workers: 43.5 k / 33.9 k.  Time 352 -> 225 us and 1240 -> 870 us; 128 x 2048 x 64: 278 -> 187.
+#include <type_traits>
 #include "tileops.cuh"
 
 namespace path {
@@ -285,7 +286,6 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         const int pos = (chunk_ % p.N) * kT + tid;
         return pos < p.L ? p.beta[(size_t)(chunk_ / p.N) * p.L + pos] : 0.f;
     };
-    if (tid < kT && (int)blockIdx.x < nchunks) bt[tid] = beta_floor(beta_of(blockIdx.x));
     if (HD == 64) {  // second panel of W must read as zeros when W^T is used with M = 128
         for (int i = tid; i < (int)(kPanelB / 16); i += kThreads) reinterpret_cast<uint4*>(sW + kPanelB)[i] = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
@@ -294,6 +294,10 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();
+    grid_launch();
+    if (p.clear && blockIdx.x == 0 && tid < 64) p.status[tid] = 0u;   // the workspace's status block (256 bytes)
+    if (tid < kT && (int)blockIdx.x < nchunks) bt[tid] = beta_floor(beta_of(blockIdx.x));
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t base_ = smem_u32(smem);
     constexpr int KS = HD / 16;  // k-steps over the head dimension
@@ -618,23 +622,18 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
 
 }  // namespace
 
-cudaError_t launch_chunk_prep(const PrepTensorMaps& tm, const PrepParams& p, int hd, int save, int nchunks,
+cudaError_t launch_chunk_prep(const PrepTensorMaps& tm, const PrepParams& p, int hd, int mode, int nchunks,
                               cudaStream_t st) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    const cudaError_t e = sm_count(sms);
     if (e != cudaSuccess) return e;
     const int grid = nchunks < sms ? nchunks : sms;
-    auto go = [&](auto kern) -> cudaError_t {
-        cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PrepSmem::alloc);
-        if (e2 != cudaSuccess) return e2;
-        kern<<<grid, kThreads, PrepSmem::alloc, st>>>(tm, p, nchunks);
-        return cudaGetLastError();
-    };
-    if (save == PREP_KEYS) return hd == 64 ? go(chunk_prep_kernel<64, PREP_KEYS>) : go(chunk_prep_kernel<128, PREP_KEYS>);
-    if (hd == 64) return save ? go(chunk_prep_kernel<64, PREP_SAVE>) : go(chunk_prep_kernel<64, PREP_FWD>);
-    return save ? go(chunk_prep_kernel<128, PREP_SAVE>) : go(chunk_prep_kernel<128, PREP_FWD>);
+    auto go = [&](auto which) { return launch<decltype(which)::value>(grid, kThreads, PrepSmem::alloc, st, tm, p, nchunks); };
+#define PREP(HD, MODE) go(std::integral_constant<decltype(&chunk_prep_kernel<HD, MODE>), &chunk_prep_kernel<HD, MODE>>{})
+    if (mode == PREP_KEYS) return hd == 64 ? PREP(64, PREP_KEYS) : PREP(128, PREP_KEYS);
+    if (hd == 64) return mode == PREP_SAVE ? PREP(64, PREP_SAVE) : PREP(64, PREP_FWD);
+    return mode == PREP_SAVE ? PREP(128, PREP_SAVE) : PREP(128, PREP_FWD);
+#undef PREP
 }
 
 }  // namespace path

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include "launch.cuh"
 
 namespace path {
 
@@ -180,6 +181,7 @@ struct PrepParams {
     const float* beta;            // [S][L]
     uint32_t* status;
     int N, L;                     // chunks per slice, positions per slice
+    int clear;                    // zero the status block first (the call's first kernel)
 };
 
 // `mode`: what the kernel produces (see chunk_prep.cu).
@@ -244,10 +246,11 @@ cudaError_t launch_decode_step(const void* q_t, const void* k_t, const void* v_t
                                const float* log_f_t, float* kc, void* vc, float* gc, int t, int cap, void* o_t, float* lse_t,
                                int S, int hd, float scale, float* part, cudaStream_t st);
 // Float32 forward (PATH_FP32): q, k, v, w, o are [S][L][hd] float, G the gate prefix [S][ldG] or nullptr; `scratch` holds
-// fp32_scratch_bytes(S, L, hd), or is nullptr (slower).
+// fp32_scratch_bytes(S, L, hd), or is nullptr (slower); `clear`: the
+// workspace's status block, zeroed.
 size_t fp32_scratch_bytes(int S, int L, int hd);
 cudaError_t launch_fp32_fwd(const float* q, const float* k, const float* v, const float* w, const float* beta, const float* G,
-                            float* o, float* lse, int S, int L, int ldG, int hd, float scale, float* scratch, cudaStream_t st);
+                            float* o, float* lse, int S, int L, int ldG, int hd, float scale, float* scratch, uint32_t* clear, cudaStream_t st);
 // Layer front-end (paper Sec. 2.2 footnote, Sec. 2.4 gate): z [B][L][H*hd] bf16 and logits [B][L][H] -> w [B][H][L][hd] bf16,
 // beta / log f [B][H][L]; and the backward (dcw must be zero on entry: CTAs add into it).
 cudaError_t launch_frontend_fwd(const void* z, const float* cw, const float* bl, const float* gl, void* w, float* beta,

@@ -43,6 +43,8 @@ __global__ void __launch_bounds__(32 * kWarps, 3) decode_update_kernel(
     const __nv_bfloat16* __restrict__ q_t, const __nv_bfloat16* __restrict__ k_t, const __nv_bfloat16* __restrict__ v_t,
     const __nv_bfloat16* __restrict__ w_t, const float* __restrict__ beta_t, const float* __restrict__ log_f_t, float* kc,
     __nv_bfloat16* vc, float* gc, int t, int cap, int per_cta, float scale, float* __restrict__ part) {
+    grid_wait();
+    grid_launch();
     constexpr int NP = HD / 64;          // 64-element panels per row
     constexpr int NH = 2 * kWarps;       // half-warps per CTA
     constexpr int U = 4 / NP;            // positions per half-warp and step
@@ -215,6 +217,8 @@ __global__ void __launch_bounds__(32 * kWarps, 3) decode_update_kernel(
 template <int HD>
 __global__ void __launch_bounds__(HD) decode_merge_kernel(const float* __restrict__ part, int nsplit, __nv_bfloat16* __restrict__ o_t,
                                                          float* __restrict__ lse_t) {
+    grid_wait();
+    grid_launch();
     constexpr int kAhead = 8;
     __shared__ float sf[kMaxSplits];
     __shared__ float sm_x[HD / 32], sl_x[HD / 32];
@@ -266,19 +270,19 @@ cudaError_t launch_decode_step(const void* q_t, const void* k_t, const void* v_t
     typedef __nv_bfloat16 bf;
     const int n = splits(S, t + 1), per_cta = (t + n - 1) / n;
     for (int s0 = 0; s0 < S; s0 += 65535) {   // (a grid's second dimension ends there)
-        const int ns = S - s0 < 65535 ? S - s0 : 65535;
+        const dim3 grid(n, S - s0 < 65535 ? S - s0 : 65535);
         const size_t x = (size_t)s0 * hd, y = (size_t)s0 * cap;
-        auto go = [&](auto kern) {
-            kern<<<dim3(n, ns), 32 * kWarps, 0, st>>>((const bf*)q_t + x, (const bf*)k_t + x, (const bf*)v_t + x, (const bf*)w_t + x,
-                                                      beta_t + s0, log_f_t ? log_f_t + s0 : nullptr, kc + y * hd, (bf*)vc + y * hd,
-                                                      gc ? gc + y : nullptr, t, cap, per_cta, scale, part + (size_t)s0 * n * (hd + 2));
-        };
-        if (hd == 64) go(decode_update_kernel<64>);
-        else go(decode_update_kernel<128>);
+        const bf *q = (const bf*)q_t + x, *k = (const bf*)k_t + x, *v = (const bf*)v_t + x, *w = (const bf*)w_t + x;
+        const float *b = beta_t + s0, *f = log_f_t ? log_f_t + s0 : nullptr;
+        float *kcs = kc + y * hd, *gcs = gc ? gc + y : nullptr, *ps = part + (size_t)s0 * n * (hd + 2);
+        bf* vcs = (bf*)vc + y * hd;
+        const cudaError_t e =
+            hd == 64 ? launch<decode_update_kernel<64>>(grid, 32 * kWarps, 0, st, q, k, v, w, b, f, kcs, vcs, gcs, t, cap, per_cta, scale, ps)
+                     : launch<decode_update_kernel<128>>(grid, 32 * kWarps, 0, st, q, k, v, w, b, f, kcs, vcs, gcs, t, cap, per_cta, scale, ps);
+        if (e != cudaSuccess) return e;
     }
-    if (hd == 64) decode_merge_kernel<64><<<S, 64, 0, st>>>(part, n, (bf*)o_t, lse_t);
-    else decode_merge_kernel<128><<<S, 128, 0, st>>>(part, n, (bf*)o_t, lse_t);
-    return cudaGetLastError();
+    return hd == 64 ? launch<decode_merge_kernel<64>>(S, 64, 0, st, (const float*)part, n, (bf*)o_t, lse_t)
+                    : launch<decode_merge_kernel<128>>(S, 128, 0, st, (const float*)part, n, (bf*)o_t, lse_t);
 }
 
 }  // namespace path

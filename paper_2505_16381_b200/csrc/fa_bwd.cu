@@ -172,6 +172,8 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();
+    grid_launch();
     constexpr uint32_t colS = 0, colDP = 128, colDV = 256, colDK = 384;
     // k-th work item of this CTA
     auto item_of = [&](int k, int& J, int& s) {
@@ -569,6 +571,8 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();
+    grid_launch();
     constexpr uint32_t colS = 0, colDP = 256, colDQ = 384;   // two S tiles at 0 and 128
     // k-th work item of this CTA; query chunk I has I steps (t = 0..I-1, key chunk J = I-1-t)
     auto item_of = [&](int k, int& I, int& s) {
@@ -818,6 +822,8 @@ template <int HD>
 __global__ void rowstats_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                                 const float* __restrict__ lse, const float* __restrict__ G, float* __restrict__ delta,
                                 float* __restrict__ lse2, int L, int Lp) {
+    grid_wait();
+    grid_launch();
     constexpr int TPR = HD / 8;                 // threads per row: 16 bytes (8 values) of o and of dO each
     const int s = blockIdx.y;
     const int i = blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
@@ -847,38 +853,14 @@ __global__ void rowstats_kernel(const __nv_bfloat16* __restrict__ o, const __nv_
     }
 }
 
-template <class K>
-cudaError_t set_smem(K kern, int bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
-constexpr int kDkvSmem = kSmemAlloc;
-constexpr int kDqSmem = kSmemAlloc;
-
 template <int HD, bool GATE>
 cudaError_t launch_one(const BwdTensorMaps& tm, const BwdParams& p, int which, cudaStream_t st) {
-    if (which == 0) {
-        cudaError_t e = set_smem(dkv_kernel<HD, GATE>, kDkvSmem);
-        if (e != cudaSuccess) return e;
-        int dev = 0, sms = 0;
-        e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        const int pairs = (p.N * p.S + 1) / 2;
-        dkv_kernel<HD, GATE><<<dim3(pairs < sms ? pairs : sms), 384, kDkvSmem, st>>>(tm, p);
-    } else {
-        cudaError_t e = set_smem(dq_kernel<HD, GATE>, kDqSmem);
-        if (e != cudaSuccess) return e;
-        int dev = 0, sms = 0;
-        e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        const int pairs = (p.N * p.S + 1) / 2;
-        dq_kernel<HD, GATE><<<dim3(pairs < sms ? pairs : sms), 384, kDqSmem, st>>>(tm, p);
-    }
-    return cudaGetLastError();
+    int sms = 0;
+    const cudaError_t e = sm_count(sms);
+    if (e != cudaSuccess) return e;
+    const int pairs = (p.N * p.S + 1) / 2, grid = pairs < sms ? pairs : sms;
+    return which == 0 ? launch<dkv_kernel<HD, GATE>>(grid, 384, kSmemAlloc, st, tm, p)
+                      : launch<dq_kernel<HD, GATE>>(grid, 384, kSmemAlloc, st, tm, p);
 }
 
 }  // namespace
@@ -893,11 +875,9 @@ cudaError_t launch_rowstats(const void* o, const void* d_o, const float* lse, co
                             int S, int L, int Lp, int hd, cudaStream_t st) {
     const int rows_per_cta = 256 / (hd / 8);
     dim3 grid((Lp + rows_per_cta - 1) / rows_per_cta, S);
-    if (hd == 64)
-        rowstats_kernel<64><<<grid, 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, G, delta, lse2, L, Lp);
-    else
-        rowstats_kernel<128><<<grid, 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, G, delta, lse2, L, Lp);
-    return cudaGetLastError();
+    typedef __nv_bfloat16 bf;
+    return hd == 64 ? launch<rowstats_kernel<64>>(grid, 256, 0, st, (const bf*)o, (const bf*)d_o, lse, G, delta, lse2, L, Lp)
+                    : launch<rowstats_kernel<128>>(grid, 256, 0, st, (const bf*)o, (const bf*)d_o, lse, G, delta, lse2, L, Lp);
 }
 
 }  // namespace path

@@ -267,6 +267,8 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();
+    grid_launch();
     // tensor memory columns: S of stream x at x*128 (P aliases its first 64 columns), O of stream x at 256 + x*128
     // k-th work item of this CTA: one if there are CTAs enough, otherwise pairs (long, short) of one slice, slice after slice
     const bool single = (int)gridDim.x >= items;
@@ -662,6 +664,8 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();
+    grid_launch();
     // tensor-memory columns of stream x: S at x * 128, O at 256 + x * HD, P over S or (d = 64) at 384 + x * 64
     auto colP = [](int x) { return SEP ? 384u + (uint32_t)x * 64u : (uint32_t)x * 128u; };
     auto decode = [&](int idx, int& k, int& s) {
@@ -1013,20 +1017,6 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
     }
 }
 
-static cudaError_t sm_count(int& sms) {
-    int dev = 0;
-    const cudaError_t e = cudaGetDevice(&dev);
-    return e != cudaSuccess ? e : cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-}
-
-template <class K>
-static cudaError_t launch_one(K kern, int grid, uint32_t smem, const FwdTensorMaps& tm, const FwdParams& p, cudaStream_t st) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, 384, smem, st>>>(tm, p);
-    return cudaGetLastError();
-}
-
 // Slices per group of the item list: what about 64 MB of keys, values and versions (half of L2) come from, but enough that
 // a group's items fill the GPU twice.
 static int slices_per_group(const FwdParams& p, int hd, int sms, int key_rows) {
@@ -1049,13 +1039,13 @@ static cudaError_t launch_hd(const FwdTensorMaps& tm, FwdParams p, cudaStream_t 
     // items are short and there are more chunks than SMs (S = 64, L = 512: 19 against 23 us).
     if (pairs < sms && (chunks <= sms || p.N >= 8)) {
         const int grid = chunks <= sms ? chunks : ((chunks + 1) / 2 < sms ? (chunks + 1) / 2 : sms);
-        return p.G ? launch_one(fa_split_kernel<HD, true>, grid, SplitSmem::alloc, tm, p, st)
-                   : launch_one(fa_split_kernel<HD, false>, grid, SplitSmem::alloc, tm, p, st);
+        return p.G ? launch<fa_split_kernel<HD, true>>(grid, 384, SplitSmem::alloc, st, tm, p)
+                   : launch<fa_split_kernel<HD, false>>(grid, 384, SplitSmem::alloc, st, tm, p);
     }
     p.group = slices_per_group(p, HD, sms, 2 * p.Lp + p.vl.ek * CHUNK);
     const int grid = pairs < sms ? pairs : sms;
-    return p.G ? launch_one(fa_fwd_kernel<HD, true, false>, grid, FwdSmem::alloc, tm, p, st)
-               : launch_one(fa_fwd_kernel<HD, false, false>, grid, FwdSmem::alloc, tm, p, st);
+    return p.G ? launch<fa_fwd_kernel<HD, true, false>>(grid, 384, FwdSmem::alloc, st, tm, p)
+               : launch<fa_fwd_kernel<HD, false, false>>(grid, 384, FwdSmem::alloc, st, tm, p);
 }
 
 cudaError_t launch_fa_fwd(const FwdTensorMaps& tm, const FwdParams& p, int hd, cudaStream_t st) {
@@ -1070,7 +1060,7 @@ static cudaError_t launch_cross_hd(const FwdTensorMaps& tm, FwdParams p, cudaStr
     if (!p.G || !p.Gk || p.Nk < 1) return cudaErrorInvalidValue;
     const int pairs = (p.N + 1) / 2 * p.S;
     p.group = slices_per_group(p, HD, sms, 2 * p.Lkp);
-    return launch_one(fa_fwd_kernel<HD, true, true>, pairs < sms ? pairs : sms, FwdSmem::alloc, tm, p, st);
+    return launch<fa_fwd_kernel<HD, true, true>>(pairs < sms ? pairs : sms, 384, FwdSmem::alloc, st, tm, p);
 }
 
 cudaError_t launch_fa_fwd_cross(const FwdTensorMaps& tm, const FwdParams& p, int hd, cudaStream_t st) {

@@ -12,7 +12,7 @@
 // fp32_fwd_kernel: a warp owns RW queries of one block, lane j the block's key j: two dot products per lane with rows from
 // shared memory (u0 broadcast), then the lanes turn to the head dimension for the update of u and for P V.  What bounds it
 // at the sizes it is for (a few slices, a few hundred tokens) is the chain of dependent phases of one block, L / 32 times.
-// B=1, H=2, L=256, d=64: 69.7 -> 26.6 us per call (one key per step: 520 cycles each).
+// B=1, H=2, L=256, d=64: 69.7 -> 20.5 us per call (one key per step: 520 cycles each).
 #include "common.cuh"
 
 namespace path {
@@ -34,7 +34,10 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b) {
 template <int HD>
 __global__ void __launch_bounds__(256) fp32_block_kernel(const float* __restrict__ k, const float* __restrict__ w,
                                                          const float* __restrict__ beta, float* __restrict__ kr,
-                                                         float* __restrict__ wt, float* __restrict__ ym, int L) {
+                                                         float* __restrict__ wt, float* __restrict__ ym, uint32_t* clear, int L) {
+    grid_wait();
+    grid_launch();
+    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 64) clear[threadIdx.x] = 0u;   // the workspace's status block
     constexpr int LD = ld<HD>(), LC = kBlk + 4;
     __shared__ __align__(16) float sw[kBlk][LD], sk[kBlk][LD], sc[kBlk][LC], skw[kBlk][LC];
     __shared__ float sb[kBlk];
@@ -133,6 +136,8 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
                                                                const float* __restrict__ ym, const float* __restrict__ G,
                                                                float* __restrict__ o, float* __restrict__ lse, int S, int L,
                                                                int ldG, float scale) {
+    grid_wait();
+    grid_launch();
     constexpr int LD = ld<HD>(), E = HD / 32, TILE = kBlk * LD, GROUPS = kBlk / (kWarps * RW);
     extern __shared__ __align__(16) float sm[];      // [2 stages][W, Kr, Wt, V][32][LD], then per warp u [RW][HD], t and p [RW][32]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -296,6 +301,8 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) fp32_walk_kernel(const float
                                                                    const float* __restrict__ beta, const float* __restrict__ G,
                                                                    float* __restrict__ o, float* __restrict__ lse, int S, int L,
                                                                    int ldG, float scale) {
+    grid_wait();
+    grid_launch();
     constexpr int E = HD / 32;   // elements per lane
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nblk = (L + kRowsPerCta - 1) / kRowsPerCta;
@@ -377,17 +384,14 @@ template <int HD, int RW>
 cudaError_t launch_rows(const float* q, const float* k, const float* v, const float* w, const float* kr, const float* wt,
                         const float* ym, const float* G, float* o, float* lse, int S, int L, int ldG, float scale, cudaStream_t st) {
     const int smem = (8 * kBlk * ld<HD>() + kWarps * RW * (HD + 2 * kBlk)) * 4;
-    const cudaError_t e = cudaFuncSetAttribute(fp32_fwd_kernel<HD, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
     const int nblk = (L + kBlk - 1) / kBlk;
-    fp32_fwd_kernel<HD, RW><<<(unsigned)((size_t)S * nblk * (kBlk / (kWarps * RW))), 32 * kWarps, smem, st>>>(
-        q, k, v, w, kr, wt, ym, G, o, lse, S, L, ldG, scale);
-    return cudaGetLastError();
+    return launch<fp32_fwd_kernel<HD, RW>>((unsigned)((size_t)S * nblk * (kBlk / (kWarps * RW))), 32 * kWarps, smem, st, q, k, v, w, kr,
+                                           wt, ym, G, o, lse, S, L, ldG, scale);
 }
 
 template <int HD>
 cudaError_t launch_hd(const float* q, const float* k, const float* v, const float* w, const float* beta, const float* G, float* o,
-                      float* lse, int S, int L, int ldG, float scale, float* scratch, cudaStream_t st) {
+                      float* lse, int S, int L, int ldG, float scale, float* scratch, uint32_t* clear, cudaStream_t st) {
     const size_t nblk = (L + kBlk - 1) / kBlk, rows = (size_t)S * nblk * kBlk;
     float* kr = scratch;
     float* wt = kr + rows * HD;
@@ -395,9 +399,8 @@ cudaError_t launch_hd(const float* q, const float* k, const float* v, const floa
     for (int s0 = 0; s0 < S; s0 += 65535) {   // (a grid's second dimension ends there)
         const int ns = S - s0 < 65535 ? S - s0 : 65535;
         const size_t in = (size_t)s0 * L, out = (size_t)s0 * nblk * kBlk;
-        fp32_block_kernel<HD><<<dim3((unsigned)nblk, ns), 256, 0, st>>>(k + in * HD, w + in * HD, beta + in, kr + out * HD, wt + out * HD,
-                                                                      ym + out * kBlk, L);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch<fp32_block_kernel<HD>>(dim3((unsigned)nblk, ns), 256, 0, st, k + in * HD, w + in * HD, beta + in,
+                                                            kr + out * HD, wt + out * HD, ym + out * kBlk, s0 == 0 ? clear : nullptr, L);
         if (e != cudaSuccess) return e;
     }
     // One query per warp while that still leaves SMs without work; four share a warp's tile reads otherwise.
@@ -413,15 +416,16 @@ size_t fp32_scratch_bytes(int S, int L, int hd) {
 }
 
 cudaError_t launch_fp32_fwd(const float* q, const float* k, const float* v, const float* w, const float* beta, const float* G,
-                            float* o, float* lse, int S, int L, int ldG, int hd, float scale, float* scratch, cudaStream_t st) {
+                            float* o, float* lse, int S, int L, int ldG, int hd, float scale, float* scratch, uint32_t* clear, cudaStream_t st) {
     if (!scratch) {
         const dim3 grid((unsigned)((size_t)S * ((L + kRowsPerCta - 1) / kRowsPerCta)));
-        if (hd == 64) fp32_walk_kernel<64><<<grid, 32 * kRowsPerCta, 0, st>>>(q, k, v, w, beta, G, o, lse, S, L, ldG, scale);
-        else fp32_walk_kernel<128><<<grid, 32 * kRowsPerCta, 0, st>>>(q, k, v, w, beta, G, o, lse, S, L, ldG, scale);
-        return cudaGetLastError();
+        const cudaError_t e = cudaMemsetAsync(clear, 0, 256, st);
+        if (e != cudaSuccess) return e;
+        return hd == 64 ? launch<fp32_walk_kernel<64>>(grid, 32 * kRowsPerCta, 0, st, q, k, v, w, beta, G, o, lse, S, L, ldG, scale)
+                        : launch<fp32_walk_kernel<128>>(grid, 32 * kRowsPerCta, 0, st, q, k, v, w, beta, G, o, lse, S, L, ldG, scale);
     }
-    return hd == 64 ? launch_hd<64>(q, k, v, w, beta, G, o, lse, S, L, ldG, scale, scratch, st)
-                    : launch_hd<128>(q, k, v, w, beta, G, o, lse, S, L, ldG, scale, scratch, st);
+    return hd == 64 ? launch_hd<64>(q, k, v, w, beta, G, o, lse, S, L, ldG, scale, scratch, clear, st)
+                    : launch_hd<128>(q, k, v, w, beta, G, o, lse, S, L, ldG, scale, scratch, clear, st);
 }
 
 }  // namespace path

@@ -48,6 +48,8 @@ __device__ __forceinline__ void setup(Ctx& c, uint8_t* smem_raw, uint32_t bar_of
     tc_fence_after_sync();
     c.tmem = *tmem_slot;
     c.tl = c.tmem + ((uint32_t)((c.warp & 3) * 32) << 16);
+    grid_wait();
+    grid_launch();
 }
 template <int NCOLS>
 __device__ __forceinline__ void teardown(Ctx& c, uint32_t* status) {
@@ -297,6 +299,7 @@ __device__ __forceinline__ int highest_level_reached(const LevelParams& p, int i
 template <int HD>
 __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int is_key = blockIdx.y, s = blockIdx.x / p.N, ch = blockIdx.x % p.N;
+    grid_wait();   // (the block-skipping counts)
     // levels to build: all of them, or for a gated problem up to the highest one a kept chunk pair uses (see level_bwd)
     const int lim = min(p.l, highest_level_reached(p, is_key, s, ch) + 1);
     int l1, b, src, l2 = 1;
@@ -370,6 +373,7 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
 template <int HD>
 __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int l1 = p.l, cnt = p.lv.dy_cnt[l1];
+    grid_wait();   // (the block-skipping counts, and the zeros below)
     const int s = blockIdx.x / cnt, b = blockIdx.x % cnt;
     const long mat = p.lv.dy_off[l1] / (HD * HD) + (long)s * cnt + b;
     const int is_key = b & 1;
@@ -717,15 +721,6 @@ __global__ void __launch_bounds__(256, 2) apply_product_kernel(const __grid_cons
     teardown<128>(c, p.status);
 }
 
-template <class K>
-cudaError_t launch(K kern, dim3 grid, uint32_t slots, const LevelTensorMaps& tm, const LevelParams& p, cudaStream_t st) {
-    const uint32_t bytes = smem_bytes(slots);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, 256, bytes, st>>>(tm, p);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const LevelParams& p, int hd, cudaStream_t st) {
@@ -733,35 +728,35 @@ cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const Leve
         case LEVEL_DYADIC_FUSED: {
             const int half_w = 1 << (p.fuse - 1);
             dim3 g(p.S * ((p.lv.dy_cnt[p.l + 1] + half_w - 1) / half_w));
-            return hd == 64 ? launch(dyadic_fused_kernel<64>, g, 6, tm, p, st) : launch(dyadic_fused_kernel<128>, g, 6, tm, p, st);
+            return hd == 64 ? launch<dyadic_fused_kernel<64>>(g, 256, smem_bytes(6), st, tm, p) : launch<dyadic_fused_kernel<128>>(g, 256, smem_bytes(6), st, tm, p);
         }
         case LEVEL_DYADIC_FWD: {
             dim3 g(p.S * p.lv.dy_cnt[p.l + 1]);
-            return hd == 64 ? launch(dyadic_fwd_kernel<64>, g, 4, tm, p, st) : launch(dyadic_fwd_kernel<128>, g, 4, tm, p, st);
+            return hd == 64 ? launch<dyadic_fwd_kernel<64>>(g, 256, smem_bytes(4), st, tm, p) : launch<dyadic_fwd_kernel<128>>(g, 256, smem_bytes(4), st, tm, p);
         }
         case LEVEL_VERSION_FWD: {
             dim3 g(p.S * p.N, 2);
-            return hd == 64 ? launch(version_fwd_kernel<64>, g, 3, tm, p, st) : launch(version_fwd_kernel<128>, g, 3, tm, p, st);
+            return hd == 64 ? launch<version_fwd_kernel<64>>(g, 256, smem_bytes(3), st, tm, p) : launch<version_fwd_kernel<128>>(g, 256, smem_bytes(3), st, tm, p);
         }
         case LEVEL_BWD: {
             dim3 g(p.S * p.lv.dy_cnt[p.l]);
-            return hd == 64 ? launch(level_bwd_kernel<64>, g, 7, tm, p, st) : launch(level_bwd_kernel<128>, g, 7, tm, p, st);
+            return hd == 64 ? launch<level_bwd_kernel<64>>(g, 256, smem_bytes(7), st, tm, p) : launch<level_bwd_kernel<128>>(g, 256, smem_bytes(7), st, tm, p);
         }
         case LEVEL_KEY_CACHE: {
             dim3 g(p.S, hd / 64, p.nseg > 1 ? p.nseg : 1);
-            return hd == 64 ? launch(key_cache_kernel<64, false>, g, 5, tm, p, st) : launch(key_cache_kernel<128, false>, g, 5, tm, p, st);
+            return hd == 64 ? launch<key_cache_kernel<64, false>>(g, 256, smem_bytes(5), st, tm, p) : launch<key_cache_kernel<128, false>>(g, 256, smem_bytes(5), st, tm, p);
         }
         case LEVEL_QUERY_EDGE: {
             dim3 g(p.S, hd / 64);
-            return hd == 64 ? launch(key_cache_kernel<64, true>, g, 5, tm, p, st) : launch(key_cache_kernel<128, true>, g, 5, tm, p, st);
+            return hd == 64 ? launch<key_cache_kernel<64, true>>(g, 256, smem_bytes(5), st, tm, p) : launch<key_cache_kernel<128, true>>(g, 256, smem_bytes(5), st, tm, p);
         }
         case LEVEL_SUFFIX: {
             dim3 g(p.S, hd / 64);
-            return hd == 64 ? launch(suffix_kernel<64>, g, 4, tm, p, st) : launch(suffix_kernel<128>, g, 4, tm, p, st);
+            return hd == 64 ? launch<suffix_kernel<64>>(g, 256, smem_bytes(4), st, tm, p) : launch<suffix_kernel<128>>(g, 256, smem_bytes(4), st, tm, p);
         }
         case LEVEL_APPLY_PRODUCT: {
             dim3 g(p.S * p.N);
-            return hd == 64 ? launch(apply_product_kernel<64>, g, 3, tm, p, st) : launch(apply_product_kernel<128>, g, 3, tm, p, st);
+            return hd == 64 ? launch<apply_product_kernel<64>>(g, 256, smem_bytes(3), st, tm, p) : launch<apply_product_kernel<128>>(g, 256, smem_bytes(3), st, tm, p);
         }
         default:
             return cudaErrorInvalidValue;

@@ -8,6 +8,8 @@ namespace path {
 namespace {
 
 __global__ void pad_rows_kernel(const void* __restrict__ src, void* __restrict__ dst, int L, int Lp, int rowbytes16) {
+    grid_wait();
+    grid_launch();
     // one 16-byte vector per thread; grid.y = slice, grid.x covers Lp * rowbytes16
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const long total = (long)Lp * rowbytes16;
@@ -20,7 +22,10 @@ __global__ void pad_rows_kernel(const void* __restrict__ src, void* __restrict__
 
 // One CTA (1024 threads) per slice: each thread scans a contiguous segment, then a block scan of the segment sums.
 __global__ void __launch_bounds__(1024) gate_prefix_kernel(const float* __restrict__ g, float* __restrict__ G, int L,
-                                                           int Lp) {
+                                                           int Lp, uint32_t* clear) {
+    grid_wait();
+    grid_launch();
+    if (clear && blockIdx.x == 0 && threadIdx.x < 64) clear[threadIdx.x] = 0u;   // the workspace's status block (256 bytes)
     __shared__ float part[1024];
     const int tid = threadIdx.x;
     const int seg = (Lp + 1023) / 1024;
@@ -46,6 +51,8 @@ __global__ void __launch_bounds__(1024) gate_prefix_kernel(const float* __restri
 
 // rs[chunk*128 + i] = sum_k dsd[chunk][i][k]; one warp per row (a lane reads four adjacent entries), four rows in flight.
 __global__ void __launch_bounds__(256) dsd_rowsum_kernel(const float* __restrict__ dsd, float* __restrict__ rs) {
+    grid_wait();
+    grid_launch();
     const float4* base = reinterpret_cast<const float4*>(dsd + (size_t)blockIdx.x * CHUNK * CHUNK);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll 1
@@ -69,6 +76,8 @@ __global__ void __launch_bounds__(256) dsd_rowsum_kernel(const float* __restrict
 __global__ void __launch_bounds__(1024) gate_suffix_kernel(const float* __restrict__ dGa, const float* __restrict__ dGb,
                                                            const float* __restrict__ dGc, float* __restrict__ out, int L,
                                                            int Lp) {
+    grid_wait();
+    grid_launch();
     __shared__ float part[1024];
     const int tid = threadIdx.x;
     const int seg = (L + 1023) / 1024;
@@ -108,6 +117,8 @@ __global__ void __launch_bounds__(256) tile_stats_kernel(const __nv_bfloat16* __
                                                         const __nv_bfloat16* __restrict__ w, const float* __restrict__ beta,
                                                         const float* __restrict__ G, float* __restrict__ stats, int L, int Lp,
                                                         int hd, float scale) {
+    grid_wait();
+    grid_launch();
     __shared__ float red[8][6];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lpr = hd / 8, grp = lane / lpr, li = lane % lpr, rows_w = 32 / lpr;
@@ -169,6 +180,8 @@ __global__ void __launch_bounds__(256) tile_stats_kernel(const __nv_bfloat16* __
 
 __global__ void __launch_bounds__(128) tile_keep_kernel(const float* __restrict__ stats, int* __restrict__ nkeep, int S, int N,
                                                        float ascale) {
+    grid_wait();
+    grid_launch();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= S * N) return;
     const int sl = idx / N, I = idx % N;
@@ -192,6 +205,8 @@ __global__ void __launch_bounds__(128) tile_keep_kernel(const float* __restrict_
 // reaches.  Also counts the kept pairs.
 __global__ void __launch_bounds__(128) tile_stair_kernel(int* __restrict__ nkeep, int* __restrict__ nvisit,
                                                         unsigned long long* counters, int S, int N) {
+    grid_wait();
+    grid_launch();
     // one CTA per slice; the two serial scans run on a copy in shared memory when it fits (N <= kStairMax chunks, i.e.
     // sequences up to a million tokens), else directly on global memory
     constexpr int kStairMax = 8192;
@@ -244,6 +259,8 @@ __global__ void __launch_bounds__(128) tile_stair_kernel(int* __restrict__ nkeep
 // ---- context-parallel path: gate terms of a segment, merge of partial softmax results
 __global__ void cp_gate_kernel(const float* __restrict__ G, float* __restrict__ gq, float* __restrict__ gk,
                                float* __restrict__ gtot, int L, int Lp) {
+    grid_wait();
+    grid_launch();
     const int s = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
     const float tot = G ? G[(size_t)s * Lp + L - 1] : 0.f;
     if (i == 0) gtot[s] = tot;
@@ -255,6 +272,8 @@ __global__ void cp_gate_kernel(const float* __restrict__ G, float* __restrict__ 
 // one thread per 4 outputs of a row
 __global__ void cp_merge_kernel(float* __restrict__ o_acc, float* __restrict__ lse_acc, const float* __restrict__ o_t,
                                 const float* __restrict__ lse_t, size_t rows, int hd4) {
+    grid_wait();
+    grid_launch();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * hd4) return;
     const size_t r = i / hd4;
@@ -269,6 +288,8 @@ __global__ void cp_merge_kernel(float* __restrict__ o_acc, float* __restrict__ l
 }
 __global__ void cp_finish_kernel(const float* __restrict__ o_acc, const float* __restrict__ lse_acc, __nv_bfloat16* __restrict__ o,
                                  float* __restrict__ lse, size_t rows, int hd4) {
+    grid_wait();
+    grid_launch();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * hd4) return;
     const float4 a = reinterpret_cast<const float4*>(o_acc)[i];
@@ -279,9 +300,15 @@ __global__ void cp_finish_kernel(const float* __restrict__ o_acc, const float* _
 
 // ---- forward-state record and the wait self-test
 __global__ void state_write_kernel(StateRecord* dst, const StateRecord rec) {
+    grid_wait();
+    grid_launch();
     if (threadIdx.x == 0) *dst = rec;
 }
 __global__ void state_check_kernel(const StateRecord* have, const StateRecord want, uint32_t* status) {
+    grid_wait();
+    grid_launch();
+    if (threadIdx.x < 8) status[threadIdx.x] = 0u;   // the status word and the sweeps' item counters; the rest is the forward's
+    __syncwarp();
     if (threadIdx.x != 0) return;
     const StateRecord h = *have;
     const bool same = h.magic == want.magic && h.q == want.q && h.k == want.k && h.v == want.v && h.w == want.w &&
@@ -312,25 +339,21 @@ __global__ void selftest_wait_kernel(uint32_t* status, long long ticks) {
 
 cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* dGc, float* out, int S, int L, int Lp,
                                cudaStream_t st) {
-    gate_suffix_kernel<<<S, 1024, 0, st>>>(dGa, dGb, dGc, out, L, Lp);
-    return cudaGetLastError();
+    return launch<gate_suffix_kernel>(S, 1024, 0, st, dGa, dGb, dGc, out, L, Lp);
 }
 cudaError_t launch_dsd_rowsum(const float* dsd, float* rs, int nchunks, cudaStream_t st) {
-    dsd_rowsum_kernel<<<nchunks, 256, 0, st>>>(dsd, rs);
-    return cudaGetLastError();
+    return launch<dsd_rowsum_kernel>(nchunks, 256, 0, st, dsd, rs);
 }
 
 cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, int f32, cudaStream_t st) {
     const int rowbytes16 = d * (f32 ? 4 : 2) / 16;
     const long total = (long)Lp * rowbytes16;
     dim3 grid((unsigned)((total + 255) / 256), S);
-    pad_rows_kernel<<<grid, 256, 0, st>>>(src, dst, L, Lp, rowbytes16);
-    return cudaGetLastError();
+    return launch<pad_rows_kernel>(grid, 256, 0, st, src, dst, L, Lp, rowbytes16);
 }
 
-cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, cudaStream_t st) {
-    gate_prefix_kernel<<<S, 1024, 0, st>>>(g, G, L, Lp);
-    return cudaGetLastError();
+cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, uint32_t* clear, cudaStream_t st) {
+    return launch<gate_prefix_kernel>(S, 1024, 0, st, g, G, L, Lp, clear);
 }
 
 cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const float* beta, const float* G, float* stats,
@@ -338,44 +361,35 @@ cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const 
                              cudaStream_t st) {
     typedef __nv_bfloat16 bf;
     const int N = Lp / CHUNK;
-    tile_stats_kernel<<<S * N, 256, 0, st>>>((const bf*)q, (const bf*)k, (const bf*)w, beta, G, stats, L, Lp, hd, scale);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch<tile_stats_kernel>(S * N, 256, 0, st, (const bf*)q, (const bf*)k, (const bf*)w, beta, G, stats, L, Lp, hd, scale);
     if (e != cudaSuccess) return e;
-    tile_keep_kernel<<<(S * N + 127) / 128, 128, 0, st>>>(stats, nkeep, S, N, fabsf(scale));
-    e = cudaGetLastError();
+    e = launch<tile_keep_kernel>((S * N + 127) / 128, 128, 0, st, stats, nkeep, S, N, fabsf(scale));
     if (e != cudaSuccess) return e;
-    tile_stair_kernel<<<S, 128, 0, st>>>(nkeep, nvisit, counters, S, N);
-    return cudaGetLastError();
+    return launch<tile_stair_kernel>(S, 128, 0, st, nkeep, nvisit, counters, S, N);
 }
 
 cudaError_t launch_cp_gate(const float* G, float* gq, float* gk, float* gtot, int S, int L, int Lp, cudaStream_t st) {
-    cp_gate_kernel<<<dim3((Lp + 255) / 256, S), 256, 0, st>>>(G, gq, gk, gtot, L, Lp);
-    return cudaGetLastError();
+    return launch<cp_gate_kernel>(dim3((Lp + 255) / 256, S), 256, 0, st, G, gq, gk, gtot, L, Lp);
 }
 cudaError_t launch_cp_merge(float* o_acc, float* lse_acc, const float* o_t, const float* lse_t, size_t rows, int hd,
                             cudaStream_t st) {
     const size_t n = rows * (hd / 4);
-    cp_merge_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(o_acc, lse_acc, o_t, lse_t, rows, hd / 4);
-    return cudaGetLastError();
+    return launch<cp_merge_kernel>((unsigned)((n + 255) / 256), 256, 0, st, o_acc, lse_acc, o_t, lse_t, rows, hd / 4);
 }
 cudaError_t launch_cp_finish(const float* o_acc, const float* lse_acc, void* o, float* lse, size_t rows, int hd,
                              cudaStream_t st) {
     const size_t n = rows * (hd / 4);
-    cp_finish_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(o_acc, lse_acc, (__nv_bfloat16*)o, lse, rows, hd / 4);
-    return cudaGetLastError();
+    return launch<cp_finish_kernel>((unsigned)((n + 255) / 256), 256, 0, st, o_acc, lse_acc, (__nv_bfloat16*)o, lse, rows, hd / 4);
 }
 
 cudaError_t launch_state_write(void* record, const StateRecord& rec, cudaStream_t st) {
-    state_write_kernel<<<1, 32, 0, st>>>((StateRecord*)record, rec);
-    return cudaGetLastError();
+    return launch<state_write_kernel>(1, 32, 0, st, (StateRecord*)record, rec);
 }
 cudaError_t launch_state_check(const void* record, const StateRecord& want, uint32_t* status, cudaStream_t st) {
-    state_check_kernel<<<1, 32, 0, st>>>((const StateRecord*)record, want, status);
-    return cudaGetLastError();
+    return launch<state_check_kernel>(1, 32, 0, st, (const StateRecord*)record, want, status);
 }
 cudaError_t launch_selftest_wait(uint32_t* status, long long ticks, cudaStream_t st) {
-    selftest_wait_kernel<<<1, 32, 0, st>>>(status, ticks);
-    return cudaGetLastError();
+    return (selftest_wait_kernel<<<1, 32, 0, st>>>(status, ticks), cudaGetLastError());
 }
 
 }  // namespace path

@@ -7,8 +7,8 @@ namespace path {
 
 // dst[S][Lp][d] <- src[S][L][d] (zero tail); bf16 elements when !f32.
 cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, int f32, cudaStream_t st);
-// G[S][Lp] <- inclusive prefix sum of g[S][L] (tail repeats the last value).
-cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, cudaStream_t st);
+// G[S][Lp] <- inclusive prefix sum of g[S][L] (tail repeats the last value).  `clear` (or nullptr): 256 bytes to zero on the way.
+cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, uint32_t* clear, cudaStream_t st);
 
 // out[S][L] <- reverse inclusive prefix sum of (dGa + dGb + dGc)[S][Lp] over positions < L.
 cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* dGc, float* out, int S, int L, int Lp,

@@ -256,7 +256,7 @@ static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const
             return PATH_ERR_LAUNCH;
         }
         PrepParams pp{};
-        pp.beta = beta; pp.N = p.N; pp.L = p.L;
+        pp.beta = beta; pp.N = p.N; pp.L = p.L; pp.clear = !p.gate;   // (gated: the gate prefix has done it)
         if (!(make_map(&tm.ql, at<void>(ws, p.Qv16), rows, d) && make_map(&tm.kr, at<void>(ws, p.Kv16), rows, d) &&
               make_map(&tm.xq, at<void>(ws, p.Xq), rows, CHUNK) && make_map(&tm.y, at<void>(ws, p.Y), rows, CHUNK) &&
               make_map_box(&tm.ph, at<void>(ws, p.Dyh), (uint64_t)nch * d, d, d) &&
@@ -294,9 +294,22 @@ static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const
     return PATH_OK;
 }
 
+// A thread that has made no CUDA call yet (an autograd worker) has no current context, which encoding a tensor map needs.
+static cudaError_t bind_context(int dev) {
+    typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
+    static const CtxGetCurrentFn get = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        return cudaGetDriverEntryPoint("cuCtxGetCurrent", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess
+                   ? (CtxGetCurrentFn)p : (CtxGetCurrentFn) nullptr;
+    }();
+    CUcontext c = nullptr;
+    return get && get(&c) == CUDA_SUCCESS && c ? cudaSuccess : cudaSetDevice(dev);
+}
+
 static int check_arch() {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return PATH_ERR_LAUNCH;
+    if (cudaGetDevice(&dev) != cudaSuccess || bind_context(dev) != cudaSuccess) return PATH_ERR_LAUNCH;
     int major = 0;
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return PATH_ERR_LAUNCH;
     return major == 10 ? PATH_OK : PATH_ERR_ARCH;
@@ -421,14 +434,13 @@ int path_attn_fwd(const void* q, const void* k, const void* v, const void* w, co
         int rc32 = check_arch();
         if (rc32 != PATH_OK) return rc32;
         cudaStream_t st32 = (cudaStream_t)cuda_stream;
-        CK(cudaMemsetAsync(workspace, 0, 256, st32));
         float* G = nullptr;
         if (log_f) {
             G = at<float>(workspace, p.G);
-            LAUNCH(launch_gate_prefix(log_f, G, p.S, L, p.Lp, st32));
+            LAUNCH(launch_gate_prefix(log_f, G, p.S, L, p.Lp, nullptr, st32));
         }
         LAUNCH(launch_fp32_fwd((const float*)q, (const float*)k, (const float*)v, (const float*)w, beta, G, (float*)o, lse,
-                               p.S, L, p.Lp, d, scale, tiles ? at<float>(workspace, p.f32) : nullptr, st32));
+                               p.S, L, p.Lp, d, scale, tiles ? at<float>(workspace, p.f32) : nullptr, at<uint32_t>(workspace, p.status), st32));
         if (tiles) ++g_launches;
         return PATH_OK;
     }
@@ -447,11 +459,10 @@ int path_attn_fwd(const void* q, const void* k, const void* v, const void* w, co
     int rc = check_arch();
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    CK(cudaMemsetAsync(workspace, 0, 256, st));
-
+    // (the call's first kernel, the gate prefix or the chunk preparation, clears the status block)
     prof_reset(STG_PREP, STG_PREP_BWD);
     if (log_f) {
-        LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
+        LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, at<uint32_t>(workspace, p.status), st));
         rc = run_gate_skip(p, workspace, q, k, w, beta, scale, st);
         if (rc != PATH_OK) return rc;
     }
@@ -499,8 +510,6 @@ static int backward_entry(const void* q, const void* k, const void* v, const voi
     int rc = check_arch();
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // the status word, and what a reused forward left only if it is not reused: the block-skipping counters and the record
-    CK(cudaMemsetAsync(workspace, 0, reuse ? kSkipCounterOffset : 256, st));
     prof_reset(STG_PREP_BWD, STG_COUNT);
     if (reuse) {
         // the record the forward left must describe this very problem (for a gated one the scale too: the block-skipping
@@ -510,7 +519,7 @@ static int backward_entry(const void* q, const void* k, const void* v, const voi
     }
     if (!reuse) {
         if (log_f) {
-            LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
+            LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, at<uint32_t>(workspace, p.status), st));
             rc = run_gate_skip(p, workspace, q, k, w, beta, scale, st);
             if (rc != PATH_OK) return rc;
         }
@@ -660,9 +669,8 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
     int rc = check_arch();
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    CK(cudaMemsetAsync(workspace, 0, 256, st));
     if (log_f) {
-        LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
+        LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, at<uint32_t>(workspace, p.status), st));
         rc = run_gate_skip(p, workspace, q, k, w, beta, scale, st);
         if (rc != PATH_OK) return rc;
     }
@@ -783,8 +791,7 @@ int path_attn_prefill_cache(const void* k, const void* v, const void* w, const f
     int rc = check_arch();
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    CK(cudaMemsetAsync(workspace, 0, 256, st));
-    if (log_f) LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, st));
+    if (log_f) LAUNCH(launch_gate_prefix(log_f, at<float>(workspace, p.G), p.S, p.L, p.Lp, at<uint32_t>(workspace, p.status), st));
     // the chunk preparation needs no queries for the key side: the keys stand in for them
     rc = run_prep(p, workspace, k, k, w, beta, false, st, false, true);
     if (rc != PATH_OK) return rc;
