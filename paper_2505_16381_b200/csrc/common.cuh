@@ -220,7 +220,7 @@ struct BwdParams {
     __nv_bfloat16* dqv;  // gradients of the query versions (placed like the versions), bf16
     __nv_bfloat16* dkv;  // same for the key versions
     void* dv;            // [S, L, d] bf16, final
-    float* dsd;          // [S*N][128 q][128 k] lower(dS) of the diagonal chunks, unscaled; written for gated problems only
+    float* dsd;          // [S*N][4][128 q] row sums of lower(dS) of the diagonal chunks, by quarters of the keys; gated problems only
     __nv_bfloat16* dsdt; // [S*N][128 k][128 q] (scale * lower(dS))^T in bf16: the chain rule's operand
     float* dG;           // [S][Lp] minus the column sums of dS (gated problems only)
     float* dGrow;        // [S][Lp] row sums of dS over the off-diagonal chunks (gated problems only)

@@ -6,7 +6,7 @@
 //   dQv[l][I] = scale sum_{J at level l} dS Kv[l][J]
 //   gate prefix:  dG_m = sum_j dS_mj - sum_i dS_im  (row sums are written by dq_kernel, column sums by dkv_kernel;
 //                 the row sums vanish in exact arithmetic but cancel the rounding of delta in the suffix sums)
-//   diagonal chunk: dSd = lower(dS) (unscaled) is stored for the per-chunk chain rule.
+//   diagonal chunk: (scale lower(dS))^T is stored for the per-chunk chain rule; its row sums in float32 if gated.
 //
 // Two kernels so that every accumulator stays in tensor memory and nothing is added atomically:
 //   dkv_kernel: one CTA per key chunk J, sweeps the query chunks I = J..N-1 with transposed tiles
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
             store_acc_bf16<CW>(p.dkv + ((size_t)krow(lvl, J) + row) * HD + h * CW, tlane + colDK + h * CW, p.scale);
         };
         auto step = [&](auto first_tag, const int t) {
-            constexpr bool FIRST = decltype(first_tag)::value;   // the diagonal chunk: causal mask, dSd written out
+            constexpr bool FIRST = decltype(first_tag)::value;   // the diagonal chunk: causal mask, dS^T written out
             const int gs = g + t;                                // running step number: ring slot and phase
             const float* st_ = rowstat + (gs & 1) * 2 * kTile;   // [0,128): -lse2 (+gate), [128,256): -delta of the queries
             const int c0 = h * 64;               // query columns of this thread
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                         if (GATE) dsum += (d[0] + d[1]) + (d[2] + d[3]);
                         pk[x >> 1] = pack_bf16(d[0], d[1]);
                         pk[(x >> 1) + 1] = pack_bf16(d[2], d[3]);
-                        if (FIRST) {   // (scale * dS)^T of the diagonal chunk for the chain rule; unscaled float copy if gated
+                        if (FIRST) {   // (scale * dS)^T of the diagonal chunk for the chain rule; and float32 row sums if gated
                             dsw[c * 16 + (x >> 1)] = pack_bf16(d[0] * p.scale, d[1] * p.scale);
                             dsw[c * 16 + (x >> 1) + 1] = pack_bf16(d[2] * p.scale, d[3] * p.scale);
                             if (GATE) {
@@ -437,10 +437,16 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                         }
                     }
                     tmem_st16(tlane + colDP + c0 + c * 16, pk);
-                    if (FIRST && GATE) {
-                        float* dsd = p.dsd + ((size_t)(s * p.N + J) * kTile) * kTile;
+                    if (FIRST && GATE) {   // row sums of dS over this warp's 32 keys: lane q of the warp ends up with query column q
 #pragma unroll
-                        for (int x = 0; x < 32; ++x) dsd[(size_t)(c0 + c * 32 + x) * kTile + row] = __uint_as_float(dp[x]);
+                        for (int off = 16; off >= 1; off >>= 1)
+#pragma unroll
+                            for (int x = 0; x < off; ++x) {
+                                const bool up = lane & off;
+                                const float keep = __uint_as_float(up ? dp[x + off] : dp[x]), give = __uint_as_float(up ? dp[x] : dp[x + off]);
+                                dp[x] = __float_as_uint(keep + __shfl_xor_sync(0xffffffffu, give, off));
+                            }
+                        p.dsd[((size_t)(s * p.N + J) * 4 + q4) * kTile + c0 + c * 32 + lane] = __uint_as_float(dp[0]);
                     }
                 }
                 tmem_st_wait();

@@ -1,5 +1,5 @@
 // Memory-bound helpers: zero-padding of ragged inputs, prefix sum of the log gate (PaTH-FoX, paper Sec. 2.2),
-// suffix sum of its gradient, row sums of the diagonal-chunk dS.
+// suffix sum of its gradient, block skipping.
 #include "linear.cuh"
 #include "tc5.cuh"
 
@@ -20,84 +20,86 @@ __global__ void pad_rows_kernel(const void* __restrict__ src, void* __restrict__
     ((uint4*)dst)[((long)blockIdx.y * Lp + row) * rowbytes16 + col] = v;
 }
 
-// One CTA (1024 threads) per slice: each thread scans a contiguous segment, then a block scan of the segment sums.
+// Inclusive scan of `x` over a CTA of 1024 threads; `total` = the sum over all of them.
+__device__ __forceinline__ float block_scan(float x, float* part, float& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+    }
+    if (lane == 31) part[warp] = x;
+    __syncthreads();
+    float w = part[lane];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, w, off);
+        if (lane >= off) w += y;
+    }
+    total = __shfl_sync(0xffffffffu, w, 31);
+    const float before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    __syncthreads();   // (`part` is written again by the next call)
+    return warp > 0 ? x + before : x;
+}
+
+// One CTA (1024 threads) per slice, 4096 positions at a time, four neighbouring ones per thread.  Latency-bound (32 KB per
+// slice).  One contiguous segment per thread with a shared-memory scan of 20 barriers took 32 us at 32 slices x 8192 positions;
+// the warp scans of this file together take 47 us off the training step of that shape and 27 us off one of 16 x 3001 x 64.
 __global__ void __launch_bounds__(1024) gate_prefix_kernel(const float* __restrict__ g, float* __restrict__ G, int L,
                                                            int Lp, uint32_t* clear) {
     grid_wait();
     grid_launch();
     if (clear && blockIdx.x == 0 && threadIdx.x < 64) clear[threadIdx.x] = 0u;   // the workspace's status block (256 bytes)
-    __shared__ float part[1024];
-    const int tid = threadIdx.x;
-    const int seg = (Lp + 1023) / 1024;
-    const int lo = tid * seg, hi = min(lo + seg, Lp);
+    __shared__ float part[32];
     const float* gs = g + (size_t)blockIdx.x * L;
     float* Gs = G + (size_t)blockIdx.x * Lp;
-    float acc = 0.f;
-    for (int i = lo; i < hi; ++i) acc += (i < L) ? gs[i] : 0.f;
-    part[tid] = acc;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        float v = (tid >= off) ? part[tid - off] : 0.f;
-        __syncthreads();
-        part[tid] += v;
-        __syncthreads();
-    }
-    acc = (tid > 0) ? part[tid - 1] : 0.f;
-    for (int i = lo; i < hi; ++i) {
-        acc += (i < L) ? gs[i] : 0.f;
-        Gs[i] = acc;
+    float carry = 0.f;
+    for (int base = 0; base < Lp; base += 4096) {
+        const int i0 = base + threadIdx.x * 4;
+        float v[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) v[x] = i0 + x < L ? gs[i0 + x] : 0.f;
+        v[1] += v[0]; v[2] += v[1]; v[3] += v[2];
+        float total;
+        const float before = carry + block_scan(v[3], part, total) - v[3];
+        if (i0 < Lp) *reinterpret_cast<float4*>(Gs + i0) = make_float4(before + v[0], before + v[1], before + v[2], before + v[3]);
+        carry += total;
     }
 }
 
-// rs[chunk*128 + i] = sum_k dsd[chunk][i][k]; one warp per row (a lane reads four adjacent entries), four rows in flight.
-__global__ void __launch_bounds__(256) dsd_rowsum_kernel(const float* __restrict__ dsd, float* __restrict__ rs) {
-    grid_wait();
-    grid_launch();
-    const float4* base = reinterpret_cast<const float4*>(dsd + (size_t)blockIdx.x * CHUNK * CHUNK);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll 1
-    for (int r0 = warp * 16; r0 < warp * 16 + 16; r0 += 4) {
-        float4 v[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) v[x] = base[(r0 + x) * (CHUNK / 4) + lane];
-        float acc[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) acc[x] = (v[x].x + v[x].y) + (v[x].z + v[x].w);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) acc[x] += __shfl_xor_sync(0xffffffffu, acc[x], off);
-        if (lane < 4)
-            rs[(size_t)blockIdx.x * CHUNK + r0 + lane] = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
-    }
-}
-
-// dlog_f[t] = sum_{m >= t} (dGa + dGb + dGc)[m]: reverse inclusive scan per slice (inputs [S][Lp], output [S][L]).
+// out[s][i] = sum over positions t >= i of dG + dGrow + the four partial row sums of the diagonal chunks' dS ([chunk][4][128]).
+// One CTA per slice, from the end, 4096 positions at a time (see gate_prefix_kernel).
 __global__ void __launch_bounds__(1024) gate_suffix_kernel(const float* __restrict__ dGa, const float* __restrict__ dGb,
-                                                           const float* __restrict__ dGc, float* __restrict__ out, int L,
-                                                           int Lp) {
+                                                           const float* __restrict__ diag, float* __restrict__ out, int L, int Lp) {
     grid_wait();
     grid_launch();
-    __shared__ float part[1024];
-    const int tid = threadIdx.x;
-    const int seg = (L + 1023) / 1024;
-    const int hi = L - tid * seg, lo = max(hi - seg, 0);  // this thread owns positions [lo, hi), scanning downwards
+    __shared__ float part[32];
     const size_t so = (size_t)blockIdx.x * Lp;
     float* os = out + (size_t)blockIdx.x * L;
-    float acc = 0.f;
-    for (int i = hi - 1; i >= lo; --i) acc += (dGa[so + i] + dGb[so + i]) + dGc[so + i];
-    part[tid] = acc;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        float v = (tid >= off) ? part[tid - off] : 0.f;
-        __syncthreads();
-        part[tid] += v;
-        __syncthreads();
-    }
-    acc = (tid > 0) ? part[tid - 1] : 0.f;
-    for (int i = hi - 1; i >= lo; --i) {
-        acc += (dGa[so + i] + dGb[so + i]) + dGc[so + i];
-        os[i] = acc;
+    float carry = 0.f;
+    for (int top = Lp; top > 0; top -= 4096) {
+        const int i0 = top - 4 - (int)threadIdx.x * 4;   // this thread: positions i0 + 3, i0 + 2, i0 + 1, i0
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        if (i0 >= 0) {
+            const float4 a = *reinterpret_cast<const float4*>(dGa + so + i0), b = *reinterpret_cast<const float4*>(dGb + so + i0);
+            v[0] = a.w + b.w; v[1] = a.z + b.z; v[2] = a.y + b.y; v[3] = a.x + b.x;
+            const float* d = diag + (so + (i0 & ~(CHUNK - 1))) * 4 + (i0 & (CHUNK - 1));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 c = *reinterpret_cast<const float4*>(d + q * CHUNK);
+                v[0] += c.w; v[1] += c.z; v[2] += c.y; v[3] += c.x;
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (i0 + 3 - x >= L) v[x] = 0.f;   // the padded tail
+        }
+        v[1] += v[0]; v[2] += v[1]; v[3] += v[2];
+        float total;
+        const float before = carry + block_scan(v[3], part, total) - v[3];
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+            if (i0 >= 0 && i0 + 3 - x < L) os[i0 + 3 - x] = before + v[x];
+        carry += total;
     }
 }
 
@@ -134,25 +136,36 @@ __global__ void __launch_bounds__(256) tile_stats_kernel(const __nv_bfloat16* __
         }
         return acc;
     };
-    for (int r = warp * rows_w + grp; r < CHUNK; r += 8 * rows_w) {
-        const int t = c * CHUNK + r;
-        const size_t row = (size_t)sl * L + t;
-        uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a, x = a;
-        if (t < L) {
-            a = *reinterpret_cast<const uint4*>(q + row * hd + li * 8);
-            b = *reinterpret_cast<const uint4*>(k + row * hd + li * 8);
-            x = *reinterpret_cast<const uint4*>(w + row * hd + li * 8);
+    constexpr int U = 4;   // rows per lane group in flight (CHUNK / (8 * rows_w) is 4 or 8)
+    for (int r0 = warp * rows_w + grp; r0 < CHUNK; r0 += 8 * rows_w * U) {
+        uint4 a[U], b[U], x[U];
+        float g[U], bt[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int t = c * CHUNK + r0 + u * 8 * rows_w;
+            const size_t row = (size_t)sl * L + t;
+            a[u] = b[u] = x[u] = make_uint4(0u, 0u, 0u, 0u);
+            bt[u] = 0.f;
+            if (t < L) {
+                a[u] = *reinterpret_cast<const uint4*>(q + row * hd + li * 8);
+                b[u] = *reinterpret_cast<const uint4*>(k + row * hd + li * 8);
+                x[u] = *reinterpret_cast<const uint4*>(w + row * hd + li * 8);
+                bt[u] = beta[row];
+            }
+            g[u] = G[(size_t)sl * Lp + t];
         }
-        float qq = dot8(a, a), kk = dot8(b, b), qk = dot8(a, b), ww = dot8(x, x);
-        for (int off = lpr / 2; off >= 1; off >>= 1) {
-            qq += __shfl_xor_sync(0xffffffffu, qq, off); kk += __shfl_xor_sync(0xffffffffu, kk, off);
-            qk += __shfl_xor_sync(0xffffffffu, qk, off); ww += __shfl_xor_sync(0xffffffffu, ww, off);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            float qq = dot8(a[u], a[u]), kk = dot8(b[u], b[u]), qk = dot8(a[u], b[u]), ww = dot8(x[u], x[u]);
+            for (int off = lpr / 2; off >= 1; off >>= 1) {
+                qq += __shfl_xor_sync(0xffffffffu, qq, off); kk += __shfl_xor_sync(0xffffffffu, kk, off);
+                qk += __shfl_xor_sync(0xffffffffu, qk, off); ww += __shfl_xor_sync(0xffffffffu, ww, off);
+            }
+            qn = fmaxf(qn, sqrtf(qq)); kn = fmaxf(kn, sqrtf(kk));
+            gmax = fmaxf(gmax, g[u]); gmin = fminf(gmin, g[u]);
+            if (c * CHUNK + r0 + u * 8 * rows_w < L) mlo = fminf(mlo, scale * qk);
+            gam += logf(fmaxf(1.f, fabsf(1.f - bt[u] * ww)));
         }
-        const float g = G[(size_t)sl * Lp + t], bt = t < L ? beta[row] : 0.f;
-        qn = fmaxf(qn, sqrtf(qq)); kn = fmaxf(kn, sqrtf(kk));
-        gmax = fmaxf(gmax, g); gmin = fminf(gmin, g);
-        if (t < L) mlo = fminf(mlo, scale * qk);
-        gam += logf(fmaxf(1.f, fabsf(1.f - bt * ww)));
     }
     // the lanes of a group hold the same values; combine the groups of the warp (the growth sum counts each group once)
     for (int off = lpr; off < 32; off <<= 1) {
@@ -178,70 +191,74 @@ __global__ void __launch_bounds__(256) tile_stats_kernel(const __nv_bfloat16* __
     }
 }
 
-__global__ void __launch_bounds__(128) tile_keep_kernel(const float* __restrict__ stats, int* __restrict__ nkeep, int S, int N,
-                                                       float ascale) {
+// One CTA per slice.  First, a warp per query chunk I finds the farthest key chunk that fails the test (lanes over the key
+// chunks, the growth summed up by a warp scan).  Then the kept ranges are made a staircase: the first kept key chunk of a query
+// chunk never lies after that of a later query chunk (ranges only grow, which is always safe).  Then "key chunk J is kept by
+// query chunk I" holds for exactly the I in J .. far(J), so the key-major sweep of the backward (nvisit[J] = far(J) - J + 1 query
+// chunks) computes the same pairs as the query-major sweeps, and every version a sweep asks for lies within the levels its
+// chunk reaches.  Also counts the kept pairs.  (Two kernels with one serial thread per query chunk and per slice took
+// 30 us at 32 slices x 64 chunks.)
+__global__ void __launch_bounds__(1024) tile_ranges_kernel(const float* __restrict__ stats, int* __restrict__ nkeep,
+                                                           int* __restrict__ nvisit, unsigned long long* counters, int N,
+                                                           float ascale) {
     grid_wait();
     grid_launch();
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= S * N) return;
-    const int sl = idx / N, I = idx % N;
-    const float* me = stats + (size_t)idx * 8;
-    const float qn = me[0], gmax = me[2], need = me[4] - kSkipMargin;
-    float acc = 0.f;
-    int keep = 1;
-    for (int n = 0; n <= I; ++n) {
-        const float* o = stats + ((size_t)sl * N + I - n) * 8;
-        acc += o[5];
-        const float bound = ascale * qn * o[1] * expf(acc) + gmax - o[3];
-        if (!(bound < need)) keep = n + 1;   // also keeps everything when a NaN or an infinity is around
-    }
-    nkeep[idx] = keep;
-}
-
-// One CTA per slice.  First the kept ranges are made a staircase: the first kept key chunk of a query chunk never lies
-// after that of a later query chunk (ranges only grow, which is always safe).  Then "key chunk J is kept by query chunk I"
-// holds for exactly the I in J .. far(J), so the key-major sweep of the backward (nvisit[J] = far(J) - J + 1 query chunks)
-// computes the same pairs as the query-major sweeps, and every version a sweep asks for lies within the levels its chunk
-// reaches.  Also counts the kept pairs.
-__global__ void __launch_bounds__(128) tile_stair_kernel(int* __restrict__ nkeep, int* __restrict__ nvisit,
-                                                        unsigned long long* counters, int S, int N) {
-    grid_wait();
-    grid_launch();
-    // one CTA per slice; the two serial scans run on a copy in shared memory when it fits (N <= kStairMax chunks, i.e.
-    // sequences up to a million tokens), else directly on global memory
-    constexpr int kStairMax = 8192;
-    __shared__ int snk[kStairMax];
-    const int sl = blockIdx.x;
+    // the ranges sit in shared memory when they fit (N <= kMax chunks, i.e. sequences up to a million tokens)
+    constexpr int kMax = 8192;
+    __shared__ int snk[kMax];
+    const int sl = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float* st = stats + (size_t)sl * N * 8;
     int* gk = nkeep + (size_t)sl * N;
     int* gv = nvisit + (size_t)sl * N;
-    const bool in_smem = N <= kStairMax;
-    if (in_smem) {
-        for (int i = threadIdx.x; i < N; i += blockDim.x) snk[i] = gk[i];
-        __syncthreads();
+    int* nk = N <= kMax ? snk : gk;
+    for (int I = warp; I < N; I += 32) {
+        const float* me = st + (size_t)I * 8;
+        const float qn = me[0], gmax = me[2], need = me[4] - kSkipMargin;
+        float grown = 0.f;
+        int keep = 1;
+        for (int n0 = 0; n0 <= I; n0 += 32) {
+            const int n = n0 + lane;
+            const bool in = n <= I;
+            const float* o = st + (size_t)(in ? I - n : 0) * 8;
+            float acc = in ? o[5] : 0.f;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const float y = __shfl_up_sync(0xffffffffu, acc, off);
+                if (lane >= off) acc += y;
+            }
+            const float bound = ascale * qn * o[1] * expf(grown + acc) + gmax - o[3];
+            const unsigned kept = __ballot_sync(0xffffffffu, in && !(bound < need));   // a NaN or an infinity keeps as well
+            if (kept) keep = n0 + 32 - __clz((int)kept);
+            grown += __shfl_sync(0xffffffffu, acc, 31);
+        }
+        if (lane == 0) nk[I] = keep;
     }
-    if (threadIdx.x == 0) {
-        int* nk = in_smem ? snk : gk;
+    __syncthreads();
+    if (warp == 0) {   // from the last chunk down: start(I) = min over I' >= I of the first kept chunk
         unsigned long long kept = 0;
         int start = N;
-        for (int I = N - 1; I >= 0; --I) {
-            start = min(start, I - nk[I] + 1);
-            nk[I] = I - start + 1;
-            kept += (unsigned long long)nk[I];
-        }
-        if (in_smem) {   // nvisit is written below by all threads from the staircase
-            atomicAdd(&counters[0], kept);
-        } else {
-            int far = 0;
-            for (int J = 0; J < N; ++J) {
-                far = max(far, J);
-                while (far + 1 < N && far + 1 - nk[far + 1] + 1 <= J) ++far;
-                gv[J] = far - J + 1;
+        for (int top = N; top > 0; top -= 32) {
+            const int I = top - 1 - lane;
+            int first = I >= 0 ? I - nk[I] + 1 : N;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, first, off);
+                if (lane >= off) first = min(first, y);
             }
-            atomicAdd(&counters[0], kept);
+            first = min(first, start);
+            if (I >= 0) {
+                nk[I] = I - first + 1;
+                kept += (unsigned long long)nk[I];
+            }
+            start = __shfl_sync(0xffffffffu, first, 31);
         }
-        atomicAdd(&counters[1], (unsigned long long)N * (N + 1) / 2);
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, off);
+        if (lane == 0) {
+            atomicAdd(&counters[0], kept);
+            atomicAdd(&counters[1], (unsigned long long)N * (N + 1) / 2);
+        }
     }
-    if (!in_smem) return;
     __syncthreads();
     // far(J) = the last I whose first kept key chunk I - nk[I] + 1 is <= J; those first chunks do not decrease with I, so a
     // binary search per J finds it
@@ -249,10 +266,10 @@ __global__ void __launch_bounds__(128) tile_stair_kernel(int* __restrict__ nkeep
         int lo = J, hi = N - 1;   // invariant: chunk lo keeps J (a chunk always keeps itself)
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (mid - snk[mid] + 1 <= J) lo = mid; else hi = mid - 1;
+            if (mid - nk[mid] + 1 <= J) lo = mid; else hi = mid - 1;
         }
         gv[J] = lo - J + 1;
-        gk[J] = snk[J];
+        if (nk != gk) gk[J] = nk[J];
     }
 }
 
@@ -337,12 +354,9 @@ __global__ void selftest_wait_kernel(uint32_t* status, long long ticks) {
 
 }  // namespace
 
-cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* dGc, float* out, int S, int L, int Lp,
+cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* diag, float* out, int S, int L, int Lp,
                                cudaStream_t st) {
-    return launch<gate_suffix_kernel>(S, 1024, 0, st, dGa, dGb, dGc, out, L, Lp);
-}
-cudaError_t launch_dsd_rowsum(const float* dsd, float* rs, int nchunks, cudaStream_t st) {
-    return launch<dsd_rowsum_kernel>(nchunks, 256, 0, st, dsd, rs);
+    return launch<gate_suffix_kernel>(S, 1024, 0, st, dGa, dGb, diag, out, L, Lp);
 }
 
 cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, int f32, cudaStream_t st) {
@@ -361,11 +375,9 @@ cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const 
                              cudaStream_t st) {
     typedef __nv_bfloat16 bf;
     const int N = Lp / CHUNK;
-    cudaError_t e = launch<tile_stats_kernel>(S * N, 256, 0, st, (const bf*)q, (const bf*)k, (const bf*)w, beta, G, stats, L, Lp, hd, scale);
+    const cudaError_t e = launch<tile_stats_kernel>(S * N, 256, 0, st, (const bf*)q, (const bf*)k, (const bf*)w, beta, G, stats, L, Lp, hd, scale);
     if (e != cudaSuccess) return e;
-    e = launch<tile_keep_kernel>((S * N + 127) / 128, 128, 0, st, stats, nkeep, S, N, fabsf(scale));
-    if (e != cudaSuccess) return e;
-    return launch<tile_stair_kernel>(S, 128, 0, st, nkeep, nvisit, counters, S, N);
+    return launch<tile_ranges_kernel>(S, 1024, 0, st, (const float*)stats, nkeep, nvisit, counters, N, fabsf(scale));
 }
 
 cudaError_t launch_cp_gate(const float* G, float* gq, float* gk, float* gtot, int S, int L, int Lp, cudaStream_t st) {

@@ -10,11 +10,10 @@ cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, in
 // G[S][Lp] <- inclusive prefix sum of g[S][L] (tail repeats the last value).  `clear` (or nullptr): 256 bytes to zero on the way.
 cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, uint32_t* clear, cudaStream_t st);
 
-// out[S][L] <- reverse inclusive prefix sum of (dGa + dGb + dGc)[S][Lp] over positions < L.
-cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* dGc, float* out, int S, int L, int Lp,
+// out[S][L] <- reverse inclusive prefix sum of dGa + dGb [S][Lp] + diag [S*N][4][128] (four partial sums per row of a chunk)
+// over positions < L.
+cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* diag, float* out, int S, int L, int Lp,
                                cudaStream_t st);
-// rs[chunk][i] = sum_k dsd[chunk][i][k]
-cudaError_t launch_dsd_rowsum(const float* dsd, float* rs, int nchunks, cudaStream_t st);
 
 // Gated problems (PaTH-FoX): which key chunks a query chunk can skip because the accumulated gate has made every logit
 // of the pair negligible.  stats: [S*N][8] floats of scratch; nkeep: [S*N] key chunks each query chunk visits (counted

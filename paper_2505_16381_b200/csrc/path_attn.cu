@@ -122,7 +122,7 @@ struct Plan {
     // offsets (bytes)
     size_t status, G, tstats, nkeep, nvisit, Dyh, Dyl, Xq, Y, Qv16, Kv16;
     // backward only
-    size_t delta, lse2, dQv, dKv, dSd, dSdT, dG, dGrow, dGdiag, dDy;
+    size_t delta, lse2, dQv, dKv, dSd, dSdT, dG, dGrow, dDy;
     size_t sTh, sTl, sXk, sU, f32;   // bf16 tiles kept by the chunk preparation for the chain rule
     size_t dy_bytes, dy_mats;
 };
@@ -182,8 +182,8 @@ static bool make_plan(int B, int H, int L, int d, int dt, int gate, int bwd, Pla
     if (bwd) {
         p.delta = bump(cur, SL * 4); p.lse2 = bump(cur, SL * 4);
         p.dQv = bump(cur, p.rows_q * d * 2); p.dKv = bump(cur, p.rows_k * d * 2);   // bf16
-        p.dSd = bump(cur, gate ? SNBB * 4 : 0); p.dSdT = bump(cur, SNBB * 2); p.dG = bump(cur, SL * 4);
-        p.dGrow = bump(cur, gate ? SL * 4 : 0); p.dGdiag = bump(cur, gate ? SL * 4 : 0);
+        p.dSd = bump(cur, gate ? SL * 4 * 4 : 0); p.dSdT = bump(cur, SNBB * 2); p.dG = bump(cur, SL * 4);
+        p.dGrow = bump(cur, gate ? SL * 4 : 0);
         // bf16, each matrix written once by the CTA that owns it.  The backward never reads the run products' low planes
         // (gradient products take single bf16 operands), so their gradients take that place.
         p.dDy = p.Dyl;
@@ -238,7 +238,7 @@ static int run_gate_skip(const Plan& p, void* ws, const void* q, const void* k, 
     LAUNCH(launch_gate_skip(q, k, w, beta, at<float>(ws, p.G), at<float>(ws, p.tstats), at<int>(ws, p.nkeep),
                             at<int>(ws, p.nvisit), at<unsigned long long>(ws, p.status + kSkipCounterOffset), p.S, p.L, p.Lp,
                             p.d, scale, st));
-    g_launches += 2;
+    ++g_launches;
     return PATH_OK;
 }
 
@@ -397,8 +397,7 @@ static int run_backward(const Plan& p, void* ws, const void* q, const void* k, c
     prof_mark(STG_CHAIN, 1, st);
     prof_mark(STG_GATE, 0, st);
     if (dlog_f) {
-        LAUNCH(launch_dsd_rowsum(at<float>(ws, p.dSd), at<float>(ws, p.dGdiag), p.S * p.N, st));
-        LAUNCH(launch_gate_suffix(at<float>(ws, p.dG), at<float>(ws, p.dGrow), at<float>(ws, p.dGdiag), dlog_f, p.S, p.L,
+        LAUNCH(launch_gate_suffix(at<float>(ws, p.dG), at<float>(ws, p.dGrow), at<float>(ws, p.dSd), dlog_f, p.S, p.L,
                                   p.Lp, st));
     }
     prof_mark(STG_GATE, 1, st);
