@@ -120,7 +120,8 @@ struct FwdParams {
     float scale;
     int out_fp32;
     // segment-against-segment sweep of the context-parallel path only (launch_fa_fwd_cross): the key segment's padded
-    // length and chunk count, and its gate terms [S, Lkp] (G then holds the query rows' terms; logit += G_i - Gk_j)
+    // length and chunk count, and its gate terms [S, Lkp] (G then holds the query rows' terms; logit += G_i - Gk_j); o
+    // (float32) and lse hold the running result of earlier sweeps, which the new one is merged into
     const float* Gk;
     int Lkp, Nk;
     int* next_item;     // work-item counter in the status block (zero on entry)
@@ -154,6 +155,7 @@ struct LevelParams {
     __nv_bfloat16* ddy16;         // gradients of the run products, same placement as the run products themselves
     float* kc;                    // edge kernels: [S][cap][d] float32 out (rows < L of every slice), or nullptr
     int cap, L;
+    __nv_bfloat16 *edge_q, *edge_k;   // version forward: [S][Lp][d] out, queries at the segment's start / keys at its end, or nullptr
     __nv_bfloat16* edge16;        // edge kernels: [S][L][d] bf16 out, or nullptr
     __nv_bfloat16* pseg;          // edge kernels: [S][nseg][2][d][d] product of the walked range as bf16 hi, lo; or nullptr
     __nv_bfloat16* sfx;           // suffix kernel: [S][nseg][2][d][d] out
@@ -164,7 +166,7 @@ struct LevelParams {
     uint32_t* status;
 };
 
-enum { LEVEL_DYADIC_FWD = 0, LEVEL_DYADIC_FUSED, LEVEL_VERSION_FWD, LEVEL_BWD, LEVEL_KEY_CACHE, LEVEL_QUERY_EDGE, LEVEL_SUFFIX, LEVEL_APPLY_PRODUCT };
+enum { LEVEL_DYADIC_FWD = 0, LEVEL_DYADIC_FUSED, LEVEL_VERSION_FWD, LEVEL_BWD, LEVEL_KEY_CACHE, LEVEL_SEGMENT_PRODUCT, LEVEL_SUFFIX, LEVEL_APPLY_PRODUCT };
 cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const LevelParams& p, int hd, cudaStream_t st);
 
 struct PrepTensorMaps {

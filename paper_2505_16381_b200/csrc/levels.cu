@@ -296,32 +296,69 @@ __device__ __forceinline__ int highest_level_reached(const LevelParams& p, int i
     return T > 0 ? msb32((unsigned)(ch ^ (ch - T))) : 0;
 }
 
+// Where a chain stands: at chunk boundary e (a query chunk I starts at e = I and goes down to 0, a key chunk J at J + 1 and up to
+// N).  The next step multiplies by the largest stored run product that is aligned at e and fits: level a, index idx, new
+// boundary e2.  As long as e is the boundary of one of the chunk's versions, the steps are those of version_step.
+__device__ __forceinline__ bool chain_step(int is_key, int e, int N, int top, int& a, int& idx, int& e2) {
+    if (e == (is_key ? N : 0)) return false;
+    a = min(lowest_set((unsigned)e), top);
+    if (is_key) {
+        while (e + (1 << a) > N) --a;
+        idx = e >> a;
+        e2 = e + (1 << a);
+    } else {
+        idx = (e >> a) - 1;
+        e2 = e - (1 << a);
+    }
+    return true;
+}
+// Level of the version whose boundary is e, or -1 if chunk ch has none there.
+__device__ __forceinline__ int version_at(int is_key, int ch, int e, int N, int nlev) {
+    if (e == 0 || e == N) return -1;
+    const int lv = lowest_set((unsigned)e);
+    return lv < nlev && (((ch >> lv) + is_key) << lv) == e ? lv : -1;
+}
+
+// With p.edge_q / p.edge_k the chains go on to the sequence's start / end (context-parallel path, paper Sec. 3.5: queries
+// pulled back to the start of the segment, keys advanced to its end, bf16 [S][Lp][d]): at most about 2 log2(N) products per
+// chunk, all chunks at once.  (Walking the chunks one after the other per slice took 105 us for the two sides of 64 slices of
+// 8 chunks at d = 128, on top of this kernel's 23; the extended chains take 45 in all, and the product of the segment comes from the run products.)
 template <int HD>
 __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int is_key = blockIdx.y, s = blockIdx.x / p.N, ch = blockIdx.x % p.N;
     grid_wait();   // (the block-skipping counts)
-    // levels to build: all of them, or for a gated problem up to the highest one a kept chunk pair uses (see level_bwd)
+    // levels to store: all of them, or for a gated problem up to the highest one a kept chunk pair uses (see level_bwd)
     const int lim = min(p.l, highest_level_reached(p, is_key, s, ch) + 1);
-    int l1, b, src, l2 = 1;
-    for (; l2 < lim; ++l2)
-        if (version_step(is_key, ch, l2, p.N, l1, b, src)) break;
-    if (l2 >= lim) return;
+    const int top = max(p.nlev - 2, 0);
+    __nv_bfloat16* edge = is_key ? p.edge_k : p.edge_q;
+    int e = ch + is_key, a, idx, e2, lv;
+    // the next step, if there is one to take: a version to store, or an edge to reach
+    auto next = [&]() {
+        if (!chain_step(is_key, e, p.N, top, a, idx, e2)) return false;
+        lv = version_at(is_key, ch, e2, p.N, p.nlev);
+        if (lv >= lim) lv = -1;
+        return edge != nullptr || lv >= 0;
+    };
+    const long row_first = (long)s * p.Lp + (long)ch * kT;   // plane 0: the boundary-adjusted tile
+    if (!next()) {
+        if (edge) {   // already at the edge
+            const uint4* src = reinterpret_cast<const uint4*>((is_key ? p.kv : p.qv) + row_first * HD);
+            uint4* dst = reinterpret_cast<uint4*>(edge + row_first * HD);
+            for (int i = threadIdx.x; i < kT * HD / 8; i += 256) dst[i] = src[i];
+        }
+        return;
+    }
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
     setup<128>(c, smem_raw, kBar3);
     uint8_t* sm = c.smem;   // slots: 0 current version, 1 Dy hi, 2 Dy lo
-    bool first = true;
+    bool first = true, more = true;
 #pragma unroll 1
-    for (; l2 < lim && c.ok; ++l2) {
-        if (!version_step(is_key, ch, l2, p.N, l1, b, src)) continue;
-        const long mat = p.lv.dy_off[l1] / (HD * HD) + (long)s * p.lv.dy_cnt[l1] + b;
-        const long row_dst = is_key ? kver_row(p.vl, s, l2, ch) : qver_row(p.vl, s, l2, ch);
+    while (more && c.ok) {
+        const long mat = p.lv.dy_off[a] / (HD * HD) + (long)s * p.lv.dy_cnt[a] + idx;
         if (c.warp == 0 && elect_one()) {
             mbar_expect_tx(&c.bars[0], (first ? 3 : 2) * kT * HD * 2);
-            if (first) {
-                const long row_src = is_key ? kver_row(p.vl, s, l1, ch) : qver_row(p.vl, s, l1, ch);
-                tma_tile(sm, is_key ? &tm.kv : &tm.qv, &c.bars[0], HD, (int)row_src);
-            }
+            if (first) tma_tile(sm, is_key ? &tm.kv : &tm.qv, &c.bars[0], HD, (int)row_first);
             tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
             tma_tile(sm + 2 * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat * HD));
         }
@@ -329,28 +366,96 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
         if (!first) publish();   // the left operand was written by this CTA's threads
         if (leader(c)) {
             tc_fence_after_sync();
-            const uint32_t a = smem_u32(sm);
+            const uint32_t t = smem_u32(sm);
             if (is_key) {
-                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, a, a + kTileB, false);
-                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, true);
+                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, t, t + kTileB, false);
+                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, true);
             } else {
-                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + kTileB, false);
-                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, true);
+                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + kTileB, false);
+                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, true);
             }
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
+        __nv_bfloat16* out = nullptr;
+        if (lv >= 0) out = (is_key ? p.kv + kver_row(p.vl, s, lv, ch) * HD : p.qv + qver_row(p.vl, s, lv, ch) * HD);
+        else if (e2 == (is_key ? p.N : 0)) out = edge + row_first * HD;
         if (c.ok) {
             float v[32];
-            __nv_bfloat16* out = (is_key ? p.kv : p.qv) + (size_t)row_dst * HD;
             for (int i = 0; i < HD / 64; ++i) {
                 const int c0 = c.half * (HD / 2) + i * 32;
                 tmem_row32(c.tl + c0, v);
-                gstore_bf16x32(out + (size_t)c.row * HD + c0, v);
+                if (out) gstore_bf16x32(out + (size_t)c.row * HD + c0, v);
                 tile_store32(sm, c.row, c0, v);
             }
         }
         first = false;
+        e = e2;
+        more = next();
+    }
+    teardown<128>(c, p.status);
+}
+
+// ---------------------------------------------------------------------------------------------- product of a whole segment
+// grid = S.  P_{N-1} ... P_0 as a bf16 hi + lo pair (p.pseg, [S][2][d][d]) from the stored run products, last run first:
+// R <- R Dy[a][idx].
+template <int HD>
+__global__ void __launch_bounds__(256, 1) segment_product_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    Ctx c;
+    setup<128>(c, smem_raw, kBar4);
+    uint8_t* sm = c.smem;   // slots: 0 R hi, 1 R lo, 2 Dy hi, 3 Dy lo
+    const int s = blockIdx.x, top = max(p.nlev - 2, 0);
+    int e = p.N, a, idx, e2;
+    auto load = [&](int slot) {   // the run below boundary e
+        const long mat = p.lv.dy_off[a] / (HD * HD) + (long)s * p.lv.dy_cnt[a] + idx;
+        if (c.warp == 0 && elect_one()) {
+            mbar_expect_tx(&c.bars[0], 2 * kT * HD * 2);
+            tma_tile(sm + slot * kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
+            tma_tile(sm + (slot + 1) * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat * HD));
+        }
+        loads_wait(c);
+        e = e2;
+    };
+    chain_step(0, e, p.N, top, a, idx, e2);
+    __nv_bfloat16* out = p.pseg + (size_t)s * 2 * HD * HD;
+    if (e2 == 0) {   // one run is the whole segment
+        const size_t mat = p.lv.dy_off[a] + ((size_t)s * p.lv.dy_cnt[a] + idx) * HD * HD;
+        for (int i = c.tid; i < HD * HD / 8; i += 256) {
+            reinterpret_cast<uint4*>(out)[i] = reinterpret_cast<const uint4*>(p.dyh + mat)[i];
+            reinterpret_cast<uint4*>(out + HD * HD)[i] = reinterpret_cast<const uint4*>(p.dyl + mat)[i];
+        }
+        teardown<128>(c, p.status);
+        return;
+    }
+    load(0);
+#pragma unroll 1
+    while (c.ok && chain_step(0, e, p.N, top, a, idx, e2)) {
+        load(2);
+        publish();
+        if (leader(c)) {
+            tc_fence_after_sync();
+            const uint32_t t = smem_u32(sm);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, false);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 3 * kTileB, true);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t + kTileB, t + 2 * kTileB, true);
+            umma_commit(&c.bars[1]);
+        }
+        mma_wait(c);
+        if (!c.ok) break;
+        float v[32];
+        uint32_t hi[16], lo[16];
+        for (int i = 0; i < HD / 64; ++i) {
+            const int c0 = c.half * (HD / 2) + i * 32;
+            tmem_row32(c.tl + c0, v);
+            split32(v, hi, lo);
+            tile_store_w16(sm, c.row, c0, hi);
+            tile_store_w16(sm + kTileB, c.row, c0, lo);
+            if (e == 0) {
+                gstore_bf16_w16(out + (size_t)c.row * HD + c0, hi, c.row < HD);
+                gstore_bf16_w16(out + (size_t)HD * HD + (size_t)c.row * HD + c0, lo, c.row < HD);
+            }
+        }
     }
     teardown<128>(c, p.status);
 }
@@ -525,18 +630,15 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
 // Both products act on the columns of R independently, so a CTA carries only 64 columns of R (and writes those columns
 // of the result): at d = 128 two CTAs share a slice (four with 32 columns each were no faster per step and, at 4096
 // tokens, more CTAs than SMs).
-// QUERY = true is the mirror image for the context-parallel path (paper Sec. 3.5): the queries pulled back to the start of
-// the segment,  x_I = Qleft_I R_I  with  R_I = P_{I-1} ... P_0,  walking the chunks upwards with  R <- P_I R;  the last R is
-// the product of the whole segment, which the segment hands to the devices holding later queries.
 // Results leave as float32 rows (p.kc, the decoding cache) and / or bf16 rows (p.edge16).
-template <int HD, bool QUERY>
+template <int HD>
 __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
     setup<256>(c, smem_raw, kBar5);
     constexpr int NC = 64;                      // columns of R per CTA
     const int s = blockIdx.x, col0 = blockIdx.y * NC;
-    uint8_t* sm = c.smem;   // slots: 0 Kright_J / Qleft_I, 1 P hi, 2 P lo, 3 R hi, 4 R lo ([d x 64] in the first panel)
+    uint8_t* sm = c.smem;   // slots: 0 Kright_J, 1 P hi, 2 P lo, 3 R hi, 4 R lo ([d x 64] in the first panel)
     {   // R = I[:, col0 .. col0+63]; the tiles' unused parts read as zeros (P^T enters with M = 128: its second panel when d = 64)
         for (int i = c.tid; i < (int)(4 * kTileB / 16); i += 256) reinterpret_cast<uint4*>(sm + kTileB)[i] = make_uint4(0, 0, 0, 0);
         __syncthreads();
@@ -550,7 +652,7 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
     auto issue = [&](int J) {
         const long mat = p.lv.dy_off[0] / (HD * HD) + (long)s * p.lv.dy_cnt[0] + J;
         mbar_expect_tx(&c.bars[0], 3 * kT * HD * 2);
-        tma_tile(sm, QUERY ? &tm.qv : &tm.kv, &c.bars[0], HD, (int)((long)s * p.Lp + (long)J * kT));   // version slot 0
+        tma_tile(sm, &tm.kv, &c.bars[0], HD, (int)((long)s * p.Lp + (long)J * kT));   // version slot 0
         tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
         tma_tile(sm + 2 * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat * HD));
     };
@@ -560,14 +662,14 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
     // chain of dependent products, so this is what lets a long prompt use all SMs.
     const int c_lo = p.nseg > 1 ? (int)blockIdx.z * p.seg_chunks : 0;
     const int c_hi = p.nseg > 1 ? min(p.N, c_lo + p.seg_chunks) : p.N, cnt = c_hi - c_lo;
-    const int first = QUERY ? c_lo : c_hi - 1, step = QUERY ? 1 : -1;
+    const int first = c_hi - 1, step = -1;
     if (cnt <= 0) { teardown<256>(c, p.status); return; }
     if (c.warp == 0 && elect_one()) issue(first);
 #pragma unroll 1
     for (int n = 0, J = first; n < cnt && c.ok; ++n, J += step) {
         const bool more = n + 1 < cnt;
-        // the query side also wants the product of the whole segment; so does every key range but the first
-        const bool update = QUERY || more || (p.nseg > 1 && blockIdx.z > 0);
+        // every range but the first also wants its whole product
+        const bool update = more || (p.nseg > 1 && blockIdx.z > 0);
         loads_wait(c);
         publish();
         if (leader(c)) {
@@ -576,7 +678,7 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
             mma<OP_K, OP_MN, HD / 16, NC>(c.tmem, a, a + 3 * kTileB, false);                       // X R
             mma<OP_K, OP_MN, HD / 16, NC>(c.tmem, a, a + 4 * kTileB, true);
             if (update) {
-                constexpr int pop = QUERY ? OP_K : OP_MN;                                          // P R  /  P^T R
+                constexpr int pop = OP_MN;                                                         // P^T R
                 mma<pop, OP_MN, HD / 16, NC>(c.tmem + 128, a + 1 * kTileB, a + 3 * kTileB, false);
                 mma<pop, OP_MN, HD / 16, NC>(c.tmem + 128, a + 2 * kTileB, a + 3 * kTileB, true);
                 mma<pop, OP_MN, HD / 16, NC>(c.tmem + 128, a + 1 * kTileB, a + 4 * kTileB, true);
@@ -744,11 +846,11 @@ cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const Leve
         }
         case LEVEL_KEY_CACHE: {
             dim3 g(p.S, hd / 64, p.nseg > 1 ? p.nseg : 1);
-            return hd == 64 ? launch<key_cache_kernel<64, false>>(g, 256, smem_bytes(5), st, tm, p) : launch<key_cache_kernel<128, false>>(g, 256, smem_bytes(5), st, tm, p);
+            return hd == 64 ? launch<key_cache_kernel<64>>(g, 256, smem_bytes(5), st, tm, p) : launch<key_cache_kernel<128>>(g, 256, smem_bytes(5), st, tm, p);
         }
-        case LEVEL_QUERY_EDGE: {
-            dim3 g(p.S, hd / 64);
-            return hd == 64 ? launch<key_cache_kernel<64, true>>(g, 256, smem_bytes(5), st, tm, p) : launch<key_cache_kernel<128, true>>(g, 256, smem_bytes(5), st, tm, p);
+        case LEVEL_SEGMENT_PRODUCT: {
+            dim3 g(p.S);
+            return hd == 64 ? launch<segment_product_kernel<64>>(g, 256, smem_bytes(4), st, tm, p) : launch<segment_product_kernel<128>>(g, 256, smem_bytes(4), st, tm, p);
         }
         case LEVEL_SUFFIX: {
             dim3 g(p.S, hd / 64);

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(1024) tile_ranges_kernel(const float* __restri
     }
 }
 
-// ---- context-parallel path: gate terms of a segment, merge of partial softmax results
+// ---- context-parallel path: gate terms of a segment, final result
 __global__ void cp_gate_kernel(const float* __restrict__ G, float* __restrict__ gq, float* __restrict__ gk,
                                float* __restrict__ gtot, int L, int Lp) {
     grid_wait();
@@ -287,22 +287,6 @@ __global__ void cp_gate_kernel(const float* __restrict__ G, float* __restrict__ 
     gk[(size_t)s * Lp + i] = i < L ? g - tot : 1e30f;
 }
 // one thread per 4 outputs of a row
-__global__ void cp_merge_kernel(float* __restrict__ o_acc, float* __restrict__ lse_acc, const float* __restrict__ o_t,
-                                const float* __restrict__ lse_t, size_t rows, int hd4) {
-    grid_wait();
-    grid_launch();
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * hd4) return;
-    const size_t r = i / hd4;
-    const float la = lse_acc[r], lt = lse_t[r];
-    const float m = fmaxf(la, lt);
-    const float wa = __expf(la - m), wt = __expf(lt - m), inv = 1.f / (wa + wt);
-    const float4 a = reinterpret_cast<const float4*>(o_acc)[i], t = reinterpret_cast<const float4*>(o_t)[i];
-    reinterpret_cast<float4*>(o_acc)[i] = make_float4((a.x * wa + t.x * wt) * inv, (a.y * wa + t.y * wt) * inv,
-                                                      (a.z * wa + t.z * wt) * inv, (a.w * wa + t.w * wt) * inv);
-    __syncwarp();   // (the lanes of a row read lse_acc before one of them replaces it: a row's hd4 lanes sit in one warp)
-    if (i % hd4 == 0) lse_acc[r] = m + __logf(wa + wt);
-}
 __global__ void cp_finish_kernel(const float* __restrict__ o_acc, const float* __restrict__ lse_acc, __nv_bfloat16* __restrict__ o,
                                  float* __restrict__ lse, size_t rows, int hd4) {
     grid_wait();
@@ -382,11 +366,6 @@ cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const 
 
 cudaError_t launch_cp_gate(const float* G, float* gq, float* gk, float* gtot, int S, int L, int Lp, cudaStream_t st) {
     return launch<cp_gate_kernel>(dim3((Lp + 255) / 256, S), 256, 0, st, G, gq, gk, gtot, L, Lp);
-}
-cudaError_t launch_cp_merge(float* o_acc, float* lse_acc, const float* o_t, const float* lse_t, size_t rows, int hd,
-                            cudaStream_t st) {
-    const size_t n = rows * (hd / 4);
-    return launch<cp_merge_kernel>((unsigned)((n + 255) / 256), 256, 0, st, o_acc, lse_acc, o_t, lse_t, rows, hd / 4);
 }
 cudaError_t launch_cp_finish(const float* o_acc, const float* lse_acc, void* o, float* lse, size_t rows, int hd,
                              cudaStream_t st) {

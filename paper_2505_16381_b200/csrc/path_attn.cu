@@ -244,7 +244,8 @@ static int run_gate_skip(const Plan& p, void* ws, const void* q, const void* k, 
 
 // Chunk preparation + dyadic run products + version chains (paper Sec. 3.1, 3.3).  Shared by forward and backward.
 static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const void* w, const float* beta, bool in_backward,
-                    cudaStream_t st, bool with_levels = true, bool keys_only = false) {
+                    cudaStream_t st, bool with_levels = true, bool keys_only = false, __nv_bfloat16* edge_q = nullptr,
+                    __nv_bfloat16* edge_k = nullptr) {
     const int d = p.d, nch = p.S * p.N;
     const int stg_prep = in_backward ? STG_PREP_BWD : STG_PREP, stg_lev = in_backward ? STG_LEVELS_BWDPREP : STG_LEVELS;
     // fused per-chunk kernel: UT transform, boundary-adjusted tiles (version slot 0), chunk products (level 0)
@@ -276,7 +277,7 @@ static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const
         LAUNCH(launch_chunk_prep(tm, pp, d, keys_only ? PREP_KEYS : (p.bwd ? PREP_SAVE : PREP_FWD), nch, st));
         prof_mark(stg_prep, 1, st);
     }
-    if (p.nlev < 2 || !with_levels) return PATH_OK;
+    if ((p.nlev < 2 && !edge_q) || !with_levels) return PATH_OK;
     LevelTensorMaps tm;
     if (!make_level_maps(p, ws, tm)) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
     LevelParams lp = level_params(p, ws);
@@ -289,6 +290,7 @@ static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const
         l += lp.fuse;
     }
     lp.l = p.nlev;                                // query and key versions: one CTA per chunk walks its chain
+    lp.edge_q = edge_q; lp.edge_k = edge_k;
     LAUNCH(launch_level_kernel(LEVEL_VERSION_FWD, tm, lp, d, st));
     prof_mark(stg_lev, 1, st);
     return PATH_OK;
@@ -617,7 +619,6 @@ struct CpLayout {
     int S, L, Lp, N, d;
     size_t x, gq, o_acc, lse_acc, state_total;        // state: query tiles pulled back so far, their gate terms, running result
     size_t kend, v, pseg, gk, gtot, message_total;    // message: what a segment hands to the holders of later queries
-    size_t o_t, lse_t, step_total;                    // scratch of one step (after the 256-byte status block)
 };
 static bool cp_layout(int B, int H, int L, int d, CpLayout& c) {
     Plan p;
@@ -631,9 +632,6 @@ static bool cp_layout(int B, int H, int L, int d, CpLayout& c) {
     c.kend = bump(cur, SLpd * 2); c.v = bump(cur, SLpd * 2); c.pseg = bump(cur, (size_t)p.S * 2 * d * d * 2);
     c.gk = bump(cur, SLp * 4); c.gtot = bump(cur, (size_t)p.S * 4);
     c.message_total = cur;
-    cur = 256;
-    c.o_t = bump(cur, SLd * 4); c.lse_t = bump(cur, SL * 4);
-    c.step_total = cur;
     return true;
 }
 
@@ -649,7 +647,7 @@ size_t path_attn_cp_workspace_bytes(int B, int H, int L, int d, int has_gate) {
     CpLayout c;
     Plan p;
     if (!cp_layout(B, H, L, d, c) || !make_plan(B, H, L, d, PATH_BF16, has_gate ? 1 : 0, 0, p)) return 0;
-    return p.total > c.step_total ? p.total : c.step_total;
+    return p.total;
 }
 
 int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void* w, const float* beta, const float* log_f,
@@ -673,7 +671,8 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
         rc = run_gate_skip(p, workspace, q, k, w, beta, scale, st);
         if (rc != PATH_OK) return rc;
     }
-    rc = run_prep(p, workspace, q, k, w, beta, false, st);
+    // versions, and on the way the keys advanced to the segment's end and the queries pulled back to its start
+    rc = run_prep(p, workspace, q, k, w, beta, false, st, true, false, at<__nv_bfloat16>(state, c.x), at<__nv_bfloat16>(message, c.kend));
     if (rc != PATH_OK) return rc;
     // the segment's own (causal) attention, as a float32 running result
     {
@@ -692,17 +691,13 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
         if (log_f) fp.nkeep = at<int>(workspace, p.nkeep);
         LAUNCH(launch_fa_fwd(tm, fp, d, st));
     }
-    // keys advanced to the segment's end, queries pulled back to its start, the product of the whole segment
+    // the product of the whole segment
     {
         LevelTensorMaps tm;
         if (!make_level_maps(p, workspace, tm)) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
         LevelParams lp = level_params(p, workspace);
-        lp.L = p.Lp; lp.cap = p.Lp;   // (whole padded chunks: the padded rows of the prepared tiles are zero)
-        lp.edge16 = at<__nv_bfloat16>(message, c.kend);
-        LAUNCH(launch_level_kernel(LEVEL_KEY_CACHE, tm, lp, d, st));
-        lp.edge16 = at<__nv_bfloat16>(state, c.x);
         lp.pseg = at<__nv_bfloat16>(message, c.pseg);
-        LAUNCH(launch_level_kernel(LEVEL_QUERY_EDGE, tm, lp, d, st));
+        LAUNCH(launch_level_kernel(LEVEL_SEGMENT_PRODUCT, tm, lp, d, st));
     }
     // (a sweep reads the message's values in whole chunks)
     if (p.L == p.Lp) CK(cudaMemcpyAsync(at<void>(message, c.v), v, (size_t)p.S * p.Lp * d * 2, cudaMemcpyDeviceToDevice, st));
@@ -719,7 +714,7 @@ int path_attn_cp_step(void* state, const void* message, int B, int H, int Lq, in
     CpLayout cq, ck;
     if (!cp_layout(B, H, Lq, d, cq) || !cp_layout(B, H, Lk, d, ck)) return PATH_ERR_SHAPE;
     if (((uintptr_t)workspace & 255) || ((uintptr_t)state & 255) || ((uintptr_t)message & 255)) return PATH_ERR_ALIGN;
-    if (workspace_bytes < cq.step_total) return PATH_ERR_WORKSPACE;
+    if (workspace_bytes < 256) return PATH_ERR_WORKSPACE;   // (a step needs the status block only)
     int rc = check_arch();
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -734,15 +729,13 @@ int path_attn_cp_step(void* state, const void* message, int B, int H, int Lq, in
         if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
         tm.q_raw = tm.k_raw = tm.xq = tm.y = tm.qv;   // unused by this sweep, but every descriptor gets prefetched
         FwdParams fp{};
-        fp.o = at<float>(workspace, cq.o_t); fp.lse = at<float>(workspace, cq.lse_t);
+        fp.o = at<float>(state, cq.o_acc); fp.lse = at<float>(state, cq.lse_acc);
         fp.G = at<float>(state, cq.gq); fp.Gk = at<float>(msg, ck.gk);
         fp.status = (uint32_t*)workspace;
         fp.next_item = at<int>(workspace, kNextItemOffset);
         fp.S = cq.S; fp.L = Lq; fp.Lp = cq.Lp; fp.N = cq.N; fp.Nk = ck.N; fp.Lkp = ck.Lp; fp.scale = scale; fp.out_fp32 = 1;
         LAUNCH(launch_fa_fwd_cross(tm, fp, d, st));
     }
-    LAUNCH(launch_cp_merge(at<float>(state, cq.o_acc), at<float>(state, cq.lse_acc), at<float>(workspace, cq.o_t),
-                           at<float>(workspace, cq.lse_t), (size_t)cq.S * Lq, d, st));
     // the queries move on past the attended segment: x <- x P(segment), gate terms += the segment's total
     {
         LevelTensorMaps tm;
