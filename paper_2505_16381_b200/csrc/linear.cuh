@@ -23,6 +23,9 @@ cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const 
                              int* nkeep, int* nvisit, unsigned long long* counters, int S, int L, int Lp, int hd, float scale,
                              cudaStream_t st);
 
+// Decoding cache from a prompt: vc[S][cap][hd] <- v[S][L][hd] (bf16), gc[S][cap] <- G[S][Lp] (gc may be nullptr).
+cudaError_t launch_cache_rows(const void* v, void* vc, const float* G, float* gc, int S, int L, int Lp, int cap, int hd, cudaStream_t st);
+
 // Context-parallel path (paper Sec. 3.5), gate terms of a segment from its prefix sums G [S][Lp] (nullptr = no gate):
 // gq[S][Lp] <- G (the query rows' terms), gk[S][Lp] <- G - G[L-1] for positions < L and a huge value for the padded tail
 // (which masks those keys), gtot[S] <- G[L-1].

@@ -818,10 +818,7 @@ int path_attn_prefill_cache(const void* k, const void* v, const void* w, const f
         lp.kc = kc; lp.L = L; lp.edge16 = nullptr; lp.qv = edge; lp.gq = nullptr;
         LAUNCH(launch_level_kernel(LEVEL_APPLY_PRODUCT, tm2, lp, d, st));
     }
-    CK(cudaMemcpy2DAsync(vc, (size_t)cap * d * 2, v, (size_t)L * d * 2, (size_t)L * d * 2, (size_t)p.S, cudaMemcpyDeviceToDevice, st));
-    if (gc)
-        CK(cudaMemcpy2DAsync(gc, (size_t)cap * 4, at<float>(workspace, p.G), (size_t)p.Lp * 4, (size_t)L * 4, (size_t)p.S,
-                             cudaMemcpyDeviceToDevice, st));
+    LAUNCH(launch_cache_rows(v, vc, gc ? at<float>(workspace, p.G) : nullptr, gc, p.S, L, p.Lp, cap, d, st));
     return PATH_OK;
 }
 
