@@ -271,6 +271,10 @@ struct GemmParams {
     int ldc, c_atomic;
     uint32_t* status;
 };
+// C[M, N] = A B, contraction over R = 64 or 128: A [M][R] and C [M][N] (maps with boxes of 128 rows x 64), B [N][R] (the same box) or,
+// with b_mn, [R][N] (box 64 x 64).
+cudaError_t launch_wide(const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_c, int M, int N, int R, int b_mn,
+                        uint32_t* status, cudaStream_t st);
 cudaError_t launch_gemm(const CUtensorMap& map_a, const CUtensorMap& map_b, const GemmParams& p, int split_k, cudaStream_t st);
 
 }  // namespace path

@@ -100,6 +100,8 @@ template <int HD>
 __global__ void __launch_bounds__(kThreads, 4) frontend_fwd_kernel(
     const __nv_bfloat16* __restrict__ z, const float* __restrict__ cw, const float* __restrict__ bl, const float* __restrict__ gl,
     __nv_bfloat16* __restrict__ w, float* __restrict__ beta, float* __restrict__ logf, int B, int H, int L, int nblk, float eps) {
+    grid_wait();
+    grid_launch();
     constexpr int kR = FwdR<HD>::value, kFwdRows = fwd_rows(kR);
     typedef Geo<HD, kR> Ge;
     extern __shared__ uint4 queue[];   // [stage][row][thread]: every slot is written and read by the same thread
@@ -192,6 +194,8 @@ __global__ void __launch_bounds__(kThreads, 2) frontend_bwd_kernel(
     const __nv_bfloat16* __restrict__ dw, const float* __restrict__ dbeta, const float* __restrict__ dlogf,
     __nv_bfloat16* __restrict__ dz, float* dcw, float* __restrict__ dbl, float* __restrict__ dgl, int B, int H, int L, int nblk,
     float eps) {
+    grid_wait();
+    grid_launch();
     constexpr int kR = BwdR<HD>::value, kBwdRows = bwd_rows(kR);
     typedef Geo<HD, kR> Ge;
     extern __shared__ uint4 queue[];   // [stage][row][thread]; reused for the reduction of the filter gradient at the end
@@ -327,10 +331,8 @@ __global__ void __launch_bounds__(kThreads, 2) frontend_bwd_kernel(
 // CTAs per head: as many as fit on the device at once at `per_sm` resident CTAs per SM (rounded down: one CTA too
 // many would run alone in a second wave and double the time), at least one, never more than there are blocks
 cudaError_t ctas_per_head(int B, int H, int nblk, int per_sm, int* out) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    const cudaError_t e = sm_count(sms);
     if (e != cudaSuccess) return e;
     long long want = (long long)sms * per_sm / H;
     if (want < 1) want = 1;
@@ -352,16 +354,8 @@ cudaError_t launch_frontend_fwd(const void* z, const float* cw, const float* bl,
     const dim3 grid((unsigned)((size_t)H * W));
     auto smem_of = [](int R) { return kFwdStages * (fwd_rows(R) * (int)sizeof(uint4) + 2 * (int)sizeof(float)) * kThreads; };
     const int smem = smem_of(hd == 64 ? FwdR<64>::value : FwdR<128>::value);
-    if (hd == 64) {
-        e = cudaFuncSetAttribute(frontend_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        frontend_fwd_kernel<64><<<grid, kThreads, smem, st>>>((const bf*)z, cw, bl, gl, (bf*)w, beta, logf, B, H, L, nblk, eps);
-    } else {
-        e = cudaFuncSetAttribute(frontend_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        frontend_fwd_kernel<128><<<grid, kThreads, smem, st>>>((const bf*)z, cw, bl, gl, (bf*)w, beta, logf, B, H, L, nblk, eps);
-    }
-    return cudaGetLastError();
+    return hd == 64 ? launch<frontend_fwd_kernel<64>>(grid, kThreads, smem, st, (const bf*)z, cw, bl, gl, (bf*)w, beta, logf, B, H, L, nblk, eps)
+                    : launch<frontend_fwd_kernel<128>>(grid, kThreads, smem, st, (const bf*)z, cw, bl, gl, (bf*)w, beta, logf, B, H, L, nblk, eps);
 }
 
 cudaError_t launch_frontend_bwd(const void* z, const float* cw, const float* bl, const float* gl, const void* dw,
@@ -379,18 +373,10 @@ cudaError_t launch_frontend_bwd(const void* z, const float* cw, const float* bl,
     static_assert(kBwdStages * bwd_rows(1) * (int)sizeof(uint4) * kThreads >= kWarps * 4 * 64 * 3 * (int)sizeof(float) &&
                       kBwdStages * bwd_rows(1) * (int)sizeof(uint4) * kThreads >= kWarps * 2 * 128 * 3 * (int)sizeof(float),
                   "the queue also holds the filter-gradient partials");
-    if (hd == 64) {
-        e = cudaFuncSetAttribute(frontend_bwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        frontend_bwd_kernel<64><<<grid, kThreads, smem, st>>>((const bf*)z, cw, bl, gl, (const bf*)dw, dbeta, dlogf, (bf*)dz, dcw,
-                                                           dbl, dgl, B, H, L, nblk, eps);
-    } else {
-        e = cudaFuncSetAttribute(frontend_bwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        frontend_bwd_kernel<128><<<grid, kThreads, smem, st>>>((const bf*)z, cw, bl, gl, (const bf*)dw, dbeta, dlogf, (bf*)dz, dcw,
-                                                            dbl, dgl, B, H, L, nblk, eps);
-    }
-    return cudaGetLastError();
+    return hd == 64 ? launch<frontend_bwd_kernel<64>>(grid, kThreads, smem, st, (const bf*)z, cw, bl, gl, (const bf*)dw, dbeta, dlogf, (bf*)dz, dcw, dbl, dgl, B,
+                                                       H, L, nblk, eps)
+                    : launch<frontend_bwd_kernel<128>>(grid, kThreads, smem, st, (const bf*)z, cw, bl, gl, (const bf*)dw, dbeta, dlogf, (bf*)dz, dcw, dbl, dgl, B,
+                                                       H, L, nblk, eps);
 }
 
 }  // namespace path

@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(1024) tile_ranges_kernel(const float* __restri
 }
 
 // Values and gate prefix of a prompt into the decoding cache: vc[S][cap][d] <- v[S][L][d], gc[S][cap] <- G[S][Lp] (L rows of every
-// slice).  grid = (blocks of 1024 16-byte vectors, slices), four vectors per thread in flight: 85 us for 32 x 32768 x 128 (6.3 TB/s),
+// slice).  grid = (blocks of 1024 16-byte vectors, slices), four vectors per thread in flight: 99 us for 32 x 32768 x 128 (5.4 TB/s),
 // where cudaMemcpy2DAsync took 273.
 __global__ void __launch_bounds__(256) cache_rows_kernel(const uint4* __restrict__ v, uint4* __restrict__ vc, const float* __restrict__ G,
                                                          float* __restrict__ gc, long n16, long cap16, int L, int Lp, int cap, int S) {

@@ -870,6 +870,16 @@ static int run_gemm(const void* a, int a_mn, const void* b, int b_mn, void* c, i
     return PATH_OK;
 }
 
+// C[M, N] = A op(B) with the contraction over r (lowrank.cu, wide_kernel).
+static int run_wide(const void* a, const void* b, int b_mn, void* c, int M, int N, int R, uint32_t* status, cudaStream_t st) {
+    CUtensorMap ma, mb, mc;
+    const bool ok = make_map_box(&ma, a, (uint64_t)M, (uint64_t)R, 128) && make_map_box(&mc, c, (uint64_t)M, (uint64_t)N, 128) &&
+                    (b_mn ? make_map_box(&mb, b, (uint64_t)R, (uint64_t)N, 64) : make_map_box(&mb, b, (uint64_t)N, (uint64_t)R, 128));
+    if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
+    LAUNCH(launch_wide(ma, mb, mc, M, N, R, b_mn, status, st));
+    return PATH_OK;
+}
+
 static bool lowrank_shape_ok(long long M, int D, int r, int C) {
     return M >= 1 && M <= (1LL << 30) && D >= 64 && D % 64 == 0 && D <= (1 << 20) && (r == 64 || r == 128) && C >= 64 &&
            C % 64 == 0 && C <= (1 << 20);
@@ -896,7 +906,7 @@ int path_attn_lowrank_fwd(const void* x, const void* w1, const void* w2, void* t
     CK(cudaMemsetAsync(workspace, 0, 256, st));
     rc = run_gemm(x, 0, w1, 0, t, 0, (int)M, r, D, (uint32_t*)workspace, st);         // t = x W1^T
     if (rc != PATH_OK) return rc;
-    return run_gemm(t, 0, w2, 0, z, 0, (int)M, C, r, (uint32_t*)workspace, st);       // z = t W2^T
+    return run_wide(t, w2, 0, z, (int)M, C, r, (uint32_t*)workspace, st);             // z = t W2^T
 }
 
 int path_attn_lowrank_bwd(const void* x, const void* w1, const void* w2, const void* t, const void* dz, void* dx, float* dw1,
@@ -922,7 +932,7 @@ int path_attn_lowrank_bwd(const void* x, const void* w1, const void* w2, const v
     if (rc != PATH_OK) return rc;
     rc = run_gemm(dz, 1, t, 1, dw2, 1, C, r, (int)M, status, st);                     // dW2 = dz^T t
     if (rc != PATH_OK) return rc;
-    rc = run_gemm(dt, 0, w1, 1, dx, 0, (int)M, D, r, status, st);                     // dx = dt W1
+    rc = run_wide(dt, w1, 1, dx, (int)M, D, r, status, st);                           // dx = dt W1
     if (rc != PATH_OK) return rc;
     return run_gemm(dt, 1, x, 1, dw1, 1, r, D, (int)M, status, st);                   // dW1 = dt^T x
 }

@@ -173,6 +173,25 @@ def test_lowrank_layer_matches_oracle(binding, B, L, D, r, C):
         assert (a - b_).abs().max().item() <= 1e-5 * a.abs().max().item()
 
 
+@pytest.mark.parametrize("M,D,r,C", [
+    (128 * 300 + 1, 960, 64, 192),      # dx: 301 x 8 tiles, the last one 64 wide; z: 301 x 2; one row in the last row tile
+    (128 * 160 - 1, 192, 128, 1088),    # z: 160 x 9 tiles; dx: 160 x 2
+])
+def test_lowrank_many_output_tiles_per_block(binding, M, D, r, C):
+    """z and dx where every block walks over several row tiles and several column tiles of each, with ragged edges."""
+    g = torch.Generator().manual_seed(M + r)
+    x = torch.randn(1, M, D, generator=g).bfloat16()
+    w1 = (torch.randn(r, D, generator=g) / D ** 0.5).bfloat16()
+    w2 = (torch.randn(C, r, generator=g) / r ** 0.5).bfloat16()
+    dz = torch.randn(1, M, C, generator=g).bfloat16()
+    z, t = binding.path_attn_lowrank_fwd(x.cuda(), w1.cuda(), w2.cuda())
+    dx, _, _ = binding.path_attn_lowrank_bwd(x.cuda(), w1.cuda(), w2.cuda(), t, dz.cuda())
+    z_ref = f64(t).reshape(M, r) @ f64(w2).T                        # from the t the kernel stored: only z's own rounding is left
+    dt = (f64(dz).reshape(M, C) @ f64(w2))
+    assert close_bf16(f64(z).reshape(M, C), z_ref)
+    assert rel_fro(f64(dx).reshape(M, D), dt @ f64(w1)) <= 5e-3     # (dt enters rounded to bf16)
+
+
 def test_lowrank_layer_argument_errors(binding):
     x = torch.zeros(4, 96, dtype=torch.bfloat16, device="cuda")                   # D not a multiple of 64
     with pytest.raises(binding.PathAttnError) as e:
