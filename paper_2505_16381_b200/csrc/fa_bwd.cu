@@ -19,8 +19,8 @@
 // The elementwise work of a step is split in two so that it overlaps the tensor pipe: part A turns S into P (the
 // exponentials) as soon as S is there, while the dP product still runs; part B forms dS once dP has arrived.  The
 // products are issued in the order  dV(t), S(t+1), dK(t), dP(t+1)  (dkv) and  dQ(t), dP(t+1), S(t+2)  (dq, which has
-// room for two S tiles), so the pipe always has the next step's logits in flight.
-// Warps: 0 = TMA producer, 1 = tcgen05 MMA issuer, 2-3 idle (their registers go to the others), 4-11 = elementwise
+// room for two S tiles), so the pipe always has the next step's logits in flight.  (dq_kernel goes further: see there.)
+// Warps of dkv_kernel: 0 = TMA producer, 1 = tcgen05 MMA issuer, 2-3 idle (their registers go to the others), 4-11 = elementwise
 // math (two warps per TMEM lane quadrant, each taking 64 of the 128 columns of a row).
 #include <type_traits>
 #include "common.cuh"
@@ -537,28 +537,109 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
 }
 
 // ------------------------------------------------------------------------------------------------ dQ
-// Persistent like the dK/dV sweep: items are the query chunks of a slice, paired (longest, shortest).
-enum { Q_QFULL = 0, Q_QEMPTY, Q_DOFULL, Q_DOEMPTY, Q_KFULL, Q_KEMPTY = Q_KFULL + 3, Q_VFULL = Q_KEMPTY + 3,
-       Q_VEMPTY = Q_VFULL + 2, Q_SFULL = Q_VEMPTY + 2, Q_DPFULL = Q_SFULL + 2, Q_DSFULL, Q_ACCFULL, Q_ACCFREE,
-       Q_GKFULL, Q_GKEMPTY = Q_GKFULL + 2, Q_COUNT = Q_GKEMPTY + 2 };
-constexpr uint32_t kDqGk = 7 * kSlotBytes + 256;              // [2][128] gate prefix of the key chunk, [128] exchange
-constexpr uint32_t kDqTotal = kDqGk + 3 * kTile * 4;
+// Persistent like the dK/dV sweep: items are the query chunks of a slice, paired (longest, shortest).  The steps of all
+// items of a CTA form one sequence.  Round i of the elementwise warps does part A of step i and part B of step i - 1 in one
+// pass over 16 columns at a time, so that exponentials, products and tensor-memory traffic of two steps share the issue
+// slots: one after the other they took 1600 + 1200 cycles of which the exponentials alone are 1024.  What a round needs is
+// produced while the previous one runs: S(i) alternates between two tiles, dP(i - 1) is released as soon as every thread
+// has it in registers, and dS(i - 1) goes into the columns of S(i) that its thread has just read.  Everything else is kept
+// out of these warps: the K producer describes each step in shared memory, four more warps write finished levels out.
+// 8 x 16 x 2048 x 64: 150 -> 123 us (a round takes 2050 cycles, 1290 of them the pass itself); 4 x 16 x 4096 x 128: 342 ->
+// 314 us, where the products alone are 1560 of 2500 cycles a round and the power limit is reached.
+// Warps: 0 = producer of Q, K, gate prefix and step descriptions, 1 = tcgen05 issue of S and dQ, 2 = producer of dO and V,
+// 3 = tcgen05 issue of dP, 4-11 = elementwise math, 12-15 = write-out.
+enum { Q_QFULL = 0, Q_QEMPTY = 2, Q_DOFULL = 4, Q_DOEMPTY = 6, Q_KFULL = 8, Q_KEMPTY = Q_KFULL + 6, Q_VFULL = Q_KEMPTY + 6,
+       Q_VEMPTY = Q_VFULL + 4, Q_GKEMPTY = Q_VEMPTY + 4, Q_READY = Q_GKEMPTY + 2, Q_DPFREE = Q_READY + 2, Q_ROUND, Q_ACCFULL = Q_ROUND + 2,
+       Q_ACCFREE, Q_SUM, Q_COUNT = Q_SUM + 3 };
+constexpr uint32_t kDqDesc = 7 * kSlotBytes + 336;            // [8] step descriptions
+constexpr uint32_t kDqGk = kDqDesc + 8 * 16;                  // [2][128] gate prefix of the key chunk, [3][128] row sums of an item
+constexpr uint32_t kDqTotal = kDqGk + 5 * kTile * 4;
+static_assert(Q_COUNT * 8 + 8 <= 336 && kDqTotal <= kSmemAlloc, "shared memory of the dQ sweep");
+
+// A CTA's steps one after the other: items come from `item_of(k, chunk, slice)`, their step counts from
+// `steps_of(chunk, slice)`, fetched one item ahead; `skipped(chunk, slice)` sees the items without a step.
+template <class ItemOf, class StepsOf, class Skipped>
+struct Flow {
+    ItemOf item_of;
+    StepsOf steps_of;
+    Skipped skipped;
+    int c = 0, s = 0, t = -1, T = 0;              // current step: chunk, slice, step t of T
+    int nc = 0, ns = 0, nT = 0, k = 0;            // the next item with steps, if there is one
+    bool more;
+    __device__ Flow(ItemOf io, StepsOf so, Skipped sk) : item_of(io), steps_of(so), skipped(sk) { fetch(); }
+    __device__ void fetch() {
+        while ((more = item_of(k++, nc, ns))) {
+            nT = steps_of(nc, ns);
+            if (nT > 0) break;
+            skipped(nc, ns);
+        }
+    }
+    __device__ bool next() {
+        if (++t < T) return true;
+        if (!more) return false;
+        c = nc; s = ns; T = nT; t = 0;
+        fetch();
+        return true;
+    }
+};
+template <class ItemOf, class StepsOf, class Skipped>
+__device__ __forceinline__ Flow<ItemOf, StepsOf, Skipped> make_flow(ItemOf io, StepsOf so, Skipped sk) {
+    return Flow<ItemOf, StepsOf, Skipped>(io, so, sk);
+}
+template <class ItemOf, class StepsOf>
+__device__ __forceinline__ auto make_flow(ItemOf io, StepsOf so) { return make_flow(io, so, [](int, int) {}); }
+enum { FL_VALID = 1, FL_FIRST = 2, FL_LAST = 4, FL_LVL0 = 8, FL_LVL1 = 16 };   // a step: first / last of its item / of a level
+
+template <int N>
+__device__ __forceinline__ void set_fewer_regs() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void set_more_regs() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+// Waits for this thread's tensor-memory loads; nothing that uses r may be moved in front of it.
+__device__ __forceinline__ void tmem_ld_wait16(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                   "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+}
+
+// D[tmem] (+)= A B with A in tensor memory: the 16 contraction indices of step kk in the 8 columns at a_col + 16 kk.
+__device__ __forceinline__ void mma_t16(uint32_t d_tmem, uint32_t a_col, uint32_t b0, uint32_t idesc, bool acc) {
+    uint32_t b_lo = umma_desc_lo(b0, kPanelBytes);
+#pragma unroll
+    for (int kk = 0; kk < kTile / 16; ++kk) {
+        umma_ts(d_tmem, a_col + kk * 16, umma_desc_join(b_lo), idesc, (acc || kk > 0) ? 1u : 0u);
+        b_lo += 128u;
+    }
+}
 
 template <int HD, bool GATE>
-__global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdTensorMaps tm, const BwdParams p) {
+__global__ void __launch_bounds__(512, 1) dq_kernel(const __grid_constant__ BwdTensorMaps tm, const BwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     if ((uint32_t)(smem - smem_raw) + kDqTotal > kSmemAlloc) {   // uniform over the CTA
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_DQ_PRODUCER);
         return;
     }
+    // Tiles in flight.  K is needed from S(i + 2) to dQ(i - 1), four steps; V only for dP.
+    constexpr int NQ = HD == 64 ? 2 : 1, NDO = NQ, NK = HD == 64 ? 6 : 4, NV = HD == 64 ? 4 : 1;
+    constexpr uint32_t kBytes = kTile * HD * 2;
+    // Registers.  Without a gate a math thread fetches its 64 columns of dP at once, so that the next dP can start early, and a
+    // level is written out 32 columns at a time.  With one (more live values, and with block skipping a level may be one step
+    // long) dP comes 16 columns at a time and a level is read whole, so that the next one can start.  dQ sweep, us, early / late:
+    // d = 128, 4 x 16 x 4096 ungated 316 / 361; 2 x 16 x 8192 gated 154 / 144;  d = 64, 8 x 16 x 2048 ungated 121 / 146.
+    constexpr bool EARLY = !GATE;
+    constexpr int kRegsMath = EARLY ? 200 : 168, kRegsOut = EARLY ? 56 : 112, kRegsIssue = EARLY ? 56 : 64;
+    static_assert(256 * kRegsMath + 128 * (kRegsOut + kRegsIssue) <= 65536, "no more than the block was launched with");
+    static_assert((NQ + NDO + NK + NV) * kBytes == 7 * kSlotBytes, "tiles fill the 7 slots");
     uint8_t* sQ = smem;
-    uint8_t* sDO = sQ + kSlotBytes;
-    uint8_t* sK = sDO + kSlotBytes;        // ring of 3
-    uint8_t* sV = sK + 3 * kSlotBytes;     // ring of 2
+    uint8_t* sDO = sQ + NQ * kBytes;
+    uint8_t* sK = sDO + NDO * kBytes;
+    uint8_t* sV = sK + NK * kBytes;
     uint64_t* bars = (uint64_t*)(smem + 7 * kSlotBytes);
     uint32_t* tmem_slot = (uint32_t*)(bars + Q_COUNT);
     volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);
+    int4* desc = (int4*)(smem + kDqDesc);   // flags, first row of the query chunk, -, the same of the next item (-1: none)
     float* gk = (float*)(smem + kDqGk);
     float* dsum_x = gk + 2 * kTile;
 
@@ -567,11 +648,14 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < Q_COUNT; ++i)
-            mbar_init(&bars[i], (i == Q_DSFULL || i == Q_ACCFREE || i == Q_GKEMPTY || i == Q_GKEMPTY + 1) ? 256u : 1u);
+            mbar_init(&bars[i], i == Q_READY || i == Q_READY + 1 ? 3u
+                              : i == Q_DPFREE || i == Q_ROUND || i == Q_ROUND + 1 || i == Q_GKEMPTY || i == Q_GKEMPTY + 1 ? 256u
+                              : i >= Q_SUM ? 256u : i == Q_ACCFREE ? 128u : 1u);
         *abort_flag = 0;
         mbar_fence_init();
     }
-    if (warp == 2 && lane < 8) tma_prefetch_desc(reinterpret_cast<const CUtensorMap*>(&tm) + lane);
+    if (GATE && threadIdx.x < 3 * kTile) dsum_x[threadIdx.x] = 0.f;
+    if (warp == 3 && lane < 8) tma_prefetch_desc(reinterpret_cast<const CUtensorMap*>(&tm) + lane);
     if (warp == 1) tmem_alloc(tmem_slot, 512);
     tc_fence_before_sync();
     __syncthreads();
@@ -589,227 +673,298 @@ __global__ void __launch_bounds__(384, 1) dq_kernel(const __grid_constant__ BwdT
         I = (j & 1) ? (j >> 1) : p.N - 1 - (j >> 1);
         return true;
     };
-    int I = 0, s = 0;
-    auto qrow = [&](int lvl, int chunk) { return qver_row(p.vl, s, lvl, chunk); };   // first row of a version tile
-    auto krow = [&](int lvl, int chunk) { return kver_row(p.vl, s, lvl, chunk); };
-    auto row0 = [&](int chunk) { return (long)s * p.Lp + (long)chunk * kTile; };      // plane 0
-    auto level = [&](int t) { return msb32((unsigned)(I ^ (I - 1 - t))); };
     // earlier key chunks this query chunk visits (J = I-1 .. I-T): all of them, or fewer when the gate has made the far
     // ones negligible (every warp role reads the same precomputed number; the diagonal chunk is not part of this sweep)
     auto steps_of = [&](int I, int s) { return p.nkeep ? min(I, p.nkeep[s * p.N + I] - 1) : I; };
+    auto level = [](int I, int t) { return msb32((unsigned)(I ^ (I - 1 - t))); };
+    auto flags_of = [](int I, int t, int T, int l) {   // level l covers the key chunks whose low l bits run from all ones down to zero
+        const int J = I - 1 - t, m = (1 << l) - 1, last = t + 1 == T;
+        return FL_VALID | (t == 0 ? FL_FIRST : 0) | (last ? FL_LAST : 0) | ((J & m) == m ? FL_LVL0 : 0) |
+               (last || (J & m) == 0 ? FL_LVL1 : 0);
+    };
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        set_fewer_regs<kRegsIssue>();
         if (warp == 0 && elect_one()) {
+            auto flow = make_flow(item_of, steps_of);
             bool ok = true;
-            int nq = 0, nd = 0, kn = 0, vn = 0;   // fills so far: Q, dO, K ring, V ring (= gate ring)
+            int nq = 0, n = 0;   // Q tiles, steps so far
             auto wait_empty = [&](int bar, int use) {
                 if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_DQ_PRODUCER)) ok = false;
+                return ok;
             };
 #pragma unroll 1
-            for (int it = 0; ok && item_of(it, I, s); ++it) {
-                const int T = steps_of(I, s);
-                if (T == 0) continue;
-                wait_empty(Q_DOEMPTY, nd);
-                if (!ok) break;
-                mbar_expect_tx(&bars[Q_DOFULL], kTile * HD * 2);
-                tma_rows(sDO, &tm.d_o, &bars[Q_DOFULL], HD, I * kTile, s);
-                ++nd;
-#pragma unroll 1
-                for (int t = 0; t < T && ok; ++t) {
-                    const int J = I - 1 - t, l = level(t);
-                    if (t == 0 || l != level(t - 1)) {
-                        wait_empty(Q_QEMPTY, nq);
-                        if (!ok) break;
-                        mbar_expect_tx(&bars[Q_QFULL], kTile * HD * 2);
-                        tma_tile(sQ, &tm.qv, &bars[Q_QFULL], HD, (int)qrow(l, I));
-                        ++nq;
-                    }
-                    wait_empty(Q_KEMPTY + kn % 3, kn / 3);
-                    if (!ok) break;
-                    mbar_expect_tx(&bars[Q_KFULL + kn % 3], kTile * HD * 2);
-                    tma_tile(sK + (kn % 3) * kSlotBytes, &tm.kv, &bars[Q_KFULL + kn % 3], HD, (int)krow(l, J));
-                    ++kn;
-                    wait_empty(Q_VEMPTY + (vn & 1), vn >> 1);
-                    if (!ok) break;
-                    mbar_expect_tx(&bars[Q_VFULL + (vn & 1)], kTile * HD * 2);
-                    tma_rows(sV + (vn & 1) * kSlotBytes, &tm.v, &bars[Q_VFULL + (vn & 1)], HD, J * kTile, s);
-                    if (GATE) {   // gate prefix of the key chunk
-                        wait_empty(Q_GKEMPTY + (vn & 1), vn >> 1);
-                        if (!ok) break;
-                        mbar_expect_tx(&bars[Q_GKFULL + (vn & 1)], kTile * 4);
-                        bulk_load(gk + (vn & 1) * kTile, p.G + (size_t)s * p.Lp + J * kTile, kTile * 4,
-                                  &bars[Q_GKFULL + (vn & 1)]);
-                    }
-                    ++vn;
+            for (; ok; ++n) {
+                const bool more = flow.next();
+                // K(n - NK) is released after round n - NK + 1, past the last look at description n - 8
+                if (!wait_empty(Q_KEMPTY + n % NK, n / NK)) break;
+                if (!more) {
+                    desc[n & 7] = make_int4(0, 0, 0, -1);
+                    mbar_arrive(&bars[Q_KFULL + n % NK]);
+                    break;
                 }
+                const int I = flow.c, s = flow.s, J = I - 1 - flow.t, l = level(I, flow.t), f = flags_of(I, flow.t, flow.T, l);
+                desc[n & 7] = make_int4(f, s * p.Lp + I * kTile, 0, flow.more ? flow.ns * p.Lp + flow.nc * kTile : -1);
+                mbar_expect_tx(&bars[Q_KFULL + n % NK], kBytes + (GATE ? kTile * 4 : 0));
+                tma_tile(sK + (n % NK) * kBytes, &tm.kv, &bars[Q_KFULL + n % NK], HD, (int)kver_row(p.vl, s, l, J));
+                if (f & FL_LVL0) {
+                    const int b = nq % NQ;
+                    if (!wait_empty(Q_QEMPTY + b, nq / NQ)) break;
+                    mbar_expect_tx(&bars[Q_QFULL + b], kBytes);
+                    tma_tile(sQ + b * kBytes, &tm.qv, &bars[Q_QFULL + b], HD, (int)qver_row(p.vl, s, l, I));
+                    ++nq;
+                }
+                if (GATE) {   // gate prefix of the key chunk (counted with K)
+                    if (!wait_empty(Q_GKEMPTY + (n & 1), n >> 1)) break;
+                    bulk_load(gk + (n & 1) * kTile, p.G + (size_t)s * p.Lp + J * kTile, kTile * 4, &bars[Q_KFULL + n % NK]);
+                }
+            }
+        } else if (warp == 2 && elect_one()) {
+            auto flow = make_flow(item_of, steps_of);
+            bool ok = true;
+            int nd = 0;
+            auto wait_empty = [&](int bar, int use) {
+                if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_DQ_PRODUCER)) ok = false;
+                return ok;
+            };
+#pragma unroll 1
+            for (int n = 0; flow.next(); ++n) {
+                if (flow.t == 0) {
+                    const int b = nd % NDO;
+                    if (!wait_empty(Q_DOEMPTY + b, nd / NDO)) break;
+                    mbar_expect_tx(&bars[Q_DOFULL + b], kBytes);
+                    tma_rows(sDO + b * kBytes, &tm.d_o, &bars[Q_DOFULL + b], HD, flow.c * kTile, flow.s);
+                    ++nd;
+                }
+                if (!wait_empty(Q_VEMPTY + n % NV, n / NV)) break;
+                mbar_expect_tx(&bars[Q_VFULL + n % NV], kBytes);
+                tma_rows(sV + (n % NV) * kBytes, &tm.v, &bars[Q_VFULL + n % NV], HD, (flow.c - 1 - flow.t) * kTile, flow.s);
             }
         } else if (warp == 1 && elect_one()) {
             constexpr uint32_t idescS = umma_idesc(128, 128, 0, 0);
             constexpr uint32_t idescD = umma_idesc(128, HD, 0, 1);
             bool ok = true;
-            int nq = 0, nd = 0, g = 0, na = 0;   // Q / dO fills consumed, steps before this item, items with steps so far
-            int T = 0;
+            int nq = 0, na = 0;   // Q tiles so far, levels finished so far
             auto wait = [&](int bar, int parity) {
                 if (ok && !mbar_wait(&bars[bar], parity & 1, abort_flag, ST_DQ_MMA)) ok = false;
+                return ok;
             };
-            auto issue_s = [&](int t) {      // S(t) into the tile of running step g + t
-                const int gs = g + t;
-                if (t == 0 || level(t) != level(t - 1)) { wait(Q_QFULL, nq); ++nq; }
-                wait(Q_KFULL + gs % 3, gs / 3);
-                tc_fence_after_sync();
-                if (!ok) return;
-                mma_kk(tmem + colS + (gs & 1) * 128, smem_u32(sQ), smem_u32(sK + (gs % 3) * kSlotBytes), HD, idescS, false);
-                umma_commit(&bars[Q_SFULL + (gs & 1)]);
-                if (t + 1 >= T || level(t + 1) != level(t)) umma_commit(&bars[Q_QEMPTY]);
-            };
-            auto issue_dp = [&](int t) {
-                const int gs = g + t;
-                wait(Q_VFULL + (gs & 1), gs >> 1);
-                tc_fence_after_sync();
-                if (!ok) return;
-                mma_kk(tmem + colDP, smem_u32(sDO), smem_u32(sV + (gs & 1) * kSlotBytes), HD, idescS, false);
-                umma_commit(&bars[Q_DPFULL]);
-                umma_commit(&bars[Q_VEMPTY + (gs & 1)]);
-                if (t + 1 >= T) umma_commit(&bars[Q_DOEMPTY]);   // the item's last use of dO
-            };
-#pragma unroll 1
-            for (int it = 0; ok && item_of(it, I, s); ++it) {
-                T = steps_of(I, s);
-                if (T == 0) continue;
-                wait(Q_DOFULL, nd); ++nd;
-                issue_s(0);
-                issue_dp(0);
-                if (T > 1) issue_s(1);
-#pragma unroll 1
-                for (int t = 0; t < T && ok; ++t) {
-                    const int gs = g + t;
-                    // dQ += dS K.  dP of the next step overwrites dS, S(t+2) the tile whose P every thread has taken
-                    // into registers before it delivered dS: in-order execution keeps both behind what they replace.
-                    wait(Q_DSFULL, gs);
-                    if (t == 0 && na > 0) wait(Q_ACCFREE, na - 1);   // the previous item's dQ has been read
+            // S of step g; returns the step's flags, 0 after the last one.  A round begins on three arrivals: S, dP, and one
+            // that hands the description on.
+            auto issue_s = [&](int g) {
+                if (!wait(Q_KFULL + g % NK, g / NK)) return 0;
+                const int f = desc[g & 7].x;
+                if (f) {
+                    if (f & FL_LVL0) { wait(Q_QFULL + nq % NQ, nq / NQ); ++nq; }
+                    const int b = (nq - 1) % NQ;
                     tc_fence_after_sync();
-                    if (!ok) break;
-                    mma_tn(tmem + colDQ, tmem + colDP, smem_u32(sK + (gs % 3) * kSlotBytes), idescD,
-                           !(t == 0 || level(t) != level(t - 1)));
-                    umma_commit(&bars[Q_KEMPTY + gs % 3]);
-                    if (t + 1 < T) issue_dp(t + 1);
-                    if (t + 2 < T) issue_s(t + 2);
-                    if (t == T - 1) umma_commit(&bars[Q_ACCFULL]);
+                    if (!ok) return 0;
+                    mma_kk(tmem + colS + (g & 1) * 128, smem_u32(sQ + b * kBytes), smem_u32(sK + (g % NK) * kBytes), HD, idescS, false);
+                    umma_commit(&bars[Q_READY + (g & 1)]);
+                    if (f & FL_LVL1) umma_commit(&bars[Q_QEMPTY + b]);
+                } else {   // the last round has no S: its tile is free once dQ(g - 3) has retired
+                    umma_commit(&bars[Q_READY + (g & 1)]);
                 }
-                g += T;
-                ++na;
+                mbar_arrive(&bars[Q_READY + (g & 1)]);
+                return f;
+            };
+            int fm = 0, f0 = issue_s(0), f1 = f0 ? issue_s(1) : 0;   // steps i - 1, i, i + 1
+            if (ok) mbar_arrive(&bars[Q_READY]);                     // (no dP before round 0)
+#pragma unroll 1
+            for (int i = 0; ok && (f0 | fm); ++i) {
+                if (!wait(Q_ROUND + (i & 1), i >> 1)) break;
+                if (fm) {                    // dQ (+)= dS(i - 1) K
+                    if ((fm & FL_LVL0) && na > 0 && !wait(Q_ACCFREE, na - 1)) break;   // the previous level has been read
+                    tc_fence_after_sync();
+                    mma_t16(tmem + colDQ, tmem + colS + (i & 1) * 128, smem_u32(sK + ((i - 1) % NK) * kBytes), idescD, !(fm & FL_LVL0));
+                    umma_commit(&bars[Q_KEMPTY + (i - 1) % NK]);
+                    if (fm & FL_LVL1) { umma_commit(&bars[Q_ACCFULL]); ++na; }
+                }
+                // in-order execution keeps S(i + 2) behind the product that reads dS(i - 1) from the same tile
+                const int f2 = f1 ? issue_s(i + 2) : 0;
+                fm = f0; f0 = f1; f1 = f2;
+            }
+        } else if (warp == 3 && elect_one()) {
+            // dP has an issuing thread of its own: its waits and those for S and dQ are not paid one after the other
+            constexpr uint32_t idescS = umma_idesc(128, 128, 0, 0);
+            auto flow = make_flow(item_of, steps_of);
+            bool ok = true;
+            auto wait = [&](int bar, int parity) {
+                if (ok && !mbar_wait(&bars[bar], parity & 1, abort_flag, ST_DQ_MMA)) ok = false;
+                return ok;
+            };
+#pragma unroll 1
+            for (int i = 0, nd = 0; flow.next(); ++i) {
+                if (flow.t == 0) { wait(Q_DOFULL + nd % NDO, nd / NDO); ++nd; }
+                const int b = (nd - 1) % NDO;
+                wait(Q_VFULL + i % NV, i / NV);
+                if (i > 0) wait(Q_DPFREE, i - 1);   // every thread holds dP(i - 1)
+                tc_fence_after_sync();
+                if (!ok) break;
+                mma_kk(tmem + colDP, smem_u32(sDO + b * kBytes), smem_u32(sV + (i % NV) * kBytes), HD, idescS, false);
+                umma_commit(&bars[Q_READY + ((i + 1) & 1)]);
+                umma_commit(&bars[Q_VEMPTY + i % NV]);
+                if (flow.t + 1 == flow.T) umma_commit(&bars[Q_DOEMPTY + b]);
             }
         }
+    } else if (warp >= 12) {
+        // ---------------------------------------------------------------- write-out of finished levels, one row per thread
+        set_fewer_regs<kRegsOut>();
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t tacc = tmem + ((uint32_t)((warp & 3) * 32) << 16) + colDQ;
+        // no key chunk visited (chunk 0, or block skipping left only the diagonal): the boundary-adjusted queries get a
+        // zero gradient from the sweep.  Levels that a shortened sweep does not reach stay unwritten: the version
+        // chain rule starts at the highest level reached.
+        auto zero_item = [&](int I, int s) {
+            uint4* dst = reinterpret_cast<uint4*>(p.dqv + ((size_t)s * p.Lp + (size_t)I * kTile) * HD);
+            for (int x = threadIdx.x - 384; x < kTile * HD / 8; x += 128) dst[x] = make_uint4(0u, 0u, 0u, 0u);
+            if (GATE) p.dGrow[(size_t)s * p.Lp + I * kTile + row] = 0.f;
+        };
+        auto flow = make_flow(item_of, steps_of, zero_item);
+#pragma unroll 1
+        for (int na = 0, nsum = 0; flow.next();) {
+            const int l = level(flow.c, flow.t), f = flags_of(flow.c, flow.t, flow.T, l);
+            if (!(f & FL_LVL1)) continue;
+            bool ok = mbar_wait(&bars[Q_ACCFULL], na & 1, abort_flag, ST_DQ_COMPUTE);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after_sync();
+            __nv_bfloat16* dst = p.dqv + ((size_t)qver_row(p.vl, flow.s, l, flow.c) + row) * HD;
+            constexpr int PIECES = EARLY ? 1 : HD / 32;   // of 32 columns, held at a time
+#pragma unroll 1
+            for (int c0 = 0; c0 < HD / 32; c0 += PIECES) {
+                uint32_t w[PIECES][16];
+#pragma unroll
+                for (int c = 0; c < PIECES; ++c) {
+                    float v[32];
+                    tile::tmem_row32(tacc + (c0 + c) * 32, v);
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) w[c][x] = pack_bf16(v[2 * x] * p.scale, v[2 * x + 1] * p.scale);
+                }
+                if (c0 + PIECES == HD / 32) {
+                    if (GATE && (f & FL_LAST)) {   // before the accumulators are handed back: three items on, the buffer is in use again
+                        const int buf = nsum % 3;
+                        if (!mbar_wait(&bars[Q_SUM + buf], (nsum / 3) & 1, abort_flag, ST_DQ_COMPUTE)) break;
+                        p.dGrow[(size_t)flow.s * p.Lp + flow.c * kTile + row] = dsum_x[buf * kTile + row];
+                        dsum_x[buf * kTile + row] = 0.f;
+                        ++nsum;
+                    }
+                    tc_fence_before_sync();
+                    mbar_arrive(&bars[Q_ACCFREE]);
+                }
+#pragma unroll
+                for (int c = 0; c < PIECES; ++c) tile::gstore_bf16_w16(dst + (c0 + c) * 32, w[c]);
+            }
+            ++na;
+        }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
+        set_more_regs<kRegsMath>();
         const int q4 = warp & 3, h = (warp - 4) >> 2, row = q4 * 32 + lane;
-        const uint32_t tlane = tmem + ((uint32_t)(q4 * 32) << 16);
+        const uint32_t tlane = tmem + ((uint32_t)(q4 * 32) << 16) + h * 64;   // this thread's 64 key columns
         const float sl2 = p.scale * kLog2e;
         const uint64_t sl2x2 = pack2(sl2, sl2), nlog2 = pack2(-kLog2e, -kLog2e);
-        bool ok = true;
-        int g = 0, na = 0;
-        constexpr int CW = HD / 2;
-        auto flush_dq = [&](int lvl) {
-            store_acc_bf16<CW>(p.dqv + ((size_t)qrow(lvl, I) + row) * HD + h * CW, tlane + colDQ + h * CW, p.scale);
-        };
-#pragma unroll 1
-        for (int it = 0; item_of(it, I, s); ++it) {
-            const int T = steps_of(I, s);
-            auto zero_dq = [&](int slot) {   // a whole [128 x HD] version gradient tile, by the 256 math threads
-                uint4* dst = reinterpret_cast<uint4*>(p.dqv + (size_t)row0(I) * HD);
-                for (int i = threadIdx.x - 128; i < kTile * HD / 8; i += 256) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-            };
-            // no key chunk visited (chunk 0, or block skipping left only the diagonal): the boundary-adjusted queries get a
-            // zero gradient from the sweep.  Levels that a shortened sweep does not reach stay unwritten: the version
-            // chain rule starts at the highest level reached.
-            if (T == 0) {
-                zero_dq(0);
-                if (GATE && h == 0) p.dGrow[(size_t)s * p.Lp + I * kTile + row] = 0.f;
-                continue;
+        float nl_n = 0.f, nd_n = 0.f, nd_a = 0.f;   // minus lse2 (plus gate prefix) and minus delta: next item; delta of A's row
+        uint64_t nl2 = 0, nd2 = 0;               // of A's row, of B's row
+        float dsum = 0.f;
+        float pr[64];                            // P of step i - 1, then of step i
+        int nsum = 0;
+        // One round: part A of step i from its S tile, part B of step i - 1 into it.
+        auto round = [&](auto a_tag, auto b_tag, const int i) {
+            constexpr bool A = decltype(a_tag)::value, B = decltype(b_tag)::value;
+            const uint32_t ts = tlane + colS + (i & 1) * 128;
+            constexpr int DC = EARLY ? 4 : 2;          // 16-column pieces of dP held at a time
+            uint32_t dp[DC][16], sv[2][16];
+            if (B) {
+#pragma unroll
+                for (int c = 0; c < DC - (EARLY ? 0 : 1); ++c) tmem_ld16(tlane + colDP + c * 16, dp[c]);
             }
-            const size_t qi = (size_t)s * p.Lp + I * kTile + row;
-            const float ndelta = p.delta[qi];            // minus delta
-            const float nl = p.lse2[qi];                 // minus lse2, plus the gate prefix of the row when gated
-            const uint64_t nl2 = pack2(nl, nl), nd2 = pack2(ndelta, ndelta);
-            float dsum = 0.f;
-#pragma unroll 1
-            for (int t = 0; t < T; ++t) {
-                const int gs = g + t;
-                const int c0 = h * 64;               // key columns of this thread
-                uint32_t pr[2][32];                  // S, then P (float bits)
-                // ---- part A: P = exp2(S * scale - lse)
-                if (GATE && ok && !mbar_wait(&bars[Q_GKFULL + (gs & 1)], (gs >> 1) & 1, abort_flag, ST_DQ_COMPUTE)) ok = false;
-                if (ok && !mbar_wait(&bars[Q_SFULL + (gs & 1)], (gs >> 1) & 1, abort_flag, ST_DQ_COMPUTE)) ok = false;
-                ok = __all_sync(0xffffffffu, ok);
-                tc_fence_after_sync();
-                if (ok) {
-                    tmem_ld32(tlane + colS + (gs & 1) * 128 + c0, pr[0]);
-                    tmem_ld32(tlane + colS + (gs & 1) * 128 + c0 + 32, pr[1]);
-                    tmem_ld_wait();
-                    const float* g_ = gk + (gs & 1) * kTile + c0;
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-#pragma unroll
-                        for (int x = 0; x < 32; x += 4) {
-                            uint64_t v01 = fma2(pack2(__uint_as_float(pr[c][x]), __uint_as_float(pr[c][x + 1])), sl2x2, nl2);
-                            uint64_t v23 = fma2(pack2(__uint_as_float(pr[c][x + 2]), __uint_as_float(pr[c][x + 3])), sl2x2, nl2);
-                            if (GATE) {
-                                const float4 g4 = *reinterpret_cast<const float4*>(g_ + c * 32 + x);
-                                v01 = fma2(pack2(g4.x, g4.y), nlog2, v01);
-                                v23 = fma2(pack2(g4.z, g4.w), nlog2, v23);
-                            }
-                            float e[4];
-                            unpack2(v01, e[0], e[1]);
-                            unpack2(v23, e[2], e[3]);
-#pragma unroll
-                            for (int y = 0; y < 4; ++y) pr[c][x + y] = __float_as_uint(ex2(e[y]));
-                        }
-                }
-                // ---- part B: dS = P o (dP - delta)
-                if (ok && !mbar_wait(&bars[Q_DPFULL], gs & 1, abort_flag, ST_DQ_COMPUTE)) ok = false;
-                ok = __all_sync(0xffffffffu, ok);
-                tc_fence_after_sync();
-                // dP ready means every product issued before it has retired: dQ of a finished level can be flushed
-                if (ok && t >= 1 && level(t) != level(t - 1)) flush_dq(level(t - 1));
-                if (ok) {
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        uint32_t dp[32], pk[16];
-                        tmem_ld32(tlane + colDP + c0 + c * 32, dp);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int x = 0; x < 32; x += 2) {
-                            const uint64_t d01 = mul2(pack2(__uint_as_float(pr[c][x]), __uint_as_float(pr[c][x + 1])),
-                                                      add2(pack2(__uint_as_float(dp[x]), __uint_as_float(dp[x + 1])), nd2));
-                            float d0, d1;
-                            unpack2(d01, d0, d1);
-                            if (GATE) dsum += d0 + d1;
-                            pk[x >> 1] = pack_bf16(d0, d1);
-                        }
-                        tmem_st16(tlane + colDP + c0 + c * 16, pk);
-                    }
-                    tmem_st_wait();
-                }
+            if (A) tmem_ld16(ts, sv[0]);
+            auto release_dp = [&]() {
                 tc_fence_before_sync();
-                mbar_arrive(&bars[Q_DSFULL]);
-                if (GATE) mbar_arrive(&bars[Q_GKEMPTY + (gs & 1)]);
+                mbar_arrive(&bars[Q_DPFREE]);
+            };
+            const float* g_ = gk + (i & 1) * kTile + h * 64;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (B && (c == 0 || !EARLY)) tmem_ld_wait16(dp[c % DC]);
+                if (A) tmem_ld_wait16(sv[c & 1]);
+                if (B && EARLY && c == 0) {
+#pragma unroll
+                    for (int x = 1; x < DC; ++x) tmem_ld_wait16(dp[x]);
+                    release_dp();
+                }
+                if (B && !EARLY && c < 3) tmem_ld16(tlane + colDP + (c + 1) * 16, dp[(c + 1) % DC]);
+                if (A && c < 3) tmem_ld16(ts + (c + 1) * 16, sv[(c + 1) & 1]);
+                if (B && !EARLY && c == 3) release_dp();
+                if (B) {   // dS = P o (dP - delta)
+                    uint32_t pk[8];
+#pragma unroll
+                    for (int x = 0; x < 16; x += 2) {
+                        const uint32_t* d_ = &dp[c % DC][x];
+                        const uint64_t d01 = mul2(pack2(pr[c * 16 + x], pr[c * 16 + x + 1]),
+                                                  add2(pack2(__uint_as_float(d_[0]), __uint_as_float(d_[1])), nd2));
+                        float d0, d1;
+                        unpack2(d01, d0, d1);
+                        if (GATE) dsum += d0 + d1;
+                        pk[x >> 1] = pack_bf16(d0, d1);
+                    }
+                    tmem_st8(ts + c * 16, pk);
+                }
+                if (A) {   // P = exp2(S * scale - lse)
+#pragma unroll
+                    for (int x = 0; x < 16; x += 4) {
+                        const uint32_t* s_ = &sv[c & 1][x];
+                        uint64_t v01 = fma2(pack2(__uint_as_float(s_[0]), __uint_as_float(s_[1])), sl2x2, nl2);
+                        uint64_t v23 = fma2(pack2(__uint_as_float(s_[2]), __uint_as_float(s_[3])), sl2x2, nl2);
+                        if (GATE) {
+                            const float4 g4 = *reinterpret_cast<const float4*>(g_ + c * 16 + x);
+                            v01 = fma2(pack2(g4.x, g4.y), nlog2, v01);
+                            v23 = fma2(pack2(g4.z, g4.w), nlog2, v23);
+                        }
+                        float e[4];
+                        unpack2(v01, e[0], e[1]);
+                        unpack2(v23, e[2], e[3]);
+#pragma unroll
+                        for (int y = 0; y < 4; ++y) pr[c * 16 + x + y] = ex2(e[y]);
+                    }
+                }
             }
-            g += T;
-            if (ok && !mbar_wait(&bars[Q_ACCFULL], na & 1, abort_flag, ST_DQ_COMPUTE)) ok = false;
-            ++na;
-            ok = __all_sync(0xffffffffu, ok);
-            tc_fence_after_sync();
-            if (GATE) {
-                if (h == 1) dsum_x[row] = dsum;
-                { __syncwarp(); asm volatile("bar.sync 1, 256;" ::: "memory"); }
-                if (h == 0 && ok) p.dGrow[qi] = dsum + dsum_x[row];
-                { __syncwarp(); asm volatile("bar.sync 1, 256;" ::: "memory"); }
-            }
-            if (ok) flush_dq(level(T - 1));
+            if (B) tmem_st_wait();
             tc_fence_before_sync();
-            mbar_arrive(&bars[Q_ACCFREE]);
+            // (two barriers: round i + 1 does not wait for the slowest warp of round i, round i + 2 does)
+            mbar_arrive(&bars[Q_ROUND + (i & 1)]);
+            if (GATE && A) mbar_arrive(&bars[Q_GKEMPTY + (i & 1)]);
+        };
+        int fb = 0;   // flags of step i - 1
+#pragma unroll 1
+        for (int i = 0;; ++i) {
+            bool ok = mbar_wait(&bars[Q_READY + (i & 1)], (i >> 1) & 1, abort_flag, ST_DQ_COMPUTE);
+            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
+            tc_fence_after_sync();
+            const int4 de = desc[i & 7];
+            const int fa = de.x;
+            if (fb & FL_FIRST) nd2 = pack2(nd_a, nd_a);
+            if (fa & FL_FIRST) {   // this item's row constants were requested when the previous item began
+                if (i == 0) { nl_n = p.lse2[de.y + row]; nd_n = p.delta[de.y + row]; }
+                nl2 = pack2(nl_n, nl_n);
+                nd_a = nd_n;
+                if (de.w >= 0) { nl_n = p.lse2[de.w + row]; nd_n = p.delta[de.w + row]; }
+            }
+            if (fa) {
+                if (fb) round(std::true_type{}, std::true_type{}, i);
+                else round(std::true_type{}, std::false_type{}, i);
+            } else {
+                if (fb) round(std::false_type{}, std::true_type{}, i);
+            }
+            if (GATE && (fb & FL_LAST)) {   // the two threads of a row add their halves (two addends: in any order)
+                const int buf = nsum++ % 3;
+                atomicAdd(dsum_x + buf * kTile + row, dsum);
+                mbar_arrive(&bars[Q_SUM + buf]);
+                dsum = 0.f;
+            }
+            if (!fa) break;
+            fb = fa;
         }
     }
     tc_fence_before_sync();
@@ -866,7 +1021,7 @@ cudaError_t launch_one(const BwdTensorMaps& tm, const BwdParams& p, int which, c
     if (e != cudaSuccess) return e;
     const int pairs = (p.N * p.S + 1) / 2, grid = pairs < sms ? pairs : sms;
     return which == 0 ? launch<dkv_kernel<HD, GATE>>(grid, 384, kSmemAlloc, st, tm, p)
-                      : launch<dq_kernel<HD, GATE>>(grid, 384, kSmemAlloc, st, tm, p);
+                      : launch<dq_kernel<HD, GATE>>(grid, 512, kSmemAlloc, st, tm, p);
 }
 
 }  // namespace

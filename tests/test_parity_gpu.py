@@ -166,6 +166,34 @@ def test_forward_pairs_of_query_chunks(binding, oracle, B, H, L, d, gate, scale)
     compare_all(binding, oracle, inp, scale=scale, idx=idx, backward=False)
 
 
+@pytest.mark.parametrize("B,H,L,d,gate", [
+    (5, 61, 300, 64, True),       # items of 2, 0 and 1 steps, three pairs of items per CTA
+    (2, 150, 200, 128, False),    # items of one step or none
+    (2, 37, 1500, 64, False),     # 0 .. 11 steps, several levels per item, ragged tail
+    (1, 40, 2176, 128, True),     # odd chunk count, block skipping
+])
+def test_backward_rounds_across_items(binding, B, H, L, d, gate):
+    """Steps of different items follow one another in the sweeps' pipelines: a slice's gradients must not depend on the
+    slices that share its CTAs (equal to the bit: the same sums in the same order)."""
+    g = torch.Generator(device="cuda").manual_seed(900 + L)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    q, k, v, d_o = (n(B, H, L, d).bfloat16() for _ in range(4))
+    w = torch.nn.functional.normalize(n(B, H, L, d), dim=-1).bfloat16()
+    beta = 2 * torch.sigmoid(n(B, H, L))
+    log_f = torch.nn.functional.logsigmoid(n(B, H, L) + 3) if gate else None
+    o, lse = binding.path_attn_fwd(q, k, v, w, beta, log_f)
+
+    def grads(pick):
+        a = [x[pick].contiguous() if x is not None else None for x in (q, k, v, w, beta, o, lse, d_o, log_f)]
+        return binding.path_attn_bwd(*a)
+
+    full = grads((slice(None), slice(None)))
+    for b, h in ((0, 0), (B // 2, H // 2), (B - 1, H - 1)):
+        one = grads((slice(b, b + 1), slice(h, h + 1)))
+        for name in ("dq", "dk", "dv", "dw"):
+            assert torch.isfinite(full[name]).all() and torch.equal(full[name][b, h], one[name][0, 0]), (name, b, h)
+
+
 def _random_cases(n, seed=20250516):
     """Seeded list of small problems: lengths below, at and across chunk boundaries, both head sizes, gate, scale sign."""
     import random
