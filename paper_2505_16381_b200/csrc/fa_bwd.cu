@@ -9,7 +9,7 @@
 //   diagonal chunk: (scale lower(dS))^T is stored for the per-chunk chain rule; its row sums in float32 if gated.
 //
 // Two kernels so that every accumulator stays in tensor memory and nothing is added atomically:
-//   dkv_kernel: one CTA per key chunk J, sweeps the query chunks I = J..N-1 with transposed tiles
+//   dkv_kernel, dkv64_kernel: one CTA per key chunk J, sweeps the query chunks I = J..N-1 with transposed tiles
 //               (TMEM lanes = keys): S^T = K Q^T, dP^T = V dO^T, dV += P^T dO, dK += dS^T Q.
 //   dq_kernel : one CTA per query chunk I, sweeps J = I-1..0: S = Q K^T, dP = dO V^T, dQ += dS K.
 // The accumulator of a version is flushed to global memory when the sweep crosses into the next level.
@@ -17,9 +17,10 @@
 // read, as packed bf16, and enter the second products as tensor-memory A operands.
 //
 // The elementwise work of a step is split in two so that it overlaps the tensor pipe: part A turns S into P (the
-// exponentials) as soon as S is there, while the dP product still runs; part B forms dS once dP has arrived.  The
-// products are issued in the order  dV(t), S(t+1), dK(t), dP(t+1)  (dkv) and  dQ(t), dP(t+1), S(t+2)  (dq, which has
-// room for two S tiles), so the pipe always has the next step's logits in flight.  (dq_kernel goes further: see there.)
+// exponentials) as soon as S is there, while the dP product still runs; part B forms dS once dP has arrived.  dkv_kernel
+// issues its products in the order  dV(t), S(t+1), dK(t), dP(t+1),  so the pipe always has the next step's logits in flight.
+// Where tensor memory has room for two S tiles (dq_kernel; dkv64_kernel for d = 64 without a gate) the two parts of
+// neighbouring steps share one pass.
 // Warps of dkv_kernel: 0 = TMA producer, 1 = tcgen05 MMA issuer, 2-3 idle (their registers go to the others), 4-11 = elementwise
 // math (two warps per TMEM lane quadrant, each taking 64 of the 128 columns of a row).
 #include <type_traits>
@@ -606,7 +607,7 @@ __device__ __forceinline__ void tmem_ld_wait16(uint32_t (&r)[16]) {
 // D[tmem] (+)= A B with A in tensor memory: the 16 contraction indices of step kk in the 8 columns at a_col + 16 kk.
 __device__ __forceinline__ void mma_t16(uint32_t d_tmem, uint32_t a_col, uint32_t b0, uint32_t idesc, bool acc) {
     uint32_t b_lo = umma_desc_lo(b0, kPanelBytes);
-#pragma unroll
+#pragma unroll 2
     for (int kk = 0; kk < kTile / 16; ++kk) {
         umma_ts(d_tmem, a_col + kk * 16, umma_desc_join(b_lo), idesc, (acc || kk > 0) ? 1u : 0u);
         b_lo += 128u;
@@ -844,7 +845,9 @@ __global__ void __launch_bounds__(512, 1) dq_kernel(const __grid_constant__ BwdT
                 if (c0 + PIECES == HD / 32) {
                     if (GATE && (f & FL_LAST)) {   // before the accumulators are handed back: three items on, the buffer is in use again
                         const int buf = nsum % 3;
-                        if (!mbar_wait(&bars[Q_SUM + buf], (nsum / 3) & 1, abort_flag, ST_DQ_COMPUTE)) break;
+                        ok = mbar_wait(&bars[Q_SUM + buf], (nsum / 3) & 1, abort_flag, ST_DQ_COMPUTE);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
                         p.dGrow[(size_t)flow.s * p.Lp + flow.c * kTile + row] = dsum_x[buf * kTile + row];
                         dsum_x[buf * kTile + row] = 0.f;
                         ++nsum;
@@ -976,6 +979,441 @@ __global__ void __launch_bounds__(512, 1) dq_kernel(const __grid_constant__ BwdT
     }
 }
 
+// ------------------------------------------------------------------------------------------------ dK, dV for d = 64, no gate
+// dkv_kernel's sweep in the rounds of dq_kernel: at d = 64 the accumulators leave room for two S^T tiles, and the products
+// (1050 cycles a step) are not what bounds it.  Round i of the math warps turns S^T(i) into P^T(i) and forms dS^T(i - 1); of the 16
+// columns of a group of S^T(i) P^T(i) takes the first 8 and dS^T(i - 1) the last 8.  A round takes 1900 cycles (4400 one half after
+// the other), 2000 to 3000 more on the diagonal step, whose passes are fetched anew each time.  Then dK (+)= dS^T(i - 1) Q, dV (+)= P^T(i) dO
+// and S^T(i + 2) into the same tile follow in order.
+// Warps: 0 = producer of Q (ring of 4), K (2), Xq, row constants (4) and step descriptions, 1 = tcgen05 issue of S, dK and dV,
+// 2 = producer of dO (ring of 4) and V, 3 = tcgen05 issue of dP, 4-11 = elementwise math, 12-15 = write-out.
+// Y of a diagonal step takes two entries of the dO ring, in halves of 64 columns.  Ring sizes: S(i + 2) is issued before
+// Q(i) is released, and dO(i + 1) is still held when Y of a step i + 2 has to be there.
+enum { D_QFULL = 0, D_QEMPTY = 4, D_DOFULL = 8, D_DOEMPTY = 12, D_KFULL = 16, D_KEMPTY = 18, D_VFULL = 20, D_VEMPTY, D_XFULL, D_XEMPTY, D_STEMPTY,
+       D_READY = D_STEMPTY + 4, D_DPFREE = D_READY + 2, D_ROUND, D_DKFULL = D_ROUND + 2, D_DKFREE, D_DVFULL, D_DVFREE, D_COUNT };
+constexpr uint32_t kD64Tile = kTile * 64 * 2;
+constexpr uint32_t kD64Bars = 13 * kD64Tile, kD64Desc = kD64Bars + 384, kD64Stat = kD64Desc + 8 * 8;
+constexpr uint32_t kD64Total = kD64Stat + 4 * 2 * kTile * 4;
+static_assert(D_COUNT * 8 + 8 <= 384 && kD64Total + 1024 <= kSmemAlloc, "shared memory of the d = 64 dK/dV sweep");
+
+__global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ BwdTensorMaps tm, const BwdParams p) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    constexpr int HD = 64, NQ = 4, ND = 4;
+    uint8_t* sQ = smem;
+    uint8_t* sDO = sQ + NQ * kD64Tile;
+    uint8_t* sK = sDO + ND * kD64Tile;
+    uint8_t* sV = sK + 2 * kD64Tile;
+    uint8_t* sX = sV + kD64Tile;                  // two panels
+    uint64_t* bars = (uint64_t*)(smem + kD64Bars);
+    uint32_t* tmem_slot = (uint32_t*)(bars + D_COUNT);
+    volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);
+    int2* desc = (int2*)(smem + kD64Desc);        // flags, first row of the key chunk
+    float* stat = (float*)(smem + kD64Stat);      // [4][2][128]: -lse2, -delta of the queries of a step
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int items = p.N * p.S;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < D_COUNT; ++i)
+            mbar_init(&bars[i], i == D_READY || i == D_READY + 1 ? 3u
+                              : i >= D_DOEMPTY && i < D_DOEMPTY + ND ? 2u        // dO serves dP and dV
+                              : i == D_DPFREE || i == D_ROUND || i == D_ROUND + 1 || (i >= D_STEMPTY && i < D_READY) ? 256u
+                              : i == D_DKFREE || i == D_DVFREE ? 128u : 1u);
+        *abort_flag = 0;
+        mbar_fence_init();
+    }
+    if (warp == 3 && lane < 8) tma_prefetch_desc(reinterpret_cast<const CUtensorMap*>(&tm) + lane);
+    if (warp == 1) tmem_alloc(tmem_slot, 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+    grid_wait();
+    grid_launch();
+    constexpr uint32_t colS = 0, colDP = 256, colDV = 384, colDK = 448;   // two S tiles at 0 and 128
+    static_assert(256 * 200 + 256 * 56 <= 65536, "registers: no more than the block was launched with");
+    // items and steps as in dkv_kernel
+    auto item_of = [&](int k, int& J, int& s) {
+        const int w = 2 * ((int)blockIdx.x + (k >> 1) * (int)gridDim.x) + (k & 1);
+        if (w >= items) return false;
+        s = w / p.N;
+        const int j = w % p.N;
+        J = (j & 1) ? p.N - 1 - (j >> 1) : (j >> 1);
+        return true;
+    };
+    auto steps_of = [&](int J, int s) { return p.N - J; };
+    auto level = [](int J, int t) { return msb32((unsigned)((J + t) ^ J)); };   // t >= 1
+    auto flags_of = [](int J, int t, int T, int l) {   // level l covers the query chunks whose low l bits run from zero up to all ones
+        const int I = J + t, m = (1 << l) - 1, last = t + 1 == T;
+        if (t == 0) return FL_VALID | FL_FIRST | FL_LVL0 | FL_LVL1 | (last ? FL_LAST : 0);   // raw q and k: a level of its own
+        return FL_VALID | (last ? FL_LAST : 0) | ((I & m) == 0 ? FL_LVL0 : 0) | (last || (I & m) == m ? FL_LVL1 : 0);
+    };
+
+    if (warp < 4) {
+        set_fewer_regs<56>();
+        if (warp == 0 && elect_one()) {
+            auto flow = make_flow(item_of, steps_of);
+            bool ok = true;
+            int nk = 0, nx = 0, n = 0;   // K tiles, items, steps (Q ring entries) so far
+            auto wait_empty = [&](int bar, int use) {
+                if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_DKV_PRODUCER)) ok = false;
+                return ok;
+            };
+#pragma unroll 1
+            for (; ok; ++n) {
+                const bool more = flow.next();
+                if (!wait_empty(D_QEMPTY + n % NQ, n / NQ)) break;
+                if (!more) {
+                    desc[n & 7] = make_int2(0, 0);
+                    mbar_arrive(&bars[D_QFULL + n % NQ]);
+                    break;
+                }
+                const int J = flow.c, s = flow.s, I = J + flow.t, l = flow.t ? level(J, flow.t) : 0, f = flags_of(J, flow.t, flow.T, l);
+                desc[n & 7] = make_int2(f, s * p.Lp + J * kTile);
+                // the row constants of the step travel with Q
+                const int sb = n & 3, q0 = n % NQ;
+                mbar_expect_tx(&bars[D_QFULL + q0], kD64Tile + 2 * kTile * 4);
+                if (f & FL_FIRST) tma_rows(sQ + q0 * kD64Tile, &tm.q_raw, &bars[D_QFULL + q0], HD, J * kTile, s);
+                else tma_tile(sQ + q0 * kD64Tile, &tm.qv, &bars[D_QFULL + q0], HD, (int)qver_row(p.vl, s, l, I));
+                if (!wait_empty(D_STEMPTY + sb, n >> 2)) break;
+                const size_t gi = (size_t)s * p.Lp + I * kTile;
+                bulk_load(stat + sb * 2 * kTile, p.lse2 + gi, kTile * 4, &bars[D_QFULL + q0]);
+                bulk_load(stat + sb * 2 * kTile + kTile, p.delta + gi, kTile * 4, &bars[D_QFULL + q0]);
+                if (f & FL_LVL0) {
+                    const int b = nk & 1;
+                    if (!wait_empty(D_KEMPTY + b, nk >> 1)) break;
+                    mbar_expect_tx(&bars[D_KFULL + b], kD64Tile);
+                    if (f & FL_FIRST) tma_rows(sK + b * kD64Tile, &tm.k_raw, &bars[D_KFULL + b], HD, J * kTile, s);
+                    else tma_tile(sK + b * kD64Tile, &tm.kv, &bars[D_KFULL + b], HD, (int)kver_row(p.vl, s, l, J));
+                    ++nk;
+                }
+                if (f & FL_FIRST) {
+                    if (!wait_empty(D_XEMPTY, nx)) break;
+                    mbar_expect_tx(&bars[D_XFULL], 2 * kD64Tile);
+                    tma_tile(sX, &tm.xq, &bars[D_XFULL], kTile, s * p.Lp + J * kTile);
+                    ++nx;
+                }
+            }
+        } else if (warp == 2 && elect_one()) {
+            auto flow = make_flow(item_of, steps_of);
+            bool ok = true;
+            int dn = 0, nv = 0;
+            auto wait_empty = [&](int bar, int use) {
+                if (ok && !mbar_wait(&bars[bar], (use & 1) ^ 1, abort_flag, ST_DKV_PRODUCER)) ok = false;
+                return ok;
+            };
+            auto entry = [&]() { return wait_empty(D_DOEMPTY + dn % ND, dn / ND); };
+#pragma unroll 1
+            while (ok && flow.next()) {
+                const int J = flow.c, s = flow.s;
+                if (flow.t == 0) {
+                    if (dn & 1) {   // the halves of Y lie one after the other: an entry is left out
+                        if (!entry()) break;
+                        mbar_arrive(&bars[D_DOFULL + dn % ND]);
+                        ++dn;
+                    }
+                    for (int h = 0; h < 2; ++h, ++dn) {
+                        if (!entry()) break;
+                        mbar_expect_tx(&bars[D_DOFULL + dn % ND], kD64Tile);
+                        tma_load_2d(sDO + (dn % ND) * kD64Tile, &tm.y, &bars[D_DOFULL + dn % ND], h * 64, s * p.Lp + J * kTile);
+                    }
+                    if (!wait_empty(D_VEMPTY, nv)) break;
+                    mbar_expect_tx(&bars[D_VFULL], kD64Tile);
+                    tma_rows(sV, &tm.v, &bars[D_VFULL], HD, J * kTile, s);
+                    ++nv;
+                }
+                if (!entry()) break;
+                mbar_expect_tx(&bars[D_DOFULL + dn % ND], kD64Tile);
+                tma_rows(sDO + (dn % ND) * kD64Tile, &tm.d_o, &bars[D_DOFULL + dn % ND], HD, (J + flow.t) * kTile, s);
+                ++dn;
+            }
+        } else if (warp == 1 && elect_one()) {
+            constexpr uint32_t idescT = umma_idesc(128, 128, 0, 0);
+            constexpr uint32_t idescD = umma_idesc(128, HD, 0, 1);
+            bool ok = true;
+            int dn = 0, nk = 0, nx = 0, ndk = 0, ndv = 0;   // entries of the dO ring, K tiles, items, levels and items finished so far
+            int d2 = 0;                                     // ring entry of dO of the step that issue_s looked at last
+            auto wait = [&](int bar, int parity) {
+                if (ok && !mbar_wait(&bars[bar], parity & 1, abort_flag, ST_DKV_MMA)) ok = false;
+                return ok;
+            };
+            // S^T of step g; returns its flags, 0 after the last step (see dq_kernel)
+            auto issue_s = [&](int g) {
+                if (!wait(D_QFULL + g % NQ, g / NQ)) return 0;
+                const int f = desc[g & 7].x;
+                if (f) {
+                    if (f & FL_LVL0) { wait(D_KFULL + (nk & 1), nk >> 1); ++nk; }
+                    const int kb = (nk - 1) & 1;
+                    if (f & FL_FIRST) {
+                        if (dn & 1) {
+                            wait(D_DOFULL + dn % ND, dn / ND);
+                            mbar_arrive(&bars[D_DOEMPTY + dn % ND]);
+                            mbar_arrive(&bars[D_DOEMPTY + dn % ND]);
+                            ++dn;
+                        }
+                        for (int h = 0; h < 2; ++h) wait(D_DOFULL + (dn + h) % ND, (dn + h) / ND);
+                        wait(D_XFULL, nx);
+                        ++nx;
+                    }
+                    tc_fence_after_sync();
+                    if (!ok) return 0;
+                    mma_kk(tmem + colS + (g & 1) * 128, smem_u32(sK + kb * kD64Tile), smem_u32(sQ + (g % NQ) * kD64Tile), HD, idescT, false);
+                    if (f & FL_FIRST) {   // S^T -= Y^T Xq^T: Y as stored ([contraction][keys], MN-major), Xq K-major
+                        const uint32_t a_lo = umma_desc_lo(smem_u32(sDO + (dn % ND) * kD64Tile), kPanelBytes), b_lo = umma_desc_lo(smem_u32(sX), 16);
+#pragma unroll
+                        for (int kk = 0; kk < kTile / 16; ++kk)
+                            umma_ss(tmem + colS + (g & 1) * 128, umma_desc_join(a_lo + kk * 128u),
+                                    umma_desc_join(b_lo + (uint32_t)(kk >> 2) * (kPanelBytes >> 4) + (uint32_t)(kk & 3) * 2u),
+                                    umma_idesc(128, 128, 1, 0) | (1u << 13), 1u);
+                        umma_commit(&bars[D_QEMPTY + g % NQ]);   // (raw q serves no other product)
+                        umma_commit(&bars[D_XEMPTY]);
+                        for (int h = 0; h < 4; ++h) umma_commit(&bars[D_DOEMPTY + (dn + (h & 1)) % ND]);
+                        dn += 2;
+                    }
+                    d2 = dn++;
+                    umma_commit(&bars[D_READY + (g & 1)]);
+                    if (f & FL_LVL1) umma_commit(&bars[D_KEMPTY + kb]);
+                } else {   // the last round has no S: its tile is free once the products that read it have retired
+                    umma_commit(&bars[D_READY + (g & 1)]);
+                }
+                mbar_arrive(&bars[D_READY + (g & 1)]);
+                return f;
+            };
+            int fm = 0;                                  // flags of step i - 1
+            int f0 = issue_s(0), d0 = d2;                // step i
+            int f1 = f0 ? issue_s(1) : 0, d1 = d2;
+            if (ok) mbar_arrive(&bars[D_READY]);         // (no dP before round 0)
+#pragma unroll 1
+            for (int i = 0; ok && (f0 | fm); ++i) {
+                if (!wait(D_ROUND + (i & 1), i >> 1)) break;
+                const uint32_t tile = tmem + colS + (i & 1) * 128;
+                if (fm && !(fm & FL_FIRST)) {            // dK (+)= dS^T(i - 1) Q
+                    if ((fm & FL_LVL0) && ndk > 0 && !wait(D_DKFREE, ndk - 1)) break;
+                    tc_fence_after_sync();
+                    mma_t16(tmem + colDK, tile + 8, smem_u32(sQ + ((i - 1) % NQ) * kD64Tile), idescD, !(fm & FL_LVL0));
+                    umma_commit(&bars[D_QEMPTY + (i - 1) % NQ]);
+                    if (fm & FL_LVL1) { umma_commit(&bars[D_DKFULL]); ++ndk; }
+                }
+                if (f0) {                                // dV (+)= P^T(i) dO
+                    if ((f0 & FL_FIRST) && ndv > 0 && !wait(D_DVFREE, ndv - 1)) break;
+                    if (!wait(D_DOFULL + d0 % ND, d0 / ND)) break;
+                    tc_fence_after_sync();
+                    mma_t16(tmem + colDV, tile, smem_u32(sDO + (d0 % ND) * kD64Tile), idescD, !(f0 & FL_FIRST));
+                    umma_commit(&bars[D_DOEMPTY + d0 % ND]);
+                    if (f0 & FL_LAST) { umma_commit(&bars[D_DVFULL]); ++ndv; }
+                }
+                const int f2 = f1 ? issue_s(i + 2) : 0;
+                fm = f0;
+                f0 = f1; d0 = d1;
+                f1 = f2; d1 = d2;
+            }
+        } else if (warp == 3 && elect_one()) {
+            constexpr uint32_t idescT = umma_idesc(128, 128, 0, 0);
+            auto flow = make_flow(item_of, steps_of);
+            bool ok = true;
+            int dn = 0, nv = 0;
+            auto wait = [&](int bar, int parity) {
+                if (ok && !mbar_wait(&bars[bar], parity & 1, abort_flag, ST_DKV_MMA)) ok = false;
+                return ok;
+            };
+#pragma unroll 1
+            for (int i = 0; flow.next(); ++i) {
+                if (flow.t == 0) {
+                    dn = ((dn + 1) & ~1) + 2;
+                    wait(D_VFULL, nv);
+                    ++nv;
+                }
+                // Every thread holds dP(i - 1).  This comes first: it says that S(i) is there, hence Y and all entries before it, which
+                // this thread does not wait for; a slot's phase below is then the current one.
+                if (i > 0) wait(D_DPFREE, i - 1);
+                wait(D_DOFULL + dn % ND, dn / ND);
+                tc_fence_after_sync();
+                if (!ok) break;
+                mma_kk(tmem + colDP, smem_u32(sV), smem_u32(sDO + (dn % ND) * kD64Tile), HD, idescT, false);
+                umma_commit(&bars[D_READY + ((i + 1) & 1)]);
+                umma_commit(&bars[D_DOEMPTY + dn % ND]);
+                if (flow.t + 1 == flow.T) umma_commit(&bars[D_VEMPTY]);
+                ++dn;
+            }
+        }
+    } else if (warp >= 12) {
+        // ---------------------------------------------------------------- write-out of finished levels and items, one row per thread
+        set_fewer_regs<56>();
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        auto flow = make_flow(item_of, steps_of);
+        int ndk = 0, ndv = 0;
+        bool ok = true;
+        auto ready = [&](int bar, int n) {
+            ok = mbar_wait(&bars[bar], n & 1, abort_flag, ST_DKV_COMPUTE);
+            ok = __all_sync(0xffffffffu, ok);
+            tc_fence_after_sync();
+            return ok;
+        };
+        auto write = [&](uint32_t col, float mul, int free_bar, __nv_bfloat16* dst, bool valid) {
+#pragma unroll 1
+            for (int c = 0; c < 2; ++c) {
+                float v[32];
+                uint32_t w[16];
+                tile::tmem_row32(tl + col + c * 32, v);
+                if (c == 1) {
+                    tc_fence_before_sync();
+                    mbar_arrive(&bars[free_bar]);
+                }
+#pragma unroll
+                for (int x = 0; x < 16; ++x) w[x] = pack_bf16(v[2 * x] * mul, v[2 * x + 1] * mul);
+                tile::gstore_bf16_w16(dst + c * 32, w, valid);
+            }
+        };
+#pragma unroll 1
+        while (flow.next()) {
+            const int J = flow.c, s = flow.s, kj = J * kTile + row;
+            const bool last = flow.t + 1 == flow.T;
+            if (last) {   // dV first: the next item's first product waits for it
+                if (!ready(D_DVFULL, ndv)) break;
+                write(colDV, 1.f, D_DVFREE, (__nv_bfloat16*)p.dv + ((size_t)s * p.L + (kj < p.L ? kj : 0)) * HD, kj < p.L);
+                ++ndv;
+            }
+            if (flow.t == 0) {
+                if (last) {   // no later query chunk met: the boundary-adjusted keys get a zero gradient from the sweep
+                    uint4* dst = reinterpret_cast<uint4*>(p.dkv + ((size_t)s * p.Lp + kj) * HD);
+                    for (int x = 0; x < HD / 8; ++x) dst[x] = make_uint4(0u, 0u, 0u, 0u);
+                }
+                continue;
+            }
+            const int l = level(J, flow.t);
+            if (!(flags_of(J, flow.t, flow.T, l) & FL_LVL1)) continue;
+            if (!ready(D_DKFULL, ndk)) break;
+            write(colDK, p.scale, D_DKFREE, p.dkv + ((size_t)kver_row(p.vl, s, l, J) + row) * HD, true);
+            ++ndk;
+        }
+    } else {
+        set_more_regs<200>();
+        const int q4 = warp & 3, h = (warp - 4) >> 2, row = q4 * 32 + lane;
+        const uint32_t tlane = tmem + ((uint32_t)(q4 * 32) << 16) + h * 64;   // this thread's 64 query columns
+        // (a scale of zero: far below one ulp of any exponent instead, so that a masked logit still vanishes)
+        const float sl2 = p.scale == 0.f ? 1e-30f : p.scale * kLog2e;
+        const uint32_t masked = sl2 > 0.f ? 0xff800000u : 0x7f800000u;   // times sl2: minus infinity
+        const uint64_t sl2x2 = pack2(sl2, sl2);
+        float pr[64];                              // P^T of step i - 1, then of step i
+#pragma unroll
+        for (int x = 0; x < 64; ++x) pr[x] = 0.f;
+        // One round: part A of step i from its S^T tile, part B of step i - 1 into it.  The first and the last round use this code too
+        // (the half without a step works on what it finds and nothing reads its results), and so do the diagonal steps: instruction
+        // fetch is what a round waits for most, and a copy of this code that runs once per item cost 3000 cycles each time.
+        auto round = [&](const int i, const int fa, const int fb) {
+            const uint32_t ts = tlane + colS + (i & 1) * 128;
+            if (fa & FL_FIRST) {   // causal mask of the diagonal chunk, put into the logits
+#pragma unroll 1
+                for (int c = 0; c < 64; c += 16) {
+                    uint32_t m[16];
+                    tmem_ld16(ts + c, m);
+                    tmem_ld_wait16(m);
+#pragma unroll
+                    for (int x = 0; x < 16; ++x)
+                        if (h * 64 + c + x < row) m[x] = masked;
+                    tmem_st16(ts + c, m);
+                }
+                tmem_st_wait();
+            }
+            uint32_t dp[4][16], sv[2][16];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tmem_ld16(tlane + colDP + c * 16, dp[c]);
+            tmem_ld16(ts, sv[0]);
+            const float* ls_ = stat + (i & 3) * 2 * kTile + h * 64;                    // -lse2 of step i
+            const float* dl_ = stat + ((i - 1) & 3) * 2 * kTile + kTile + h * 64;      // -delta of step i - 1
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                tmem_ld_wait16(sv[c & 1]);
+                if (c == 0) {   // dP too has arrived
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) tmem_ld_wait16(dp[x]);
+                    tc_fence_before_sync();
+                    if (fb) mbar_arrive(&bars[D_DPFREE]);
+                }
+                if (c < 3) tmem_ld16(ts + (c + 1) * 16, sv[(c + 1) & 1]);
+                uint32_t pk[16];   // P^T(i), dS^T(i - 1)
+#pragma unroll
+                for (int x = 0; x < 16; x += 4) {   // dS^T = P^T o (dP^T - delta)
+                    const uint32_t* d_ = &dp[c][x];
+                    const float4 dl = *reinterpret_cast<const float4*>(dl_ + c * 16 + x);
+                    float d[4];
+                    unpack2(mul2(pack2(pr[c * 16 + x], pr[c * 16 + x + 1]),
+                                 add2(pack2(__uint_as_float(d_[0]), __uint_as_float(d_[1])), pack2(dl.x, dl.y))), d[0], d[1]);
+                    unpack2(mul2(pack2(pr[c * 16 + x + 2], pr[c * 16 + x + 3]),
+                                 add2(pack2(__uint_as_float(d_[2]), __uint_as_float(d_[3])), pack2(dl.z, dl.w))), d[2], d[3]);
+                    pk[8 + (x >> 1)] = pack_bf16(d[0], d[1]);
+                    pk[9 + (x >> 1)] = pack_bf16(d[2], d[3]);
+                }
+#pragma unroll
+                for (int x = 0; x < 16; x += 4) {   // P^T = exp2(S^T * scale - lse)
+                    const uint32_t* s_ = &sv[c & 1][x];
+                    const float4 ls = *reinterpret_cast<const float4*>(ls_ + c * 16 + x);
+                    uint64_t v01 = fma2(pack2(__uint_as_float(s_[0]), __uint_as_float(s_[1])), sl2x2, pack2(ls.x, ls.y));
+                    uint64_t v23 = fma2(pack2(__uint_as_float(s_[2]), __uint_as_float(s_[3])), sl2x2, pack2(ls.z, ls.w));
+                    float e[4];
+                    unpack2(v01, e[0], e[1]);
+                    unpack2(v23, e[2], e[3]);
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) pr[c * 16 + x + y] = ex2(e[y]);
+                    pk[x >> 1] = pack_bf16(pr[c * 16 + x], pr[c * 16 + x + 1]);
+                    pk[(x >> 1) + 1] = pack_bf16(pr[c * 16 + x + 2], pr[c * 16 + x + 3]);
+                }
+                tmem_st16(ts + c * 16, pk);
+            }
+            tmem_st_wait();
+            tc_fence_before_sync();
+            mbar_arrive(&bars[D_ROUND + (i & 1)]);
+            if (fb) mbar_arrive(&bars[D_STEMPTY + ((i - 1) & 3)]);
+        };
+        // The diagonal chunk's (scale * dS)^T in bf16 for the chain rule; `base` = the chunk's first row.
+        auto diagonal = [&](const int i, const int base) {
+            const float* dl_ = stat + (i & 3) * 2 * kTile + kTile + h * 64;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t dp[16], w[8];
+                float d[16];
+                tmem_ld16(tlane + colDP + c * 16, dp);
+                tmem_ld_wait16(dp);
+#pragma unroll
+                for (int x = 0; x < 16; x += 4) {
+                    const float4 dl = *reinterpret_cast<const float4*>(dl_ + c * 16 + x);
+                    d[x] = pr[c * 16 + x] * (__uint_as_float(dp[x]) + dl.x);
+                    d[x + 1] = pr[c * 16 + x + 1] * (__uint_as_float(dp[x + 1]) + dl.y);
+                    d[x + 2] = pr[c * 16 + x + 2] * (__uint_as_float(dp[x + 2]) + dl.z);
+                    d[x + 3] = pr[c * 16 + x + 3] * (__uint_as_float(dp[x + 3]) + dl.w);
+                }
+#pragma unroll
+                for (int x = 0; x < 8; ++x) w[x] = pack_bf16(d[2 * x] * p.scale, d[2 * x + 1] * p.scale);
+                tile::st_global_v8(p.dsdt + ((size_t)base + row) * kTile + h * 64 + c * 16, w);
+            }
+        };
+        int fb = 0, base = 0;   // step i - 1: flags, first row of the key chunk
+#pragma unroll 1
+        for (int i = 0;; ++i) {
+            bool ok = mbar_wait(&bars[D_READY + (i & 1)], (i >> 1) & 1, abort_flag, ST_DKV_COMPUTE);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after_sync();
+            const int2 de = desc[i & 7];
+            const int fa = de.x;
+            if (!(fa | fb)) break;
+            if (fb & FL_FIRST) diagonal(i - 1, base);
+            round(i, fa, fb);
+            if (!fa) break;
+            fb = fa;
+            base = de.y;
+        }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    if (warp == 1) {
+        tc_fence_after_sync();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
 // Per-row constants of the backward sweeps, stored negated so that they enter as addends:
 //   delta[i] = -(dO_i . O_i),   lse2[i] = (G_i - lse_i) * log2(e)   (G: gate prefix, absent = 0),
 // padded to Lp (tail rows: delta 0, lse2 -1e30 so that their probabilities vanish).  One warp per row.
@@ -1020,8 +1458,14 @@ cudaError_t launch_one(const BwdTensorMaps& tm, const BwdParams& p, int which, c
     const cudaError_t e = sm_count(sms);
     if (e != cudaSuccess) return e;
     const int pairs = (p.N * p.S + 1) / 2, grid = pairs < sms ? pairs : sms;
-    return which == 0 ? launch<dkv_kernel<HD, GATE>>(grid, 384, kSmemAlloc, st, tm, p)
-                      : launch<dq_kernel<HD, GATE>>(grid, 512, kSmemAlloc, st, tm, p);
+    // dK/dV sweep, us, dkv64_kernel / dkv_kernel: 8 x 16 x 2048 x 64 226 / 275, 4 x 32 x 4096 x 64 742 / 950; gated, its further
+    // live values and passes cost more than the rounds give (2 x 8 x 3001 x 64: 75 / 68)
+    if constexpr (HD == 64 && !GATE) {
+        if (which == 0) return launch<dkv64_kernel>(grid, 512, kD64Total + 1024, st, tm, p);
+    } else {
+        if (which == 0) return launch<dkv_kernel<HD, GATE>>(grid, 384, kSmemAlloc, st, tm, p);
+    }
+    return launch<dq_kernel<HD, GATE>>(grid, 512, kSmemAlloc, st, tm, p);
 }
 
 }  // namespace

@@ -170,6 +170,7 @@ def test_forward_pairs_of_query_chunks(binding, oracle, B, H, L, d, gate, scale)
     (5, 61, 300, 64, True),       # items of 2, 0 and 1 steps, three pairs of items per CTA
     (2, 150, 200, 128, False),    # items of one step or none
     (2, 37, 1500, 64, False),     # 0 .. 11 steps, several levels per item, ragged tail
+    (3, 100, 256, 64, False),     # 2 and 1 steps in turn, four items per CTA: diagonal steps next to one another
     (1, 40, 2176, 128, True),     # odd chunk count, block skipping
 ])
 def test_backward_rounds_across_items(binding, B, H, L, d, gate):
