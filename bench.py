@@ -47,13 +47,13 @@ UNIT = "TFLOP/s"
 # DRAM bytes per launch PER (batch, head) SLICE at the C3 shape (L=4096, d=128), from the ncu captures at batch 1
 # (16 slices) summarised under profiles/; slices are independent, so a launch over S slices moves S times this.
 NCU_TRAFFIC_BYTES_PER_SLICE = {
-    "chunk_prep": 12.71e6,         # backward instance (the step's forward runs on the shared workspace)
-    "levels_fwd": 2.13e6 + 6.35e6,   # dyadic_fused (one launch for three levels) + version_fwd
-    "fa_fwd": 11.18e6,
-    "fa_bwd_dkv": 15.24e6,
-    "fa_bwd_dq": 8.62e6,
-    "bwd_levels": 12.64e6,         # level_bwd (4 launches)
-    "bwd_chunk_chain": 18.29e6,
+    "chunk_prep": 9.83e6,            # backward instance (the step's forward runs on the shared workspace)
+    "levels_fwd": 2.10e6 + 6.10e6,   # dyadic_fused (one launch for three levels) + version_fwd
+    "fa_fwd": 10.88e6,
+    "fa_bwd_dkv": 14.97e6,
+    "fa_bwd_dq": 8.31e6,
+    "bwd_levels": 12.45e6,           # level_bwd (4 launches)
+    "bwd_chunk_chain": 15.58e6,
 }
 
 # DRAM bytes per launch of frontend_bwd_kernel PER BATCH ROW at H=32, L=4096, d=64 with the gate, from the ncu capture at
@@ -455,11 +455,11 @@ def run_ours(args, cfg):
     t_d, t_b = CHUNK * d * 2, CHUNK * CHUNK * 2                 # bytes of a [128 x d] / [128 x 128] bf16 tile
     prep_bytes = nch * (3 * t_d + 2 * t_d + 2 * t_b + 2 * d * d * 2)
     lev_f, lev_b = level_bytes(S, N, d)
-    # (the step's forward runs on the backward-sized workspace: its chunk preparation also stores T~ and (I+N)^-1 as
-    # hi + lo, Xk [128 x 128] and U [128 x d]; the chain rule reads w, q, k, U, seven [128 x 128] tiles, (s dSd)^T, bf16
-    # dQl / dKr / dP and writes dq, dk, dw)
-    stage_bytes = {"chunk_prep": prep_bytes + nch * (5 * t_b + t_d), "bwd_chunk_prep": prep_bytes + nch * (5 * t_b + t_d),
-                   "bwd_chunk_chain": nch * (4 * t_d + 7 * t_b + t_b + 2 * t_d + d * d * 2 + 3 * t_d),
+    # (the step's forward runs on the backward-sized workspace: its chunk preparation also stores T~ as hi + lo, Xk
+    # [128 x 128] and U [128 x d]; the chain rule reads w, q, k, U, five [128 x 128] tiles, (s dSd)^T, bf16 dQl / dKr / dP
+    # and writes dq, dk, dw)
+    stage_bytes = {"chunk_prep": prep_bytes + nch * (3 * t_b + t_d), "bwd_chunk_prep": prep_bytes + nch * (3 * t_b + t_d),
+                   "bwd_chunk_chain": nch * (4 * t_d + 5 * t_b + t_b + 2 * t_d + d * d * 2 + 3 * t_d),
                    "levels_fwd": lev_f, "bwd_levels": lev_b, "bwd_levels_fwd": lev_f}
     if cfg["gate"]:   # version chains are built only up to the levels the kept pairs use: no closed-form byte count
         for k_ in ("levels_fwd", "bwd_levels", "bwd_levels_fwd"):
