@@ -15,6 +15,9 @@ cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, u
 cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* diag, float* out, int S, int L, int Lp,
                                cudaStream_t st);
 
+// Zeroes up to three buffers of 32-bit words in one launch (a buffer may be absent: 0 words).
+cudaError_t launch_clear(void* a, size_t na, void* b, size_t nb, void* c, size_t nc, cudaStream_t st);
+
 // Gated problems (PaTH-FoX): which key chunks a query chunk can skip because the accumulated gate has made every logit
 // of the pair negligible.  stats: [S*N][8] floats of scratch; nkeep: [S*N] key chunks each query chunk visits (counted
 // from the diagonal); nvisit: [S*N] query chunks each key chunk meets (the same pairs, key-major); counters: {kept pairs,

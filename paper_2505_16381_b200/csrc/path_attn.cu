@@ -903,7 +903,7 @@ int path_attn_lowrank_fwd(const void* x, const void* w1, const void* w2, void* t
     int rc = check_arch();
     if (rc != PATH_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    CK(cudaMemsetAsync(workspace, 0, 256, st));
+    LAUNCH(launch_clear(workspace, 64, nullptr, 0, nullptr, 0, st));
     rc = run_gemm(x, 0, w1, 0, t, 0, (int)M, r, D, (uint32_t*)workspace, st);         // t = x W1^T
     if (rc != PATH_OK) return rc;
     return run_wide(t, w2, 0, z, (int)M, C, r, (uint32_t*)workspace, st);             // z = t W2^T
@@ -925,9 +925,7 @@ int path_attn_lowrank_bwd(const void* x, const void* w1, const void* w2, const v
     cudaStream_t st = (cudaStream_t)cuda_stream;
     uint32_t* status = (uint32_t*)workspace;
     void* dt = (uint8_t*)workspace + 256;
-    CK(cudaMemsetAsync(workspace, 0, 256, st));
-    CK(cudaMemsetAsync(dw1, 0, (size_t)r * D * sizeof(float), st));
-    CK(cudaMemsetAsync(dw2, 0, (size_t)C * r * sizeof(float), st));
+    LAUNCH(launch_clear(workspace, 64, dw1, (size_t)r * D, dw2, (size_t)C * r, st));
     rc = run_gemm(dz, 0, w2, 1, dt, 0, (int)M, r, C, status, st);                     // dt = dz W2
     if (rc != PATH_OK) return rc;
     rc = run_gemm(dz, 1, t, 1, dw2, 1, C, r, (int)M, status, st);                     // dW2 = dz^T t
