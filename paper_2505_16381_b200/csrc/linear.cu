@@ -20,7 +20,8 @@ __global__ void pad_rows_kernel(const void* __restrict__ src, void* __restrict__
     ((uint4*)dst)[((long)blockIdx.y * Lp + row) * rowbytes16 + col] = v;
 }
 
-// Inclusive scan of `x` over a CTA of 1024 threads; `total` = the sum over all of them.
+// Sum of `x` over the threads before this one in a CTA of 1024; `total` = the sum over all of them.  Nothing is added and taken
+// off again: the sums in front of a huge or infinite value (a gate that resets) must not feel it.
 __device__ __forceinline__ float block_scan(float x, float* part, float& total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -37,9 +38,9 @@ __device__ __forceinline__ float block_scan(float x, float* part, float& total) 
         if (lane >= off) w += y;
     }
     total = __shfl_sync(0xffffffffu, w, 31);
-    const float before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    const float warps = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0), lanes = __shfl_up_sync(0xffffffffu, x, 1);
     __syncthreads();   // (`part` is written again by the next call)
-    return warp > 0 ? x + before : x;
+    return (warp > 0 ? warps : 0.f) + (lane > 0 ? lanes : 0.f);
 }
 
 // One CTA (1024 threads) per slice, 4096 positions at a time, four neighbouring ones per thread.  Latency-bound (32 KB per
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(1024) gate_prefix_kernel(const float* __restri
         for (int x = 0; x < 4; ++x) v[x] = i0 + x < L ? gs[i0 + x] : 0.f;
         v[1] += v[0]; v[2] += v[1]; v[3] += v[2];
         float total;
-        const float before = carry + block_scan(v[3], part, total) - v[3];
+        const float before = carry + block_scan(v[3], part, total);
         if (i0 < Lp) *reinterpret_cast<float4*>(Gs + i0) = make_float4(before + v[0], before + v[1], before + v[2], before + v[3]);
         carry += total;
     }
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(1024) gate_suffix_kernel(const float* __restri
         }
         v[1] += v[0]; v[2] += v[1]; v[3] += v[2];
         float total;
-        const float before = carry + block_scan(v[3], part, total) - v[3];
+        const float before = carry + block_scan(v[3], part, total);
 #pragma unroll
         for (int x = 0; x < 4; ++x)
             if (i0 >= 0 && i0 + 3 - x < L) os[i0 + 3 - x] = before + v[x];

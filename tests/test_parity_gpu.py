@@ -613,3 +613,33 @@ def test_strong_gate_with_a_ragged_tail(binding, oracle, L, d, shift):
     gen = torch.Generator().manual_seed(4801 + L)
     inp["log_f"] = torch.nn.functional.logsigmoid(torch.randn(2, 2, L, generator=gen) + shift).contiguous()
     compare_all(binding, oracle, inp)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("p", [5, 6, 7, 133, 4097, 8190])
+@pytest.mark.parametrize("value", [-1e4, -1e6, -1e30, -float("inf")])
+def test_gate_reset_leaves_earlier_rows_alone(binding, dtype, p, value):
+    """log f of one position far below the others: the gate prefix of the positions before it, and with it their rows, is what
+    it was (equal to the bit), wherever that position lies in the scan's groups of four, 128 and 4096."""
+    L = 300 if p < 300 else 8192 + 40
+    dev = to_dev(synth.make_inputs(1, 1, L, 64, dtype, gate=True, seed=41))
+    run = lambda: binding.path_attn_fwd(*(dev[n] for n in ("q", "k", "v", "w", "beta", "log_f")))
+    (o0, l0), log_f = run(), dev["log_f"].clone()
+    dev["log_f"] = log_f.index_fill(2, torch.tensor([p], device="cuda"), value)
+    o, lse = run()
+    assert torch.equal(o[:, :, :p], o0[:, :, :p]) and torch.equal(lse[:, :, :p], l0[:, :, :p])
+
+
+@pytest.mark.parametrize("p", [4, 5, 6, 7, 300, 4099])
+def test_gate_gradient_of_later_positions_ignores_a_large_row(binding, p):
+    """d log f of the positions after p sums rows after p only: a d_o of 1e6 in row p must not reach them (equal to the bit)."""
+    L = 400 if p < 400 else 4500
+    dev = to_dev(synth.make_inputs(1, 1, L, 64, "bf16", gate=True, seed=42))
+    a = [dev[n] for n in ("q", "k", "v", "w", "beta")]
+    o, lse = binding.path_attn_fwd(*a, dev["log_f"])
+    g0 = binding.path_attn_bwd(*a, o, lse, dev["d_o"], dev["log_f"])["dlog_f"]
+    big = dev["d_o"].clone()
+    big[:, :, p] *= 1e6
+    g = binding.path_attn_bwd(*a, o, lse, big, dev["log_f"])["dlog_f"]
+    assert torch.equal(g[:, :, p + 1:], g0[:, :, p + 1:])
+    assert not torch.equal(g[:, :, :p + 1], g0[:, :, :p + 1])
