@@ -389,10 +389,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
                 const int c0 = half * (HD / 2) + c * 32;
                 tmem_row32(tl + cB + c0, v);
                 add_row(wq, pre_q, c, v);
-                gstore_bf16x32(p.dq + urow * HD + c0, v, row_valid);
+                gstore_bf16x32<true>(p.dq + urow * HD + c0, v, row_valid);
                 tmem_row32(tl + cG + c0, v);
                 add_row(wk, pre_k, c, v);
-                gstore_bf16x32(p.dk + urow * HD + c0, v, row_valid);
+                gstore_bf16x32<true>(p.dk + urow * HD + c0, v, row_valid);
             }
         }
         mma_wait(B_MMA2);                                           // the last of dw
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         for (int c = 0; c < NI; ++c) {
             const int c0 = half * (HD / 2) + c * 32;
             tmem_row32(tl + cDW + c0, v);
-            gstore_bf16x32(p.dw + urow * HD + c0, v, row_valid);
+            gstore_bf16x32<true>(p.dw + urow * HD + c0, v, row_valid);
         }
         publish(B_R1);   // the next chunk's first products overwrite the accumulators read above
     }

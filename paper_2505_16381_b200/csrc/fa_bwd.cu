@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
             mbar_arrive(&bars[K_STEMPTY + (gs & 1)]);
             if constexpr (FIRST) {   // rows = keys (this warp's 32 lanes), 64 query columns = 128 bytes per row
                 if (ok)
-                    warp_store_rows128(p.dsdt + ((size_t)(s * p.N + J) * kTile + q4 * 32) * kTile + h * 64, (size_t)kTile * 2,
+                    warp_store_rows128<false>(p.dsdt + ((size_t)(s * p.N + J) * kTile + q4 * 32) * kTile + h * 64, (size_t)kTile * 2,
                                        dsw);
             }
         };
@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                     w[16 + x] = pack_bf16(__uint_as_float(r1[2 * x]), __uint_as_float(r1[2 * x + 1]));
                 }
                 const int row0 = J * kTile + q4 * 32;
-                warp_store_rows128((__nv_bfloat16*)p.dv + ((size_t)s * p.L + row0) * HD + h * CW, (size_t)HD * 2, w,
+                warp_store_rows128<true>((__nv_bfloat16*)p.dv + ((size_t)s * p.L + row0) * HD + h * CW, (size_t)HD * 2, w,
                                    p.L - row0);
             } else {
                 uint32_t r[32];
@@ -1250,7 +1250,7 @@ __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ B
             tc_fence_after_sync();
             return ok;
         };
-        auto write = [&](uint32_t col, float mul, int free_bar, __nv_bfloat16* dst, bool valid) {
+        auto write = [&](auto caller, uint32_t col, float mul, int free_bar, __nv_bfloat16* dst, bool valid) {
 #pragma unroll 1
             for (int c = 0; c < 2; ++c) {
                 float v[32];
@@ -1262,7 +1262,7 @@ __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ B
                 }
 #pragma unroll
                 for (int x = 0; x < 16; ++x) w[x] = pack_bf16(v[2 * x] * mul, v[2 * x + 1] * mul);
-                tile::gstore_bf16_w16(dst + c * 32, w, valid);
+                tile::gstore_bf16_w16<decltype(caller)::value>(dst + c * 32, w, valid);
             }
         };
 #pragma unroll 1
@@ -1271,7 +1271,7 @@ __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ B
             const bool last = flow.t + 1 == flow.T;
             if (last) {   // dV first: the next item's first product waits for it
                 if (!ready(D_DVFULL, ndv)) break;
-                write(colDV, 1.f, D_DVFREE, (__nv_bfloat16*)p.dv + ((size_t)s * p.L + (kj < p.L ? kj : 0)) * HD, kj < p.L);
+                write(std::true_type{}, colDV, 1.f, D_DVFREE, (__nv_bfloat16*)p.dv + ((size_t)s * p.L + (kj < p.L ? kj : 0)) * HD, kj < p.L);
                 ++ndv;
             }
             if (flow.t == 0) {
@@ -1284,7 +1284,7 @@ __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ B
             const int l = level(J, flow.t);
             if (!(flags_of(J, flow.t, flow.T, l) & FL_LVL1)) continue;
             if (!ready(D_DKFULL, ndk)) break;
-            write(colDK, p.scale, D_DKFREE, p.dkv + ((size_t)kver_row(p.vl, s, l, J) + row) * HD, true);
+            write(std::false_type{}, colDK, p.scale, D_DKFREE, p.dkv + ((size_t)kver_row(p.vl, s, l, J) + row) * HD, true);
             ++ndk;
         }
     } else {
@@ -1385,7 +1385,7 @@ __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ B
                 }
 #pragma unroll
                 for (int x = 0; x < 8; ++x) w[x] = pack_bf16(d[2 * x] * p.scale, d[2 * x + 1] * p.scale);
-                tile::st_global_v8(p.dsdt + ((size_t)base + row) * kTile + h * 64 + c * 16, w);
+                st_global_32<false>(p.dsdt + ((size_t)base + row) * kTile + h * 64 + c * 16, w);
             }
         };
         int fb = 0, base = 0;   // step i - 1: flags, first row of the key chunk

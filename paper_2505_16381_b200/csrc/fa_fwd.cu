@@ -570,7 +570,7 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
             if (CW == 64 && !p.out_fp32) {   // the warp's 32 rows, whole 128-byte pieces per store instruction
                 const int row0 = I * kTile + q4 * 32;
                 if (CW == 64)
-                    warp_store_rows128((__nv_bfloat16*)p.o + ((size_t)s * p.L + row0) * HD + x * CW, (size_t)HD * 2,
+                    warp_store_rows128<true>((__nv_bfloat16*)p.o + ((size_t)s * p.L + row0) * HD + x * CW, (size_t)HD * 2,
                                        reinterpret_cast<uint32_t(&)[32]>(wrow), p.L - row0);
             }
             if (live) {
@@ -1011,7 +1011,7 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
 #pragma unroll
                         for (int e = 0; e < 16; ++e)
                             w[c * 16 + e] = pack_bf16(__uint_as_float(o[c][2 * e]) * inv, __uint_as_float(o[c][2 * e + 1]) * inv);
-                    warp_store_rows128((__nv_bfloat16*)p.o + ((size_t)s * p.L + row0) * HD + h * 64, (size_t)HD * 2, w, p.L - row0);
+                    warp_store_rows128<true>((__nv_bfloat16*)p.o + ((size_t)s * p.L + row0) * HD + h * 64, (size_t)HD * 2, w, p.L - row0);
                 }
             }
             if (live) p.lse[(size_t)s * p.L + qi] = lse2 * 0.6931471805599453f;

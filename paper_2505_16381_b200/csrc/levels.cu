@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
         float v[32];
         uint32_t hi[16], lo[16];
         tmem_row32(c.tl + c0, v);
-        if (p.kc) gstore_f32x32(p.kc + ((size_t)s * p.cap + pos) * HD + col0 + c0, v, pos < p.L);
+        if (p.kc) gstore_f32x32<true>(p.kc + ((size_t)s * p.cap + pos) * HD + col0 + c0, v, pos < p.L);
         if (p.edge16) gstore_bf16x32(p.edge16 + ((size_t)s * p.L + pos) * HD + col0 + c0, v, pos < p.L);
         if (update) {
             tmem_row32(c.tl + 128 + c0, v);
@@ -816,7 +816,7 @@ __global__ void __launch_bounds__(256, 2) apply_product_kernel(const __grid_cons
         for (int i = 0; i < HD / 64; ++i) {
             const int c0 = c.half * (HD / 2) + i * 32;
             tmem_row32(c.tl + c0, v);
-            if (p.kc) gstore_f32x32(p.kc + ((size_t)s * p.cap + pos) * HD + c0, v, pos < p.L);
+            if (p.kc) gstore_f32x32<true>(p.kc + ((size_t)s * p.cap + pos) * HD + c0, v, pos < p.L);
             else gstore_bf16x32(p.qv + ((size_t)row0 + c.row) * HD + c0, v);
         }
     }

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(192, 2) gemm_kernel(const __grid_constant__ CU
                                          "f"(v[x + 2]), "f"(v[x + 3]) : "memory");
                     }
                 } else {   // bf16, N a multiple of 32 (checked on the host)
-                    tile::gstore_bf16x32((__nv_bfloat16*)p.c + (size_t)(m < p.M ? m : 0) * p.ldc + n, v, m < p.M);
+                    tile::gstore_bf16x32<true>((__nv_bfloat16*)p.c + (size_t)(m < p.M ? m : 0) * p.ldc + n, v, m < p.M);
                 }
             }
         }

@@ -273,8 +273,22 @@ __device__ __forceinline__ void rot4_pieces(uint32_t (&w)[32], int j) {   // pie
         w[24 + x] = b1 ? a1 : a3;
     }
 }
-// `base`: address of row 0's 128-byte segment (warp-uniform, 32-byte aligned), `stride`: bytes between rows
+// Stores 32 bytes.  A workspace address is 32-byte aligned; a caller's tensor (CALLER) is promised to start at a multiple of 16
+// only, and where it does the row goes out as two halves.
+template <bool CALLER>
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&v)[8]) {
+    if (CALLER && ((uintptr_t)p & 16)) {
+        reinterpret_cast<uint4*>(p)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<uint4*>(p)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    } else {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                     "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                     : "memory");
+    }
+}
+// `base`: address of row 0's 128-byte segment (warp-uniform; aligned as st_global_32 wants it), `stride`: bytes between rows
 // (multiple of 32).  Rows >= nrows are not written.  Destroys w.
+template <bool CALLER>
 __device__ __forceinline__ void warp_store_rows128(void* base, size_t stride, uint32_t (&w)[32], int nrows = 32) {
     const int lane = threadIdx.x & 31, j = lane & 3, g4 = lane & ~3;
     rot4_pieces(w, j);
@@ -284,12 +298,7 @@ __device__ __forceinline__ void warp_store_rows128(void* base, size_t stride, ui
 #pragma unroll
         for (int x = 0; x < 8; ++x) v[x] = r == 0 ? w[x] : __shfl_xor_sync(0xffffffffu, w[8 * r + x], r);
         const int row = g4 + (j ^ r);
-        if (row < nrows) {
-            uint8_t* dst = (uint8_t*)base + (size_t)row * stride + 32 * j;
-            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]),
-                         "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                         : "memory");
-        }
+        if (row < nrows) st_global_32<CALLER>((uint8_t*)base + (size_t)row * stride + 32 * j, v);
     }
 }
 }  // namespace tc5

@@ -52,18 +52,15 @@ __device__ __forceinline__ void tile_store32(uint8_t* t, int row, int c0, const 
 // Row transfers between registers and global memory.  Lane L of a warp owns one row segment (32 consecutive values
 // starting at its own pointer).  All 32 lanes must call together: the lanes of a group first swap 32-byte pieces so
 // that one instruction covers whole rows (full 128- or 64-byte runs) instead of 32 scattered 16-byte pieces.
-// `valid` = false: the lane's row is not written / reads as zero.
-__device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&v)[8]) {
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                 : "memory");
-}
+// `valid` = false: the lane's row is not written / reads as zero.  CALLER: the row lies in a caller's tensor (16-byte aligned),
+// not in a workspace (see st_global_32).
 __device__ __forceinline__ void ld_global_v8(const void* p, uint32_t (&v)[8]) {
     asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                  : "l"(p)
                  : "memory");
 }
+template <bool CALLER = false>
 __device__ __forceinline__ void gstore_f32x32(float* dst, const float (&v)[32], bool valid = true) {
     const int j = threadIdx.x & 3;
     uint32_t w[32];
@@ -78,7 +75,7 @@ __device__ __forceinline__ void gstore_f32x32(float* dst, const float (&v)[32], 
         for (int x = 0; x < 8; ++x) d[x] = r == 0 ? w[x] : __shfl_xor_sync(0xffffffffu, w[8 * r + x], r);
         const unsigned long long ptr = r == 0 ? mine : __shfl_xor_sync(0xffffffffu, mine, r);
         const bool ok = r == 0 ? valid : (bool)__shfl_xor_sync(0xffffffffu, (int)valid, r);
-        if (ok) st_global_v8((uint8_t*)ptr + 32 * j, d);
+        if (ok) st_global_32<CALLER>((uint8_t*)ptr + 32 * j, d);
     }
 }
 // The load in two halves, so that a caller can put other work between the request and the first use of the data.
@@ -116,6 +113,7 @@ __device__ __forceinline__ void gload_f32x32(const float* src, float (&v)[32], b
     gload_f32x32_finish(d, v);
 }
 // 32 bf16 = 64 bytes per row: pairs of lanes.  `w`: the row segment as 16 packed words.
+template <bool CALLER = false>
 __device__ __forceinline__ void gstore_bf16_w16(__nv_bfloat16* dst, const uint32_t (&w)[16], bool valid = true) {
     const bool odd = threadIdx.x & 1;
     uint32_t first[8], second[8];   // halves [32 * odd, +32) of the even lane's row and of the odd lane's row
@@ -127,17 +125,18 @@ __device__ __forceinline__ void gstore_bf16_w16(__nv_bfloat16* dst, const uint32
     }
     const unsigned long long mine = (unsigned long long)dst, other = __shfl_xor_sync(0xffffffffu, mine, 1);
     const bool ovalid = (bool)__shfl_xor_sync(0xffffffffu, (int)valid, 1);
-    if (odd ? ovalid : valid) st_global_v8((uint8_t*)(odd ? other : mine) + 32 * (int)odd, first);
-    if (odd ? valid : ovalid) st_global_v8((uint8_t*)(odd ? mine : other) + 32 * (int)odd, second);
+    if (odd ? ovalid : valid) st_global_32<CALLER>((uint8_t*)(odd ? other : mine) + 32 * (int)odd, first);
+    if (odd ? valid : ovalid) st_global_32<CALLER>((uint8_t*)(odd ? mine : other) + 32 * (int)odd, second);
 }
 __device__ __forceinline__ void pack32(const float (&v)[32], uint32_t (&w)[16]) {
 #pragma unroll
     for (int x = 0; x < 16; ++x) w[x] = pack_bf16(v[2 * x], v[2 * x + 1]);
 }
+template <bool CALLER = false>
 __device__ __forceinline__ void gstore_bf16x32(__nv_bfloat16* dst, const float (&v)[32], bool valid = true) {
     uint32_t w[16];
     pack32(v, w);
-    gstore_bf16_w16(dst, w, valid);
+    gstore_bf16_w16<CALLER>(dst, w, valid);
 }
 // t = hi + lo with hi = bf16(t) and lo = bf16(t - hi), both packed two per word.
 __device__ __forceinline__ void split32(const float (&t)[32], uint32_t (&hi)[16], uint32_t (&lo)[16]) {

@@ -643,3 +643,56 @@ def test_gate_gradient_of_later_positions_ignores_a_large_row(binding, p):
     g = binding.path_attn_bwd(*a, o, lse, big, dev["log_f"])["dlog_f"]
     assert torch.equal(g[:, :, p + 1:], g0[:, :, p + 1:])
     assert not torch.equal(g[:, :, :p + 1], g0[:, :, :p + 1])
+
+
+def off16(shape, dtype):
+    """An output at an address that is a multiple of 16 and not of 32, which is all the interface asks for; with guard bands."""
+    n = int(np.prod(shape)) * torch.empty(0, dtype=dtype).element_size()
+    raw = torch.full((GUARD + 16 + n + GUARD,), 0x5A, dtype=torch.uint8, device="cuda")
+    t = raw[GUARD + 16:GUARD + 16 + n].view(dtype).view(*shape)
+    assert t.data_ptr() % 32 == 16
+    return t, lambda: bool((raw[:GUARD + 16] == 0x5A).all()) and bool((raw[GUARD + 16 + n:] == 0x5A).all())
+
+
+@pytest.mark.parametrize("S,L,d,gate", [(4, 300, 64, False), (4, 300, 128, True), (150, 200, 64, True), (150, 200, 128, False),
+                                        (150, 256, 64, False)])
+def test_outputs_on_odd_multiples_of_16_bytes(binding, S, L, d, gate):
+    """Both forward sweeps (few and many slices), the backward and the prompt's key cache: the bits of the aligned call."""
+    dev = to_dev(synth.make_inputs(1, S, L, d, "bf16", gate=gate, seed=51))
+    a = [dev[n] for n in ("q", "k", "v", "w", "beta")]
+    o0, lse0 = binding.path_attn_fwd(*a, dev["log_f"])
+    (o, ok), (lse, ok2) = off16(o0.shape, o0.dtype), off16(lse0.shape, lse0.dtype)
+    binding.path_attn_fwd(*a, dev["log_f"], out=(o, lse))
+    assert torch.equal(o, o0) and torch.equal(lse, lse0) and ok() and ok2()
+    g0 = binding.path_attn_bwd(*a, o0, lse0, dev["d_o"], dev["log_f"])
+    outs = {n: off16(t.shape, t.dtype) for n, t in g0.items()}
+    binding.path_attn_bwd(*a, o0, lse0, dev["d_o"], dev["log_f"], out={n: t for n, (t, _) in outs.items()})
+    for n, (t, ok) in outs.items():
+        assert torch.equal(t, g0[n]) and ok(), n
+    c0 = binding.alloc_cache(1, S, L, d, gate)
+    binding.path_attn_prefill_cache(a[1], a[2], a[3], a[4], c0, dev["log_f"])
+    kc, ok = off16(c0["kc"].shape, torch.float32)
+    binding.path_attn_prefill_cache(a[1], a[2], a[3], a[4], dict(c0, kc=kc), dev["log_f"])
+    assert torch.equal(kc, c0["kc"]) and ok()
+
+
+def test_long_prompt_cache_on_an_odd_multiple_of_16_bytes(binding):
+    """One slice of 40 chunks: the chunk walk in ranges, whose last kernel writes the keys."""
+    dev = to_dev(synth.make_inputs(1, 1, 5100, 128, "bf16", seed=52))
+    a = [dev[n] for n in ("k", "v", "w", "beta")]
+    c0 = binding.alloc_cache(1, 1, 5100, 128, False)
+    binding.path_attn_prefill_cache(*a, c0)
+    kc, ok = off16(c0["kc"].shape, torch.float32)
+    binding.path_attn_prefill_cache(*a, dict(c0, kc=kc))
+    assert torch.equal(kc, c0["kc"]) and ok()
+
+
+def test_lowrank_output_on_an_odd_multiple_of_16_bytes(binding):
+    g = torch.Generator(device="cuda").manual_seed(53)
+    x, w1, w2 = (torch.randn(*s, generator=g, device="cuda").bfloat16() for s in ((300, 128), (64, 128), (192, 64)))
+    z0, t0 = binding.path_attn_lowrank_fwd(x, w1, w2)
+    (z, ok), (t, ok2) = off16(z0.shape, z0.dtype), off16(t0.shape, t0.dtype)
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    rc = binding.load().path_attn_lowrank_fwd(x.data_ptr(), w1.data_ptr(), w2.data_ptr(), t.data_ptr(), z.data_ptr(), 300, 128, 64, 192,
+                                              ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
+    assert rc == 0 and torch.equal(z, z0) and torch.equal(t, t0) and ok() and ok2()
