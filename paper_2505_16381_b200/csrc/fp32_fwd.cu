@@ -6,13 +6,15 @@
 // t = W u0 (32 dot products at once),
 //     T = (I + C)^-1,  C_jm = beta_m w_j . w_m  (m > j),      Y = strictUpper(K W^T) D T
 //     logits of the block:  K u0 - Y t = (K - Y W) u0 = Kr u0,      u after the block:  u0 - ((D T)^T W)^T t = u0 - Wt^T t
-// Kr, Wt and Y belong to the keys alone: fp32_block_kernel makes them once per block.  A query's own block uses K, Y and t with
-// the entries after the query set to zero.
+// Kr, Wt and Y belong to the keys alone: fp32_block_kernel makes them once per block.  A query's own block uses K, Y and t up to
+// the query.  Entries that the definition does not use are left out, not multiplied by zero: an infinity or NaN at one position
+// stays out of every row before it, as in the walk.
 //
 // fp32_fwd_kernel: a warp owns RW queries of one block, lane j the block's key j: two dot products per lane with rows from
 // shared memory (u0 broadcast), then the lanes turn to the head dimension for the update of u and for P V.  What bounds it
 // at the sizes it is for (a few slices, a few hundred tokens) is the chain of dependent phases of one block, L / 32 times.
-// B=1, H=2, L=256, d=64: 69.7 -> 20.5 us per call (one key per step: 520 cycles each).
+// B=1, H=2, L=256, d=64: 69.7 -> 21.0 us per call (one key per step: 520 cycles each).
+#include <type_traits>
 #include "common.cuh"
 
 namespace path {
@@ -69,31 +71,35 @@ __global__ void __launch_bounds__(256) fp32_block_kernel(const float* __restrict
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const int m = part + 8 * x;
-            sc[row][m] = m > row ? sb[m] * a[x] : 0.f;
-            skw[row][m] = m > row ? b[x] : 0.f;
+            sc[m][row] = m > row ? sb[m] * a[x] : 0.f;   // (C transposed: the substitution goes column by column)
+            skw[row][m] = b[x];
         }
     }
     __syncthreads();
     if (tid < kBlk) {   // column tid of T by back substitution, in registers; D T replaces C
         float x[kBlk];
 #pragma unroll
-        for (int j = kBlk - 1; j >= 0; --j) {
-            float acc[4] = {j == tid ? 1.f : 0.f, 0.f, 0.f, 0.f};
+        for (int j = 0; j < kBlk; ++j) x[j] = j == tid ? 1.f : 0.f;
 #pragma unroll
-            for (int m = j + 1; m < kBlk; ++m) acc[m & 3] = fmaf(-sc[j][m], x[m], acc[m & 3]);
-            x[j] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-        }
+        for (int j = kBlk - 1; j > 0; --j)
+#pragma unroll
+            for (int i = 0; i < j; ++i) x[i] = j <= tid ? fmaf(-sc[j][i], x[j], x[i]) : x[i];
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < kBlk; ++j) sc[j][tid] = sb[j] * x[j];
+        for (int j = 0; j < kBlk; ++j) sc[j][tid] = j <= tid ? sb[j] * x[j] : 0.f;
     }
     __syncthreads();
-    float y[4] = {0.f, 0.f, 0.f, 0.f};   // Y[row][4 part ..]
-#pragma unroll 8
-    for (int p = 0; p < kBlk; ++p) {
+    const int r4 = row & ~3;             // the warp's rows are r4 .. r4 + 3
+    float y[4] = {0.f, 0.f, 0.f, 0.f};   // Y[row][4 part ..]: over row < p <= column
+#pragma unroll 4
+    for (int p = r4; p < kBlk; ++p) {
         const float c = skw[row][p];
         const float4 d4 = *reinterpret_cast<const float4*>(&sc[p][4 * part]);
-        y[0] = fmaf(c, d4.x, y[0]); y[1] = fmaf(c, d4.y, y[1]); y[2] = fmaf(c, d4.z, y[2]); y[3] = fmaf(c, d4.w, y[3]);
+        const int last = p > row ? 4 * part : -8;
+        y[0] = p <= last ? fmaf(c, d4.x, y[0]) : y[0];
+        y[1] = p <= last + 1 ? fmaf(c, d4.y, y[1]) : y[1];
+        y[2] = p <= last + 2 ? fmaf(c, d4.z, y[2]) : y[2];
+        y[3] = p <= last + 3 ? fmaf(c, d4.w, y[3]) : y[3];
     }
     *reinterpret_cast<float4*>(ym + dst * kBlk + 4 * part) = make_float4(y[0], y[1], y[2], y[3]);
     __syncthreads();
@@ -102,20 +108,24 @@ __global__ void __launch_bounds__(256) fp32_block_kernel(const float* __restrict
     float ok[HD / 8], ow[HD / 8];
 #pragma unroll
     for (int c = 0; c < HD / 8; ++c) { ok[c] = sk[row][(c >> 2) * 32 + part * 4 + (c & 3)]; ow[c] = 0.f; }
-#pragma unroll 4
-    for (int m = 0; m < kBlk; ++m) {
-        const float cy = skw[row][m], ct = sc[m][row];
+    // Kr takes the keys after the row, Wt those up to it
+    auto add = [&](float (&out)[HD / 8], const float x, const int m) {
 #pragma unroll
         for (int c = 0; c < HD / 32; ++c) {
             const float4 wm = *reinterpret_cast<const float4*>(&sw[m][c * 32 + part * 4]);
-            const float t[4] = {wm.x, wm.y, wm.z, wm.w};
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                ok[4 * c + x] = fmaf(-cy, t[x], ok[4 * c + x]);
-                ow[4 * c + x] = fmaf(ct, t[x], ow[4 * c + x]);
-            }
+            out[4 * c] = fmaf(x, wm.x, out[4 * c]); out[4 * c + 1] = fmaf(x, wm.y, out[4 * c + 1]);
+            out[4 * c + 2] = fmaf(x, wm.z, out[4 * c + 2]); out[4 * c + 3] = fmaf(x, wm.w, out[4 * c + 3]);
         }
+    };
+#pragma unroll 4
+    for (int m = 0; m < r4; ++m) add(ow, sc[m][row], m);
+#pragma unroll
+    for (int m = r4; m < r4 + 4; ++m) {
+        if (m > row) add(ok, -skw[row][m], m);
+        else add(ow, sc[m][row], m);
     }
+#pragma unroll 4
+    for (int m = r4 + 4; m < kBlk; ++m) add(ok, -skw[row][m], m);
 #pragma unroll
     for (int c = 0; c < HD / 32; ++c) {
         *reinterpret_cast<float4*>(kr + dst * HD + c * 32 + part * 4) = make_float4(ok[4 * c], ok[4 * c + 1], ok[4 * c + 2], ok[4 * c + 3]);
@@ -179,10 +189,11 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
         Gi[r] = G && i[r] < L ? G[(size_t)s * ldG + i[r]] : 0.f;
     }
     __syncwarp();
-#pragma unroll 1
-    for (int n = nb; n >= 0; --n) {
+    auto step = [&](auto own_tag, const int n) {
+        // The block of the warp's own queries runs once and is kept short: as long as the others it costs 5 % at d = 128 (97 us for
+        // 4 x 512 positions, 93 like this) in instruction fetch.
+        constexpr bool own = decltype(own_tag)::value;
         const int stage = (nb - n) & 1;
-        const bool own = n == nb;
         if (n > 0) {
             request(n - 1, stage ^ 1);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -198,7 +209,7 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
         for (int r = 0; r < RW; ++r)
 #pragma unroll
             for (int x = 0; x < 4; ++x) t[r][x] = a[r][x] = 0.f;
-#pragma unroll 8
+#pragma unroll (own ? 2 : 8)
         for (int e = 0; e < HD; e += 4) {
             const float4 w4 = *reinterpret_cast<const float4*>(tw + e), k4 = *reinterpret_cast<const float4*>(tw + TILE + e);
 #pragma unroll
@@ -218,13 +229,22 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
             lg[r] = (a[r][0] + a[r][1]) + (a[r][2] + a[r][3]);
         }
         __syncwarp();
-        if (own) {   // logits of the own block: K q - Y t
+        if constexpr (own) {   // logits of the own block: K q - Y t
             const float4* yr = reinterpret_cast<const float4*>(ym + (((size_t)s * nblk + n) * kBlk + lane) * kBlk);
 #pragma unroll
             for (int c = 0; c < kBlk / 4; ++c) {
                 const float4 y4 = yr[c];
+                const float y[4] = {y4.x, y4.y, y4.z, y4.w};
 #pragma unroll
-                for (int r = 0; r < RW; ++r) lg[r] -= dot4(y4, *reinterpret_cast<const float4*>(st + r * kBlk + 4 * c));
+                for (int r = 0; r < RW; ++r) {
+                    const float4 t4 = *reinterpret_cast<const float4*>(st + r * kBlk + 4 * c);
+                    const float tt[4] = {t4.x, t4.y, t4.z, t4.w};
+                    float d = 0.f;
+#pragma unroll
+                    for (int x = 0; x < 4; ++x)
+                        if (4 * c + x > lane && 4 * c + x <= r0 + r) d = fmaf(y[x], tt[x], d);
+                    lg[r] -= d;
+                }
             }
         }
 #pragma unroll
@@ -249,8 +269,8 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
 #pragma unroll
             for (int e = 0; e < E; ++e) du[r][e] = 0.f;
         const float* cw = sm + stage * 4 * TILE + 2 * TILE + lane;
-#pragma unroll 4
-        for (int j = 0; j < kBlk; j += 4) {
+#pragma unroll (own ? 1 : 4)
+        for (int j = 0; j < (own ? (r0 + RW + 3) & ~3 : kBlk); j += 4) {
             float4 t4[RW], p4[RW];
 #pragma unroll
             for (int r = 0; r < RW; ++r) {
@@ -266,6 +286,7 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
                     for (int r = 0; r < RW; ++r) {
                         const float tj = y == 0 ? t4[r].x : y == 1 ? t4[r].y : y == 2 ? t4[r].z : t4[r].w;
                         const float pj = y == 0 ? p4[r].x : y == 1 ? p4[r].y : y == 2 ? p4[r].z : p4[r].w;
+                        if (own && j + y > r0 + r) continue;
                         du[r][e] = fmaf(tj, ww, du[r][e]);
                         acc[r][e] = fmaf(pj, vv, acc[r][e]);
                     }
@@ -276,7 +297,10 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
 #pragma unroll
             for (int e = 0; e < E; ++e) su[r * HD + e * 32 + lane] -= du[r][e];
         __syncthreads();   // everyone is done with this stage's tiles
-    }
+    };
+    step(std::true_type{}, nb);
+#pragma unroll 1
+    for (int n = nb - 1; n >= 0; --n) step(std::false_type{}, n);
 #pragma unroll
     for (int r = 0; r < RW; ++r) {
 #pragma unroll

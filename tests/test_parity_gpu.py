@@ -696,3 +696,19 @@ def test_lowrank_output_on_an_odd_multiple_of_16_bytes(binding):
     rc = binding.load().path_attn_lowrank_fwd(x.data_ptr(), w1.data_ptr(), w2.data_ptr(), t.data_ptr(), z.data_ptr(), 300, 128, 64, 192,
                                               ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
     assert rc == 0 and torch.equal(z, z0) and torch.equal(t, t0) and ok() and ok2()
+
+
+@pytest.mark.parametrize("name", ["q", "k", "v", "w", "beta", "log_f"])
+@pytest.mark.parametrize("S,d,p,value", [(2, 64, 0, "nan"), (2, 64, 45, "nan"), (2, 128, 63, "inf"), (40, 128, 33, "nan"), (40, 64, 97, "inf")])
+def test_float32_rows_before_a_nan_or_infinity(binding, name, S, d, p, value):
+    """The float32 forward is causal to the bit: a NaN or infinity at position p changes no row before p (one and four queries
+    per warp), and none at all where it is in w or beta of position 0, which no logit uses."""
+    dev = to_dev(synth.make_inputs(1, S, 150, d, "fp32", gate=True, seed=61))
+    run = lambda: binding.path_attn_fwd(*(dev[n] for n in ("q", "k", "v", "w", "beta", "log_f")))
+    o0, l0 = run()
+    dev[name][:, :, p] = float(value) if name != "log_f" or value == "nan" else -float(value)
+    o, lse = run()
+    c = 150 if p == 0 and name in ("w", "beta") else p
+    assert torch.equal(o[:, :, :c], o0[:, :, :c]) and torch.equal(lse[:, :, :c], l0[:, :, :c])
+    if c < 150:
+        assert not torch.isfinite(o[:, :, p:]).all(), "the value must reach its own row or a later one"
