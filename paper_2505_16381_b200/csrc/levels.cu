@@ -10,6 +10,7 @@
 //     Kv[l2][J]  = Kv[l1][J] Dy[l1][(J >> l1) + 1]^T            l1 < l2 consecutive clear bits of J
 // and the backward kernel (level_bwd) applies the chain rule to exactly these products, level by level.  Run products are stored as bf16
 // hi + lo pairs (they are multiplied up to log2(N) times); versions are bf16, the values the sweep consumes.
+#include <type_traits>
 #include "tileops.cuh"
 
 namespace path {
@@ -321,27 +322,29 @@ __device__ __forceinline__ int version_at(int is_key, int ch, int e, int N, int 
 
 // With p.edge_q / p.edge_k the chains go on to the sequence's start / end (context-parallel path, paper Sec. 3.5: queries
 // pulled back to the start of the segment, keys advanced to its end, bf16 [S][Lp][d]): at most about 2 log2(N) products per
-// chunk, all chunks at once.  (Walking the chunks one after the other per slice took 105 us for the two sides of 64 slices of
-// 8 chunks at d = 128, on top of this kernel's 23; the extended chains take 45 in all, and the product of the segment comes from the run products.)
-template <int HD>
+// chunk, all chunks at once.  What goes on from step to step is then a bf16 pair in tensor memory, a version and what it
+// lacks: rounded to bf16 at every step, as the versions are, the keys at the end of a segment of 8 chunks with unit w of four directions and beta = 2 were 2.9e-3
+// off (2.3e-3 with the pair, which leaves the first tile's and the last rounding; outputs of sharp attention 8.3e-3 against 7.5e-3).  (Walking the chunks one after the other per slice took 105 us for the two sides of 64 slices of
+// 8 chunks at d = 128, on top of this kernel's 23; the extended chains take 49 in all, and the product of the segment comes from the run products.)
+template <int HD, bool EDGE>
 __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int is_key = blockIdx.y, s = blockIdx.x / p.N, ch = blockIdx.x % p.N;
     grid_wait();   // (the block-skipping counts)
     // levels to store: all of them, or for a gated problem up to the highest one a kept chunk pair uses (see level_bwd)
     const int lim = min(p.l, highest_level_reached(p, is_key, s, ch) + 1);
     const int top = max(p.nlev - 2, 0);
-    __nv_bfloat16* edge = is_key ? p.edge_k : p.edge_q;
+    __nv_bfloat16* edge = !EDGE ? nullptr : is_key ? p.edge_k : p.edge_q;
     int e = ch + is_key, a, idx, e2, lv;
     // the next step, if there is one to take: a version to store, or an edge to reach
     auto next = [&]() {
         if (!chain_step(is_key, e, p.N, top, a, idx, e2)) return false;
         lv = version_at(is_key, ch, e2, p.N, p.nlev);
         if (lv >= lim) lv = -1;
-        return edge != nullptr || lv >= 0;
+        return EDGE || lv >= 0;
     };
     const long row_first = (long)s * p.Lp + (long)ch * kT;   // plane 0: the boundary-adjusted tile
     if (!next()) {
-        if (edge) {   // already at the edge
+        if (EDGE) {   // already at the edge
             const uint4* src = reinterpret_cast<const uint4*>((is_key ? p.kv : p.qv) + row_first * HD);
             uint4* dst = reinterpret_cast<uint4*>(edge + row_first * HD);
             for (int i = threadIdx.x; i < kT * HD / 8; i += 256) dst[i] = src[i];
@@ -350,8 +353,10 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
     }
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<128>(c, smem_raw, kBar3);
-    uint8_t* sm = c.smem;   // slots: 0 current version, 1 Dy hi, 2 Dy lo
+    constexpr int kCols = EDGE ? 256 : 128;
+    constexpr uint32_t colHi = 128, colLo = 128 + HD / 2;   // EDGE: the running pair
+    setup<kCols>(c, smem_raw, kBar3);
+    uint8_t* sm = c.smem;   // slots: 0 current version (EDGE: the first one only), 1 Dy hi, 2 Dy lo
     bool first = true, more = true;
 #pragma unroll 1
     while (more && c.ok) {
@@ -362,38 +367,78 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
             tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
             tma_tile(sm + 2 * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat * HD));
         }
+        // A stored version is the product of the one before it alone, here as in the plain instance; what the rest of the pair adds
+        // comes in a product of its own.
+        const bool apart = EDGE && !first && lv >= 0;
         loads_wait(c);
         if (!first) publish();   // the left operand was written by this CTA's threads
         if (leader(c)) {
             tc_fence_after_sync();
             const uint32_t t = smem_u32(sm);
-            if (is_key) {
-                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, t, t + kTileB, false);
-                mma<OP_K, OP_K, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, true);
-            } else {
-                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + kTileB, false);
-                mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, true);
-            }
+            auto products = [&](auto bop) {
+                constexpr int BOP = decltype(bop)::value;
+                if (!EDGE || first) {
+                    mma<OP_K, BOP, HD / 16, HD>(c.tmem, t, t + kTileB, false);
+                    mma<OP_K, BOP, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, true);
+                } else {
+                    mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colHi, t + kTileB, false);
+                    mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colHi, t + 2 * kTileB, true);
+                    if (!apart) mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colLo, t + kTileB, true);
+                }
+            };
+            if (is_key) products(std::integral_constant<int, OP_K>{});
+            else products(std::integral_constant<int, OP_MN>{});
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
         __nv_bfloat16* out = nullptr;
         if (lv >= 0) out = (is_key ? p.kv + kver_row(p.vl, s, lv, ch) * HD : p.qv + qver_row(p.vl, s, lv, ch) * HD);
         else if (e2 == (is_key ? p.N : 0)) out = edge + row_first * HD;
+        uint32_t hi[EDGE ? HD / 64 : 1][16];
         if (c.ok) {
             float v[32];
+#pragma unroll
             for (int i = 0; i < HD / 64; ++i) {
                 const int c0 = c.half * (HD / 2) + i * 32;
                 tmem_row32(c.tl + c0, v);
                 if (out) gstore_bf16x32(out + (size_t)c.row * HD + c0, v);
-                tile_store32(sm, c.row, c0, v);
+                if (!EDGE) tile_store32(sm, c.row, c0, v);
+                else pack32(v, hi[EDGE ? i : 0]);
             }
+        }
+        if (apart) {
+            tc_fence_before_sync();
+            __syncthreads();
+            if (leader(c)) {
+                tc_fence_after_sync();
+                const uint32_t t = smem_u32(sm) + kTileB;
+                if (is_key) mma_ta<OP_K, HD / 16, HD>(c.tmem, c.tmem + colLo, t, true);
+                else mma_ta<OP_MN, HD / 16, HD>(c.tmem, c.tmem + colLo, t, true);
+                umma_commit(&c.bars[1]);
+            }
+            mma_wait(c);
+        }
+        if (EDGE && c.ok) {
+            float v[32];
+            uint32_t lo[16];
+#pragma unroll
+            for (int i = 0; i < HD / 64; ++i) {
+                const int c0 = c.half * (HD / 2) + i * 32;
+                const uint32_t (&h)[16] = hi[EDGE ? i : 0];
+                tmem_row32(c.tl + c0, v);
+#pragma unroll
+                for (int x = 0; x < 16; ++x)
+                    lo[x] = pack_bf16(v[2 * x] - __uint_as_float(h[x] << 16), v[2 * x + 1] - __uint_as_float(h[x] & 0xffff0000u));
+                tmem_st16(c.tl + colHi + c0 / 2, h);
+                tmem_st16(c.tl + colLo + c0 / 2, lo);
+            }
+            tmem_st_wait();
         }
         first = false;
         e = e2;
         more = next();
     }
-    teardown<128>(c, p.status);
+    teardown<kCols>(c, p.status);
 }
 
 // ---------------------------------------------------------------------------------------------- product of a whole segment
@@ -838,7 +883,11 @@ cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const Leve
         }
         case LEVEL_VERSION_FWD: {
             dim3 g(p.S * p.N, 2);
-            return hd == 64 ? launch<version_fwd_kernel<64>>(g, 256, smem_bytes(3), st, tm, p) : launch<version_fwd_kernel<128>>(g, 256, smem_bytes(3), st, tm, p);
+            if (p.edge_q)
+                return hd == 64 ? launch<version_fwd_kernel<64, true>>(g, 256, smem_bytes(3), st, tm, p)
+                                : launch<version_fwd_kernel<128, true>>(g, 256, smem_bytes(3), st, tm, p);
+            return hd == 64 ? launch<version_fwd_kernel<64, false>>(g, 256, smem_bytes(3), st, tm, p)
+                            : launch<version_fwd_kernel<128, false>>(g, 256, smem_bytes(3), st, tm, p);
         }
         case LEVEL_BWD: {
             dim3 g(p.S * p.lv.dy_cnt[p.l]);

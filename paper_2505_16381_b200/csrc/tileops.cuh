@@ -39,6 +39,18 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a_tile, uint32_t b
     }
 }
 
+// The same with A in tensor memory: packed bf16, 8 columns per step, from column `a_tmem` on.
+template <int BOP, int KSTEPS, int N>
+__device__ __forceinline__ void mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_tile, bool acc) {
+    constexpr uint32_t idesc = umma_idesc(128, N, OP_K, BOP);
+    const uint32_t b_lo = umma_desc_lo(b_tile, BOP == OP_K ? 16u : kPanelB);
+#pragma unroll
+    for (int kk = 0; kk < KSTEPS; ++kk) {
+        const uint32_t ko = (uint32_t)(kk >> 2) * (kPanelB >> 4) + (uint32_t)(kk & 3) * 2u, mo = (uint32_t)kk * 128u;
+        umma_ts(d_tmem, a_tmem + kk * 8, umma_desc_join(b_lo + (BOP == OP_K ? ko : mo)), idesc, (acc || kk > 0) ? 1u : 0u);
+    }
+}
+
 // Stores columns c0 .. c0+31 of `row` of a swizzled bf16 tile.
 __device__ __forceinline__ void tile_store32(uint8_t* t, int row, int c0, const float (&v)[32]) {
     uint8_t* panel = t + (c0 >> 6) * kPanelB;

@@ -44,6 +44,32 @@ def test_virtual_ring_matches_the_oracle(oracle, B, H, L, d, gate, cuts, scale):
     assert np.abs(f(lse) - lse_ref).max() <= 2e-3 * max(1.0, np.abs(lse_ref).max())
 
 
+@pytest.mark.parametrize("L,d", [(256, 64), (1024, 64), (1024, 128), (1500, 128)])
+def test_edge_tiles_are_rounded_twice_at_most(L, d):
+    """Keys at the segment's end and queries at its start: a prepared tile (rounded to bf16 once) moved through the run products of
+    up to 12 chunks and rounded once more.  Two roundings of half an ulp, uniform over it, are at most
+    sqrt(2) 2^-8 / sqrt(3) = 3.2e-3 of a value (its mantissa at the low end) and 2.3e-3 on average over mantissas; a third would
+    make that 2.8e-3.  Directions that repeat, at beta = 2, leave the norm alone, so nothing else sets the scale."""
+    from paper_2505_16381_b200 import binding
+    g = torch.Generator(device="cuda").manual_seed(L + d)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    q, k, v = (n(1, 2, L, d).bfloat16() for _ in range(3))
+    w = torch.nn.functional.normalize(n(1, 2, 4, d), dim=-1)[:, :, torch.randint(4, (L,), generator=g, device="cuda")].bfloat16()
+    beta = torch.full((1, 2, L), 2.0, device="cuda")
+    state, message, _ = binding.path_attn_cp_prepare(q, k, v, w, beta)
+    Lp = (L + 127) // 128 * 128
+    tiles = lambda b: b[:2 * Lp * d * 2].view(torch.bfloat16).view(1, 2, Lp, d)[:, :, :L].double()
+    kr, x, W = k.double().clone(), q.double().clone(), w.double()
+    for t in range(L):                       # every earlier key through H_t
+        c = 2.0 * (kr[:, :, :t] @ W[:, :, t, :, None])
+        kr[:, :, :t] -= c * W[:, :, t, None]
+    for t in range(L - 1, -1, -1):           # every query from t on through H_t
+        c = 2.0 * (x[:, :, t:] @ W[:, :, t, :, None])
+        x[:, :, t:] -= c * W[:, :, t, None]
+    for got, ref in ((tiles(message), kr), (tiles(state), x)):
+        assert (got - ref).norm() <= 2.55e-3 * ref.norm()
+
+
 def test_one_segment_is_the_ordinary_forward(oracle):
     from paper_2505_16381_b200 import binding, ring
     inp = synth.make_inputs(1, 2, 640, 128, "bf16", gate=True, seed=9200)
