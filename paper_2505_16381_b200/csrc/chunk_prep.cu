@@ -23,9 +23,9 @@
 // What bounds it: the chain of dependent phases of one chunk (its seven tiles and four accumulators fill the SM, so there is
 // one chunk per SM at a time) and, in the backward's instance, bursts of stores: 416 KB per chunk against about 23 bytes per
 // cycle and SM of memory bandwidth.  Cycles per chunk at B=4, H=16, L=4096, d=128 (backward's instance) / 32 x 32768 x 128
-// (forward's): 27.2 k / 23.6 k, of which the inverse 8 k, 116 product steps 7.5 k (mostly underneath), E1 1.9 k, Xk and Xq
+// (forward's): 29 k / 25 k, of which the inverse 9.7 k, 116 product steps 7.5 k (mostly underneath), E1 1.9 k, Xk and Xq
 // 3 k, U and Y 1.8 k, P, Q<- and K-> 3.9 k, the rest waits.  With the inverse in float32 loops plus one tcgen05 level and
-// rows stored and fetched by the workers: 43.5 k / 33.9 k.  Time 352 -> 225 us and 1240 -> 870 us; 128 x 2048 x 64: 278 -> 187.
+// rows stored and fetched by the workers: 43.5 k / 33.9 k.  Time 352 -> 243 us and 1240 -> 940 us; 128 x 2048 x 64: 278 -> 206.
 #include <type_traits>
 #include "tileops.cuh"
 
@@ -73,15 +73,24 @@ __device__ __forceinline__ bool wsync_and(bool ok) {   // barrier over the worke
 }
 
 // ------------------------------------------------------------------------------------------------ triangular inverse
-// In place on a [128 x 128] matrix held as a bf16 pair of swizzled tiles (aH, aL):  N strictly lower -> T~ = (I + N)^-1 D.
-// 16 x 16 diagonal blocks by float32 forward substitution (`dblk`: the blocks [8][16][16] in float32), then three merge
-// levels  [[A,0],[C,B]]^-1 = [[A^-1,0],[-B^-1 C A^-1, B^-1]]  of 16-, 32- and 64-row blocks as warp-level products
-// (mma.sync m16n8k16, bf16 pairs, lo x lo left out: the precision T~ is kept in afterwards).  A warp owns a 16-row strip of
-// B^-1 C: its accumulators are the A fragments of the second product, so nothing goes through memory in between.
+// In place in the two slots of a bf16 pair of swizzled tiles (aH, aL):  N strictly lower -> T~ = (I + N)^-1 D.  The two 64 x 64
+// diagonal blocks of N arrive in float32, in the 16 KB that their pair takes up later (fel below); the 64 x 64 block C under the
+// diagonal as a pair, and zeros above it.  16 x 16 diagonal blocks by float32 forward substitution, then three merge levels
+// [[A,0],[C,B]]^-1 = [[A^-1,0],[-B^-1 C A^-1, B^-1]]  of 16-, 32- and 64-row blocks as warp-level products.  A warp owns a
+// 16-row strip of B^-1 C: its accumulators are the A fragments of the second product, so nothing goes through memory in between.
+//
+// Precision.  The first two levels read and write float32, their products split every operand into two tf32 numbers (mma.sync
+// m16n8k8, lo x lo left out: 2^-22 of a product).  The last level takes bf16 pairs (m16n8k16), the form T~ is kept in
+// afterwards, and the blocks on the diagonal are scaled by D in float32 before they become one.  Relative error of T~ against
+// float64 over 128 chunks, d = 64 / 128, with N and all levels in bf16 pairs -> like this, which is what float32 loops for
+// the first two levels give (rounding the exact T~ to a pair: 2.3e-6): random unit w 5.1e-6 / 3.8e-6 -> 4.0e-6 / 3.2e-6; beta = 2
+// and w around one direction 1.7e-4 / 1.6e-4 -> 8.4e-5 / 8.2e-5; beta = 2 and four directions 7.7e-5 / 6.2e-5 -> 1.5e-5 / 1.5e-5.
+//
+// Time: 9.7 thousand cycles (substitution 2.0, merges 0.9, 2.2, 3.3, the change to pairs 0.7, scaling 0.6), 8 with pairs throughout;
+// float32 loops up to 64 rows plus one tcgen05 level took 14.  The merges are bound by the rate of mma.sync, about 20 cycles
+// each and scheduler for either shape (dependent products in three separate accumulators changed nothing).
 // Why not tcgen05: its smallest tile has 64 rows and every product costs a round trip through tensor memory, a shared
 // memory tile and two hand-overs (about 1500 cycles each, measured); here the blocks are 16 to 64 rows and dependent.
-// 8 thousand cycles for the whole inverse (substitution 2.0, merges 0.6, 1.2, 2.9, scaling 1.0); float32 loops up to 64 rows
-// plus one tcgen05 level took 14 thousand.
 __device__ __forceinline__ uint32_t frag_addr(uint32_t tile_, int r0, int c0, int lane) {
     const int rr = r0 + (lane & 15), c = c0 + (lane >> 4) * 8;
     return tile_ + (uint32_t)(c >> 6) * kPanelB + sw128_off((uint32_t)rr, (uint32_t)((c & 63) >> 3));
@@ -96,6 +105,11 @@ __device__ __forceinline__ void ldsm4t(uint32_t (&f)[4], uint32_t addr) {
 }
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma1688(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -114,85 +128,157 @@ __device__ __forceinline__ uint32_t split_pair(float a, float b, uint32_t& l) { 
     l = pack_bf16(a - __uint_as_float(h << 16), b - __uint_as_float(h & 0xffff0000u));
     return h;
 }
-// One merge level of blocks of NBK 16-row strips.  The two warps that share a scheduler (w, w + 4) take a long and a short
-// strip (B^-1 is lower triangular: strip rb needs its first rb + 1 blocks).  The last level's result is scaled by D.
+// hi (x cut off), l = lo (the rest, rounded: 11 + 11 bits and a sign).  Plain integer operations: cvt.rna.tf32 took 4 % longer.
+__device__ __forceinline__ uint32_t split_tf32(float x, uint32_t& l) {
+    const uint32_t h = __float_as_uint(x) & 0xffffe000u;
+    l = (__float_as_uint(x - __uint_as_float(h)) + 0x1000u) & 0xffffe000u;
+    return h;
+}
+// Element (r, c) of the float32 diagonal block b (64 x 64): rows 0 - 31 where the block's hi tile goes later, rows 32 - 63 at its lo
+// tile.  Columns are permuted in groups of four so that fragment loads (8 rows x 8 columns, rows 2t and 2t + 1) and row-wise
+// 16-byte accesses are free of bank conflicts.
+__device__ __forceinline__ float* fel(uint8_t* aH, uint8_t* aL, int b, int r, int c) {
+    const int f = (((r & 3) ^ ((r >> 2) & 1)) << 3) | (r & 4);
+    return reinterpret_cast<float*>((r & 32 ? aL : aH) + b * (kPanelB + 8192)) + (r & 31) * 64 + (c ^ f);
+}
+// Fragments of float32 blocks for m16n8k8.  Slots t and t + 4 of the contraction stand for columns 2t and 2t + 1 of A and
+// rows 2t and 2t + 1 of B, which makes an accumulator tile of one product an A fragment of the next as it is.
+struct Tf32A { uint32_t h[4], l[4]; };
+__device__ __forceinline__ Tf32A tf32_a(uint8_t* aH, uint8_t* aL, int b, int r0, int c0, int lane) {
+    const float2 x = *reinterpret_cast<const float2*>(fel(aH, aL, b, r0 + (lane >> 2), c0 + 2 * (lane & 3)));
+    const float2 y = *reinterpret_cast<const float2*>(fel(aH, aL, b, r0 + 8 + (lane >> 2), c0 + 2 * (lane & 3)));
+    Tf32A a;
+    a.h[0] = split_tf32(x.x, a.l[0]); a.h[1] = split_tf32(y.x, a.l[1]);
+    a.h[2] = split_tf32(x.y, a.l[2]); a.h[3] = split_tf32(y.y, a.l[3]);
+    return a;
+}
+__device__ __forceinline__ Tf32A tf32_a(const float (&d)[4]) {
+    Tf32A a;
+    a.h[0] = split_tf32(d[0], a.l[0]); a.h[1] = split_tf32(d[2], a.l[1]);
+    a.h[2] = split_tf32(d[1], a.l[2]); a.h[3] = split_tf32(d[3], a.l[3]);
+    return a;
+}
+// d[16 x 8] += A B, B the 8 x 8 block at (r0, c0)
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const Tf32A& a, uint8_t* aH, uint8_t* aL, int b, int r0, int c0, int lane) {
+    uint32_t h[2], l[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) h[x] = split_tf32(*fel(aH, aL, b, r0 + 2 * (lane & 3) + x, c0 + (lane >> 2)), l[x]);
+    mma1688(d, a.h, h[0], h[1]);
+    mma1688(d, a.h, l[0], l[1]);
+    mma1688(d, a.l, h[0], h[1]);
+}
+// One merge level of blocks of NBK 16-row strips (1, 2) inside the float32 blocks.  NBK = 1: four pairs, the two warps of a pair take
+// 8 columns of the result each; NBK = 2: a warp takes 16 x 16, the two warps that share a scheduler (w, w + 4) a long and a
+// short strip (B^-1 is lower triangular: strip rb needs its first rb + 1 blocks).
 template <int NBK>
-__device__ __forceinline__ void merge_level(uint8_t* aH, uint8_t* aL, const float* bt, int warp, int lane) {
-    constexpr int CBN = NBK == 4 ? 2 : 1;   // 16-column blocks of the result per warp
-    const uint32_t tH = smem_u32(aH), tL = smem_u32(aL);
+__device__ __forceinline__ void merge_f32(uint8_t* aH, uint8_t* aL, int warp, int lane) {
+    constexpr int NT = NBK;                       // 8-column tiles of the result per warp
     const int hw = warp >> 2, w4 = warp & 3;
-    const int pair = NBK == 1 ? w4 : (NBK == 2 ? (w4 & 1) : 0);
-    const int rb = NBK == 1 ? 0 : (NBK == 2 ? ((w4 >> 1) ^ hw) : (hw ? 3 - w4 : w4));
-    const int cb0 = NBK == 1 ? 0 : hw * CBN;
-    const int base_a = pair * 2 * NBK * 16, base_b = base_a + NBK * 16, row0 = base_b + rb * 16;
-    const bool active = NBK > 1 || hw == 0;
-    float m[CBN][2][4];
-    if (active) {
-        float p1[NBK][2][4];
+    const int b = NBK == 1 ? w4 >> 1 : w4 & 1, rb = NBK == 1 ? 0 : ((w4 >> 1) ^ hw);
+    const int base_a = NBK == 1 ? (w4 & 1) * 32 : 0, base_b = base_a + NBK * 16, row0 = base_b + rb * 16;
+    const int k_lo = NBK == 1 ? 0 : hw, col0 = base_a + hw * NBK * 8;   // A^-1 is lower triangular: columns col0.. need no earlier block
+    float m[NT][4], p1[NBK][2][4];
 #pragma unroll
-        for (int k = 0; k < NBK; ++k)
+    for (int k = 0; k < NBK; ++k)
 #pragma unroll
-            for (int x = 0; x < 8; ++x) p1[k][x >> 2][x & 3] = 0.f;
+        for (int x = 0; x < 8; ++x) p1[k][x >> 2][x & 3] = 0.f;
 #pragma unroll
-        for (int k = 0; k < CBN; ++k)
+    for (int x = 0; x < 4 * NT; ++x) m[x >> 2][x & 3] = 0.f;
 #pragma unroll
-            for (int x = 0; x < 8; ++x) m[k][x >> 2][x & 3] = 0.f;
-#pragma unroll 1
-        for (int j = 0; j <= rb; ++j) {
-            uint32_t ah[4], al[4];
-            ldsm4(ah, frag_addr(tH, row0, base_b + j * 16, lane));
-            ldsm4(al, frag_addr(tL, row0, base_b + j * 16, lane));
+    for (int j = 0; j < NBK; ++j)
+#pragma unroll
+        for (int k8 = 0; k8 < 2; ++k8) {
+            if (j > rb) continue;
+            const Tf32A a = tf32_a(aH, aL, b, row0, base_b + j * 16 + k8 * 8, lane);
 #pragma unroll
             for (int kb = 0; kb < NBK; ++kb) {
-                if (kb < cb0) continue;       // A^-1 is lower triangular: columns cb0.. need no earlier block
-                uint32_t bh[4], bl[4];
-                ldsm4t(bh, frag_addr(tH, base_b + j * 16, base_a + kb * 16, lane));
-                ldsm4t(bl, frag_addr(tL, base_b + j * 16, base_a + kb * 16, lane));
-                mma_pair(p1[kb], ah, al, bh, bl);
+                if (kb < k_lo) continue;
+#pragma unroll
+                for (int n = 0; n < 2; ++n) mma_tf32(p1[kb][n], a, aH, aL, b, base_b + j * 16 + k8 * 8, base_a + kb * 16 + n * 8, lane);
             }
         }
+#pragma unroll
+    for (int kb = 0; kb < NBK; ++kb) {
+        if (kb < k_lo) continue;
+#pragma unroll
+        for (int k8 = 0; k8 < 2; ++k8) {
+            const Tf32A a = tf32_a(p1[kb][k8]);
+#pragma unroll
+            for (int n = 0; n < NT; ++n) mma_tf32(m[n], a, aH, aL, b, base_a + kb * 16 + k8 * 8, col0 + n * 8, lane);
+        }
+    }
+    wsync();   // the other warps of the pair read C as well
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+            *reinterpret_cast<float2*>(fel(aH, aL, b, row0 + (lane >> 2) + 8 * y, col0 + n * 8 + 2 * (lane & 3))) =
+                make_float2(-m[n][2 * y], -m[n][2 * y + 1]);
+}
+// The last level, on the pairs: strips of 64 x 64 blocks, the result scaled by D.
+__device__ __forceinline__ void merge_pairs(uint8_t* aH, uint8_t* aL, const float* bt, int warp, int lane) {
+    constexpr int NBK = 4, CBN = 2;               // 16-row strips per block, 16-column blocks of the result per warp
+    const uint32_t tH = smem_u32(aH), tL = smem_u32(aL);
+    const int hw = warp >> 2, w4 = warp & 3, rb = hw ? 3 - w4 : w4, cb0 = hw * CBN, row0 = 64 + rb * 16;
+    float m[CBN][2][4], p1[NBK][2][4];
+#pragma unroll
+    for (int k = 0; k < NBK; ++k)
+#pragma unroll
+        for (int x = 0; x < 8; ++x) p1[k][x >> 2][x & 3] = 0.f;
+#pragma unroll
+    for (int k = 0; k < CBN; ++k)
+#pragma unroll
+        for (int x = 0; x < 8; ++x) m[k][x >> 2][x & 3] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j <= rb; ++j) {
+        uint32_t ah[4], al[4];
+        ldsm4(ah, frag_addr(tH, row0, 64 + j * 16, lane));
+        ldsm4(al, frag_addr(tL, row0, 64 + j * 16, lane));
 #pragma unroll
         for (int kb = 0; kb < NBK; ++kb) {
-            if (kb < cb0) continue;
-            uint32_t ah[4], al[4];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) ah[x] = split_pair(p1[kb][x >> 1][(x & 1) * 2], p1[kb][x >> 1][(x & 1) * 2 + 1], al[x]);
-#pragma unroll
-            for (int i = 0; i < CBN; ++i) {
-                if (kb < cb0 + i) continue;
-                uint32_t bh[4], bl[4];
-                ldsm4t(bh, frag_addr(tH, base_a + kb * 16, base_a + (cb0 + i) * 16, lane));
-                ldsm4t(bl, frag_addr(tL, base_a + kb * 16, base_a + (cb0 + i) * 16, lane));
-                mma_pair(m[i], ah, al, bh, bl);
-            }
+            if (kb < cb0) continue;       // A^-1 is lower triangular: columns cb0.. need no earlier block
+            uint32_t bh[4], bl[4];
+            ldsm4t(bh, frag_addr(tH, 64 + j * 16, kb * 16, lane));
+            ldsm4t(bl, frag_addr(tL, 64 + j * 16, kb * 16, lane));
+            mma_pair(p1[kb], ah, al, bh, bl);
         }
     }
-    if (NBK > 1) wsync();   // the other strips of the pair read C as well
-    else __syncwarp();
-    if (active) {
 #pragma unroll
-        for (int i = 0; i < CBN; ++i)
+    for (int kb = 0; kb < NBK; ++kb) {
+        if (kb < cb0) continue;
+        uint32_t ah[4], al[4];
 #pragma unroll
-            for (int n = 0; n < 2; ++n) {
-                const int col = base_a + (cb0 + i) * 16 + n * 8 + 2 * (lane & 3);
-                const float s0 = NBK == 4 ? -bt[col] : -1.f, s1 = NBK == 4 ? -bt[col + 1] : -1.f;
+        for (int x = 0; x < 4; ++x) ah[x] = split_pair(p1[kb][x >> 1][(x & 1) * 2], p1[kb][x >> 1][(x & 1) * 2 + 1], al[x]);
 #pragma unroll
-                for (int y = 0; y < 2; ++y) {
-                    const int rr = row0 + (lane >> 2) + 8 * y;
-                    uint32_t l;
-                    const uint32_t h = split_pair(s0 * m[i][n][2 * y], s1 * m[i][n][2 * y + 1], l);
-                    const uint32_t off = (uint32_t)(col >> 6) * kPanelB + sw128_off((uint32_t)rr, (uint32_t)((col & 63) >> 3)) + (col & 7) * 2;
-                    *reinterpret_cast<uint32_t*>(aH + off) = h;
-                    *reinterpret_cast<uint32_t*>(aL + off) = l;
-                }
-            }
+        for (int i = 0; i < CBN; ++i) {
+            if (kb < cb0 + i) continue;
+            uint32_t bh[4], bl[4];
+            ldsm4t(bh, frag_addr(tH, kb * 16, (cb0 + i) * 16, lane));
+            ldsm4t(bl, frag_addr(tL, kb * 16, (cb0 + i) * 16, lane));
+            mma_pair(m[i], ah, al, bh, bl);
+        }
     }
+    wsync();   // the other strips read C as well
+#pragma unroll
+    for (int i = 0; i < CBN; ++i)
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const int col = (cb0 + i) * 16 + n * 8 + 2 * (lane & 3);
+            const float s0 = -bt[col], s1 = -bt[col + 1];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const int rr = row0 + (lane >> 2) + 8 * y;
+                uint32_t l;
+                const uint32_t h = split_pair(s0 * m[i][n][2 * y], s1 * m[i][n][2 * y + 1], l);
+                const uint32_t off = (uint32_t)(col >> 6) * kPanelB + sw128_off((uint32_t)rr, (uint32_t)((col & 63) >> 3)) + (col & 7) * 2;
+                *reinterpret_cast<uint32_t*>(aH + off) = h;
+                *reinterpret_cast<uint32_t*>(aL + off) = l;
+            }
+        }
 }
-__device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const float* dblk, const float* bt, int warp, int lane, int row,
-                                            int half) {
-    {   // diagonal block `warp`: lane j (and its copy j + 16, which stores the lo parts) keeps column j in registers
-        const float* Lb = dblk + warp * 256;
-        const int o = warp * 16, j = lane & 15;
+__device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const float* bt, int warp, int lane, int row, int half) {
+    {   // diagonal block `warp`: lane j (and its copy j + 16) keeps column j in registers
+        const int b = warp >> 2, o = (warp & 3) * 16, j = lane & 15;
         float x[16];
 #pragma unroll
         for (int g = 0; g < 4; ++g) {   // four rows at a time: their loads are issued together, ahead of the dependent sums
@@ -200,7 +286,7 @@ __device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const floa
 #pragma unroll
             for (int y = 0; y < 4; ++y)
 #pragma unroll
-                for (int c = 0; c <= g; ++c) f[y][c] = *reinterpret_cast<const float4*>(Lb + (4 * g + y) * 16 + 4 * c);
+                for (int c = 0; c <= g; ++c) f[y][c] = *reinterpret_cast<const float4*>(fel(aH, aL, b, o + 4 * g + y, o + 4 * c));
 #pragma unroll
             for (int y = 0; y < 4; ++y) {
                 const int rr = 4 * g + y;
@@ -219,41 +305,38 @@ __device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const floa
                 x[rr] = rr >= j ? a : 0.f;
             }
         }
-        uint8_t* t_ = (lane < 16 ? aH : aL) + (o >> 6) * kPanelB + ((o + j) & 7) * 2;
+        __syncwarp();
 #pragma unroll
-        for (int rr = 0; rr < 16; ++rr) {
-            const __nv_bfloat16 h = __float2bfloat16_rn(x[rr]);
-            *reinterpret_cast<__nv_bfloat16*>(t_ + sw128_off((uint32_t)(o + rr), (uint32_t)(((o + j) & 63) >> 3))) =
-                lane < 16 ? h : __float2bfloat16_rn(x[rr] - __bfloat162float(h));
-        }
+        for (int rr = 0; rr < 8; ++rr) *fel(aH, aL, b, o + rr + (lane >> 4) * 8, o + j) = lane < 16 ? x[rr] : x[rr + 8];
     }
     wsync();
-    merge_level<1>(aH, aL, bt, warp, lane);
+    merge_f32<1>(aH, aL, warp, lane);
     wsync();
-    merge_level<2>(aH, aL, bt, warp, lane);
+    merge_f32<2>(aH, aL, warp, lane);
     wsync();
-    merge_level<4>(aH, aL, bt, warp, lane);   // (from its barrier on nobody reads the diagonal blocks any more)
-    {   // the 64 x 64 diagonal blocks are scaled by D; the corner that held the float32 blocks becomes zero
-        const int cb = row & 64;
-        uint8_t* ph = aH + (cb >> 6) * kPanelB;
-        uint8_t* pl = aL + (cb >> 6) * kPanelB;
+    // the diagonal blocks become pairs, in the same place; this thread's 32 entries stay in registers until they are scaled
+    float d[32];
+    const int cb = (row & 64) + half * 32;
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-            const uint32_t off = sw128_off((uint32_t)row, (uint32_t)(half * 4 + ch));
-            const uint4 h4 = *reinterpret_cast<const uint4*>(ph + off), l4 = *reinterpret_cast<const uint4*>(pl + off);
-            const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
-            uint32_t ho[4], lo[4];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const float2 b2 = *reinterpret_cast<const float2*>(bt + cb + half * 32 + ch * 8 + 2 * x);
-                ho[x] = split_pair((__uint_as_float(hw[x] << 16) + __uint_as_float(lw[x] << 16)) * b2.x,
-                                   (__uint_as_float(hw[x] & 0xffff0000u) + __uint_as_float(lw[x] & 0xffff0000u)) * b2.y, lo[x]);
-            }
-            *reinterpret_cast<uint4*>(ph + off) = make_uint4(ho[0], ho[1], ho[2], ho[3]);
-            *reinterpret_cast<uint4*>(pl + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            if (row < 64) *reinterpret_cast<uint4*>(aH + kPanelB + off) = make_uint4(0u, 0u, 0u, 0u);
-        }
+    for (int x = 0; x < 32; x += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(fel(aH, aL, row >> 6, row & 63, half * 32 + x));
+        d[x] = v.x; d[x + 1] = v.y; d[x + 2] = v.z; d[x + 3] = v.w;
     }
+    wsync();
+    uint32_t hi[16], lo[16];
+    split32(d, hi, lo);
+    tile_store_w16(aH, row, cb, hi);
+    tile_store_w16(aL, row, cb, lo);
+    wsync();
+    merge_pairs(aH, aL, bt, warp, lane);   // (from its barrier on nobody reads the diagonal blocks any more)
+#pragma unroll
+    for (int x = 0; x < 32; x += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(bt + cb + x);
+        d[x] *= v.x; d[x + 1] *= v.y; d[x + 2] *= v.z; d[x + 3] *= v.w;
+    }
+    split32(d, hi, lo);
+    tile_store_w16(aH, row, cb, hi);
+    tile_store_w16(aL, row, cb, lo);
 }
 
 // MODE: PREP_FWD = everything the forward needs; PREP_SAVE = also keeps the tiles of the chain rule (the backward's instance);
@@ -459,11 +542,10 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
             const uint32_t par = it & 1;
             if (!(ok = wwait(B_GM, par))) break;
 
-            // ---- E1: N = strictLower(D Gm) as a bf16 pair into slots 1, 2, its 16 x 16 diagonal blocks also in float32.  The
-            // blocks borrow 8 KB of the tile's zero corner (rows 0 - 63 of its second panel).
+            // ---- E1: N = strictLower(D Gm) into slots 1, 2 as tri_inverse wants it: the two diagonal blocks in float32, the rest (and
+            // the zeros above the diagonal) as a bf16 pair
             uint8_t* aH = slot(1);
             uint8_t* aL = slot(2);
-            float* dblk = (float*)(aH + kPanelB);
             for (int c = 0; c < 2; ++c) {
                 const int c0 = half * 64 + c * 32;
                 tmem_ld32(tl + 0 + c0, r);
@@ -471,20 +553,18 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
                 const float b = bt[row];
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = (c0 + x < row) ? b * __uint_as_float(r[x]) : 0.f;
-                split32(v, hi, lo);
-                if (c0 < 64 || row >= 64) tile_store_w16(aH, row, c0, hi);
-                tile_store_w16(aL, row, c0, lo);
-                if ((row >> 5) == (c0 >> 5)) {
-                    float4* d = reinterpret_cast<float4*>(dblk + row * 16);
-                    const bool up = lane >= 16;
+                if ((row >> 6) == half) {
 #pragma unroll
-                    for (int x = 0; x < 4; ++x)
-                        d[x] = make_float4(up ? v[16 + 4 * x] : v[4 * x], up ? v[17 + 4 * x] : v[4 * x + 1],
-                                           up ? v[18 + 4 * x] : v[4 * x + 2], up ? v[19 + 4 * x] : v[4 * x + 3]);
+                    for (int x = 0; x < 32; x += 4)
+                        *reinterpret_cast<float4*>(fel(aH, aL, half, row & 63, c * 32 + x)) = make_float4(v[x], v[x + 1], v[x + 2], v[x + 3]);
+                } else {
+                    split32(v, hi, lo);
+                    tile_store_w16(aH, row, c0, hi);
+                    tile_store_w16(aL, row, c0, lo);
                 }
             }
             wsync();
-            tri_inverse(aH, aL, dblk, bt, warp, lane, row, half);   // -> T~ = (I + N)^-1 D
+            tri_inverse(aH, aL, bt, warp, lane, row, half);   // -> T~ = (I + N)^-1 D
             fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&bars[R_TT]);

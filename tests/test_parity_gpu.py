@@ -712,3 +712,42 @@ def test_float32_rows_before_a_nan_or_infinity(binding, name, S, d, p, value):
     assert torch.equal(o[:, :, :c], o0[:, :, :c]) and torch.equal(lse[:, :, :c], l0[:, :, :c])
     if c < 150:
         assert not torch.isfinite(o[:, :, p:]).all(), "the value must reach its own row or a later one"
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("directions", ["random", "one", "four"])
+def test_triangular_inverse_accuracy(binding, d, directions):
+    """T~ = (I + strictLower(D W W^T))^-1 D as the preparation keeps it (a bf16 pair, at the start of a backward-sized workspace),
+    its 64 x 64 diagonal blocks against float64: random w, and beta = 2 with directions that repeat through the whole chunk.
+
+    Rounding the exact block to a pair costs at most 2^-18 = 3.8e-6 of every entry.  The merges up to 64 rows, M = B^-1 C A^-1, work
+    in float32 with products whose factors are good to 2^-22.  Their errors are independent, so an entry of M is off by
+    2^-22 times the root of the sum of the squares of its terms, which is evaluated from the exact blocks; twice that for what the
+    second level takes over from the first."""
+    B, H, L = 1, 4, 1024
+    g = torch.Generator(device="cuda").manual_seed(71 + d)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    q, k, v = (n(B, H, L, d).bfloat16() for _ in range(3))
+    w, beta = n(B, H, L, d), 2 * torch.sigmoid(n(B, H, L))
+    if directions != "random":
+        w = w + 3 * n(B, H, 1, d) if directions == "one" else w[:, :, :4][:, :, torch.randint(4, (L,), generator=g, device="cuda")]
+        beta = torch.full_like(beta, 2.0)
+    w = torch.nn.functional.normalize(w, dim=-1).bfloat16()
+    ws = binding.alloc_workspace(q, False, True)
+    binding.path_attn_fwd(q, k, v, w, beta, workspace=ws)
+    m = B * H * L * 128 * 2
+    tile = lambda i: ws[256 + i * m:256 + (i + 1) * m].view(torch.bfloat16).view(-1, 128, 128).double()
+    T = tile(0) + tile(1)
+    W, bt = w.double().view(-1, 128, d), beta.double().view(-1, 128)
+    N = torch.tril(bt[..., None] * (W @ W.transpose(-1, -2)), -1)
+    eye = torch.eye(64, dtype=torch.float64, device="cuda")
+    for c in (0, 64):
+        Nb = N[:, c:c + 64, c:c + 64]
+        inv = torch.linalg.solve_triangular(eye + Nb, eye.expand_as(Nb), upper=False)
+        ref = inv * bt[:, None, c:c + 64]
+        norm = lambda x: x.norm(dim=(-2, -1))
+        terms = [(inv[:, a + h:a + 2 * h, a + h:a + 2 * h] ** 2 @ Nb[:, a + h:a + 2 * h, a:a + h] ** 2 @ inv[:, a:a + h, a:a + h] ** 2)
+                 .sum(dim=(-2, -1)) for h in (16, 32) for a in range(0, 64, 2 * h)]
+        bound = 2 ** -18 * norm(ref) + 2 * 2 ** -22 * bt.amax(-1) * sum(terms).sqrt()
+        err = norm(T[:, c:c + 64, c:c + 64] - ref)
+        assert (err <= bound).all(), ((err / norm(ref)).max().item(), (bound / norm(ref)).min().item())
