@@ -193,19 +193,6 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     bool ok = true;
     uint32_t ph_mma = 0, ph_mma2 = 0;
     float v[32];
-    auto wsync_and = [&](bool good) {   // barrier over the eight worker warps + AND of `good`
-        uint32_t r;
-        __syncwarp();
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t"
-            "setp.ne.b32 p, %1, 0;\n\t"
-            "bar.red.and.pred q, 1, 256, p;\n\t"
-            "selp.u32 %0, 1, 0, q;\n\t}"
-            : "=r"(r)
-            : "r"((uint32_t)good)
-            : "memory");
-        return r != 0;
-    };
     auto wsync = [&]() {
         __syncwarp();
         asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -216,7 +203,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         bool good = true;
         if (lane == 0) good = mbar_wait(&bars[b], ph, abort_flag, ST_CHAIN);
         ph ^= 1;
-        ok = wsync_and(good);
+        ok = barrier_and<1, 256>(good);
         tc_fence_after_sync();
     };
     // tiles written by this thread become visible to the MMA unit, its accumulator reads are ordered, the leader learns

@@ -58,19 +58,7 @@ __device__ __forceinline__ void wsync() {
     __syncwarp();
     asm volatile("bar.sync 1, 256;" ::: "memory");
 }
-__device__ __forceinline__ bool wsync_and(bool ok) {   // barrier over the worker warps + AND of `ok`
-    uint32_t r;
-    __syncwarp();
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.and.pred q, 1, 256, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)ok)
-        : "memory");
-    return r != 0;
-}
+__device__ __forceinline__ bool wsync_and(bool ok) { return barrier_and<1, 256>(ok); }
 
 // ------------------------------------------------------------------------------------------------ triangular inverse
 // In place in the two slots of a bf16 pair of swizzled tiles (aH, aL):  N strictly lower -> T~ = (I + N)^-1 D.  The two 64 x 64

@@ -223,8 +223,7 @@ __global__ void __launch_bounds__(192, R == 64 ? 2 : 1) wide_kernel(const __grid
         for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
             const int m0 = u / groups * 128, t0 = u % groups * per_unit, t1 = min(t0 + per_unit, ntiles);
             for (int t = t0; t < t1; ++t, ++nb) {
-                if (!wait(CFULL + (nb & 1), nb >> 1)) ok = false;
-                ok = __all_sync(0xffffffffu, ok);
+                ok = __all_sync(0xffffffffu, wait(CFULL + (nb & 1), nb >> 1));
                 tc_fence_after_sync();
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -242,7 +241,8 @@ __global__ void __launch_bounds__(192, R == 64 ? 2 : 1) wide_kernel(const __grid
                     }
                     // the panel's previous store (two stores ago) has read it
                     if (tid == 64) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                    sync();
+                    if (h == 0) ok = barrier_and<1, 128>(ok);   // the four warps go on, or leave after this tile, together
+                    else sync();
                     if (ok) {
                         float v[32];
 #pragma unroll

@@ -80,6 +80,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return mbar_wait_slow(bar, parity, abort_flag, code);
 }
 
+// Barrier ID over N threads (whole warps) + AND of `ok`.  Warps that meet at a named barrier leave a loop only on a vote like
+// this: if each went by its own waits, one whose wait ran out would be gone, and another, whose wait on the same barrier was
+// answered an instant later, would wait for it at the next named barrier for ever (that wait has no limit).  The instruction
+// is warp-aligned: a warp whose lanes left a loop at different times must reconverge first.
+template <int ID, int N>
+__device__ __forceinline__ bool barrier_and(bool ok) {
+    uint32_t r;
+    __syncwarp();
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, %2, %3, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)ok), "n"(ID), "n"(N)
+        : "memory");
+    return r != 0;
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
