@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
             tc_fence_after_sync();
             if (GATE) {   // the two threads of a key row add their halves of the column sum
                 if (h == 1) dsum_x[row] = dsum;
-                { __syncwarp(); asm volatile("bar.sync 1, 256;" ::: "memory"); }
+                ok = barrier_and<1, 256>(ok);   // (all warps leave below, or none)
                 if (h == 0 && ok) p.dG[(size_t)s * p.Lp + kj] = -(dsum + dsum_x[row]);
                 { __syncwarp(); asm volatile("bar.sync 1, 256;" ::: "memory"); }
             }

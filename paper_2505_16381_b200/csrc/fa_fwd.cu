@@ -498,8 +498,7 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
             // ---- merge the two streams and write O, LSE: warpgroup x handles columns [x*HD/2, (x+1)*HD/2)
             if (GATE) wg_sync();
             if (TX > 0) statx[row] = make_float2(m, l);
-            __syncwarp();
-            asm volatile("bar.sync 3, 256;" ::: "memory");
+            if (!barrier_and<3, 256>(ok)) break;   // (all warps or none: see barrier_and)
             const bool two = NS > 1;
             const float2 s0 = stat[row];
             const float2 s1 = two ? stat[kTile + row] : make_float2(-INFINITY, 0.f);
@@ -510,7 +509,7 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
             }
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after_sync();
-            if (!ok) break;
+            if (!ok) continue;                    // (to the vote of the next item)
             constexpr int CW = HD / 2;            // columns per warpgroup
             const float mm = fmaxf(s0.x, s1.x);
             const float w0 = ex2(s0.x - mm), w1 = two ? ex2(s1.x - mm) : 0.f;
