@@ -1411,35 +1411,36 @@ __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ B
 template <int HD>
 __global__ void rowstats_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                                 const float* __restrict__ lse, const float* __restrict__ G, float* __restrict__ delta,
-                                float* __restrict__ lse2, int L, int Lp) {
+                                float* __restrict__ lse2, int S, int L, int Lp) {
     grid_wait();
     grid_launch();
     constexpr int TPR = HD / 8;                 // threads per row: 16 bytes (8 values) of o and of dO each
-    const int s = blockIdx.y;
     const int i = blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
     const int sub = threadIdx.x % TPR;
-    float acc = 0.f;
-    if (i < L) {
-        const size_t base = ((size_t)s * L + i) * HD + sub * 8;
-        const uint4 a = *reinterpret_cast<const uint4*>(o + base), b = *reinterpret_cast<const uint4*>(d_o + base);
-        const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+    for (int s = blockIdx.y; s < S; s += gridDim.y) {   // (a grid's second dimension ends at 65535)
+        float acc = 0.f;
+        if (i < L) {
+            const size_t base = ((size_t)s * L + i) * HD + sub * 8;
+            const uint4 a = *reinterpret_cast<const uint4*>(o + base), b = *reinterpret_cast<const uint4*>(d_o + base);
+            const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[x]));
-            const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[x]));
-            acc += fa.x * fb.x + fa.y * fb.y;
+            for (int x = 0; x < 4; ++x) {
+                const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[x]));
+                const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw[x]));
+                acc += fa.x * fb.x + fa.y * fb.y;
+            }
         }
-    }
 #pragma unroll
-    for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (sub == 0 && i < Lp) {
-        delta[(size_t)s * Lp + i] = -acc;
-        // rows of the zero-padded tail get a huge negative value: their probabilities must come out as exact zeros.  (A
-        // plain 0 would do without a gate; with one, exp2(0 - G_j log2 e) of a strongly decayed key overflows and the
-        // product with the row's zero dP - delta is a NaN.)
-        float v = -1e30f;
-        if (i < L) v = ((G ? G[(size_t)s * Lp + i] : 0.f) - lse[(size_t)s * L + i]) * kLog2e;
-        lse2[(size_t)s * Lp + i] = v;
+        for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (sub == 0 && i < Lp) {
+            delta[(size_t)s * Lp + i] = -acc;
+            // rows of the zero-padded tail get a huge negative value: their probabilities must come out as exact zeros.  (A
+            // plain 0 would do without a gate; with one, exp2(0 - G_j log2 e) of a strongly decayed key overflows and the
+            // product with the row's zero dP - delta is a NaN.)
+            float v = -1e30f;
+            if (i < L) v = ((G ? G[(size_t)s * Lp + i] : 0.f) - lse[(size_t)s * L + i]) * kLog2e;
+            lse2[(size_t)s * Lp + i] = v;
+        }
     }
 }
 
@@ -1470,10 +1471,10 @@ cudaError_t launch_fa_bwd(const BwdTensorMaps& tm, const BwdParams& p, int hd, i
 cudaError_t launch_rowstats(const void* o, const void* d_o, const float* lse, const float* G, float* delta, float* lse2,
                             int S, int L, int Lp, int hd, cudaStream_t st) {
     const int rows_per_cta = 256 / (hd / 8);
-    dim3 grid((Lp + rows_per_cta - 1) / rows_per_cta, S);
+    const dim3 grid((Lp + rows_per_cta - 1) / rows_per_cta, S < 65535 ? S : 65535);
     typedef __nv_bfloat16 bf;
-    return hd == 64 ? launch<rowstats_kernel<64>>(grid, 256, 0, st, (const bf*)o, (const bf*)d_o, lse, G, delta, lse2, L, Lp)
-                    : launch<rowstats_kernel<128>>(grid, 256, 0, st, (const bf*)o, (const bf*)d_o, lse, G, delta, lse2, L, Lp);
+    return hd == 64 ? launch<rowstats_kernel<64>>(grid, 256, 0, st, (const bf*)o, (const bf*)d_o, lse, G, delta, lse2, S, L, Lp)
+                    : launch<rowstats_kernel<128>>(grid, 256, 0, st, (const bf*)o, (const bf*)d_o, lse, G, delta, lse2, S, L, Lp);
 }
 
 }  // namespace path

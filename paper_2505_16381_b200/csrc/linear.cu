@@ -7,17 +7,19 @@ namespace path {
 
 namespace {
 
-__global__ void pad_rows_kernel(const void* __restrict__ src, void* __restrict__ dst, int L, int Lp, int rowbytes16) {
+// Slices in a grid's second dimension, which ends at 65535: the kernels below walk on from there.
+constexpr int kMaxGridY = 65535;
+
+__global__ void pad_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int S, int L, int Lp, int rowbytes16) {
     grid_wait();
     grid_launch();
-    // one 16-byte vector per thread; grid.y = slice, grid.x covers Lp * rowbytes16
+    // one 16-byte vector per thread and slice; grid.x covers Lp * rowbytes16
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const long total = (long)Lp * rowbytes16;
     if (i >= total) return;
     const long row = i / rowbytes16, col = i % rowbytes16;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (row < L) v = ((const uint4*)src)[((long)blockIdx.y * L + row) * rowbytes16 + col];
-    ((uint4*)dst)[((long)blockIdx.y * Lp + row) * rowbytes16 + col] = v;
+    for (int s = blockIdx.y; s < S; s += gridDim.y)
+        dst[((long)s * Lp + row) * rowbytes16 + col] = row < L ? src[((long)s * L + row) * rowbytes16 + col] : make_uint4(0, 0, 0, 0);
 }
 
 // Sum of `x` over the threads before this one in a CTA of 1024; `total` = the sum over all of them.  Nothing is added and taken
@@ -297,16 +299,18 @@ __global__ void __launch_bounds__(256) cache_rows_kernel(const uint4* __restrict
 
 // ---- context-parallel path: gate terms of a segment, final result
 __global__ void cp_gate_kernel(const float* __restrict__ G, float* __restrict__ gq, float* __restrict__ gk,
-                               float* __restrict__ gtot, int L, int Lp) {
+                               float* __restrict__ gtot, int S, int L, int Lp) {
     grid_wait();
     grid_launch();
-    const int s = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
-    const float tot = G ? G[(size_t)s * Lp + L - 1] : 0.f;
-    if (i == 0) gtot[s] = tot;
-    if (i >= Lp) return;
-    const float g = G ? G[(size_t)s * Lp + i] : 0.f;
-    gq[(size_t)s * Lp + i] = i < L ? g : 0.f;
-    gk[(size_t)s * Lp + i] = i < L ? g - tot : 1e30f;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int s = blockIdx.y; s < S; s += gridDim.y) {
+        const float tot = G ? G[(size_t)s * Lp + L - 1] : 0.f;
+        if (i == 0) gtot[s] = tot;
+        if (i >= Lp) continue;
+        const float g = G ? G[(size_t)s * Lp + i] : 0.f;
+        gq[(size_t)s * Lp + i] = i < L ? g : 0.f;
+        gk[(size_t)s * Lp + i] = i < L ? g - tot : 1e30f;
+    }
 }
 // one thread per 4 outputs of a row
 __global__ void cp_finish_kernel(const float* __restrict__ o_acc, const float* __restrict__ lse_acc, __nv_bfloat16* __restrict__ o,
@@ -384,11 +388,11 @@ cudaError_t launch_clear(void* a, size_t na, void* b, size_t nb, void* c, size_t
     return launch<clear_kernel>((unsigned)(blocks < 1184 ? blocks : 1184), 256, 0, st, (uint32_t*)a, na, (uint32_t*)b, nb, (uint32_t*)c, nc);
 }
 
-cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, int f32, cudaStream_t st) {
-    const int rowbytes16 = d * (f32 ? 4 : 2) / 16;
+cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, cudaStream_t st) {
+    const int rowbytes16 = d * 2 / 16;
     const long total = (long)Lp * rowbytes16;
-    dim3 grid((unsigned)((total + 255) / 256), S);
-    return launch<pad_rows_kernel>(grid, 256, 0, st, src, dst, L, Lp, rowbytes16);
+    const dim3 grid((unsigned)((total + 255) / 256), S < kMaxGridY ? S : kMaxGridY);
+    return launch<pad_rows_kernel>(grid, 256, 0, st, (const uint4*)src, (uint4*)dst, S, L, Lp, rowbytes16);
 }
 
 cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, uint32_t* clear, cudaStream_t st) {
@@ -407,12 +411,12 @@ cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const 
 
 cudaError_t launch_cache_rows(const void* v, void* vc, const float* G, float* gc, int S, int L, int Lp, int cap, int hd, cudaStream_t st) {
     const long n16 = (long)L * hd / 8, cap16 = (long)cap * hd / 8;
-    const dim3 grid((unsigned)((n16 + 1023) / 1024), S < 65535 ? S : 65535);
+    const dim3 grid((unsigned)((n16 + 1023) / 1024), S < kMaxGridY ? S : kMaxGridY);
     return launch<cache_rows_kernel>(grid, 256, 0, st, (const uint4*)v, (uint4*)vc, G, gc, n16, cap16, L, Lp, cap, S);
 }
 
 cudaError_t launch_cp_gate(const float* G, float* gq, float* gk, float* gtot, int S, int L, int Lp, cudaStream_t st) {
-    return launch<cp_gate_kernel>(dim3((Lp + 255) / 256, S), 256, 0, st, G, gq, gk, gtot, L, Lp);
+    return launch<cp_gate_kernel>(dim3((Lp + 255) / 256, S < kMaxGridY ? S : kMaxGridY), 256, 0, st, G, gq, gk, gtot, S, L, Lp);
 }
 cudaError_t launch_cp_finish(const float* o_acc, const float* lse_acc, void* o, float* lse, size_t rows, int hd,
                              cudaStream_t st) {

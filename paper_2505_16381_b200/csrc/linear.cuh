@@ -5,8 +5,8 @@
 
 namespace path {
 
-// dst[S][Lp][d] <- src[S][L][d] (zero tail); bf16 elements when !f32.
-cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, int f32, cudaStream_t st);
+// dst[S][Lp][d] <- src[S][L][d], bf16 (zero tail).
+cudaError_t launch_pad_rows(const void* src, void* dst, int S, int L, int Lp, int d, cudaStream_t st);
 // G[S][Lp] <- inclusive prefix sum of g[S][L] (tail repeats the last value).  `clear` (or nullptr): 256 bytes to zero on the way.
 cudaError_t launch_gate_prefix(const float* g, float* G, int S, int L, int Lp, uint32_t* clear, cudaStream_t st);
 

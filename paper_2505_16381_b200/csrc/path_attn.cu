@@ -701,7 +701,7 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
     }
     // (a sweep reads the message's values in whole chunks)
     if (p.L == p.Lp) CK(cudaMemcpyAsync(at<void>(message, c.v), v, (size_t)p.S * p.Lp * d * 2, cudaMemcpyDeviceToDevice, st));
-    else LAUNCH(launch_pad_rows(v, at<void>(message, c.v), p.S, p.L, p.Lp, d, 0, st));
+    else LAUNCH(launch_pad_rows(v, at<void>(message, c.v), p.S, p.L, p.Lp, d, st));
     LAUNCH(launch_cp_gate(log_f ? at<float>(workspace, p.G) : nullptr, at<float>(state, c.gq), at<float>(message, c.gk),
                           at<float>(message, c.gtot), p.S, L, p.Lp, st));
     return PATH_OK;

@@ -751,3 +751,29 @@ def test_triangular_inverse_accuracy(binding, d, directions):
         bound = 2 ** -18 * norm(ref) + 2 * 2 ** -22 * bt.amax(-1) * sum(terms).sqrt()
         err = norm(T[:, c:c + 64, c:c + 64] - ref)
         assert (err <= bound).all(), ((err / norm(ref)).max().item(), (bound / norm(ref)).min().item())
+
+
+@pytest.mark.parametrize("gate", [False, True])
+def test_more_slices_than_a_grid_dimension(binding, gate):
+    """65540 short slices through the forward, the backward and a segment's preparation: the slices past 65535 get the bits that
+    they get alone."""
+    S, L, d = 65540, 3, 64
+    g = torch.Generator(device="cuda").manual_seed(81)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    q, k, v, d_o = (n(1, S, L, d).bfloat16() for _ in range(4))
+    w = torch.nn.functional.normalize(n(1, S, L, d), dim=-1).bfloat16()
+    beta = 2 * torch.sigmoid(n(1, S, L))
+    log_f = torch.nn.functional.logsigmoid(n(1, S, L) + 3) if gate else None
+    last = lambda x: None if x is None else x[:, -5:].clone()
+
+    def run(q, k, v, w, beta, log_f, d_o):
+        o, lse = binding.path_attn_fwd(q, k, v, w, beta, log_f)
+        out = dict(binding.path_attn_bwd(q, k, v, w, beta, o, lse, d_o, log_f), o=o, lse=lse)
+        state, _, _ = binding.path_attn_cp_prepare(q, k, v, w, beta, log_f)
+        out["seg_o"], out["seg_lse"] = binding.path_attn_cp_finish(state, *q.shape)
+        return out
+
+    ins = (q, k, v, w, beta, log_f, d_o)
+    full, one = run(*ins), run(*map(last, ins))
+    for name in one:
+        assert torch.equal(last(full[name]), one[name]), name
