@@ -3,6 +3,8 @@ rejects bad arguments on the host before touching the device."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -130,3 +132,24 @@ def test_product_path_has_no_oracle_or_cpu_fallback():
     for fn in ("binding.py", "build.py", "synth.py", "__init__.py"):
         src = open(os.path.join(ROOT, "paper_2505_16381_b200", fn)).read()
         assert "oracle" not in src.replace("the CPU oracle's tests", "").replace("CPU oracle", "") or fn == "synth.py"
+
+
+def test_import_and_planning_with_a_torch_without_cuda():
+    """torch built for CPU has no torch._C._cuda_*: the package imports, plans workspaces and refuses CPU tensors as ever."""
+    code = """
+import torch
+for name in [n for n in dir(torch._C) if n.startswith("_cuda_getCurrentRawStream") or n == "_cuda_getDevice"]:
+    delattr(torch._C, name)
+from paper_2505_16381_b200 import binding
+import paper_2505_16381_b200.autograd, paper_2505_16381_b200.ring
+assert binding.workspace_bytes(1, 2, 300, 64) > 0
+x = torch.zeros(1, 2, 300, 64, dtype=torch.bfloat16)
+try:
+    binding.path_attn_fwd(x, x, x, x, torch.zeros(1, 2, 300), workspace=torch.empty(1, dtype=torch.uint8))
+except RuntimeError as e:
+    assert "CUDA device" in str(e)
+else:
+    raise SystemExit("a CPU tensor was accepted")
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
