@@ -127,6 +127,8 @@ _get_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_d
 
 def _call(where, fn, device_index, *args):
     """``fn(*args, current stream of the device)`` with that device current; raises on a status other than PATH_OK."""
+    if device_index < 0:   # (torch takes -1 for the current device, and the kernels would be handed host pointers)
+        raise ValueError(f"{where}: expected tensors on a CUDA device")
     if _get_device() == device_index:
         rc = fn(*args, _raw_stream(device_index))
     else:

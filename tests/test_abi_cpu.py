@@ -153,3 +153,13 @@ else:
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
+
+
+def test_calls_without_tensor_checks_refuse_cpu_buffers(lib):
+    """A segment's state or a workspace on the CPU never reaches the library (its address would be a host address)."""
+    from paper_2505_16381_b200 import binding as b
+    state, message, ws = b.cp_alloc(1, 1, 128, 64, device="cpu")
+    for call in (lambda: b.path_attn_cp_step(state, message, 1, 1, 128, 128, 64, workspace=ws),
+                 lambda: b.path_attn_cp_finish(state, 1, 1, 128, 64), lambda: b.selftest_timeout(ws)):
+        with pytest.raises(ValueError, match="CUDA device"):
+            call()
