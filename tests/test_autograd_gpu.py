@@ -82,3 +82,25 @@ def test_wrappers_refuse_cpu_tensors():
     inp = synth.make_inputs(1, 1, 128, 64, "bf16", seed=1)
     with pytest.raises(Exception):
         path_attention(inp["q"], inp["k"], inp["v"], inp["w"], inp["beta"])
+
+
+class _NoGradient(torch.autograd.Function):
+    """A consumer whose backward passes an undefined gradient on."""
+
+    @staticmethod
+    def forward(ctx, x):
+        return x.sum()
+
+    @staticmethod
+    def backward(ctx, g):
+        return None
+
+
+@pytest.mark.parametrize("retain", [False, True])
+def test_undefined_upstream_gradient_is_zero(retain):
+    from paper_2505_16381_b200.autograd import path_attention
+    inp = synth.make_inputs(1, 2, 200, 64, "bf16", gate=True, seed=8300)
+    leaves = [inp[n].cuda().requires_grad_(True) for n in ("q", "k", "v", "w", "beta", "log_f")]
+    grads = torch.autograd.grad(_NoGradient.apply(path_attention(*leaves, retain_state=retain)), leaves)
+    for x, g in zip(leaves, grads):
+        assert g is not None and g.shape == x.shape and not g.any()
