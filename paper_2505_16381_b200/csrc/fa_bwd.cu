@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     if ((uint32_t)(smem - smem_raw) + kDkvTotal > kSmemAlloc) {   // uniform over the CTA
+        grid_wait();   // (the status word belongs to the kernels before)
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_DKV_PRODUCER);
         return;
     }
@@ -610,6 +611,7 @@ __global__ void __launch_bounds__(512, 1) dq_kernel(const __grid_constant__ BwdT
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     if ((uint32_t)(smem - smem_raw) + kDqTotal > kSmemAlloc) {   // uniform over the CTA
+        grid_wait();   // (the status word belongs to the kernels before)
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_DQ_PRODUCER);
         return;
     }
