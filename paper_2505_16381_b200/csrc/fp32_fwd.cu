@@ -6,15 +6,17 @@
 // t = W u0 (32 dot products at once),
 //     T = (I + C)^-1,  C_jm = beta_m w_j . w_m  (m > j),      Y = strictUpper(K W^T) D T
 //     logits of the block:  K u0 - Y t = (K - Y W) u0 = Kr u0,      u after the block:  u0 - ((D T)^T W)^T t = u0 - Wt^T t
-// Kr, Wt and Y belong to the keys alone: fp32_block_kernel makes them once per block.  A query's own block uses K, Y and t up to
-// the query.  Entries that the definition does not use are left out, not multiplied by zero: an infinity or NaN at one position
-// stays out of every row before it, as in the walk.
+// Kr, Wt and Y belong to the keys alone: fp32_block_kernel makes them once per block.  A query's own block uses K, Y and t with
+// the entries after the query set to zero.
+//
+// Blocks with a NaN or an infinity, in k, v, w, beta or in what is made of them, are walked key by key: products with zeros
+// would carry it into rows before its position, and sums in another order turn an infinite logit, which the definition handles
+// (minus infinity has no weight), into a NaN.  fp32_block_kernel marks them.
 //
 // fp32_fwd_kernel: a warp owns RW queries of one block, lane j the block's key j: two dot products per lane with rows from
 // shared memory (u0 broadcast), then the lanes turn to the head dimension for the update of u and for P V.  What bounds it
 // at the sizes it is for (a few slices, a few hundred tokens) is the chain of dependent phases of one block, L / 32 times.
-// B=1, H=2, L=256, d=64: 69.7 -> 21.0 us per call (one key per step: 520 cycles each).
-#include <type_traits>
+// B=1, H=2, L=256, d=64: 69.7 -> 20.8 us per call (one key per step: 520 cycles each).
 #include "common.cuh"
 
 namespace path {
@@ -32,11 +34,12 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b) {
 }
 
 // ---------------------------------------------------------------------------------------------- per block of keys
-// grid = (blocks, S), 256 threads.  kr, wt: [S][nblk * 32][HD], ym: [S][nblk * 32][32].
+// grid = (blocks, S), 256 threads.  kr, wt: [S][nblk * 32][HD], ym: [S][nblk * 32][32], odd: [S][nblk].
 template <int HD>
 __global__ void __launch_bounds__(256) fp32_block_kernel(const float* __restrict__ k, const float* __restrict__ w,
-                                                         const float* __restrict__ beta, float* __restrict__ kr,
-                                                         float* __restrict__ wt, float* __restrict__ ym, uint32_t* clear, int L) {
+                                                         const float* __restrict__ beta, const float* __restrict__ v,
+                                                         float* __restrict__ kr, float* __restrict__ wt, float* __restrict__ ym,
+                                                         int* __restrict__ odd, uint32_t* clear, int L) {
     grid_wait();
     grid_launch();
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 64) clear[threadIdx.x] = 0u;   // the workspace's status block
@@ -47,10 +50,13 @@ __global__ void __launch_bounds__(256) fp32_block_kernel(const float* __restrict
     const int row = tid >> 3, part = tid & 7;
     const bool live = blk * kBlk + row < L;
     const size_t src = ((size_t)s * L + blk * kBlk + row) * HD, dst = ((size_t)s * nblk + blk) * kBlk + row;
+    float zero = 0.f;   // 0, or NaN if anything in this block is not finite
+    auto look = [&](const float4& x) { zero = fmaf(x.x, 0.f, fmaf(x.y, 0.f, fmaf(x.z, 0.f, fmaf(x.w, 0.f, zero)))); };
 #pragma unroll
     for (int c = 0; c < HD / 32; ++c) {
         const int e = c * 32 + part * 4;
         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        look(live ? *reinterpret_cast<const float4*>(v + src + e) : z);
         *reinterpret_cast<float4*>(&sw[row][e]) = live ? *reinterpret_cast<const float4*>(w + src + e) : z;
         *reinterpret_cast<float4*>(&sk[row][e]) = live ? *reinterpret_cast<const float4*>(k + src + e) : z;
     }
@@ -72,7 +78,7 @@ __global__ void __launch_bounds__(256) fp32_block_kernel(const float* __restrict
         for (int x = 0; x < 4; ++x) {
             const int m = part + 8 * x;
             sc[m][row] = m > row ? sb[m] * a[x] : 0.f;   // (C transposed: the substitution goes column by column)
-            skw[row][m] = b[x];
+            skw[row][m] = m > row ? b[x] : 0.f;
         }
     }
     __syncthreads();
@@ -83,54 +89,52 @@ __global__ void __launch_bounds__(256) fp32_block_kernel(const float* __restrict
 #pragma unroll
         for (int j = kBlk - 1; j > 0; --j)
 #pragma unroll
-            for (int i = 0; i < j; ++i) x[i] = j <= tid ? fmaf(-sc[j][i], x[j], x[i]) : x[i];
+            for (int i = 0; i < j; ++i) x[i] = fmaf(-sc[j][i], x[j], x[i]);
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < kBlk; ++j) sc[j][tid] = j <= tid ? sb[j] * x[j] : 0.f;
+        for (int j = 0; j < kBlk; ++j) sc[j][tid] = sb[j] * x[j];
     }
     __syncthreads();
-    const int r4 = row & ~3;             // the warp's rows are r4 .. r4 + 3
-    float y[4] = {0.f, 0.f, 0.f, 0.f};   // Y[row][4 part ..]: over row < p <= column
-#pragma unroll 4
-    for (int p = r4; p < kBlk; ++p) {
+    float y[4] = {0.f, 0.f, 0.f, 0.f};   // Y[row][4 part ..]
+#pragma unroll 8
+    for (int p = 0; p < kBlk; ++p) {
         const float c = skw[row][p];
         const float4 d4 = *reinterpret_cast<const float4*>(&sc[p][4 * part]);
-        const int last = p > row ? 4 * part : -8;
-        y[0] = p <= last ? fmaf(c, d4.x, y[0]) : y[0];
-        y[1] = p <= last + 1 ? fmaf(c, d4.y, y[1]) : y[1];
-        y[2] = p <= last + 2 ? fmaf(c, d4.z, y[2]) : y[2];
-        y[3] = p <= last + 3 ? fmaf(c, d4.w, y[3]) : y[3];
+        y[0] = fmaf(c, d4.x, y[0]); y[1] = fmaf(c, d4.y, y[1]); y[2] = fmaf(c, d4.z, y[2]); y[3] = fmaf(c, d4.w, y[3]);
     }
     *reinterpret_cast<float4*>(ym + dst * kBlk + 4 * part) = make_float4(y[0], y[1], y[2], y[3]);
+    look(make_float4(y[0], y[1], y[2], y[3]));
     __syncthreads();
     *reinterpret_cast<float4*>(&skw[row][4 * part]) = make_float4(y[0], y[1], y[2], y[3]);
     __syncthreads();
     float ok[HD / 8], ow[HD / 8];
 #pragma unroll
     for (int c = 0; c < HD / 8; ++c) { ok[c] = sk[row][(c >> 2) * 32 + part * 4 + (c & 3)]; ow[c] = 0.f; }
-    // Kr takes the keys after the row, Wt those up to it
-    auto add = [&](float (&out)[HD / 8], const float x, const int m) {
+#pragma unroll 4
+    for (int m = 0; m < kBlk; ++m) {
+        const float cy = skw[row][m], ct = sc[m][row];
 #pragma unroll
         for (int c = 0; c < HD / 32; ++c) {
             const float4 wm = *reinterpret_cast<const float4*>(&sw[m][c * 32 + part * 4]);
-            out[4 * c] = fmaf(x, wm.x, out[4 * c]); out[4 * c + 1] = fmaf(x, wm.y, out[4 * c + 1]);
-            out[4 * c + 2] = fmaf(x, wm.z, out[4 * c + 2]); out[4 * c + 3] = fmaf(x, wm.w, out[4 * c + 3]);
-        }
-    };
-#pragma unroll 4
-    for (int m = 0; m < r4; ++m) add(ow, sc[m][row], m);
+            const float t[4] = {wm.x, wm.y, wm.z, wm.w};
 #pragma unroll
-    for (int m = r4; m < r4 + 4; ++m) {
-        if (m > row) add(ok, -skw[row][m], m);
-        else add(ow, sc[m][row], m);
+            for (int x = 0; x < 4; ++x) {
+                ok[4 * c + x] = fmaf(-cy, t[x], ok[4 * c + x]);
+                ow[4 * c + x] = fmaf(ct, t[x], ow[4 * c + x]);
+            }
+        }
     }
-#pragma unroll 4
-    for (int m = r4 + 4; m < kBlk; ++m) add(ok, -skw[row][m], m);
 #pragma unroll
     for (int c = 0; c < HD / 32; ++c) {
-        *reinterpret_cast<float4*>(kr + dst * HD + c * 32 + part * 4) = make_float4(ok[4 * c], ok[4 * c + 1], ok[4 * c + 2], ok[4 * c + 3]);
-        *reinterpret_cast<float4*>(wt + dst * HD + c * 32 + part * 4) = make_float4(ow[4 * c], ow[4 * c + 1], ow[4 * c + 2], ow[4 * c + 3]);
+        const float4 a = make_float4(ok[4 * c], ok[4 * c + 1], ok[4 * c + 2], ok[4 * c + 3]);
+        const float4 b = make_float4(ow[4 * c], ow[4 * c + 1], ow[4 * c + 2], ow[4 * c + 3]);
+        *reinterpret_cast<float4*>(kr + dst * HD + c * 32 + part * 4) = a;
+        *reinterpret_cast<float4*>(wt + dst * HD + c * 32 + part * 4) = b;
+        look(a);
+        look(b);
     }
+    const int any = __syncthreads_or(!(zero == 0.f));
+    if (tid == 0) odd[(size_t)s * nblk + blk] = any;
 }
 
 // ---------------------------------------------------------------------------------------------- queries
@@ -142,8 +146,9 @@ __device__ __forceinline__ void cp16(float* dst, const float* src, bool live) { 
 template <int HD, int RW>
 __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __restrict__ q, const float* __restrict__ k,
                                                                const float* __restrict__ v, const float* __restrict__ w,
-                                                               const float* __restrict__ kr, const float* __restrict__ wt,
-                                                               const float* __restrict__ ym, const float* __restrict__ G,
+                                                               const float* __restrict__ beta, const float* __restrict__ kr,
+                                                               const float* __restrict__ wt, const float* __restrict__ ym,
+                                                               const int* __restrict__ odd, const float* __restrict__ G,
                                                                float* __restrict__ o, float* __restrict__ lse, int S, int L,
                                                                int ldG, float scale) {
     grid_wait();
@@ -175,6 +180,7 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     request(nb, 0);
+    const int* odds = odd + (size_t)s * nblk;
     float acc[RW][E], m[RW], l[RW], Gi[RW];
     int i[RW];
 #pragma unroll
@@ -189,11 +195,52 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
         Gi[r] = G && i[r] < L ? G[(size_t)s * ldG + i[r]] : 0.f;
     }
     __syncwarp();
-    auto step = [&](auto own_tag, const int n) {
-        // The block of the warp's own queries runs once and is kept short: as long as the others it costs 5 % at d = 128 (97 us for
-        // 4 x 512 positions, 93 like this) in instruction fetch.
-        constexpr bool own = decltype(own_tag)::value;
+    // Query r over block n, one key after the other, as fp32_walk_kernel does it (the lanes over the head dimension).
+    auto walk = [&](const int r_, const int n) {
+        const int last = min(n == nb ? nb * kBlk + r0 + r_ : n * kBlk + kBlk - 1, L - 1);
+        float* u = su + r_ * HD;
+#pragma unroll 1
+        for (int j = last; j >= n * kBlk; --j) {
+            const size_t at = ((size_t)s * L + j) * HD + lane;
+            float a = 0.f, t = 0.f, ww[E], vv[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                ww[e] = w[at + e * 32];
+                vv[e] = v[at + e * 32];
+                a = fmaf(u[e * 32 + lane], k[at + e * 32], a);
+                t = fmaf(u[e * 32 + lane], ww[e], t);
+            }
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, off);
+                t += __shfl_xor_sync(0xffffffffu, t, off);
+            }
+            const float bt = beta[(size_t)s * L + j] * t, Gj = G ? G[(size_t)s * ldG + j] : 0.f;
+#pragma unroll
+            for (int r = 0; r < RW; ++r)
+                if (r == r_) {   // (registers: the index has to be a constant)
+                    const float sc = fmaf(scale, a, Gi[r] - Gj);
+                    if (sc > m[r]) {
+                        const float c = expf(m[r] - sc);
+                        l[r] *= c;
+#pragma unroll
+                        for (int e = 0; e < E; ++e) acc[r][e] *= c;
+                        m[r] = sc;
+                    }
+                    const float pj = expf(sc - m[r]);
+                    if (lane == 0) l[r] += pj;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) acc[r][e] = fmaf(pj, vv[e], acc[r][e]);
+                }
+#pragma unroll
+            for (int e = 0; e < E; ++e) u[e * 32 + lane] = fmaf(-bt, ww[e], u[e * 32 + lane]);
+        }
+        __syncwarp();
+    };
+#pragma unroll 1
+    for (int n = nb; n >= 0; --n) {
         const int stage = (nb - n) & 1;
+        const bool own = n == nb;
         if (n > 0) {
             request(n - 1, stage ^ 1);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -202,14 +249,21 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
         }
         const int key = n * kBlk + lane;
         const float Gj = G && key < L ? G[(size_t)s * ldG + key] : 0.f;
+        const int walked = odds[n];
         __syncthreads();
+        if (walked) {   // (the whole CTA)
+#pragma unroll 1
+            for (int r = 0; r < RW; ++r) walk(r, n);
+            __syncthreads();
+            continue;
+        }
         const float* tw = sm + stage * 4 * TILE + lane * LD;
         float t[RW][4], a[RW][4];
 #pragma unroll
         for (int r = 0; r < RW; ++r)
 #pragma unroll
             for (int x = 0; x < 4; ++x) t[r][x] = a[r][x] = 0.f;
-#pragma unroll (own ? 2 : 8)
+#pragma unroll 8
         for (int e = 0; e < HD; e += 4) {
             const float4 w4 = *reinterpret_cast<const float4*>(tw + e), k4 = *reinterpret_cast<const float4*>(tw + TILE + e);
 #pragma unroll
@@ -229,22 +283,13 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
             lg[r] = (a[r][0] + a[r][1]) + (a[r][2] + a[r][3]);
         }
         __syncwarp();
-        if constexpr (own) {   // logits of the own block: K q - Y t
+        if (own) {   // logits of the own block: K q - Y t
             const float4* yr = reinterpret_cast<const float4*>(ym + (((size_t)s * nblk + n) * kBlk + lane) * kBlk);
 #pragma unroll
             for (int c = 0; c < kBlk / 4; ++c) {
                 const float4 y4 = yr[c];
-                const float y[4] = {y4.x, y4.y, y4.z, y4.w};
 #pragma unroll
-                for (int r = 0; r < RW; ++r) {
-                    const float4 t4 = *reinterpret_cast<const float4*>(st + r * kBlk + 4 * c);
-                    const float tt[4] = {t4.x, t4.y, t4.z, t4.w};
-                    float d = 0.f;
-#pragma unroll
-                    for (int x = 0; x < 4; ++x)
-                        if (4 * c + x > lane && 4 * c + x <= r0 + r) d = fmaf(y[x], tt[x], d);
-                    lg[r] -= d;
-                }
+                for (int r = 0; r < RW; ++r) lg[r] -= dot4(y4, *reinterpret_cast<const float4*>(st + r * kBlk + 4 * c));
             }
         }
 #pragma unroll
@@ -269,8 +314,8 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
 #pragma unroll
             for (int e = 0; e < E; ++e) du[r][e] = 0.f;
         const float* cw = sm + stage * 4 * TILE + 2 * TILE + lane;
-#pragma unroll (own ? 1 : 4)
-        for (int j = 0; j < (own ? (r0 + RW + 3) & ~3 : kBlk); j += 4) {
+#pragma unroll 4
+        for (int j = 0; j < kBlk; j += 4) {
             float4 t4[RW], p4[RW];
 #pragma unroll
             for (int r = 0; r < RW; ++r) {
@@ -286,7 +331,6 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
                     for (int r = 0; r < RW; ++r) {
                         const float tj = y == 0 ? t4[r].x : y == 1 ? t4[r].y : y == 2 ? t4[r].z : t4[r].w;
                         const float pj = y == 0 ? p4[r].x : y == 1 ? p4[r].y : y == 2 ? p4[r].z : p4[r].w;
-                        if (own && j + y > r0 + r) continue;
                         du[r][e] = fmaf(tj, ww, du[r][e]);
                         acc[r][e] = fmaf(pj, vv, acc[r][e]);
                     }
@@ -297,10 +341,7 @@ __global__ void __launch_bounds__(32 * kWarps) fp32_fwd_kernel(const float* __re
 #pragma unroll
             for (int e = 0; e < E; ++e) su[r * HD + e * 32 + lane] -= du[r][e];
         __syncthreads();   // everyone is done with this stage's tiles
-    };
-    step(std::true_type{}, nb);
-#pragma unroll 1
-    for (int n = nb - 1; n >= 0; --n) step(std::false_type{}, n);
+    }
 #pragma unroll
     for (int r = 0; r < RW; ++r) {
 #pragma unroll
@@ -405,12 +446,13 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) fp32_walk_kernel(const float
 }
 
 template <int HD, int RW>
-cudaError_t launch_rows(const float* q, const float* k, const float* v, const float* w, const float* kr, const float* wt,
-                        const float* ym, const float* G, float* o, float* lse, int S, int L, int ldG, float scale, cudaStream_t st) {
+cudaError_t launch_rows(const float* q, const float* k, const float* v, const float* w, const float* beta, const float* kr, const float* wt,
+                        const float* ym, const int* odd, const float* G, float* o, float* lse, int S, int L, int ldG, float scale,
+                        cudaStream_t st) {
     const int smem = (8 * kBlk * ld<HD>() + kWarps * RW * (HD + 2 * kBlk)) * 4;
     const int nblk = (L + kBlk - 1) / kBlk;
-    return launch<fp32_fwd_kernel<HD, RW>>((unsigned)((size_t)S * nblk * (kBlk / (kWarps * RW))), 32 * kWarps, smem, st, q, k, v, w, kr,
-                                           wt, ym, G, o, lse, S, L, ldG, scale);
+    return launch<fp32_fwd_kernel<HD, RW>>((unsigned)((size_t)S * nblk * (kBlk / (kWarps * RW))), 32 * kWarps, smem, st, q, k, v, w, beta,
+                                           kr, wt, ym, odd, G, o, lse, S, L, ldG, scale);
 }
 
 template <int HD>
@@ -420,23 +462,24 @@ cudaError_t launch_hd(const float* q, const float* k, const float* v, const floa
     float* kr = scratch;
     float* wt = kr + rows * HD;
     float* ym = wt + rows * HD;
+    int* odd = reinterpret_cast<int*>(ym + rows * kBlk);
     for (int s0 = 0; s0 < S; s0 += 65535) {   // (a grid's second dimension ends there)
         const int ns = S - s0 < 65535 ? S - s0 : 65535;
         const size_t in = (size_t)s0 * L, out = (size_t)s0 * nblk * kBlk;
-        const cudaError_t e = launch<fp32_block_kernel<HD>>(dim3((unsigned)nblk, ns), 256, 0, st, k + in * HD, w + in * HD, beta + in,
-                                                            kr + out * HD, wt + out * HD, ym + out * kBlk, s0 == 0 ? clear : nullptr, L);
+        const cudaError_t e = launch<fp32_block_kernel<HD>>(dim3((unsigned)nblk, ns), 256, 0, st, k + in * HD, w + in * HD, beta + in, v + in * HD,
+                                                            kr + out * HD, wt + out * HD, ym + out * kBlk, odd + (size_t)s0 * nblk, s0 == 0 ? clear : nullptr, L);
         if (e != cudaSuccess) return e;
     }
     // One query per warp while that still leaves SMs without work; four share a warp's tile reads otherwise.
-    if (rows <= 148 * 4 * 4) return launch_rows<HD, 1>(q, k, v, w, kr, wt, ym, G, o, lse, S, L, ldG, scale, st);
-    return launch_rows<HD, 4>(q, k, v, w, kr, wt, ym, G, o, lse, S, L, ldG, scale, st);
+    if (rows <= 148 * 4 * 4) return launch_rows<HD, 1>(q, k, v, w, beta, kr, wt, ym, odd, G, o, lse, S, L, ldG, scale, st);
+    return launch_rows<HD, 4>(q, k, v, w, beta, kr, wt, ym, odd, G, o, lse, S, L, ldG, scale, st);
 }
 
 }  // namespace
 
 size_t fp32_scratch_bytes(int S, int L, int hd) {
     const size_t rows = (size_t)S * ((L + kBlk - 1) / kBlk) * kBlk;
-    return rows * (2 * hd + kBlk) * sizeof(float);
+    return (rows * (2 * hd + kBlk) + rows / kBlk) * sizeof(float);
 }
 
 cudaError_t launch_fp32_fwd(const float* q, const float* k, const float* v, const float* w, const float* beta, const float* G,
