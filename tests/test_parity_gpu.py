@@ -803,3 +803,18 @@ def test_float32_infinities_as_in_the_walk(binding, name, value, S, d):
     both = torch.isfinite(o1)
     assert (o[both] - o1[both]).norm() <= 1e-5 * o1[both].norm()
     assert (lse[fin] - lse1[fin]).abs().max() <= 2e-5 * max(1.0, lse1[fin].abs().max().item())
+
+
+@pytest.mark.parametrize("d,gate", [(64, False), (64, True), (128, False), (128, True)])
+@pytest.mark.parametrize("p", [0, 40, 128, 300])
+def test_dv_of_keys_after_a_nan_row(binding, d, gate, p):
+    """A NaN query at position p makes its own row and the gradients of the keys it attends to NaN: dv of the keys after p, which
+    the causal mask keeps from it, is what it was (equal to the bit)."""
+    dev = to_dev(synth.make_inputs(1, 3, 330, d, "bf16", gate=gate, seed=91))
+    ins = lambda: [dev[n] for n in ("q", "k", "v", "w", "beta")]
+    run = lambda: binding.path_attn_bwd(*ins(), *binding.path_attn_fwd(*ins(), dev["log_f"]), dev["d_o"], dev["log_f"])["dv"]
+    g0 = run()
+    dev["q"][:, :, p] = float("nan")
+    g = run()
+    assert torch.equal(g[:, :, p + 1:], g0[:, :, p + 1:])
+    assert torch.isnan(g[:, :, :p + 1]).all()
