@@ -191,7 +191,7 @@ def test_backward_rounds_across_items(binding, B, H, L, d, gate):
     full = grads((slice(None), slice(None)))
     for b, h in ((0, 0), (B // 2, H // 2), (B - 1, H - 1)):
         one = grads((slice(b, b + 1), slice(h, h + 1)))
-        for name in ("dq", "dk", "dv", "dw"):
+        for name in one:   # (dlog_f among them when gated: the row sums that items pass on through shared buffers)
             assert torch.isfinite(full[name]).all() and torch.equal(full[name][b, h], one[name][0, 0]), (name, b, h)
 
 
