@@ -21,6 +21,11 @@ namespace {
 
 constexpr int kWarps = 8, kSlots = 3 * 148, kMinKeys = 64, kMaxSplits = 96;
 
+// The number of SMs is a constant here because the workspace query, which needs no device, has to come to the same answer.
+// The merge counts on every range but the last having a position (an empty state would be a NaN in it): for one of n ranges over t
+// positions to stay empty, (n - 2) ceil(t / n) >= t, n would have to exceed 2 ceil(t / n), and ceil(t / n) is at least kMinKeys - 1.
+static_assert(kMaxSplits <= 2 * kMinKeys - 2, "a range could be empty");
+
 // CTAs per slice for n positions: one wave of the GPU (three CTAs per SM), ranges of at least 64 positions and no more states
 // than the merge reads quickly (2 heads x 20000 tokens, d = 128: 29 us with 222 states, 24 with 79).  Long ranges are cut in
 // four: with 2500 positions per CTA the wave's end is ragged (32 heads x 32768 x 128: 230 us, 220 with 600 per CTA), with

@@ -39,30 +39,6 @@ constexpr uint32_t kPanelBytes = 16384;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr uint32_t kSmemAlloc = 232448;   // everything an SM offers one CTA
 
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// Two-wide float arithmetic on register pairs.
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
     uint64_t d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -81,13 +57,6 @@ __device__ __forceinline__ void store_acc_bf16(__nv_bfloat16* dst, uint32_t tcol
         for (int x = 0; x < 16; ++x) w[x] = pack_bf16(__uint_as_float(r[2 * x]) * mul, __uint_as_float(r[2 * x + 1]) * mul);
         tile::gstore_bf16_w16(dst + c * 32, w);
     }
-}
-
-// Plain (untiled) bulk copy global -> shared, completion counted in bytes on `bar`; 16-byte aligned, size % 16 == 0.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
 }
 
 // D[tmem] (+)= A B^T with both operands K-major [rows][kdim] tiles (two 64-column panels per 128 of kdim).  Descriptors
@@ -113,11 +82,8 @@ __device__ __forceinline__ void mma_tn(uint32_t d_tmem, uint32_t a_col, uint32_t
     }
 }
 
-__device__ __forceinline__ void tma_tile(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int kdim, int row0) {
-    for (int h = 0; h < kdim / 64; ++h) tma_load_2d(dst + h * kPanelBytes, m, bar, h * 64, row0);
-}
-
 using tile::tma_rows;
+using tile::tma_tile;
 
 // ------------------------------------------------------------------------------------------------ dK, dV
 // Persistent: the work items (one key chunk of one slice each) are listed slice after slice as pairs (longest,
@@ -479,12 +445,12 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
                 mbar_arrive(&bars[K_ACCFREE]);
                 break;
             }
-            auto zero_dk = [&](int slot) {
+            auto zero_dk = [&]() {
                 uint4* dst = reinterpret_cast<uint4*>(p.dkv + ((size_t)row0(J) + row) * HD + h * CW);
                 for (int x = 0; x < CW / 8; ++x) dst[x] = make_uint4(0u, 0u, 0u, 0u);
             };
             if (T > 1) flush_dk(level(T - 1));
-            else zero_dk(0);   // no later query chunk met: the boundary-adjusted keys get a zero gradient from the sweep
+            else zero_dk();   // no later query chunk met: the boundary-adjusted keys get a zero gradient from the sweep
             // (levels that a sweep shortened by block skipping did not reach stay unwritten: the version chain rule starts
             // at the highest level reached)
             if (CW == 64) {   // 64 bf16 = one 128-byte line per row: coalesced exchange

@@ -470,7 +470,9 @@ cudaError_t launch_hd(const float* q, const float* k, const float* v, const floa
                                                             kr + out * HD, wt + out * HD, ym + out * kBlk, odd + (size_t)s0 * nblk, s0 == 0 ? clear : nullptr, L);
         if (e != cudaSuccess) return e;
     }
-    // One query per warp while that still leaves SMs without work; four share a warp's tile reads otherwise.
+    // One query per warp for few rows, four that share a warp's tile reads otherwise.  us with one / with four (slices x positions x
+    // d): 2 x 256 x 64 20 / 25, 4 x 448 x 64 49 / 42, 4 x 592 x 64 62 / 63, 8 x 512 x 64 78 / 62; 2 x 256 x 128 32 / 53,
+    // 4 x 448 x 128 88 / 89, 4 x 592 x 128 134 / 121, 8 x 512 x 128 184 / 106.  The line lies at four rows per warp of every SM.
     if (rows <= 148 * 4 * 4) return launch_rows<HD, 1>(q, k, v, w, beta, kr, wt, ym, odd, G, o, lse, S, L, ldG, scale, st);
     return launch_rows<HD, 4>(q, k, v, w, beta, kr, wt, ym, odd, G, o, lse, S, L, ldG, scale, st);
 }

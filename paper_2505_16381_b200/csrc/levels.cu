@@ -323,9 +323,11 @@ __device__ __forceinline__ int version_at(int is_key, int ch, int e, int N, int 
 // With p.edge_q / p.edge_k the chains go on to the sequence's start / end (context-parallel path, paper Sec. 3.5: queries
 // pulled back to the start of the segment, keys advanced to its end, bf16 [S][Lp][d]): at most about 2 log2(N) products per
 // chunk, all chunks at once.  What goes on from step to step is then a bf16 pair in tensor memory, a version and what it
-// lacks: rounded to bf16 at every step, as the versions are, the keys at the end of a segment of 8 chunks with unit w of four directions and beta = 2 were 2.9e-3
-// off (2.3e-3 with the pair, which leaves the first tile's and the last rounding; outputs of sharp attention 8.3e-3 against 7.5e-3).  (Walking the chunks one after the other per slice took 105 us for the two sides of 64 slices of
-// 8 chunks at d = 128, on top of this kernel's 23; the extended chains take 49 in all, and the product of the segment comes from the run products.)
+// lacks: rounded to bf16 at every step, as the versions are, the keys at the end of a segment of 8 chunks with unit w of four
+// directions and beta = 2 were 2.9e-3 off (2.3e-3 with the pair, which leaves the first tile's and the last rounding; outputs of
+// sharp attention 8.3e-3 against 7.5e-3).  (Walking the chunks one after the other per slice took 105 us for the two sides of
+// 64 slices of 8 chunks at d = 128, on top of this kernel's 23; the extended chains take 49 in all, and the product of the
+// segment comes from the run products.)
 template <int HD, bool EDGE>
 __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int is_key = blockIdx.y, s = blockIdx.x / p.N, ch = blockIdx.x % p.N;

@@ -1,5 +1,5 @@
-// Memory-bound helpers: zero-padding of ragged inputs, prefix sum of the log gate (PaTH-FoX, paper Sec. 2.2),
-// suffix sum of its gradient, block skipping.
+// Memory-bound helpers: prefix sum of the log gate (PaTH-FoX, paper Sec. 2.2) and suffix sum of its gradient, block skipping,
+// decoding cache and segment buffers (copies, gate terms, padding), the forward-state record, clearing.
 #include "linear.cuh"
 #include "tc5.cuh"
 
@@ -384,7 +384,7 @@ cudaError_t launch_gate_suffix(const float* dGa, const float* dGb, const float* 
 }
 
 cudaError_t launch_clear(void* a, size_t na, void* b, size_t nb, void* c, size_t nc, cudaStream_t st) {
-    const size_t blocks = (na + nb + nc + 1023) / 1024;
+    const size_t blocks = (na + nb + nc + 1023) / 1024;   // (at most about eight per SM: the rest is the loop's)
     return launch<clear_kernel>((unsigned)(blocks < 1184 ? blocks : 1184), 256, 0, st, (uint32_t*)a, na, (uint32_t*)b, nb, (uint32_t*)c, nc);
 }
 

@@ -1,5 +1,5 @@
 // C-ABI entry points of the PaTH attention library: argument validation, workspace planning, tensor-map
-// encoding and the launch sequence.  All arithmetic runs in the kernels of linear.cu / fa_fwd.cu / fa_bwd.cu.
+// encoding and the launch sequence.  All arithmetic runs in the kernels of the other files of this folder.
 #include "../../include/path_attn.h"
 
 #include <cstdio>
@@ -231,8 +231,9 @@ static LevelParams level_params(const Plan& p, void* ws) {
     return lp;
 }
 
-// Gated problems: which chunk pairs the sweeps can leave out (counts per query chunk and per key chunk, three small
-// kernels; the status block's pair counters are zero on entry).  Runs before the chunk preparation: the version chains stop at the highest level a kept pair uses.
+// Gated problems: which chunk pairs the sweeps can leave out (counts per query chunk and per key chunk, two small
+// kernels; the status block's pair counters are zero on entry).  Runs before the chunk preparation: the version chains stop
+// at the highest level a kept pair uses.
 static int run_gate_skip(const Plan& p, void* ws, const void* q, const void* k, const void* w, const float* beta, float scale,
                          cudaStream_t st) {
     LAUNCH(launch_gate_skip(q, k, w, beta, at<float>(ws, p.G), at<float>(ws, p.tstats), at<int>(ws, p.nkeep),
@@ -686,7 +687,7 @@ int path_attn_cp_prepare(const void* q, const void* k, const void* v, const void
         FwdParams fp{};
         fp.o = at<float>(state, c.o_acc); fp.lse = at<float>(state, c.lse_acc); fp.G = log_f ? at<float>(workspace, p.G) : nullptr;
         fp.status = at<uint32_t>(workspace, p.status);
-    fp.next_item = at<int>(workspace, p.status + kNextItemOffset);
+        fp.next_item = at<int>(workspace, p.status + kNextItemOffset);
         fp.S = p.S; fp.L = L; fp.Lp = p.Lp; fp.N = p.N; fp.scale = scale; fp.out_fp32 = 1; fp.vl = p.vl;
         if (log_f) fp.nkeep = at<int>(workspace, p.nkeep);
         LAUNCH(launch_fa_fwd(tm, fp, d, st));
@@ -861,7 +862,8 @@ static int run_gemm(const void* a, int a_mn, const void* b, int b_mn, void* c, i
     GemmParams gp{};
     gp.M = Mo; gp.N = No; gp.K = K; gp.a_mn = a_mn; gp.b_mn = b_mn; gp.c = c; gp.ldc = No; gp.c_atomic = c_atomic; gp.status = status;
     int split = 1;
-    if (c_atomic) {   // weight gradients: few output tiles, a contraction over all tokens: spread it over about two waves of CTAs
+    // weight gradients: few output tiles, a contraction over all tokens: spread it over about one wave of two CTAs per SM
+    if (c_atomic) {
         const int tiles = ((Mo + 127) / 128) * ((No + 127) / 128), stages = (K + 63) / 64;
         split = 296 / tiles;
         split = split < 1 ? 1 : (split > stages ? stages : split);
