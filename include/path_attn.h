@@ -45,8 +45,10 @@ extern "C" {
 
 /* I/O dtype of q, k, v, w, o and their gradients.
  * PATH_BF16: bf16 tensor-core products with float32 accumulation (the training path, forward and backward).
- * PATH_FP32: forward only; the definition of Sec. 2.2 evaluated in float32 on the CUDA cores (one warp per query
- * position carrying u <- H_j u over the keys), O(L^2 d) work: an accuracy path for float32 tensors, not a fast one.
+ * PATH_FP32: forward only; the definition of Sec. 2.2 evaluated in float32 on the CUDA cores (a warp carries u <- H_j u
+ * for one or four query positions, 32 keys at a time; one key at a time over keys that are not finite, or if the
+ * workspace holds less than path_attn_workspace_bytes), O(L^2 d) work: an accuracy path for float32 tensors, not a
+ * fast one.
  * path_attn_bwd and for_backward = 1 do not accept it. */
 typedef enum { PATH_BF16 = 0, PATH_FP32 = 1 } path_dtype_t;
 

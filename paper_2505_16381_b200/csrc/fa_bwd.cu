@@ -1427,8 +1427,9 @@ cudaError_t launch_one(const BwdTensorMaps& tm, const BwdParams& p, int which, c
     const cudaError_t e = sm_count(sms);
     if (e != cudaSuccess) return e;
     const int pairs = (p.N * p.S + 1) / 2, grid = pairs < sms ? pairs : sms;
-    // dK/dV sweep, us, dkv64_kernel / dkv_kernel: 8 x 16 x 2048 x 64 226 / 275, 4 x 32 x 4096 x 64 742 / 950; gated, its further
-    // live values and passes cost more than the rounds give (2 x 8 x 3001 x 64: 75 / 68)
+    // dK/dV sweep, us, dkv64_kernel / dkv_kernel: 8 x 16 x 2048 x 64 226 / 275, 4 x 32 x 4096 x 64 742 / 950 (taken with the mask in
+    // the logits, see mask_pt: 3 % more now); gated, its further live values and passes cost more than the rounds give (2 x 8 x
+    // 3001 x 64: 75 / 68)
     if constexpr (HD == 64 && !GATE) {
         if (which == 0) return launch<dkv64_kernel>(grid, 512, kD64Total + 1024, st, tm, p);
     } else {
