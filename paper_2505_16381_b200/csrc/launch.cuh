@@ -59,7 +59,9 @@ cudaError_t launch(dim3 grid, unsigned block, size_t smem, cudaStream_t st, cons
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, KERN, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, KERN, args...);
+    if (e != cudaSuccess) (void)cudaGetLastError();   // reported by the return code; the host's next CUDA call must not find it
+    return e;
 }
 
 }  // namespace path
