@@ -3,7 +3,7 @@
 //
 // With W, Q, K the rows of one 128-token chunk and D = diag(beta):
 //   Gm = W W^T,  Xq = lower(Q W^T),  Xk = strictLower(W K^T)
-//   T~ = (I + strictLower(D Gm))^-1 D        (16 x 16 blocks by float32 substitution, merged by warp-level products: tri_inverse)
+//   T~ = (I + strictLower(D Gm))^-1 D        (see invert_diagonal)
 //   U = T~ W,  Y = T~ Xk
 //   Qleft = Q - Xq U,  Kright = K - Y^T W,  P = I - W^T U
 // Xq and Y are also the bf16 operands of the diagonal-chunk correction -Xq Y of the attention sweep.
@@ -14,18 +14,21 @@
 // are read back one row per thread.  T~ is kept as a bf16 pair (hi + lo) because everything downstream
 // depends on it; the other intermediates are rounded to bf16 once, like the tiles the attention sweep consumes.
 //
-// The kernel is persistent: one CTA per SM walks over chunks.  Eight worker warps do the element-wise work (the
-// triangular inverse, accumulator read-outs, conversions); one lane of a ninth warp issues the TMA loads and stores and
-// every product as soon as its operands are published, so the products run underneath the workers' next phase and the
-// first product of the next chunk is already finished when the workers get there.  Every result leaves by a TMA store from
-// the tile that the workers have written anyway (or write for that): no worker touches global memory but for beta.
+// The kernel is persistent: one CTA per SM walks over chunks, and two chunks are in work at a time.  Eight warps compute the
+// triangular inverse of a chunk while eight others still turn the accumulators of the chunk before into operands and results.  One
+// thread issues the products as soon as their operands are published, one the two products inside the inverse, one requests and
+// stores tiles.  They meet at mbarriers only.  Every result leaves by a TMA store from the tile that the workers have written anyway
+// (or write for that): no worker touches global memory but for beta.
 //
-// What bounds it: the chain of dependent phases of one chunk (its seven tiles and four accumulators fill the SM, so there is
-// one chunk per SM at a time) and, in the backward's instance, bursts of stores: 416 KB per chunk against about 23 bytes per
-// cycle and SM of memory bandwidth.  Cycles per chunk at B=4, H=16, L=4096, d=128 (backward's instance) / 32 x 32768 x 128
-// (forward's): 29 k / 25 k, of which the inverse 9.7 k, 116 product steps 7.5 k (mostly underneath), E1 1.9 k, Xk and Xq
-// 3 k, U and Y 1.8 k, P, Q<- and K-> 3.9 k, the rest waits.  With the inverse in float32 loops plus one tcgen05 level and
-// rows stored and fetched by the workers: 43.5 k / 33.9 k.  Time 352 -> 243 us and 1240 -> 940 us; 128 x 2048 x 64: 278 -> 206.
+// What bounds it.  d = 64: the inverse, about 17 k cycles per chunk, of which its merges take 7 k (mma.sync shares the tensor pipe
+// with the products: 2.6 k when nothing else runs).  d = 128: shared memory, which moves about 2 MB per chunk (operand reads of the
+// products 1 MB, tiles in and out 0.4, the workers 0.6) = 16 k of 20 k cycles.  Both streams of code together have to fit the
+// instruction caches as well: warps went without instructions for 2.3 cycles per issue until the operand group was one loop, 0.7
+// since.  Times, before with one group of warps and one chunk at a time / now: B = 2, H = 16, L = 8192, d = 128, forward's instance
+// 220 / 180 us, backward's 238 / 195; 32 x 32768 x 128 928 / 750; 128 x 2048 x 64 185 / 166 and 199 / 180.
+// Tried: 32 x 32 blocks by substitution and a merge in float32 arithmetic (rows broadcast from shared memory: 4.3 k and 5.7 k
+// cycles, the loads' 128 bytes per cycle bound them); T~ from tensor memory at d = 128 too (Gm of the next chunk has to be ready
+// before T~: its W arrives too late, 750 -> 880 us).
 #include <type_traits>
 #include "tileops.cuh"
 
@@ -36,23 +39,25 @@ namespace {
 
 using namespace tile;
 
-// Seven 32 KB tile slots.  0: W.  1, 2: N hi, lo -> (I + N)^-1 -> T~ -> U -> Q, K once more.  3: K -> Xq hi -> P lo.
-// 4: Q -> Xq lo -> P hi.  5: Xk hi -> Y hi -> Q<-.  6: Xk lo -> Y lo -> K->.  The four results of a chunk wait in slots 3 - 6
-// for their TMA stores to read them while the next chunk's triangular inverse runs in slots 1, 2 and in registers; its Q and K
-// arrive meanwhile.
+// Seven 32 KB tile slots.  0: W.  1, 2: N -> T~ (hi, lo).  3, 4: Xk -> Y (hi, lo) -> Q, K once more -> Q<-, K->.  5, 6: Q, K ->
+// the next chunk's W (5) and Xq hi for its store (6) -> U (hi, lo) -> P (hi, lo).  At d = 64 a tile of the head dimension takes one
+// 16 KB panel: slot 0 holds the W of two chunks by turns, slot 5 the pair of Xq's panels, then U, then P, slot 6 Q and K.
 struct PrepSmem {
     static constexpr uint32_t offBar = 7 * kTileB;
-    static constexpr uint32_t offBeta = offBar + 256;                                      // [128] float
-    static constexpr uint32_t total = offBeta + kT * 4;
+    static constexpr uint32_t offBeta = offBar + 256;                                      // [2][128] float
+    static constexpr uint32_t total = offBeta + 2 * kT * 4;
     static constexpr uint32_t alloc = total + 1024;
 };
 
-// mbarriers.  Issuer -> workers: one per group of products (and the TMA load, which only the issuer waits for).
-// Workers -> issuer (256 arrivals): operands published / accumulators drained.  Each completes once per chunk.
-enum { B_LOAD = 0, B_LOADQK, B_GM, B_XQK, B_U, B_Y, B_G3A, B_G3B, B_ST, B_LOADR, R_TT, R_XK, R_XQ, R_U, R_Y, R_P, R_E3, B_COUNT };
-constexpr int kWorkers = 256, kThreads = 384;   // warps 8..11: the issuer's warpgroup (one active lane)
+// mbarriers, each completing once per chunk.  L_*: tiles have arrived.  M_*: a group of products has retired.  S_*: stores have
+// read their tiles, which may be written again.  R_*: workers (256 arrivals) have published operands or drained accumulators.
+enum { L_W = 0, L_QK, L_WN, L_ROW, M_GM, M_IX, M_IT, M_XQK, M_U, M_Y, M_GA, M_GB, S_T, S_XQ, S_XK, S_U, S_E3,
+       R_GM, R_ID, R_IX, R_TT, R_XQ, R_XK, R_U, R_Y, R_P, R_E3, B_COUNT };
+static_assert(B_COUNT * 8 + 8 <= 256, "");
+constexpr int kWorkers = 256;               // per group: warps 0 - 7 invert, warps 8 - 15 turn accumulators into operands and results
+constexpr int kThreads = 640;               // one thread each of warp 16: issues products, 17: moves tiles, 18: products of the inverse
 
-// Barriers over the eight worker warps.  bar.sync / bar.red are warp-aligned instructions: a warp whose lanes left a
+// Barriers over the eight warps that invert.  bar.sync / bar.red are warp-aligned instructions: a warp whose lanes left a
 // loop at different times must reconverge first, or the part that runs ahead is taken for the whole warp.
 __device__ __forceinline__ void wsync() {
     __syncwarp();
@@ -62,64 +67,25 @@ __device__ __forceinline__ bool wsync_and(bool ok) { return barrier_and<1, 256>(
 
 // ------------------------------------------------------------------------------------------------ triangular inverse
 // In place in the two slots of a bf16 pair of swizzled tiles (aH, aL):  N strictly lower -> T~ = (I + N)^-1 D.  The two 64 x 64
-// diagonal blocks of N arrive in float32, in the 16 KB that their pair takes up later (fel below); the 64 x 64 block C under the
-// diagonal as a pair, and zeros above it.  16 x 16 diagonal blocks by float32 forward substitution, then three merge levels
-// [[A,0],[C,B]]^-1 = [[A^-1,0],[-B^-1 C A^-1, B^-1]]  of 16-, 32- and 64-row blocks as warp-level products.  A warp owns a
-// 16-row strip of B^-1 C: its accumulators are the A fragments of the second product, so nothing goes through memory in between.
+// diagonal blocks of N arrive in float32, in the 16 KB that their pair takes up later (fel below); the 64 x 64 block C under them
+// as a pair, and zeros above.  16 x 16 diagonal blocks by float32 forward substitution, two float32 merges
+// [[A,0],[C,B]]^-1 = [[A^-1,0],[-B^-1 C A^-1, B^-1]]  to 64 rows, and the last merge by two
+// products of the tensor unit on bf16 pairs.  The columns are scaled by D in float32, before they become the pair that T~ is kept in.
 //
 // Precision.  The first two levels read and write float32, their products split every operand into two tf32 numbers (mma.sync
-// m16n8k8, lo x lo left out: 2^-22 of a product).  The last level takes bf16 pairs (m16n8k16), the form T~ is kept in
-// afterwards, and the blocks on the diagonal are scaled by D in float32 before they become one.  Relative error of T~ against
-// float64 over 128 chunks, d = 64 / 128, with N and all levels in bf16 pairs -> like this, which is what float32 loops for
-// the first two levels give (rounding the exact T~ to a pair: 2.3e-6): random unit w 5.1e-6 / 3.8e-6 -> 4.0e-6 / 3.2e-6; beta = 2
-// and w around one direction 1.7e-4 / 1.6e-4 -> 8.4e-5 / 8.2e-5; beta = 2 and four directions 7.7e-5 / 6.2e-5 -> 1.5e-5 / 1.5e-5.
-//
-// Time: 9.7 thousand cycles (substitution 2.0, merges 0.9, 2.2, 3.3, the change to pairs 0.7, scaling 0.6), 8 with pairs throughout;
-// float32 loops up to 64 rows plus one tcgen05 level took 14.  The merges are bound by the rate of mma.sync, about 20 cycles
-// each and scheduler for either shape (dependent products in three separate accumulators changed nothing).
-// Why not tcgen05: its smallest tile has 64 rows and every product costs a round trip through tensor memory, a shared
-// memory tile and two hand-overs (about 1500 cycles each, measured); here the blocks are 16 to 64 rows and dependent.
-__device__ __forceinline__ uint32_t frag_addr(uint32_t tile_, int r0, int c0, int lane) {
-    const int rr = r0 + (lane & 15), c = c0 + (lane >> 4) * 8;
-    return tile_ + (uint32_t)(c >> 6) * kPanelB + sw128_off((uint32_t)rr, (uint32_t)((c & 63) >> 3));
-}
-__device__ __forceinline__ void ldsm4(uint32_t (&f)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void ldsm4t(uint32_t (&f)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
+// m16n8k8, lo x lo left out: 2^-22 of a product).  The last level takes pairs of the blocks not yet scaled (their diagonals are
+// exact then).  Relative error of T~ against float64, 512 chunks, d = 64 / 128: random unit w 4.0e-6 / 3.2e-6 (rounding
+// the exact T~ to a pair: 2.3e-6); beta = 2 and w around one direction 8.3e-5 / 8.3e-5; beta = 2 and four directions 1.6e-5 / 1.5e-5.
+// (With T_A, T_B, the scaled blocks, as the last level's operands: 4.9e-6 / 3.9e-6 for random w.)
 __device__ __forceinline__ void mma1688(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// d[16 x 16] += (ah + al) (bh + bl) without al bl
-__device__ __forceinline__ void mma_pair(float (&d)[2][4], const uint32_t (&ah)[4], const uint32_t (&al)[4], const uint32_t (&bh)[4],
-                                         const uint32_t (&bl)[4]) {
-#pragma unroll
-    for (int n = 0; n < 2; ++n) mma16816(d[n], ah, bh[2 * n], bh[2 * n + 1]);
-#pragma unroll
-    for (int n = 0; n < 2; ++n) mma16816(d[n], ah, bl[2 * n], bl[2 * n + 1]);
-#pragma unroll
-    for (int n = 0; n < 2; ++n) mma16816(d[n], al, bh[2 * n], bh[2 * n + 1]);
-}
-__device__ __forceinline__ uint32_t split_pair(float a, float b, uint32_t& l) {   // packed hi, l = packed lo
-    const uint32_t h = pack_bf16(a, b);
-    l = pack_bf16(a - __uint_as_float(h << 16), b - __uint_as_float(h & 0xffff0000u));
-    return h;
-}
-// hi (x cut off), l = lo (the rest, rounded: 11 + 11 bits and a sign).  Plain integer operations: cvt.rna.tf32 took 4 % longer.
+// hi (x cut off), l = lo (the rest, rounded: 11 + 11 bits and a sign; the product cuts off what lies below them).
 __device__ __forceinline__ uint32_t split_tf32(float x, uint32_t& l) {
     const uint32_t h = __float_as_uint(x) & 0xffffe000u;
-    l = (__float_as_uint(x - __uint_as_float(h)) + 0x1000u) & 0xffffe000u;
+    l = __float_as_uint(x - __uint_as_float(h)) + 0x1000u;
     return h;
 }
 // Element (r, c) of the float32 diagonal block b (64 x 64): rows 0 - 31 where the block's hi tile goes later, rows 32 - 63 at its lo
@@ -146,14 +112,28 @@ __device__ __forceinline__ Tf32A tf32_a(const float (&d)[4]) {
     a.h[2] = split_tf32(d[1], a.l[2]); a.h[3] = split_tf32(d[3], a.l[3]);
     return a;
 }
-// d[16 x 8] += A B, B the 8 x 8 block at (r0, c0)
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const Tf32A& a, uint8_t* aH, uint8_t* aL, int b, int r0, int c0, int lane) {
-    uint32_t h[2], l[2];
+// d[16 x 8 T] += A B, B the 8 x 8 T block at (r0, c0)
+template <int T>
+__device__ __forceinline__ void mma_tf32(float (&d)[T][4], const Tf32A& a, uint8_t* aH, uint8_t* aL, int b, int r0, int c0, int lane) {
+    uint32_t h[T][2], l[T][2];
 #pragma unroll
-    for (int x = 0; x < 2; ++x) h[x] = split_tf32(*fel(aH, aL, b, r0 + 2 * (lane & 3) + x, c0 + (lane >> 2)), l[x]);
-    mma1688(d, a.h, h[0], h[1]);
-    mma1688(d, a.h, l[0], l[1]);
-    mma1688(d, a.l, h[0], h[1]);
+    for (int n = 0; n < T; ++n)
+#pragma unroll
+        for (int x = 0; x < 2; ++x) h[n][x] = split_tf32(*fel(aH, aL, b, r0 + 2 * (lane & 3) + x, c0 + n * 8 + (lane >> 2)), l[n][x]);
+#pragma unroll
+    for (int n = 0; n < T; ++n) mma1688(d[n], a.h, h[n][0], h[n][1]);
+#pragma unroll
+    for (int n = 0; n < T; ++n) mma1688(d[n], a.h, l[n][0], l[n][1]);
+#pragma unroll
+    for (int n = 0; n < T; ++n) mma1688(d[n], a.l, h[n][0], h[n][1]);
+}
+// x *= the 32 entries of D at bt
+__device__ __forceinline__ void scale32(float (&x)[32], const float* bt) {
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) {
+        const float4 b = *reinterpret_cast<const float4*>(bt + i);
+        x[i] *= b.x; x[i + 1] *= b.y; x[i + 2] *= b.z; x[i + 3] *= b.w;
+    }
 }
 // One merge level of blocks of NBK 16-row strips (1, 2) inside the float32 blocks.  NBK = 1: four pairs, the two warps of a pair take
 // 8 columns of the result each; NBK = 2: a warp takes 16 x 16, the two warps that share a scheduler (w, w + 4) a long and a
@@ -172,27 +152,22 @@ __device__ __forceinline__ void merge_f32(uint8_t* aH, uint8_t* aL, int warp, in
         for (int x = 0; x < 8; ++x) p1[k][x >> 2][x & 3] = 0.f;
 #pragma unroll
     for (int x = 0; x < 4 * NT; ++x) m[x >> 2][x & 3] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < 16 * (rb + 1); j += 8) {
+        const Tf32A a = tf32_a(aH, aL, b, row0, base_b + j, lane);
 #pragma unroll
-    for (int j = 0; j < NBK; ++j)
-#pragma unroll
-        for (int k8 = 0; k8 < 2; ++k8) {
-            if (j > rb) continue;
-            const Tf32A a = tf32_a(aH, aL, b, row0, base_b + j * 16 + k8 * 8, lane);
-#pragma unroll
-            for (int kb = 0; kb < NBK; ++kb) {
-                if (kb < k_lo) continue;
-#pragma unroll
-                for (int n = 0; n < 2; ++n) mma_tf32(p1[kb][n], a, aH, aL, b, base_b + j * 16 + k8 * 8, base_a + kb * 16 + n * 8, lane);
-            }
+        for (int kb = 0; kb < NBK; ++kb) {
+            if (kb < k_lo) continue;
+            mma_tf32(p1[kb], a, aH, aL, b, base_b + j, base_a + kb * 16, lane);
         }
+    }
 #pragma unroll
     for (int kb = 0; kb < NBK; ++kb) {
         if (kb < k_lo) continue;
 #pragma unroll
         for (int k8 = 0; k8 < 2; ++k8) {
             const Tf32A a = tf32_a(p1[kb][k8]);
-#pragma unroll
-            for (int n = 0; n < NT; ++n) mma_tf32(m[n], a, aH, aL, b, base_a + kb * 16 + k8 * 8, col0 + n * 8, lane);
+            mma_tf32(m, a, aH, aL, b, base_a + kb * 16 + k8 * 8, col0, lane);
         }
     }
     wsync();   // the other warps of the pair read C as well
@@ -203,107 +178,48 @@ __device__ __forceinline__ void merge_f32(uint8_t* aH, uint8_t* aL, int warp, in
             *reinterpret_cast<float2*>(fel(aH, aL, b, row0 + (lane >> 2) + 8 * y, col0 + n * 8 + 2 * (lane & 3))) =
                 make_float2(-m[n][2 * y], -m[n][2 * y + 1]);
 }
-// The last level, on the pairs: strips of 64 x 64 blocks, the result scaled by D.
-__device__ __forceinline__ void merge_pairs(uint8_t* aH, uint8_t* aL, const float* bt, int warp, int lane) {
-    constexpr int NBK = 4, CBN = 2;               // 16-row strips per block, 16-column blocks of the result per warp
-    const uint32_t tH = smem_u32(aH), tL = smem_u32(aL);
-    const int hw = warp >> 2, w4 = warp & 3, rb = hw ? 3 - w4 : w4, cb0 = hw * CBN, row0 = 64 + rb * 16;
-    float m[CBN][2][4], p1[NBK][2][4];
+// 16 x 16 diagonal blocks: half a warp each, a lane owns a column of the inverse and reads the rows all lanes of its half need.
+__device__ __forceinline__ void substitute16(uint8_t* aH, uint8_t* aL, int warp, int lane) {
+    const int o = (warp & 1) * 32 + (lane & 16), j = lane & 15;
+    uint8_t* rows = (warp & 1 ? aL : aH) + (warp >> 1) * (kPanelB + 8192) + (lane & 16) * 256;
+    uint8_t* at[2] = {rows + o * 4, rows + (o ^ 16) * 4};
+    auto piece = [&](int r, int c4) {   // fel for these rows, 16 bytes from column o + 4 c4 on
+        const int f = (((r & 3) ^ ((r >> 2) & 1)) << 3) | (r & 4);
+        return at[(f >> 4) & 1] + r * 256 + ((4 * c4) ^ (f & 12)) * 4;
+    };
+    float x[16];
 #pragma unroll
-    for (int k = 0; k < NBK; ++k)
+    for (int r = 0; r < 16; ++r) {
+        uint64_t acc[2] = {0ull, 0ull};
+        ulonglong2 f{};
 #pragma unroll
-        for (int x = 0; x < 8; ++x) p1[k][x >> 2][x & 3] = 0.f;
-#pragma unroll
-    for (int k = 0; k < CBN; ++k)
-#pragma unroll
-        for (int x = 0; x < 8; ++x) m[k][x >> 2][x & 3] = 0.f;
-#pragma unroll 1
-    for (int j = 0; j <= rb; ++j) {
-        uint32_t ah[4], al[4];
-        ldsm4(ah, frag_addr(tH, row0, 64 + j * 16, lane));
-        ldsm4(al, frag_addr(tL, row0, 64 + j * 16, lane));
-#pragma unroll
-        for (int kb = 0; kb < NBK; ++kb) {
-            if (kb < cb0) continue;       // A^-1 is lower triangular: columns cb0.. need no earlier block
-            uint32_t bh[4], bl[4];
-            ldsm4t(bh, frag_addr(tH, 64 + j * 16, kb * 16, lane));
-            ldsm4t(bl, frag_addr(tL, 64 + j * 16, kb * 16, lane));
-            mma_pair(p1[kb], ah, al, bh, bl);
+        for (int c = 0; c < (r + 3) / 4; ++c) {
+            f = *reinterpret_cast<const ulonglong2*>(piece(r, c));
+            if (4 * c + 1 < r) acc[0] = fma2(f.x, pack2(x[4 * c], x[4 * c + 1]), acc[0]);
+            if (4 * c + 3 < r) acc[1] = fma2(f.y, pack2(x[4 * c + 2], x[4 * c + 3]), acc[1]);
         }
+        float s0, s1, last = 0.f;
+        unpack2(r >= 4 ? add2(acc[0], acc[1]) : acc[0], s0, s1);
+        if (r & 1) {   // the last of an odd number of entries
+            float hi;
+            unpack2(r & 2 ? f.y : f.x, last, hi);
+            last *= x[r - 1];
+        }
+        const float sum = (s0 + s1) + last;
+        x[r] = r > j ? -sum : r == j ? 1.f : 0.f;
     }
+    __syncwarp();
 #pragma unroll
-    for (int kb = 0; kb < NBK; ++kb) {
-        if (kb < cb0) continue;
-        uint32_t ah[4], al[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) ah[x] = split_pair(p1[kb][x >> 1][(x & 1) * 2], p1[kb][x >> 1][(x & 1) * 2 + 1], al[x]);
-#pragma unroll
-        for (int i = 0; i < CBN; ++i) {
-            if (kb < cb0 + i) continue;
-            uint32_t bh[4], bl[4];
-            ldsm4t(bh, frag_addr(tH, kb * 16, (cb0 + i) * 16, lane));
-            ldsm4t(bl, frag_addr(tL, kb * 16, (cb0 + i) * 16, lane));
-            mma_pair(m[i], ah, al, bh, bl);
-        }
-    }
-    wsync();   // the other strips read C as well
-#pragma unroll
-    for (int i = 0; i < CBN; ++i)
-#pragma unroll
-        for (int n = 0; n < 2; ++n) {
-            const int col = (cb0 + i) * 16 + n * 8 + 2 * (lane & 3);
-            const float s0 = -bt[col], s1 = -bt[col + 1];
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-                const int rr = row0 + (lane >> 2) + 8 * y;
-                uint32_t l;
-                const uint32_t h = split_pair(s0 * m[i][n][2 * y], s1 * m[i][n][2 * y + 1], l);
-                const uint32_t off = (uint32_t)(col >> 6) * kPanelB + sw128_off((uint32_t)rr, (uint32_t)((col & 63) >> 3)) + (col & 7) * 2;
-                *reinterpret_cast<uint32_t*>(aH + off) = h;
-                *reinterpret_cast<uint32_t*>(aL + off) = l;
-            }
-        }
+    for (int r = 0; r < 16; ++r) *reinterpret_cast<float*>(piece(r, j >> 2) + (j & 3) * 4) = x[r];
 }
-__device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const float* bt, int warp, int lane, int row, int half) {
-    {   // diagonal block `warp`: lane j (and its copy j + 16) keeps column j in registers
-        const int b = warp >> 2, o = (warp & 3) * 16, j = lane & 15;
-        float x[16];
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {   // four rows at a time: their loads are issued together, ahead of the dependent sums
-            float4 f[4][4];
-#pragma unroll
-            for (int y = 0; y < 4; ++y)
-#pragma unroll
-                for (int c = 0; c <= g; ++c) f[y][c] = *reinterpret_cast<const float4*>(fel(aH, aL, b, o + 4 * g + y, o + 4 * c));
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const int rr = 4 * g + y;
-                float acc[4] = {rr == j ? 1.f : 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int c = 0; c < g; ++c) {
-                    acc[0] -= f[y][c].x * x[4 * c];
-                    acc[1] -= f[y][c].y * x[4 * c + 1];
-                    acc[2] -= f[y][c].z * x[4 * c + 2];
-                    acc[3] -= f[y][c].w * x[4 * c + 3];
-                }
-                float a = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-                if (y > 0) a -= f[y][g].x * x[4 * g];
-                if (y > 1) a -= f[y][g].y * x[4 * g + 1];
-                if (y > 2) a -= f[y][g].z * x[4 * g + 2];
-                x[rr] = rr >= j ? a : 0.f;
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) *fel(aH, aL, b, o + rr + (lane >> 4) * 8, o + j) = lane < 16 ? x[rr] : x[rr + 8];
-    }
+// The 64 x 64 diagonal blocks of N -> their inverses, as pairs and (d: this thread's 32 entries of a row) scaled by D in float32.
+__device__ __forceinline__ void invert_diagonal(uint8_t* aH, uint8_t* aL, const float* bt, int warp, int lane, int row, int half, float (&d)[32]) {
+    if (warp < 4) substitute16(aH, aL, warp, lane);
     wsync();
     merge_f32<1>(aH, aL, warp, lane);
     wsync();
     merge_f32<2>(aH, aL, warp, lane);
     wsync();
-    // the diagonal blocks become pairs, in the same place; this thread's 32 entries stay in registers until they are scaled
-    float d[32];
     const int cb = (row & 64) + half * 32;
 #pragma unroll
     for (int x = 0; x < 32; x += 4) {
@@ -315,16 +231,7 @@ __device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const floa
     split32(d, hi, lo);
     tile_store_w16(aH, row, cb, hi);
     tile_store_w16(aL, row, cb, lo);
-    wsync();
-    merge_pairs(aH, aL, bt, warp, lane);   // (from its barrier on nobody reads the diagonal blocks any more)
-#pragma unroll
-    for (int x = 0; x < 32; x += 4) {
-        const float4 v = *reinterpret_cast<const float4*>(bt + cb + x);
-        d[x] *= v.x; d[x + 1] *= v.y; d[x + 2] *= v.z; d[x + 3] *= v.w;
-    }
-    split32(d, hi, lo);
-    tile_store_w16(aH, row, cb, hi);
-    tile_store_w16(aL, row, cb, lo);
+    scale32(d, bt + cb);
 }
 
 // MODE: PREP_FWD = everything the forward needs; PREP_SAVE = also keeps the tiles of the chain rule (the backward's instance);
@@ -333,22 +240,27 @@ __device__ __forceinline__ void tri_inverse(uint8_t* aH, uint8_t* aL, const floa
 template <int HD, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_constant__ PrepTensorMaps tm, const PrepParams p,
                                                                       const int nchunks) {
-    constexpr bool SAVE = MODE == PREP_SAVE, KEYS = MODE == PREP_KEYS;
+    constexpr bool SAVE = MODE == PREP_SAVE, KEYS = MODE == PREP_KEYS, D64 = HD == 64;
+    // T~ as an operand: at d = 64 from tensor memory, so that the next inverse can have its tiles while U and Y are computed.  It lies
+    // where the next Gm was, which has to be ready by then: at d = 128 its W comes too late for that.
+    constexpr bool TMT = D64;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     auto slot = [&](int i) { return smem + i * kTileB; };
-    uint8_t* sW = slot(0);
-    float* bt = (float*)(smem + PrepSmem::offBeta);
+    // tiles of the head dimension in slots 5, 6
+    constexpr uint32_t oU = 5 * kTileB, oUlo = oU + (D64 ? kPanelB : kTileB);            // U, then P: hi, lo
+    constexpr uint32_t oQ = (D64 ? 6 : 5) * kTileB, oK = oQ + (D64 ? kPanelB : kTileB);  // Q, K of the chunk
+    constexpr uint32_t oXq = (D64 ? 5 : 6) * kTileB;                                      // Xq hi, for its store
+    float* betas = (float*)(smem + PrepSmem::offBeta);   // of this chunk and the next, by turns
     uint64_t* bars = (uint64_t*)(smem + PrepSmem::offBar);
     uint32_t* tmem_slot = (uint32_t*)(bars + B_COUNT);
     volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row = (warp & 3) * 32 + lane;       // accumulator row (TMEM lane) of a worker thread
-    const int half = (warp >> 2) & 1;             // which half of the accumulator's columns
+    const int half = (warp >> 2) & 1;             // which half of an accumulator's columns a worker thread has
 
     if (tid == 0) {
-        for (int i = 0; i < B_COUNT; ++i) mbar_init(&bars[i], i >= R_TT ? (uint32_t)kWorkers : 1u);
+        for (int i = 0; i < B_COUNT; ++i) mbar_init(&bars[i], i >= R_GM ? (uint32_t)kWorkers : 1u);
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -357,10 +269,10 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         const int pos = (chunk_ % p.N) * kT + tid;
         return pos < p.L ? p.beta[(size_t)(chunk_ / p.N) * p.L + pos] : 0.f;
     };
-    if (HD == 64) {  // second panel of W must read as zeros when W^T is used with M = 128
-        for (int i = tid; i < (int)(kPanelB / 16); i += kThreads) reinterpret_cast<uint4*>(sW + kPanelB)[i] = make_uint4(0, 0, 0, 0);
-        fence_proxy_async_smem();
-    }
+    // the block of T~ above the diagonal blocks stays zero: nothing is ever written there
+    for (int i = tid; i < 1024; i += kThreads)
+        reinterpret_cast<uint4*>(slot(1 + (i >> 9)) + kPanelB)[i & 511] = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -368,314 +280,441 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
     grid_wait();
     grid_launch();
     if (p.clear && blockIdx.x == 0 && tid < 64) p.status[tid] = 0u;   // the workspace's status block (256 bytes)
-    if (tid < kT && (int)blockIdx.x < nchunks) bt[tid] = beta_floor(beta_of(blockIdx.x));
+    if (tid < kT && (int)blockIdx.x < nchunks) betas[tid] = beta_floor(beta_of(blockIdx.x));
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t base_ = smem_u32(smem);
     constexpr int KS = HD / 16;  // k-steps over the head dimension
-    // tensor-memory columns:  0: Gm -> U   128: Xq -> W^T U   256: Xk -> Xq U   384: Y -> Y^T W
+    // Tensor-memory columns.  0: the next chunk's Gm, then (TMT) the pair T~, then Xq U.  128: Xq, then its pair.  256 and 384, changing places from
+    // chunk to chunk: Xk -> Y -> Y^T W, and the inverse's two products -> U -> W^T U.
+    constexpr uint32_t cG = 0, cXq = 128;
+    auto col_x = [](uint32_t it) { return 256u + (it & 1) * 128u; };
+    auto col_u = [](uint32_t it) { return 384u - (it & 1) * 128u; };
 
-    if (warp >= kWorkers / 32) {
-        // ------------------------------------------------------------------ issuer
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
-        if (warp == kWorkers / 32 && elect_one()) {
-            auto wait = [&](int b, uint32_t par) { return mbar_wait(&bars[b], par, abort_flag, ST_PREP); };
-            auto fetch = [&](const CUtensorMap* m, int i, int b, int chunk_) {
-                tma_rows(slot(i), m, &bars[b], HD, (chunk_ % p.N) * kT, chunk_ / p.N);
-            };
-            auto load_w = [&](int chunk_) {
-                mbar_expect_tx(&bars[B_LOAD], kT * HD * 2);
-                fetch(&tm.w, 0, B_LOAD, chunk_);
-            };
-            auto load_qk = [&](int chunk_) {
-                mbar_expect_tx(&bars[B_LOADQK], (KEYS ? 1 : 2) * kT * HD * 2);
-                if (!KEYS) fetch(&tm.q, 4, B_LOADQK, chunk_);
-                fetch(&tm.k, 3, B_LOADQK, chunk_);
-            };
-            auto store = [&](const CUtensorMap* m, int i, int ncols, int row0) {
-                for (int h = 0; h < ncols / 64; ++h) tma_store_2d(m, slot(i) + h * kPanelB, h * 64, row0);
-            };
-            int chunk = blockIdx.x;
-            bool ok = chunk < nchunks;
-            if (ok) {
-                load_w(chunk);
-                load_qk(chunk);
-                ok = wait(B_LOAD, 0);
-                if (ok) {
-                    tc_fence_after_sync();
-                    mma<OP_K, OP_K, KS, 128>(tmem + 0, base_, base_, false);
-                    umma_commit(&bars[B_GM]);
-                }
+    if (warp >= 2 * kWorkers / 32) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");   // 128 x 72 + 256 x 128 + 256 x 72 = 60416 of the 640 x 96
+        auto wait = [&](int b, uint32_t par) { return mbar_wait(&bars[b], par, abort_flag, ST_PREP); };
+        if (warp == 16 && elect_one()) {
+            // -------------------------------------------------------------- products
+            bool ok = (int)blockIdx.x < nchunks;
+            if (ok && (ok = wait(L_W, 0))) {
+                tc_fence_after_sync();
+                mma<OP_K, OP_K, KS, 128>(tmem + cG, base_, base_, false);
+                umma_commit(&bars[M_GM]);
             }
-            for (uint32_t it = 0; ok && chunk < nchunks; ++it, chunk += gridDim.x) {
+            for (uint32_t it = 0, chunk = blockIdx.x; ok && (int)chunk < nchunks; ++it, chunk += gridDim.x) {
                 const uint32_t par = it & 1;
-                const int r0 = chunk * kT, next = chunk + (int)gridDim.x;
+                const bool more = (int)(chunk + gridDim.x) < nchunks;
                 // (the tiles' address is made opaque once per chunk: otherwise every descriptor of every product is
                 // hoisted out of this loop and the thread's small register allotment spills)
                 uint32_t a0 = base_;
                 asm volatile("" : "+r"(a0));
                 auto t = [&](int i) { return a0 + i * kTileB; };
-                // Xq, Xk: their columns' previous contents have been read (R_P, R_E3 at the end of the previous chunk)
-                if (!(ok = wait(B_LOADQK, par))) break;
+                const uint32_t w = a0 + (D64 ? par * kPanelB : 0u);
+                const uint32_t cx = tmem + col_x(it), cu = tmem + col_u(it);
+                // Xq, Xk: P of the chunk before has been read, and with it the columns that Xk takes
+                if (!D64 && it > 0 && !(ok = wait(L_W, par))) break;
+                if (!(ok = wait(L_QK, par))) break;
+                if (it > 0 && !(ok = wait(R_P, par ^ 1))) break;
                 tc_fence_after_sync();
-                if (!KEYS) mma<OP_K, OP_K, KS, 128>(tmem + 128, t(4), t(0), false);
-                mma<OP_K, OP_K, KS, 128>(tmem + 256, t(0), t(3), false);
-                tma_store_wait_read();   // the previous chunk's Q<- and K-> tiles: Xk goes over them
-                umma_commit(&bars[B_XQK]);
-                // U = T~ W  (lo x lo terms are dropped everywhere).  In the backward's instance the tiles kept for the chain
-                // rule leave through TMA stores, straight from the operand slots.
+                if (!KEYS) mma<OP_K, OP_K, KS, 128>(tmem + cXq, a0 + oQ, w, false);
+                mma<OP_K, OP_K, KS, 128>(cx, w, a0 + oK, false);
+                umma_commit(&bars[M_XQK]);
+                // The next chunk's Gm runs underneath this chunk's inverse; what its columns held has been read: Xq U for Q<- (or the
+                // first Gm).  (K-> has been read as well, and with it the columns that U takes.)
+                if (more && !(ok = wait(L_WN, par))) break;
+                if (it > 0 && !(ok = wait(R_E3, par ^ 1))) break;
+                if ((!TMT || it == 0) && !(ok = wait(R_GM, par))) break;
+                tc_fence_after_sync();
+                if (more) {
+                    const uint32_t wn = D64 ? a0 + (par ^ 1) * kPanelB : t(5);
+                    mma<OP_K, OP_K, KS, 128>(tmem + cG, wn, wn, false);
+                    umma_commit(&bars[M_GM]);
+                }
+                // U = T~ W, Y = T~ Xk  (lo x lo terms are dropped everywhere)
                 if (!(ok = wait(R_TT, par))) break;
                 tc_fence_after_sync();
-                if (SAVE) {
-                    store(&tm.th, 1, kT, r0);
-                    store(&tm.tl, 2, kT, r0);
-                    tma_store_commit();
+                if (TMT) {
+                    mma_tap<OP_MN, 8, HD>(cu, tmem + cG, w, false);
+                    mma_tap<OP_MN, 8, HD>(cu, tmem + cG + 16, w, true);
+                } else {
+                    mma<OP_K, OP_MN, 8, HD>(cu, t(1), w, false);
+                    mma<OP_K, OP_MN, 8, HD>(cu, t(2), w, true);
                 }
-                mma<OP_K, OP_MN, 8, HD>(tmem + 0, t(1), t(0), false);
-                mma<OP_K, OP_MN, 8, HD>(tmem + 0, t(2), t(0), true);
-                umma_commit(&bars[B_U]);
-                // Y = T~ Xk
+                umma_commit(&bars[M_U]);
                 if (!(ok = wait(R_XK, par))) break;
                 tc_fence_after_sync();
-                if (SAVE) {
-                    store(&tm.xk, 5, kT, r0);
-                    tma_store_commit();
+                if (TMT) {
+                    mma_tap<OP_MN, 8, 128>(cx, tmem + cG, t(3), false);
+                    mma_tap<OP_MN, 8, 128>(cx, tmem + cG + 16, t(3), true);
+                    mma_tap<OP_MN, 8, 128>(cx, tmem + cG, t(4), true);
+                } else {
+                    mma<OP_K, OP_MN, 8, 128>(cx, t(1), t(3), false);
+                    mma<OP_K, OP_MN, 8, 128>(cx, t(2), t(3), true);
+                    mma<OP_K, OP_MN, 8, 128>(cx, t(1), t(4), true);
                 }
-                mma<OP_K, OP_MN, 8, 128>(tmem + 384, t(1), t(5), false);
-                mma<OP_K, OP_MN, 8, 128>(tmem + 384, t(2), t(5), true);
-                mma<OP_K, OP_MN, 8, 128>(tmem + 384, t(1), t(6), true);
-                // B_Y lets the workers overwrite T~ (with U) and Xk (with Y): the stores must have read them
-                if (SAVE) tma_store_wait_read();
-                umma_commit(&bars[B_Y]);
-                if (!KEYS) {
-                    if (!(ok = wait(R_XQ, par))) break;
-                    store(&tm.xq, 3, kT, r0);
-                    tma_store_commit();
-                }
-                // Xq U and W^T U
+                umma_commit(&bars[M_Y]);
+                // -W^T U, and Xq U over the next Gm once that has been read, or over T~ once Y has retired
                 if (!(ok = wait(R_U, par))) break;
                 tc_fence_after_sync();
-                tma_store_wait_read();   // Xq: the workers' next tile goes over it when this group has retired
-                if (SAVE) {
-                    store(&tm.u, 1, HD, r0);
-                    tma_store_commit();
-                }
+                mma<OP_MN, OP_MN, 8, HD, true>(cu, w, a0 + oU, false);
+                mma<OP_MN, OP_MN, 8, HD, true>(cu, w, a0 + oUlo, true);
                 if (!KEYS) {
-                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, t(3), t(1), false);
-                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, t(4), t(1), true);
-                    mma<OP_K, OP_MN, 8, HD>(tmem + 256, t(3), t(2), true);
+                    if (!(ok = TMT ? wait(M_Y, par) : !more || wait(R_GM, par ^ 1))) break;
+                    tc_fence_after_sync();
+                    mma_tap<OP_MN, 8, HD>(tmem + cG, tmem + cXq, a0 + oU, false);
+                    mma_tap<OP_MN, 8, HD>(tmem + cG, tmem + cXq + 16, a0 + oU, true);
+                    mma_tap<OP_MN, 8, HD>(tmem + cG, tmem + cXq, a0 + oUlo, true);
                 }
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, t(0), t(1), false);
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 128, t(0), t(2), true);
-                umma_commit(&bars[B_G3A]);
+                umma_commit(&bars[M_GA]);
                 // Y^T W
                 if (!(ok = wait(R_Y, par))) break;
                 tc_fence_after_sync();
+                mma<OP_MN, OP_MN, 8, HD>(cx, t(3), w, false);
+                mma<OP_MN, OP_MN, 8, HD>(cx, t(4), w, true);
+                umma_commit(&bars[M_GB]);
+            }
+        }
+        if (warp == 17 && elect_one()) {
+            // -------------------------------------------------------------- tile loads and stores
+            auto fetch = [&](const CUtensorMap* m, uint32_t off, int b, int chunk_) {
+                tma_rows(smem + off, m, &bars[b], HD, (chunk_ % p.N) * kT, chunk_ / p.N);
+            };
+            auto load_w = [&](int chunk_, uint32_t off, int b) {
+                mbar_expect_tx(&bars[b], kT * HD * 2);
+                fetch(&tm.w, off, b, chunk_);
+            };
+            auto load_qk = [&](int chunk_, uint32_t off_q, uint32_t off_k, int b) {
+                mbar_expect_tx(&bars[b], (KEYS ? 1 : 2) * kT * HD * 2);
+                if (!KEYS) fetch(&tm.q, off_q, b, chunk_);
+                fetch(&tm.k, off_k, b, chunk_);
+            };
+            auto store = [&](const CUtensorMap* m, uint32_t off, int ncols, int row0) {
+                for (int h = 0; h < ncols / 64; ++h) tma_store_2d(m, smem + off + h * kPanelB, h * 64, row0);
+            };
+            bool ok = (int)blockIdx.x < nchunks;
+            if (ok) {
+                load_w(blockIdx.x, 0, L_W);
+                load_qk(blockIdx.x, oQ, oK, L_QK);
+            }
+            for (uint32_t it = 0, chunk = blockIdx.x; ok && (int)chunk < nchunks; ++it, chunk += gridDim.x) {
+                const uint32_t par = it & 1;
+                const int r0 = chunk * kT, next = chunk + gridDim.x;
+                const bool more = next < nchunks;
+                if (!D64 && more) {   // what the next chunk reads: its slots become free late, the trip from memory is taken now
+                    const int row0 = (next % p.N) * kT, slice = next / p.N;
+                    for (int h = 0; h < HD / 64; ++h) {
+                        tma_prefetch_3d(&tm.w, h * 64, row0, slice);
+                        if (!KEYS) tma_prefetch_3d(&tm.q, h * 64, row0, slice);
+                        tma_prefetch_3d(&tm.k, h * 64, row0, slice);
+                    }
+                }
+                if (D64 && more) load_w(next, (par ^ 1) * kPanelB, L_WN);   // (M_GB of the chunk before: its W is not needed any more)
+                if (!(ok = wait(M_XQK, par))) break;
+                if (more) {
+                    if (D64) load_qk(next, oQ, oK, L_QK);
+                    else load_w(next, 5 * kTileB, L_WN);
+                }
                 if (!KEYS) {
-                    store(&tm.y, 5, kT, r0);
+                    if (!(ok = wait(R_XQ, par))) break;
+                    store(&tm.xq, oXq, kT, r0);
                     tma_store_commit();
                 }
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, t(5), t(0), false);
-                mma<OP_MN, OP_MN, 8, HD>(tmem + 384, t(6), t(0), true);
-                umma_commit(&bars[B_G3B]);
-                // U's slots take the Q and K rows once more (from L2), for the sums that finish Q<- and K->
-                if (!(ok = wait(B_G3A, par))) break;
-                mbar_expect_tx(&bars[B_LOADR], (KEYS ? 1 : 2) * kT * HD * 2);
-                fetch(&tm.k, 2, B_LOADR, chunk);
-                tma_store_wait_read();
-                mbar_arrive(&bars[B_ST]);
-                if (!KEYS) fetch(&tm.q, 1, B_LOADR, chunk);
-                // W's slot is free once this chunk's last product has retired: the next chunk's Gram matrix is ready before
-                // the workers have written the last results of this one
-                if (next < nchunks) {
-                    if (!(ok = wait(B_G3B, par))) break;
-                    load_w(next);
+                if (SAVE) {
+                    if (!(ok = wait(R_XK, par))) break;
+                    store(&tm.xk, 3 * kTileB, kT, r0);
+                    tma_store_commit();
                 }
-                if (!(ok = wait(R_P, par))) break;
-                store(&tm.ph, 4, HD, chunk * HD);
-                store(&tm.pl, 3, HD, chunk * HD);
-                tma_store_commit();
-                if (next < nchunks) {
-                    if (!(ok = wait(B_LOAD, par ^ 1))) break;
-                    tc_fence_after_sync();
-                    mma<OP_K, OP_K, KS, 128>(tmem + 0, t(0), t(0), false);
-                    umma_commit(&bars[B_GM]);
+                if (!KEYS) {
                     tma_store_wait_read();
-                    load_qk(next);
+                    mbar_arrive(&bars[S_XQ]);
+                }
+                if (SAVE) {
+                    mbar_arrive(&bars[S_XK]);
+                    if (!(ok = wait(R_TT, par))) break;
+                    store(&tm.th, 1 * kTileB, kT, r0);
+                    store(&tm.tl, 2 * kTileB, kT, r0);
+                    tma_store_commit();
+                    tma_store_wait_read();
+                    mbar_arrive(&bars[S_T]);
+                    if (!(ok = wait(R_U, par))) break;
+                    store(&tm.u, oU, HD, r0);
+                    tma_store_commit();
+                }
+                if (!KEYS) {
+                    if (!(ok = wait(R_Y, par))) break;
+                    store(&tm.y, 3 * kTileB, kT, r0);
+                    tma_store_commit();
+                }
+                if (SAVE) {
+                    tma_store_wait_read_but<1>();
+                    mbar_arrive(&bars[S_U]);
+                }
+                // once Y^T W has retired, W's slot takes the next chunk's W, Y's slots the Q and K rows once more (from L2), for the
+                // sums that finish Q<- and K->
+                if (!(ok = wait(M_GB, par))) break;
+                if (!D64 && more) load_w(next, 0, L_W);
+                if (!KEYS) tma_store_wait_read();
+                load_qk(chunk, 3 * kTileB, 4 * kTileB, L_ROW);
+                if (!(ok = wait(R_P, par))) break;
+                store(&tm.ph, oU, HD, chunk * HD);
+                store(&tm.pl, oUlo, HD, chunk * HD);
+                tma_store_commit();
+                if (!D64 && more) {
+                    tma_store_wait_read();
+                    load_qk(next, oQ, oK, L_QK);
                 }
                 if (!(ok = wait(R_E3, par))) break;
-                if (!KEYS) store(&tm.ql, 5, HD, r0);
-                store(&tm.kr, 6, HD, r0);
+                if (!KEYS) store(&tm.ql, 3 * kTileB, HD, r0);
+                store(&tm.kr, 4 * kTileB, HD, r0);
                 tma_store_commit();
+                tma_store_wait_read();
+                mbar_arrive(&bars[S_E3]);
             }
             tma_store_wait_all();
         }
+        if (warp == 18 && elect_one()) {
+            // -------------------------------------------------------------- products of the inverse
+            // in the columns that U takes afterwards, once K-> of the chunk before has been read from them
+            bool ok = true;
+            for (uint32_t it = 0, chunk = blockIdx.x; ok && (int)chunk < nchunks; ++it, chunk += gridDim.x) {
+                const uint32_t par = it & 1;
+                uint32_t tH = base_ + kTileB;
+                asm volatile("" : "+r"(tH));
+                const uint32_t tL = tH + kTileB, cu = tmem + col_u(it);
+                if (it > 0 && !(ok = wait(R_E3, par ^ 1))) break;
+                if (!(ok = wait(R_ID, par))) break;
+                tc_fence_after_sync();
+                mma<OP_K, OP_MN, 4, 64>(cu, tH, tH, false);            // rows 64 ..: X = C A^-1
+                mma<OP_K, OP_MN, 4, 64>(cu, tL, tH, true);
+                mma<OP_K, OP_MN, 4, 64>(cu, tH, tL, true);
+                umma_commit(&bars[M_IX]);
+                if (!(ok = wait(R_IX, par))) break;
+                tc_fence_after_sync();
+                mma<OP_K, OP_MN, 4, 64, true>(cu + 64, tH + kPanelB, tH + 8192, false);   // rows 64 ..: -B^-1 X
+                mma<OP_K, OP_MN, 4, 64, true>(cu + 64, tL + kPanelB, tH + 8192, true);
+                mma<OP_K, OP_MN, 4, 64, true>(cu + 64, tH + kPanelB, tL + 8192, true);
+                umma_commit(&bars[M_IT]);
+            }
+        }
         __syncwarp();
-    } else {
-        // ------------------------------------------------------------------ workers
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+    } else if (warp < kWorkers / 32) {
+        // ------------------------------------------------------------------ inverse
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
         bool ok = true;
-        uint32_t r[32];
-        float v[32];
-        uint32_t hi[16], lo[16];
         // lane 0 of every warp waits; the vote that follows is also the barrier that releases the other lanes
         auto wwait = [&](int b, uint32_t par) {
             bool good = ok;
-            if (lane == 0 && good) good = mbar_wait(&bars[b], par, abort_flag, ST_PREP);
-            good = wsync_and(good);
-            tc_fence_after_sync();
-            return good;
+            if ((tid & 31) == 0 && good) good = mbar_wait(&bars[b], par, abort_flag, ST_PREP);
+            return wsync_and(good);
+        };
+        uint8_t* aH = slot(1);
+        uint8_t* aL = slot(2);
+        const int w8 = warp;
+        // This thread's 64 entries of Gm (only those of the two diagonal blocks and of the block under them are used).
+        uint32_t g[2][32];
+        auto read_gm = [&]() {
+            tmem_ld32(tl + cG + half * 64, g[0]);
+            tmem_ld32(tl + cG + half * 64 + 32, g[1]);
+            tmem_ld_wait();
         };
         int chunk = blockIdx.x;
-        for (uint32_t it = 0; chunk < nchunks; ++it, chunk += gridDim.x) {
+        auto first_gm = [&](uint32_t par) {
+            if (!(ok = wwait(M_GM, par))) return;
+            tc_fence_after_sync();
+            read_gm();
+            tc_fence_before_sync();
+            mbar_arrive(&bars[R_GM]);
+        };
+        if (TMT) first_gm(0);
+        for (uint32_t it = 0; ok && chunk < nchunks; ++it, chunk += gridDim.x) {
             const uint32_t par = it & 1;
-            if (!(ok = wwait(B_GM, par))) break;
-
-            // ---- E1: N = strictLower(D Gm) into slots 1, 2 as tri_inverse wants it: the two diagonal blocks in float32, the rest (and
-            // the zeros above the diagonal) as a bf16 pair
-            uint8_t* aH = slot(1);
-            uint8_t* aL = slot(2);
+            // (made opaque once per chunk: otherwise every address of the inverse is kept from chunk to chunk, in registers it does not have)
+            int lane = tid & 31, warp = w8;
+            asm volatile("" : "+r"(lane), "+r"(warp));
+            const int row = (warp & 3) * 32 + lane, half = (warp >> 2) & 1;   // accumulator row (TMEM lane), half of the columns
+            const bool diag = (row >> 6) == half, below = row >= 64 && half == 0;   // (the same for a whole warp)
+            const int next = chunk + (int)gridDim.x;
+            const float* bt = betas + par * kT;
+            float next_beta = 0.f;
+            if (tid < kT && next < nchunks) next_beta = beta_of(next);
+            // N = strictLower(D Gm) into slots 1, 2 as the inverse wants it: the two diagonal blocks in float32, the block
+            // under them as a bf16 pair
+            if (!TMT) {   // (read while the products that use the T~ before it still run)
+                first_gm(par);
+                if (!ok || (it > 0 && !(ok = wwait(M_Y, par ^ 1)))) break;
+            }
+            if (SAVE && it > 0 && !(ok = wwait(S_T, par ^ 1))) break;
+            const float b = bt[row];
+#pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int c0 = half * 64 + c * 32;
-                tmem_ld32(tl + 0 + c0, r);
-                tmem_ld_wait();
-                const float b = bt[row];
+                if (diag) {
+                    const int m = c * 32 - (row & 32);   // > 0: above the diagonal, < 0: below it, 0: on it (the same for a whole warp)
+                    float v[32];
 #pragma unroll
-                for (int x = 0; x < 32; ++x) v[x] = (c0 + x < row) ? b * __uint_as_float(r[x]) : 0.f;
-                if ((row >> 6) == half) {
+                    for (int x = 0; x < 32; ++x) v[x] = m > 0 ? 0.f : b * __uint_as_float(g[c][x]);
+                    if (m == 0) {
+#pragma unroll
+                        for (int x = 0; x < 32; ++x) v[x] = x < lane ? v[x] : 0.f;
+                    }
 #pragma unroll
                     for (int x = 0; x < 32; x += 4)
                         *reinterpret_cast<float4*>(fel(aH, aL, half, row & 63, c * 32 + x)) = make_float4(v[x], v[x + 1], v[x + 2], v[x + 3]);
-                } else {
+                } else if (below) {
+                    float v[32];
+                    uint32_t hi[16], lo[16];
+#pragma unroll
+                    for (int x = 0; x < 32; ++x) v[x] = b * __uint_as_float(g[c][x]);
                     split32(v, hi, lo);
                     tile_store_w16(aH, row, c0, hi);
                     tile_store_w16(aL, row, c0, lo);
                 }
             }
             wsync();
-            tri_inverse(aH, aL, bt, warp, lane, row, half);   // -> T~ = (I + N)^-1 D
+            float d[32];
+            invert_diagonal(aH, aL, bt, warp, lane, row, half, d);
+            if (tid < kT) betas[(par ^ 1) * kT + tid] = beta_floor(next_beta);   // (nobody reads the chunk before's any more)
             fence_proxy_async_smem();
+            tc_fence_before_sync();
+            mbar_arrive(&bars[R_ID]);
+            if (TMT && next < nchunks) {   // Gm of the next chunk leaves its columns to T~
+                if (!(ok = wwait(M_GM, par ^ 1))) break;
+                tc_fence_after_sync();
+                read_gm();
+            }
+            // X = C A^-1 over C, then the block of T~ there: -B^-1 X D; a thread has 32 entries of a row in all of this.  T~ goes into
+            // tensor memory (per 32 columns 16 of hi, 16 of lo) and / or over the tiles.
+            const uint32_t cu = col_u(it) + half * 32;
+            const int cd = (row & 64) + half * 32, co = half * 32 + 64 - (row & 64);   // its columns in the diagonal block and the other one
+            uint32_t hi[16], lo[16];
+            if (!(ok = wwait(M_IX, par))) break;
+            tc_fence_after_sync();
+            if (row >= 64) {
+                float v[32];
+                tmem_row32(tl + cu, v);
+                split32(v, hi, lo);
+                tile_store_w16(aH, row, half * 32, hi);
+                tile_store_w16(aL, row, half * 32, lo);
+            }
+            fence_proxy_async_smem();
+            tc_fence_before_sync();
+            mbar_arrive(&bars[R_IX]);
+            split32(d, hi, lo);
+            if (TMT) {   // (everybody has read Gm: there was a vote since)
+                tmem_st16(tl + cG + cd, hi);
+                tmem_st16(tl + cG + cd + 16, lo);
+            }
+            if (!(ok = wwait(M_IT, par))) break;
+            tc_fence_after_sync();
+            if (!TMT || SAVE) {
+                tile_store_w16(aH, row, cd, hi);
+                tile_store_w16(aL, row, cd, lo);
+            }
+            if (row >= 64) {
+                float v[32];
+                tmem_row32(tl + cu + 64, v);
+                scale32(v, bt + half * 32);
+                split32(v, hi, lo);
+                if (!TMT || SAVE) {
+                    tile_store_w16(aH, row, co, hi);
+                    tile_store_w16(aL, row, co, lo);
+                }
+            } else {
+#pragma unroll
+                for (int x = 0; x < 16; ++x) hi[x] = lo[x] = 0u;
+            }
+            if (TMT) {
+                tmem_st16(tl + cG + co, hi);
+                tmem_st16(tl + cG + co + 16, lo);
+                tmem_st_wait();
+            }
+            if (!TMT || SAVE) fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&bars[R_TT]);
-
-            if (!(ok = wwait(B_XQK, par))) break;
-            // ---- E1b: Xk = strictLower(.) -> bf16 hi / lo tiles (slots 5, 6), then Xq = lower(.) (slots 3, 4)
-            for (int c = 0; c < 2; ++c) {
-                const int c0 = half * 64 + c * 32;
-                tmem_ld32(tl + 256 + c0, r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int x = 0; x < 32; ++x) v[x] = (c0 + x < row) ? __uint_as_float(r[x]) : 0.f;
-                split32(v, hi, lo);
-                tile_store_w16(slot(5), row, c0, hi);
-                tile_store_w16(slot(6), row, c0, lo);
-            }
+        }
+    } else {
+        // ------------------------------------------------------------------ operands and results
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        bool ok = true;
+        uint32_t r[32];
+        float v[32];
+        auto wwait = [&](int b, uint32_t par) {   // (a thread touches its own rows only: warps meet nowhere but at mbarriers)
+            return __all_sync(0xffffffffu, mbar_wait(&bars[b], par, abort_flag, ST_PREP)) != 0;
+        };
+        auto publish = [&](int b) {
             fence_proxy_async_smem();
             tc_fence_before_sync();
-            mbar_arrive(&bars[R_XK]);
-            for (int c = 0; c < (KEYS ? 0 : 2); ++c) {
-                const int c0 = half * 64 + c * 32;
-                tmem_ld32(tl + 128 + c0, r);
-                tmem_ld_wait();
+            mbar_arrive(&bars[b]);
+        };
+        int chunk = blockIdx.x;
+        for (uint32_t it = 0; chunk < nchunks; ++it, chunk += gridDim.x) {
+            const uint32_t par = it & 1, cx = col_x(it), cu = col_u(it);
+            int row = (warp & 3) * 32 + lane;
+            asm volatile("" : "+r"(row));   // (as above)
+            // Five accumulators become bf16 pairs:  Xq = lower(.) in its own columns (per 32 columns 16 of hi, 16 of lo; hi also as
+            // a tile, for its store), Xk = strictLower(.), U over Q and K, Y over Xk, P = I - W^T U over U.  One body for all of
+            // them: the two groups' straight-line code does not fit the instruction caches.
+            enum { XQ = 0, XK, UU, YY, PP };
+#pragma unroll 1
+            for (int st = KEYS ? XK : XQ; st <= PP; ++st) {
+                if (!(ok = wwait(st <= XK ? M_XQK : st == UU ? M_U : st == YY ? M_Y : M_GA, par))) break;
+                // stores that still read the tiles about to be written (at d = 64 Xq goes over the P of the chunk before)
+                const int behind = st == XQ ? (D64 ? S_E3 : -1) : st == XK ? S_E3 : st == UU ? (KEYS ? -1 : S_XQ) : !SAVE ? -1 : st == YY ? S_XK : S_U;
+                if (behind >= 0 && (st > XK || it > 0) && !(ok = wwait(behind, st > XK ? par : par ^ 1))) break;
+                tc_fence_after_sync();
+                const uint32_t col = st == XQ ? cXq : st & 1 ? cx : cu;
+                const bool head = st == UU || st == PP;   // HD columns, not 128
+                const uint32_t to_hi = head ? oU : st == XQ ? oXq : 3 * kTileB, to_lo = head ? oUlo : 4 * kTileB;
+                const int n = head ? HD / 64 : 2;
+#pragma unroll 1
+                for (int c = 0; c < n; ++c) {
+                    const int c0 = half * n * 32 + c * 32, m = st == UU || st == YY ? -1 : c0 - (warp & 3) * 32;
+                    uint32_t hi[16], lo[16];
+                    if (m > 0 && st <= XK) {   // (the warp's 32 rows and these 32 columns: above the diagonal)
 #pragma unroll
-                for (int x = 0; x < 32; ++x) v[x] = (c0 + x <= row) ? __uint_as_float(r[x]) : 0.f;
-                split32(v, hi, lo);
-                tile_store_w16(slot(3), row, c0, hi);
-                tile_store_w16(slot(4), row, c0, lo);
-            }
-            if (!KEYS) {
-                fence_proxy_async_smem();
-                tc_fence_before_sync();
-                mbar_arrive(&bars[R_XQ]);
-            }
-
-            // ---- E2: U -> hi / lo tiles over T~ (slots 1, 2) once Y = T~ Xk has retired; Y -> hi / lo tiles over Xk
-            // (slots 5, 6)
-            if (!(ok = wwait(B_U, par))) break;
-            uint32_t uh[HD / 64][16], ul[HD / 64][16];
+                        for (int x = 0; x < 16; ++x) hi[x] = lo[x] = 0u;
+                    } else {
+                        tmem_ld32(tl + col + c0, r);
+                        tmem_ld_wait();
 #pragma unroll
-            for (int c = 0; c < HD / 64; ++c) {
-                const int c0 = half * (HD / 2) + c * 32;
-                tmem_ld32(tl + 0 + c0, r);
-                tmem_ld_wait();
+                        for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(r[x]);
+                        if (m == 0) {
+                            const int last = st == XQ ? lane + 1 : st == XK ? lane : 32, one = st == PP ? lane : -1;
 #pragma unroll
-                for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(r[x]);
-                split32(v, uh[c], ul[c]);
-            }
-            if (!(ok = wwait(B_Y, par))) break;
-#pragma unroll
-            for (int c = 0; c < HD / 64; ++c) {
-                const int c0 = half * (HD / 2) + c * 32;
-                tile_store_w16(slot(1), row, c0, uh[c]);
-                tile_store_w16(slot(2), row, c0, ul[c]);
-            }
-            fence_proxy_async_smem();
-            tc_fence_before_sync();
-            mbar_arrive(&bars[R_U]);
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int c0 = half * 64 + c * 32;
-                tmem_ld32(tl + 384 + c0, r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(r[x]);
-                split32(v, hi, lo);
-                tile_store_w16(slot(5), row, c0, hi);
-                tile_store_w16(slot(6), row, c0, lo);
-            }
-            fence_proxy_async_smem();
-            tc_fence_before_sync();
-            mbar_arrive(&bars[R_Y]);
-
-            // ---- E3: P = I - W^T U, Qleft = Q - Xq U, Kright = K - Y^T W; the Q and K rows arrive in U's slots meanwhile
-            const int next = chunk + (int)gridDim.x;
-            float next_beta = 0.f;
-            if (tid < kT && next < nchunks) next_beta = beta_of(next);
-            if (!(ok = wwait(B_G3A, par))) break;
-#pragma unroll
-            for (int c = 0; c < HD / 64; ++c) {   // P: hi over Xq lo, lo over Xq hi
-                const int c0 = half * (HD / 2) + c * 32;
-                tmem_ld32(tl + 128 + c0, r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int x = 0; x < 32; ++x) v[x] = ((c0 + x == row) ? 1.f : 0.f) - __uint_as_float(r[x]);
-                split32(v, hi, lo);
-                tile_store_w16(slot(4), row, c0, hi);
-                tile_store_w16(slot(3), row, c0, lo);
-            }
-            fence_proxy_async_smem();
-            tc_fence_before_sync();
-            mbar_arrive(&bars[R_P]);
-            if (!(ok = wwait(B_G3B, par))) break;
-            // (a wait that runs out here ends everyone's loop at the next worker barrier)
-            if (!mbar_wait(&bars[B_LOADR], par, abort_flag, ST_PREP) || !mbar_wait(&bars[B_ST], par, abort_flag, ST_PREP)) ok = false;
-            if (!KEYS) {   // Qleft, over Y hi, which has been stored
-#pragma unroll
-                for (int c = 0; c < HD / 64; ++c) {
-                    const int c0 = half * (HD / 2) + c * 32;
-                    float in[32];
-                    tmem_ld32(tl + 256 + c0, r);
-                    tmem_ld_wait();
-                    tile_load32(slot(1), row, c0, in);
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) v[x] = in[x] - __uint_as_float(r[x]);
-                    tile_store32(slot(5), row, c0, v);
+                            for (int x = 0; x < 32; ++x) v[x] = x == one ? v[x] + 1.f : x < last ? v[x] : 0.f;
+                        }
+                        split32(v, hi, lo);
+                    }
+                    tile_store_w16(smem + to_hi, row, c0, hi);
+                    if (st == XQ) {
+                        tmem_st16(tl + cXq + c0, hi);
+                        tmem_st16(tl + cXq + c0 + 16, lo);
+                    } else {
+                        tile_store_w16(smem + to_lo, row, c0, lo);
+                    }
                 }
+                if (st == XQ) tmem_st_wait();
+                publish(R_XQ + st);
             }
-#pragma unroll
-            for (int c = 0; c < HD / 64; ++c) {   // Kright, over Y lo
-                const int c0 = half * (HD / 2) + c * 32;
+            if (!ok) break;
+            // ---- Qleft = Q - Xq U, Kright = K - Y^T W over the Q and K rows that have arrived in Y's slots
+            if (!(ok = wwait(M_GB, par))) break;
+            if (!(ok = wwait(L_ROW, par))) break;
+            tc_fence_after_sync();
+#pragma unroll 1
+            for (int c = KEYS ? HD / 64 : 0; c < 2 * (HD / 64); ++c) {
+                const bool is_k = c >= HD / 64;
+                const int c0 = half * (HD / 2) + (is_k ? c - HD / 64 : c) * 32;
+                uint8_t* tile_ = slot(is_k ? 4 : 3);
                 float in[32];
-                tmem_ld32(tl + 384 + c0, r);
+                tmem_ld32(tl + (is_k ? cx : cG) + c0, r);
                 tmem_ld_wait();
-                tile_load32(slot(2), row, c0, in);
+                tile_load32(tile_, row, c0, in);
 #pragma unroll
                 for (int x = 0; x < 32; ++x) v[x] = in[x] - __uint_as_float(r[x]);
-                tile_store32(slot(6), row, c0, v);
+                tile_store32(tile_, row, c0, v);
             }
-            fence_proxy_async_smem();
-            if (tid < kT) bt[tid] = beta_floor(next_beta);   // read again only after the next chunk's first wait (a worker barrier)
-            tc_fence_before_sync();
-            mbar_arrive(&bars[R_E3]);
+            publish(R_E3);
         }
     }
 

@@ -12,6 +12,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// The first 1024-byte boundary at or after p in shared memory.  (An offset, not a rounded integer: so the compiler still sees a
+// pointer into shared memory, and its accesses need no 64-bit addresses.)
+__device__ __forceinline__ uint8_t* align1024(uint8_t* p) { return p + ((0u - smem_u32(p)) & 1023u); }
+
 // True in exactly one lane of a converged warp.  The roles that issue TMA loads and products pick their thread with this
 // and not with `lane == 0`: the operands of these instructions are uniform registers, and only behind elect.sync does the
 // compiler know that a single thread is active (otherwise every such instruction is wrapped in a loop over the active
@@ -54,6 +58,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// The same with a hint how long (ns) the thread may be suspended before it looks again.
+__device__ __forceinline__ bool mbar_try_wait_for(uint64_t* bar, uint32_t parity, uint32_t ns) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
+        : "memory");
+    return ok != 0;
+}
+
 // Limit of one wait, in clock64() ticks (about one second at B200 clocks).
 constexpr long long kWaitTicks = 2000000000LL;
 
@@ -66,7 +83,7 @@ __device__ __forceinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, v
     for (;;) {
 #pragma unroll 1      // rolled on purpose: there are dozens of wait sites and the kernels must fit the instruction cache
         for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait(bar, parity)) return true;
+            if (mbar_try_wait_for(bar, parity, 20000u)) return true;
         if (*abort_flag != 0) return false;
         if (clock64() - t0 > limit_ticks) {
             atomicCAS((uint32_t*)abort_flag, 0u, code);
@@ -145,6 +162,11 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* m, uin
         : "memory");
 }
 
+// A tile of such a map on its way into L2.
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* m, int c0, int c1, int c2) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(m), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
+
 // Plain (untiled) bulk copy global -> shared, completion counted in bytes on `bar`; 16-byte aligned, size % 16 == 0.
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -162,6 +184,9 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, const void* s
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // all committed stores of this thread have finished reading shared memory / have completed
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// the same for all but the N groups committed last
+template <int N>
+__device__ __forceinline__ void tma_store_wait_read_but() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // dst[0 .. bytes/4) += src[0 .. bytes/4) as float32, done by the copy engine at the memory side (bulk async-group

@@ -51,6 +51,19 @@ __device__ __forceinline__ void mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint32_
     }
 }
 
+// The same with A as half of a bf16 pair that lies where its float32 accumulator was: per 32 elements of the contraction 16 columns
+// of hi, then 16 of lo (`a_tmem` = first column of the half).
+template <int BOP, int KSTEPS, int N>
+__device__ __forceinline__ void mma_tap(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_tile, bool acc) {
+    constexpr uint32_t idesc = umma_idesc(128, N, OP_K, BOP);
+    const uint32_t b_lo = umma_desc_lo(b_tile, BOP == OP_K ? 16u : kPanelB);
+#pragma unroll
+    for (int kk = 0; kk < KSTEPS; ++kk) {
+        const uint32_t ko = (uint32_t)(kk >> 2) * (kPanelB >> 4) + (uint32_t)(kk & 3) * 2u, mo = (uint32_t)kk * 128u;
+        umma_ts(d_tmem, a_tmem + (kk >> 1) * 32 + (kk & 1) * 8, umma_desc_join(b_lo + (BOP == OP_K ? ko : mo)), idesc, (acc || kk > 0) ? 1u : 0u);
+    }
+}
+
 // Stores columns c0 .. c0+31 of `row` of a swizzled bf16 tile.
 __device__ __forceinline__ void tile_store32(uint8_t* t, int row, int c0, const float (&v)[32]) {
     uint8_t* panel = t + (c0 >> 6) * kPanelB;
@@ -167,6 +180,14 @@ __device__ __forceinline__ void tile_store_w16(uint8_t* t, int row, int c0, cons
     for (int ch = 0; ch < 4; ++ch)
         *reinterpret_cast<uint4*>(panel + sw128_off((uint32_t)row, (uint32_t)(ch0 + ch))) =
             make_uint4(w[4 * ch], w[4 * ch + 1], w[4 * ch + 2], w[4 * ch + 3]);
+}
+__device__ __forceinline__ void tile_load_w16(const uint8_t* t, int row, int c0, uint32_t (&w)[16]) {
+    const uint8_t* panel = t + (c0 >> 6) * kPanelB;
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) {
+        const uint4 u = *reinterpret_cast<const uint4*>(panel + sw128_off((uint32_t)row, (uint32_t)(((c0 & 63) >> 3) + ch)));
+        w[4 * ch] = u.x; w[4 * ch + 1] = u.y; w[4 * ch + 2] = u.z; w[4 * ch + 3] = u.w;
+    }
 }
 __device__ __forceinline__ void unpack_bf16x32(const uint4 (&u4)[4], float (&v)[32]) {
 #pragma unroll
