@@ -32,7 +32,7 @@ template <int HD>
 __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __grid_constant__ ChainTensorMaps tm,
                                                              const ChainParams p, const int nchunks) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     uint64_t* bars = (uint64_t*)(smem + kBarOff);  // two for loads, two for product groups, two for the workers' hand-overs
     uint32_t* tmem_slot = (uint32_t*)(bars + 6);
     volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);

@@ -99,7 +99,7 @@ constexpr uint32_t kDkvTotal = kDkvStat + 2 * 2 * kTile * 4 + kTile * 4;   // + 
 template <int HD, bool GATE>
 __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ BwdTensorMaps tm, const BwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     if ((uint32_t)(smem - smem_raw) + kDkvTotal > kSmemAlloc) {   // uniform over the CTA
         grid_wait();   // (the status word belongs to the kernels before)
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_DKV_PRODUCER);
@@ -575,7 +575,7 @@ __device__ __forceinline__ void mma_t16(uint32_t d_tmem, uint32_t a_col, uint32_
 template <int HD, bool GATE>
 __global__ void __launch_bounds__(512, 1) dq_kernel(const __grid_constant__ BwdTensorMaps tm, const BwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     if ((uint32_t)(smem - smem_raw) + kDqTotal > kSmemAlloc) {   // uniform over the CTA
         grid_wait();   // (the status word belongs to the kernels before)
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_DQ_PRODUCER);
@@ -977,7 +977,7 @@ __device__ __noinline__ void mask_pt(uint32_t ts, int n) {
 
 __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ BwdTensorMaps tm, const BwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     constexpr int HD = 64, NQ = 4, ND = 4;
     uint8_t* sQ = smem;
     uint8_t* sDO = sQ + NQ * kD64Tile;

@@ -195,7 +195,7 @@ template <int HD, bool GATE>
 __global__ void __launch_bounds__(384, 1)
 fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     if ((uint32_t)(smem - smem_raw) + SplitSmem::total > SplitSmem::alloc) {   // uniform over the CTA
         grid_wait();   // (the status word belongs to the kernels before)
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_FWD_PRODUCER);
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
     constexpr bool SEP = HD == 64;
     constexpr int kOff = CROSS ? 0 : 1;                        // stream 0's step index is n - kOff
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     if ((uint32_t)(smem - smem_raw) + FwdSmem::total > FwdSmem::alloc) {   // uniform over the CTA
         grid_wait();   // (the status word belongs to the kernels before)
         if (threadIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)ST_FWD_PRODUCER);

@@ -30,7 +30,7 @@ struct Ctx {
 
 template <int NCOLS>
 __device__ __forceinline__ void setup(Ctx& c, uint8_t* smem_raw, uint32_t bar_off) {
-    c.smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    c.smem = align1024(smem_raw);
     c.bars = (uint64_t*)(c.smem + bar_off);
     uint32_t* tmem_slot = (uint32_t*)(c.bars + 2);
     c.abort_flag = (volatile uint32_t*)(tmem_slot + 1);

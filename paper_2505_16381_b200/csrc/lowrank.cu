@@ -32,7 +32,7 @@ __device__ __forceinline__ uint32_t step_lo(uint32_t tile, int mn_major, int kk)
 __global__ void __launch_bounds__(192, 2) gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                                                       const GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     uint64_t* full = (uint64_t*)(smem + kStages * kStageBytes);
     uint64_t* empty = full + kStages;
     uint64_t* done = empty + kStages;
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(192, R == 64 ? 2 : 1) wide_kernel(const __grid
                                                                     const int ntiles, const int per_unit, const int N, uint32_t* status) {
     typedef WideSmem<R, BMN> Sm;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align1024(smem_raw);
     uint64_t* bars = (uint64_t*)(smem + Sm::offBar);
     enum { AFULL = 0, AEMPTY = 2, BFULL = 4, BEMPTY = 6, CFULL = 8, CEMPTY = 10, COUNT = 12 };
     uint32_t* tmem_slot = (uint32_t*)(bars + COUNT);
