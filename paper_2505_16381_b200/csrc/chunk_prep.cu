@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
 
     if (warp >= 2 * kWorkers / 32) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");   // 128 x 72 + 256 x 128 + 256 x 72 = 60416 of the 640 x 96
-        auto wait = [&](int b, uint32_t par) { return mbar_wait(&bars[b], par, abort_flag, ST_PREP); };
+        auto wait = [&](int b, uint32_t par) { return mbar_wait<true>(&bars[b], par, abort_flag, ST_PREP); };
         if (warp == 16 && elect_one()) {
             // -------------------------------------------------------------- products
             bool ok = (int)blockIdx.x < nchunks;
@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         // lane 0 of every warp waits; the vote that follows is also the barrier that releases the other lanes
         auto wwait = [&](int b, uint32_t par) {
             bool good = ok;
-            if ((tid & 31) == 0 && good) good = mbar_wait(&bars[b], par, abort_flag, ST_PREP);
+            if ((tid & 31) == 0 && good) good = mbar_wait<true>(&bars[b], par, abort_flag, ST_PREP);
             return wsync_and(good);
         };
         uint8_t* aH = slot(1);
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         uint32_t r[32];
         float v[32];
         auto wwait = [&](int b, uint32_t par) {   // (a thread touches its own rows only: warps meet nowhere but at mbarriers)
-            return __all_sync(0xffffffffu, mbar_wait(&bars[b], par, abort_flag, ST_PREP)) != 0;
+            return __all_sync(0xffffffffu, mbar_wait<true>(&bars[b], par, abort_flag, ST_PREP)) != 0;
         };
         auto publish = [&](int b) {
             fence_proxy_async_smem();

@@ -75,7 +75,10 @@ __device__ __forceinline__ bool mbar_try_wait_for(uint64_t* bar, uint32_t parity
 constexpr long long kWaitTicks = 2000000000LL;
 
 // Waits for the phase with the given parity.  Returns false (and raises *abort_flag with
-// `code`) if the limit ran out or another thread of the CTA already gave up.
+// `code`) if the limit ran out or another thread of the CTA already gave up.  PARKED: a thread may be suspended for longer at a
+// time, which leaves the issue slots to other warps (a third of all instructions of the chunk preparation were such waits) but
+// wakes up later: the forward sweep, whose waits are short, takes 1 % longer with it.
+template <bool PARKED = false>
 __device__ __forceinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t code,
                                                long long limit_ticks = kWaitTicks) {
     long long t0 = clock64();
@@ -83,7 +86,7 @@ __device__ __forceinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, v
     for (;;) {
 #pragma unroll 1      // rolled on purpose: there are dozens of wait sites and the kernels must fit the instruction cache
         for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait_for(bar, parity, 20000u)) return true;
+            if (PARKED ? mbar_try_wait_for(bar, parity, 20000u) : mbar_try_wait(bar, parity)) return true;
         if (*abort_flag != 0) return false;
         if (clock64() - t0 > limit_ticks) {
             atomicCAS((uint32_t*)abort_flag, 0u, code);
@@ -91,10 +94,11 @@ __device__ __forceinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, v
         }
     }
 }
+template <bool PARKED = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
                                           uint32_t code) {
     if (mbar_try_wait(bar, parity)) return true;
-    return mbar_wait_slow(bar, parity, abort_flag, code);
+    return mbar_wait_slow<PARKED>(bar, parity, abort_flag, code);
 }
 
 // Barrier ID over N threads (whole warps) + AND of `ok`.  Warps that meet at a named barrier leave a loop only on a vote like
