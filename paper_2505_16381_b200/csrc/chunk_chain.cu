@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     // have retired, and these five tiles are all that the chunk's first two products read; the other two slots feed the
     // previous chunk's very last products.
     auto first_loads_a = [&](int ch) {
-        mbar_expect_tx(&bars[B_LOAD], 3 * kT * HD * 2 + 2 * kTileB);
+        mbar_expect_tx(&bars[B_LOAD], 2 * kT * HD * 2 + HD * HD * 2 + 2 * kTileB);
         tma_tile(slot(1), &tm.dql, &bars[B_LOAD], HD, ch * kT);
         tma_tile(slot(0), &tm.u, &bars[B_LOAD], HD, ch * kT);
         tma_tile(slot(3), &tm.dsdt, &bars[B_LOAD], kT, ch * kT);   // (s dSd)^T: every use takes the transposed view

@@ -136,10 +136,10 @@ struct LevelTable {
 };
 
 struct LevelTensorMaps {
-    CUtensorMap dyh, dyl;   // [matrices * d][d] bf16 hi / lo planes of the run products
+    CUtensorMap dyh, dyl;   // [matrices * d][d] bf16 hi / lo planes of the run products, box d rows
     CUtensorMap qv, kv;     // bf16 versions, rows of d elements placed by VerLayout
     CUtensorMap dqv, dkv;   // same shape: bf16 gradients of the versions (backward only)
-    CUtensorMap ddy;        // [matrices * d][d] bf16 gradients of the run products (backward only)
+    CUtensorMap ddy;        // [matrices * d][d] bf16 gradients of the run products (backward only), box d rows
 };
 
 struct LevelParams {
@@ -197,7 +197,7 @@ struct ChainTensorMaps {
     CUtensorMap y, xq, xk, th, tl;                // [S*Lp][128]; y and xq are the attention sweep's operands
     CUtensorMap dsdt;                             // [S*N*128][128] bf16: (scale * lower(dS))^T of the diagonal chunks
     CUtensorMap dql, dkr;                         // [S*Lp][d] bf16 gradients of the boundary-adjusted queries / keys
-    CUtensorMap dp;                               // [S*N*d][d] bf16 gradients of the chunk products
+    CUtensorMap dp;                               // [S*N*d][d] bf16 gradients of the chunk products, box d rows
 };
 
 struct ChainParams {

@@ -102,8 +102,26 @@ __device__ __forceinline__ bool version_step(int is_key, int c, int l2, int N, i
     return true;
 }
 
-constexpr uint32_t kBar3 = 3 * kTileB, kBar4 = 4 * kTileB, kBar5 = 5 * kTileB;
-constexpr uint32_t smem_bytes(uint32_t slots) { return slots * kTileB + 64 + 1024; }
+// Slots: a [128 x d] tile (or a d x d matrix written by all 128 rows' threads), a d x d matrix as it is loaded.  At d = 64 they are half
+// and a quarter of the 32 KB of d = 128, so that two or three CTAs share an SM.  A product's A operand has 128 rows all the same: what
+// follows a matrix of 64 rows, or the panel after a tile of 64 columns, makes rows 64 ... of a result that nobody reads.
+template <int HD> constexpr uint32_t kTS = HD * 256;
+template <int HD> constexpr uint32_t kMS = HD == 64 ? 8192 : 32768;
+template <int HD> constexpr uint32_t kTileBytes = kT * HD * 2;
+template <int HD> constexpr uint32_t kMatBytes = HD * HD * 2;
+// where a kernel's barriers are: behind its slots
+template <int HD> constexpr uint32_t kOffDyadic = 4 * kMS<HD>;
+template <int HD> constexpr uint32_t kOffFused = 6 * kTS<HD>;
+template <int HD> constexpr uint32_t kOffVersion = kTS<HD> + 2 * kMS<HD>;
+template <int HD> constexpr uint32_t kOffSegment = 2 * kTS<HD> + 2 * kMS<HD>;
+template <int HD> constexpr uint32_t kOffBwd = 3 * kMS<HD> + 4 * kTS<HD> + (HD == 64 ? kPanelB : 0);   // (the panel after the last tile)
+constexpr uint32_t kOffKeys = 5 * kTileB, kOffSuffix = 4 * kTileB;
+constexpr uint32_t smem_bytes(uint32_t bars) { return bars + 64 + 1024; }
+// Loads of d x d matrices: maps with boxes of d rows.
+template <int HD>
+__device__ __forceinline__ void tma_matrix(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, long mat) {
+    for (int h = 0; h < HD / 64; ++h) tma_load_2d(dst + h * kPanelB, m, bar, h * 64, (int)(mat * HD));
+}
 
 // ---------------------------------------------------------------------------------------------- dyadic forward
 // grid.x = S * cnt2.  Dy[l+1][b] = Dy[l][2b+1] Dy[l][2b] with hi/lo operands (three products).
@@ -111,26 +129,27 @@ template <int HD>
 __global__ void __launch_bounds__(256, 1) dyadic_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<128>(c, smem_raw, kBar4);
+    setup<128>(c, smem_raw, kOffDyadic<HD>);
+    constexpr uint32_t M = kMS<HD>;
     const int cnt2 = p.lv.dy_cnt[p.l + 1], cnt = p.lv.dy_cnt[p.l];
     const int s = blockIdx.x / cnt2, b = blockIdx.x % cnt2;
     const long mat_lo = p.lv.dy_off[p.l] / (HD * HD) + (long)s * cnt + 2 * b;        // right factor; left is +1
     const long mat_out = p.lv.dy_off[p.l + 1] / (HD * HD) + (long)s * cnt2 + b;
     uint8_t* sm = c.smem;
     if (c.warp == 0 && elect_one()) {
-        mbar_expect_tx(&c.bars[0], 4 * kT * HD * 2);
-        tma_tile(sm + 0 * kTileB, &tm.dyh, &c.bars[0], HD, (int)((mat_lo + 1) * HD));
-        tma_tile(sm + 1 * kTileB, &tm.dyl, &c.bars[0], HD, (int)((mat_lo + 1) * HD));
-        tma_tile(sm + 2 * kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat_lo * HD));
-        tma_tile(sm + 3 * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat_lo * HD));
+        mbar_expect_tx(&c.bars[0], 4 * kMatBytes<HD>);
+        tma_matrix<HD>(sm + 0 * M, &tm.dyh, &c.bars[0], mat_lo + 1);
+        tma_matrix<HD>(sm + 1 * M, &tm.dyl, &c.bars[0], mat_lo + 1);
+        tma_matrix<HD>(sm + 2 * M, &tm.dyh, &c.bars[0], mat_lo);
+        tma_matrix<HD>(sm + 3 * M, &tm.dyl, &c.bars[0], mat_lo);
     }
     loads_wait(c);
     if (leader(c)) {
         tc_fence_after_sync();
         const uint32_t a = smem_u32(sm);
-        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, false);
-        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 3 * kTileB, true);
-        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a + kTileB, a + 2 * kTileB, true);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 2 * M, false);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 3 * M, true);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a + M, a + 2 * M, true);
         umma_commit(&c.bars[1]);
     }
     mma_wait(c);
@@ -161,10 +180,11 @@ __global__ void __launch_bounds__(256, 1) dyadic_fwd_kernel(const __grid_constan
 // Six tile slots: a product's result replaces the tiles of its own left factor; B_0 waits in tensor memory (columns
 // 128..255) while A_2, A_3 and B_1 are made.  grid.x = S * groups, groups = ceil(cnt(l + 1) / 2^(fuse-1)).
 template <int HD>
-__global__ void __launch_bounds__(256, 1) dyadic_fused_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
+__global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) dyadic_fused_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<256>(c, smem_raw, 6 * kTileB);
+    setup<256>(c, smem_raw, kOffFused<HD>);
+    constexpr uint32_t T = kTS<HD>;
     const int half_w = 1 << (p.fuse - 1);                        // A products per group
     const int groups = (p.lv.dy_cnt[p.l + 1] + half_w - 1) / half_w;
     const int s = blockIdx.x / groups, g = blockIdx.x % groups;
@@ -176,9 +196,9 @@ __global__ void __launch_bounds__(256, 1) dyadic_fused_kernel(const __grid_const
         if (leader(c)) {
             tc_fence_after_sync();
             const uint32_t base = smem_u32(sm);
-            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + a * kTileB, base + b * kTileB, false);
-            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + a * kTileB, base + (b + 1) * kTileB, true);
-            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + (a + 1) * kTileB, base + b * kTileB, true);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + a * T, base + b * T, false);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + a * T, base + (b + 1) * T, true);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem + col, base + (a + 1) * T, base + b * T, true);
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
@@ -196,8 +216,8 @@ __global__ void __launch_bounds__(256, 1) dyadic_fused_kernel(const __grid_const
                 v[x] -= hi[x];
             }
             if (a >= 0) {
-                tile_store32(sm + a * kTileB, c.row, c0, hi);
-                tile_store32(sm + (a + 1) * kTileB, c.row, c0, v);
+                tile_store32(sm + a * T, c.row, c0, hi);
+                tile_store32(sm + (a + 1) * T, c.row, c0, v);
             }
             if (to_global) {
                 const size_t o = ((size_t)mat(lvl, idx) * HD + c.row) * HD + c0;
@@ -224,14 +244,14 @@ __global__ void __launch_bounds__(256, 1) dyadic_fused_kernel(const __grid_const
     // part 1 announces all four tiles and fetches the right factor, part 2 the left one (its slots free up later)
     auto request_a1 = [&](int k, int b_) {
         if (c.warp != 0 || !elect_one()) return;
-        mbar_expect_tx(lbar[k & 1], 4 * kT * HD * 2);
-        tma_tile(sm + b_ * kTileB, &tm.dyh, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k)) * HD));
-        tma_tile(sm + (b_ + 1) * kTileB, &tm.dyl, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k)) * HD));
+        mbar_expect_tx(lbar[k & 1], 4 * kMatBytes<HD>);
+        tma_matrix<HD>(sm + b_ * T, &tm.dyh, lbar[k & 1], mat(l, 2 * (a0 + k)));
+        tma_matrix<HD>(sm + (b_ + 1) * T, &tm.dyl, lbar[k & 1], mat(l, 2 * (a0 + k)));
     };
     auto request_a2 = [&](int k, int a) {
         if (c.warp != 0 || !elect_one()) return;
-        tma_tile(sm + a * kTileB, &tm.dyh, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k) + 1) * HD));
-        tma_tile(sm + (a + 1) * kTileB, &tm.dyl, lbar[k & 1], HD, (int)(mat(l, 2 * (a0 + k) + 1) * HD));
+        tma_matrix<HD>(sm + a * T, &tm.dyh, lbar[k & 1], mat(l, 2 * (a0 + k) + 1));
+        tma_matrix<HD>(sm + (a + 1) * T, &tm.dyl, lbar[k & 1], mat(l, 2 * (a0 + k) + 1));
     };
     auto wait_a = [&](int k) {
         if (!mbar_wait(lbar[k & 1], lph[k & 1], c.abort_flag, ST_LEVELS)) c.ok = false;
@@ -329,7 +349,7 @@ __device__ __forceinline__ int version_at(int is_key, int ch, int e, int N, int 
 // 64 slices of 8 chunks at d = 128, on top of this kernel's 23; the extended chains take 49 in all, and the product of the
 // segment comes from the run products.)
 template <int HD, bool EDGE>
-__global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
+__global__ void __launch_bounds__(256, HD == 64 && !EDGE ? 3 : 2) version_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int is_key = blockIdx.y, s = blockIdx.x / p.N, ch = blockIdx.x % p.N;
     grid_wait();   // (the block-skipping counts)
     // levels to store: all of them, or for a gated problem up to the highest one a kept chunk pair uses (see level_bwd)
@@ -357,17 +377,18 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
     Ctx c;
     constexpr int kCols = EDGE ? 256 : 128;
     constexpr uint32_t colHi = 128, colLo = 128 + HD / 2;   // EDGE: the running pair
-    setup<kCols>(c, smem_raw, kBar3);
+    setup<kCols>(c, smem_raw, kOffVersion<HD>);
+    constexpr uint32_t T = kTS<HD>, M = kMS<HD>;
     uint8_t* sm = c.smem;   // slots: 0 current version (EDGE: the first one only), 1 Dy hi, 2 Dy lo
     bool first = true, more = true;
 #pragma unroll 1
     while (more && c.ok) {
         const long mat = p.lv.dy_off[a] / (HD * HD) + (long)s * p.lv.dy_cnt[a] + idx;
         if (c.warp == 0 && elect_one()) {
-            mbar_expect_tx(&c.bars[0], (first ? 3 : 2) * kT * HD * 2);
+            mbar_expect_tx(&c.bars[0], (first ? kTileBytes<HD> : 0) + 2 * kMatBytes<HD>);
             if (first) tma_tile(sm, is_key ? &tm.kv : &tm.qv, &c.bars[0], HD, (int)row_first);
-            tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
-            tma_tile(sm + 2 * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat * HD));
+            tma_matrix<HD>(sm + T, &tm.dyh, &c.bars[0], mat);
+            tma_matrix<HD>(sm + T + M, &tm.dyl, &c.bars[0], mat);
         }
         // A stored version is the product of the one before it alone, here as in the plain instance; what the rest of the pair adds
         // comes in a product of its own.
@@ -380,12 +401,12 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
             auto products = [&](auto bop) {
                 constexpr int BOP = decltype(bop)::value;
                 if (!EDGE || first) {
-                    mma<OP_K, BOP, HD / 16, HD>(c.tmem, t, t + kTileB, false);
-                    mma<OP_K, BOP, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, true);
+                    mma<OP_K, BOP, HD / 16, HD>(c.tmem, t, t + T, false);
+                    mma<OP_K, BOP, HD / 16, HD>(c.tmem, t, t + T + M, true);
                 } else {
-                    mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colHi, t + kTileB, false);
-                    mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colHi, t + 2 * kTileB, true);
-                    if (!apart) mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colLo, t + kTileB, true);
+                    mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colHi, t + T, false);
+                    mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colHi, t + T + M, true);
+                    if (!apart) mma_ta<BOP, HD / 16, HD>(c.tmem, c.tmem + colLo, t + T, true);
                 }
             };
             if (is_key) products(std::integral_constant<int, OP_K>{});
@@ -413,7 +434,7 @@ __global__ void __launch_bounds__(256, 2) version_fwd_kernel(const __grid_consta
             __syncthreads();
             if (leader(c)) {
                 tc_fence_after_sync();
-                const uint32_t t = smem_u32(sm) + kTileB;
+                const uint32_t t = smem_u32(sm) + T;
                 if (is_key) mma_ta<OP_K, HD / 16, HD>(c.tmem, c.tmem + colLo, t, true);
                 else mma_ta<OP_MN, HD / 16, HD>(c.tmem, c.tmem + colLo, t, true);
                 umma_commit(&c.bars[1]);
@@ -450,16 +471,17 @@ template <int HD>
 __global__ void __launch_bounds__(256, 1) segment_product_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<128>(c, smem_raw, kBar4);
+    setup<128>(c, smem_raw, kOffSegment<HD>);
+    constexpr uint32_t T = kTS<HD>, M = kMS<HD>;
     uint8_t* sm = c.smem;   // slots: 0 R hi, 1 R lo, 2 Dy hi, 3 Dy lo
     const int s = blockIdx.x, top = max(p.nlev - 2, 0);
     int e = p.N, a, idx, e2;
-    auto load = [&](int slot) {   // the run below boundary e
+    auto load = [&](uint32_t hi, uint32_t lo) {   // the run below boundary e
         const long mat = p.lv.dy_off[a] / (HD * HD) + (long)s * p.lv.dy_cnt[a] + idx;
         if (c.warp == 0 && elect_one()) {
-            mbar_expect_tx(&c.bars[0], 2 * kT * HD * 2);
-            tma_tile(sm + slot * kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
-            tma_tile(sm + (slot + 1) * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat * HD));
+            mbar_expect_tx(&c.bars[0], 2 * kMatBytes<HD>);
+            tma_matrix<HD>(sm + hi, &tm.dyh, &c.bars[0], mat);
+            tma_matrix<HD>(sm + lo, &tm.dyl, &c.bars[0], mat);
         }
         loads_wait(c);
         e = e2;
@@ -475,17 +497,17 @@ __global__ void __launch_bounds__(256, 1) segment_product_kernel(const __grid_co
         teardown<128>(c, p.status);
         return;
     }
-    load(0);
+    load(0, T);
 #pragma unroll 1
     while (c.ok && chain_step(0, e, p.N, top, a, idx, e2)) {
-        load(2);
+        load(2 * T, 2 * T + M);
         publish();
         if (leader(c)) {
             tc_fence_after_sync();
             const uint32_t t = smem_u32(sm);
-            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 2 * kTileB, false);
-            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 3 * kTileB, true);
-            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t + kTileB, t + 2 * kTileB, true);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 2 * T, false);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t, t + 2 * T + M, true);
+            mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, t + T, t + 2 * T, true);
             umma_commit(&c.bars[1]);
         }
         mma_wait(c);
@@ -497,7 +519,7 @@ __global__ void __launch_bounds__(256, 1) segment_product_kernel(const __grid_co
             tmem_row32(c.tl + c0, v);
             split32(v, hi, lo);
             tile_store_w16(sm, c.row, c0, hi);
-            tile_store_w16(sm + kTileB, c.row, c0, lo);
+            tile_store_w16(sm + T, c.row, c0, lo);
             if (e == 0) {
                 gstore_bf16_w16(out + (size_t)c.row * HD + c0, hi, c.row < HD);
                 gstore_bf16_w16(out + (size_t)HD * HD + (size_t)c.row * HD + c0, lo, c.row < HD);
@@ -523,7 +545,7 @@ __global__ void __launch_bounds__(256, 1) segment_product_kernel(const __grid_co
 // dDy is written once, as bf16: it is only ever read as an MMA operand (by the next launch and, at level 0, by the
 // chunk chain rule as dP).  Runs with b = 0 multiply nothing (no boundary lies before chunk 0): only level 0 writes them.
 template <int HD>
-__global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
+__global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) level_bwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int l1 = p.l, cnt = p.lv.dy_cnt[l1];
     grid_wait();   // (the block-skipping counts, and the zeros below)
     const int s = blockIdx.x / cnt, b = blockIdx.x % cnt;
@@ -561,28 +583,28 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
     __nv_bfloat16* dxv = is_key ? p.dkv : p.dqv;
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<256>(c, smem_raw, 7 * kTileB);
+    setup<256>(c, smem_raw, kOffBwd<HD>);
+    constexpr uint32_t T = kTS<HD>, M = kMS<HD>;
     uint8_t* sm = c.smem;   // slots: 0 Dy, 1 dC, 2 the other factor of the level above, (3, 4) and (5, 6): g and Xv[l1] of a chunk
     constexpr uint32_t colCarry = 0, colAcc = 128;
     auto ver_row = [&](int lvl, int chx) { return is_key ? kver_row(p.vl, s, lvl, chx) : qver_row(p.vl, s, lvl, chx); };
     auto chunk_loads = [&](int chx, int buf) {
-        uint8_t* base = sm + (3 + 2 * buf) * kTileB;
+        uint8_t* base = sm + 3 * M + 2 * buf * T;
         const CUtensorMap* gm = is_key ? &tm.dkv : &tm.dqv;
         const CUtensorMap* xm = is_key ? &tm.kv : &tm.qv;
         tma_tile(base, gm, &c.bars[0], HD, (int)ver_row(l2, chx));
-        tma_tile(base + kTileB, xm, &c.bars[0], HD, (int)ver_row(l1, chx));
+        tma_tile(base + T, xm, &c.bars[0], HD, (int)ver_row(l1, chx));
     };
     if (c.warp == 0 && elect_one()) {   // first group: the run product itself, the operands of the level above, the first chunk
-        const uint32_t tile = kT * HD * 2;
-        mbar_expect_tx(&c.bars[0], (ch >= 0 ? 3 : 0) * tile + (parent ? 2 : 0) * tile);
+        mbar_expect_tx(&c.bars[0], (ch >= 0 ? kMatBytes<HD> + 2 * kTileBytes<HD> : 0) + (parent ? 2 : 0) * kMatBytes<HD>);
         if (ch >= 0) {
-            tma_tile(sm, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
+            tma_matrix<HD>(sm, &tm.dyh, &c.bars[0], mat);
             chunk_loads(ch, 0);
         }
         if (parent) {
             const long up = p.lv.dy_off[l1 + 1] / (HD * HD) + (long)s * p.lv.dy_cnt[l1 + 1] + (b >> 1);
-            tma_tile(sm + kTileB, &tm.ddy, &c.bars[0], HD, (int)(up * HD));
-            tma_tile(sm + 2 * kTileB, &tm.dyh, &c.bars[0], HD, (int)((mat + (is_key ? -1 : 1)) * HD));
+            tma_matrix<HD>(sm + M, &tm.ddy, &c.bars[0], up);
+            tma_matrix<HD>(sm + 2 * M, &tm.dyh, &c.bars[0], mat + (is_key ? -1 : 1));
         }
     }
     constexpr int NI = HD / 64;
@@ -596,8 +618,8 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
         }
     };
     auto issue_parent = [&](uint32_t a) {
-        if (is_key) mma<OP_K, OP_K, HD / 16, HD>(c.tmem + colAcc, a + kTileB, a + 2 * kTileB, false);      // dC B^T
-        else        mma<OP_MN, OP_MN, HD / 16, HD>(c.tmem + colAcc, a + 2 * kTileB, a + kTileB, false);   // A^T dC
+        if (is_key) mma<OP_K, OP_K, HD / 16, HD>(c.tmem + colAcc, a + M, a + 2 * M, false);      // dC B^T
+        else        mma<OP_MN, OP_MN, HD / 16, HD>(c.tmem + colAcc, a + 2 * M, a + M, false);   // A^T dC
     };
     int buf = 0;
     bool first = true;
@@ -612,11 +634,11 @@ __global__ void __launch_bounds__(256, 1) level_bwd_kernel(const __grid_constant
         __syncthreads();
         if (leader(c)) {
             if (nxt >= 0) {   // the other buffer's products retired before the previous mma_wait returned
-                mbar_expect_tx(&c.bars[0], 2 * kT * HD * 2);
+                mbar_expect_tx(&c.bars[0], 2 * kTileBytes<HD>);
                 chunk_loads(nxt, buf ^ 1);
             }
             tc_fence_after_sync();
-            const uint32_t a = smem_u32(sm), g = a + (3 + 2 * buf) * kTileB, x = g + kTileB;
+            const uint32_t a = smem_u32(sm), g = a + 3 * M + 2 * buf * T, x = g + T;
             if (first && parent) issue_parent(a);
             const bool acc = !first || parent;
             if (!is_key) {
@@ -682,7 +704,7 @@ template <int HD>
 __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<256>(c, smem_raw, kBar5);
+    setup<256>(c, smem_raw, kOffKeys);
     constexpr int NC = 64;                      // columns of R per CTA
     const int s = blockIdx.x, col0 = blockIdx.y * NC;
     uint8_t* sm = c.smem;   // slots: 0 Kright_J, 1 P hi, 2 P lo, 3 R hi, 4 R lo ([d x 64] in the first panel)
@@ -698,10 +720,10 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
     }
     auto issue = [&](int J) {
         const long mat = p.lv.dy_off[0] / (HD * HD) + (long)s * p.lv.dy_cnt[0] + J;
-        mbar_expect_tx(&c.bars[0], 3 * kT * HD * 2);
+        mbar_expect_tx(&c.bars[0], kTileBytes<HD> + 2 * kMatBytes<HD>);
         tma_tile(sm, &tm.kv, &c.bars[0], HD, (int)((long)s * p.Lp + (long)J * kT));   // version slot 0
-        tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(mat * HD));
-        tma_tile(sm + 2 * kTileB, &tm.dyl, &c.bars[0], HD, (int)(mat * HD));
+        tma_matrix<HD>(sm + kTileB, &tm.dyh, &c.bars[0], mat);
+        tma_matrix<HD>(sm + 2 * kTileB, &tm.dyl, &c.bars[0], mat);
     };
     // Segments (key side, p.nseg > 1): blockIdx.z walks only the chunks [z * seg_chunks, (z+1) * seg_chunks) and leaves its keys
     // advanced to the end of THAT range (bf16, p.edge16) together with the range's product (p.pseg); a second pass
@@ -766,7 +788,7 @@ template <int HD>
 __global__ void __launch_bounds__(256, 1) suffix_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<128>(c, smem_raw, kBar4);
+    setup<128>(c, smem_raw, kOffSuffix);
     constexpr int NC = 64;
     const int s = blockIdx.x, col0 = blockIdx.y * NC, c0 = c.half * 32;
     uint8_t* sm = c.smem;   // slots: 0 M hi, 1 M lo, 2 R hi, 3 R lo
@@ -796,10 +818,10 @@ __global__ void __launch_bounds__(256, 1) suffix_kernel(const __grid_constant__ 
 #pragma unroll 1
     for (int g = p.nseg - 1; g >= 1 && c.ok; --g) {
         if (c.warp == 0 && elect_one()) {
-            const long mrow = ((long)s * p.nseg + g) * 2 * HD;
-            mbar_expect_tx(&c.bars[0], 2 * kT * HD * 2);
-            tma_tile(sm, &tm.dyh, &c.bars[0], HD, (int)mrow);
-            tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(mrow + HD));
+            const long m = ((long)s * p.nseg + g) * 2;
+            mbar_expect_tx(&c.bars[0], 2 * kMatBytes<HD>);
+            tma_matrix<HD>(sm, &tm.dyh, &c.bars[0], m);
+            tma_matrix<HD>(sm + kTileB, &tm.dyh, &c.bars[0], m + 1);
         }
         loads_wait(c);
         publish();
@@ -836,24 +858,25 @@ template <int HD>
 __global__ void __launch_bounds__(256, 2) apply_product_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
-    setup<128>(c, smem_raw, kBar3);
+    setup<128>(c, smem_raw, kOffVersion<HD>);
+    constexpr uint32_t T = kTS<HD>, M = kMS<HD>;
     const int s = blockIdx.x / p.N, ch = blockIdx.x % p.N;
     uint8_t* sm = c.smem;   // slots: 0 x tile, 1 M hi, 2 M lo
     const long row0 = (long)s * p.Lp + (long)ch * kT;
     const long mi = p.nseg > 1 ? (long)s * p.nseg + ch / p.seg_chunks : (long)s;
     if (c.warp == 0 && elect_one()) {
-        mbar_expect_tx(&c.bars[0], 3 * kT * HD * 2);
+        mbar_expect_tx(&c.bars[0], kTileBytes<HD> + 2 * kMatBytes<HD>);
         tma_tile(sm, &tm.qv, &c.bars[0], HD, (int)row0);
-        tma_tile(sm + kTileB, &tm.dyh, &c.bars[0], HD, (int)(2 * mi * HD));
-        tma_tile(sm + 2 * kTileB, &tm.dyh, &c.bars[0], HD, (int)((2 * mi + 1) * HD));
+        tma_matrix<HD>(sm + T, &tm.dyh, &c.bars[0], 2 * mi);
+        tma_matrix<HD>(sm + T + M, &tm.dyh, &c.bars[0], 2 * mi + 1);
     }
     if (p.gq && c.tid < kT) p.gq[row0 + c.tid] += p.gtot[s];
     loads_wait(c);
     if (leader(c)) {
         tc_fence_after_sync();
         const uint32_t a = smem_u32(sm);
-        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + kTileB, false);
-        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + 2 * kTileB, true);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + T, false);
+        mma<OP_K, OP_MN, HD / 16, HD>(c.tmem, a, a + T + M, true);
         umma_commit(&c.bars[1]);
     }
     mma_wait(c);
@@ -877,39 +900,39 @@ cudaError_t launch_level_kernel(int which, const LevelTensorMaps& tm, const Leve
         case LEVEL_DYADIC_FUSED: {
             const int half_w = 1 << (p.fuse - 1);
             dim3 g(p.S * ((p.lv.dy_cnt[p.l + 1] + half_w - 1) / half_w));
-            return hd == 64 ? launch<dyadic_fused_kernel<64>>(g, 256, smem_bytes(6), st, tm, p) : launch<dyadic_fused_kernel<128>>(g, 256, smem_bytes(6), st, tm, p);
+            return hd == 64 ? launch<dyadic_fused_kernel<64>>(g, 256, smem_bytes(kOffFused<64>), st, tm, p) : launch<dyadic_fused_kernel<128>>(g, 256, smem_bytes(kOffFused<128>), st, tm, p);
         }
         case LEVEL_DYADIC_FWD: {
             dim3 g(p.S * p.lv.dy_cnt[p.l + 1]);
-            return hd == 64 ? launch<dyadic_fwd_kernel<64>>(g, 256, smem_bytes(4), st, tm, p) : launch<dyadic_fwd_kernel<128>>(g, 256, smem_bytes(4), st, tm, p);
+            return hd == 64 ? launch<dyadic_fwd_kernel<64>>(g, 256, smem_bytes(kOffDyadic<64>), st, tm, p) : launch<dyadic_fwd_kernel<128>>(g, 256, smem_bytes(kOffDyadic<128>), st, tm, p);
         }
         case LEVEL_VERSION_FWD: {
             dim3 g(p.S * p.N, 2);
             if (p.edge_q)
-                return hd == 64 ? launch<version_fwd_kernel<64, true>>(g, 256, smem_bytes(3), st, tm, p)
-                                : launch<version_fwd_kernel<128, true>>(g, 256, smem_bytes(3), st, tm, p);
-            return hd == 64 ? launch<version_fwd_kernel<64, false>>(g, 256, smem_bytes(3), st, tm, p)
-                            : launch<version_fwd_kernel<128, false>>(g, 256, smem_bytes(3), st, tm, p);
+                return hd == 64 ? launch<version_fwd_kernel<64, true>>(g, 256, smem_bytes(kOffVersion<64>), st, tm, p)
+                                : launch<version_fwd_kernel<128, true>>(g, 256, smem_bytes(kOffVersion<128>), st, tm, p);
+            return hd == 64 ? launch<version_fwd_kernel<64, false>>(g, 256, smem_bytes(kOffVersion<64>), st, tm, p)
+                            : launch<version_fwd_kernel<128, false>>(g, 256, smem_bytes(kOffVersion<128>), st, tm, p);
         }
         case LEVEL_BWD: {
             dim3 g(p.S * p.lv.dy_cnt[p.l]);
-            return hd == 64 ? launch<level_bwd_kernel<64>>(g, 256, smem_bytes(7), st, tm, p) : launch<level_bwd_kernel<128>>(g, 256, smem_bytes(7), st, tm, p);
+            return hd == 64 ? launch<level_bwd_kernel<64>>(g, 256, smem_bytes(kOffBwd<64>), st, tm, p) : launch<level_bwd_kernel<128>>(g, 256, smem_bytes(kOffBwd<128>), st, tm, p);
         }
         case LEVEL_KEY_CACHE: {
             dim3 g(p.S, hd / 64, p.nseg > 1 ? p.nseg : 1);
-            return hd == 64 ? launch<key_cache_kernel<64>>(g, 256, smem_bytes(5), st, tm, p) : launch<key_cache_kernel<128>>(g, 256, smem_bytes(5), st, tm, p);
+            return hd == 64 ? launch<key_cache_kernel<64>>(g, 256, smem_bytes(kOffKeys), st, tm, p) : launch<key_cache_kernel<128>>(g, 256, smem_bytes(kOffKeys), st, tm, p);
         }
         case LEVEL_SEGMENT_PRODUCT: {
             dim3 g(p.S);
-            return hd == 64 ? launch<segment_product_kernel<64>>(g, 256, smem_bytes(4), st, tm, p) : launch<segment_product_kernel<128>>(g, 256, smem_bytes(4), st, tm, p);
+            return hd == 64 ? launch<segment_product_kernel<64>>(g, 256, smem_bytes(kOffSegment<64>), st, tm, p) : launch<segment_product_kernel<128>>(g, 256, smem_bytes(kOffSegment<128>), st, tm, p);
         }
         case LEVEL_SUFFIX: {
             dim3 g(p.S, hd / 64);
-            return hd == 64 ? launch<suffix_kernel<64>>(g, 256, smem_bytes(4), st, tm, p) : launch<suffix_kernel<128>>(g, 256, smem_bytes(4), st, tm, p);
+            return hd == 64 ? launch<suffix_kernel<64>>(g, 256, smem_bytes(kOffSuffix), st, tm, p) : launch<suffix_kernel<128>>(g, 256, smem_bytes(kOffSuffix), st, tm, p);
         }
         case LEVEL_APPLY_PRODUCT: {
             dim3 g(p.S * p.N);
-            return hd == 64 ? launch<apply_product_kernel<64>>(g, 256, smem_bytes(3), st, tm, p) : launch<apply_product_kernel<128>>(g, 256, smem_bytes(3), st, tm, p);
+            return hd == 64 ? launch<apply_product_kernel<64>>(g, 256, smem_bytes(kOffVersion<64>), st, tm, p) : launch<apply_product_kernel<128>>(g, 256, smem_bytes(kOffVersion<128>), st, tm, p);
         }
         default:
             return cudaErrorInvalidValue;

@@ -211,11 +211,11 @@ static T* at(void* ws, size_t off) { return reinterpret_cast<T*>((char*)ws + off
 
 static bool make_level_maps(const Plan& p, void* ws, LevelTensorMaps& tm) {
     memset(&tm, 0, sizeof(tm));
-    return make_map(&tm.dyh, at<void>(ws, p.Dyh), (uint64_t)p.dy_mats * p.d, p.d) &&
-           make_map(&tm.dyl, at<void>(ws, p.Dyl), (uint64_t)p.dy_mats * p.d, p.d) &&
+    return make_map_box(&tm.dyh, at<void>(ws, p.Dyh), (uint64_t)p.dy_mats * p.d, p.d, p.d) &&
+           make_map_box(&tm.dyl, at<void>(ws, p.Dyl), (uint64_t)p.dy_mats * p.d, p.d, p.d) &&
            make_map(&tm.qv, at<void>(ws, p.Qv16), p.rows_q, p.d) && make_map(&tm.kv, at<void>(ws, p.Kv16), p.rows_k, p.d) &&
            (!p.bwd || (make_map(&tm.dqv, at<void>(ws, p.dQv), p.rows_q, p.d) && make_map(&tm.dkv, at<void>(ws, p.dKv), p.rows_k, p.d) &&
-                       make_map(&tm.ddy, at<void>(ws, p.dDy), (uint64_t)p.dy_mats * p.d, p.d)));
+                       make_map_box(&tm.ddy, at<void>(ws, p.dDy), (uint64_t)p.dy_mats * p.d, p.d, p.d)));
 }
 
 static LevelParams level_params(const Plan& p, void* ws) {
@@ -336,7 +336,7 @@ static int run_chunk_chain(const Plan& p, void* ws, const void* q, const void* k
               make_map(&tm.th, at<void>(ws, p.sTh), rows, CHUNK) && make_map(&tm.tl, at<void>(ws, p.sTl), rows, CHUNK) &&
               make_map(&tm.dsdt, at<void>(ws, p.dSdT), (uint64_t)p.S * p.N * CHUNK, CHUNK) &&
               make_map(&tm.dql, at<void>(ws, p.dQv), rows, d) && make_map(&tm.dkr, at<void>(ws, p.dKv), rows, d) &&
-              make_map(&tm.dp, at<void>(ws, p.dDy), (uint64_t)p.S * p.N * d, d);   // level 0 of the run-product gradients
+              make_map_box(&tm.dp, at<void>(ws, p.dDy), (uint64_t)p.S * p.N * d, d, d);   // level 0 of the run-product gradients
     if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
     ChainParams cp{};
     cp.dql = at<__nv_bfloat16>(ws, p.dQv); cp.dkr = at<__nv_bfloat16>(ws, p.dKv);   // slot 0 of the version gradients: the final sums
@@ -742,7 +742,7 @@ int path_attn_cp_step(void* state, const void* message, int B, int H, int Lq, in
         LevelTensorMaps tm;
         memset(&tm, 0, sizeof(tm));
         bool ok = make_map(&tm.qv, at<void>(state, cq.x), (uint64_t)cq.S * cq.Lp, d) &&
-                  make_map(&tm.dyh, at<void>(msg, ck.pseg), (uint64_t)ck.S * 2 * d, d);
+                  make_map_box(&tm.dyh, at<void>(msg, ck.pseg), (uint64_t)ck.S * 2 * d, d, d);
         if (!ok) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
         tm.dyl = tm.kv = tm.dqv = tm.dkv = tm.ddy = tm.qv;
         LevelParams lp{};
@@ -810,9 +810,9 @@ int path_attn_prefill_cache(const void* k, const void* v, const void* w, const f
         lp.edge16 = edge; lp.pseg = pseg; lp.sfx = sfx; lp.L = p.Lp;   // (whole padded chunks: padded rows are zero)
         LAUNCH(launch_level_kernel(LEVEL_KEY_CACHE, tm, lp, d, st));
         LevelTensorMaps tm2 = tm;
-        if (!make_map(&tm2.dyh, pseg, (uint64_t)p.S * nseg * 2 * d, d)) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
+        if (!make_map_box(&tm2.dyh, pseg, (uint64_t)p.S * nseg * 2 * d, d, d)) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
         LAUNCH(launch_level_kernel(LEVEL_SUFFIX, tm2, lp, d, st));
-        if (!(make_map(&tm2.dyh, sfx, (uint64_t)p.S * nseg * 2 * d, d) && make_map(&tm2.qv, edge, (uint64_t)p.S * p.Lp, d))) {
+        if (!(make_map_box(&tm2.dyh, sfx, (uint64_t)p.S * nseg * 2 * d, d, d) && make_map(&tm2.qv, edge, (uint64_t)p.S * p.Lp, d))) {
             g_last_cuda_error = (int)cudaErrorUnknown;
             return PATH_ERR_LAUNCH;
         }
