@@ -97,10 +97,30 @@ __device__ __forceinline__ float* fel(uint8_t* aH, uint8_t* aL, int b, int r, in
 }
 // Fragments of float32 blocks for m16n8k8.  Slots t and t + 4 of the contraction stand for columns 2t and 2t + 1 of A and
 // rows 2t and 2t + 1 of B, which makes an accumulator tile of one product an A fragment of the next as it is.
+// The permutation is split into a lane's part, computed once, and one XOR per column: computed anew for every element it took
+// the merges three times as long as their products (integer operations issue at half rate).
 struct Tf32A { uint32_t h[4], l[4]; };
-__device__ __forceinline__ Tf32A tf32_a(uint8_t* aH, uint8_t* aL, int b, int r0, int c0, int lane) {
-    const float2 x = *reinterpret_cast<const float2*>(fel(aH, aL, b, r0 + (lane >> 2), c0 + 2 * (lane & 3)));
-    const float2 y = *reinterpret_cast<const float2*>(fel(aH, aL, b, r0 + 8 + (lane >> 2), c0 + 2 * (lane & 3)));
+struct FragLane {
+    int a, xa, b[2], xb[2];
+    __device__ __forceinline__ explicit FragLane(int lane) {
+        auto perm = [](int r) { return (((r & 3) ^ ((r >> 2) & 1)) << 3) | (r & 4); };
+        const int ra = lane >> 2, ca = 2 * (lane & 3), fa = perm(ra);
+        a = ra * 256 + (ca ^ (fa & 4)) * 4;
+        xa = (fa & 24) * 4;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const int fb = perm(ca + x);
+            b[x] = (ca + x) * 256 + (ra ^ (fb & 4)) * 4;
+            xb[x] = (fb & 24) * 4;
+        }
+    }
+    // `rows`: a stripe's row that is a multiple of 8; c: a column that is
+    __device__ __forceinline__ float* at_a(uint8_t* rows, int c) const { return reinterpret_cast<float*>(rows + a + ((c * 4) ^ xa)); }
+    __device__ __forceinline__ float at_b(uint8_t* rows, int c, int x) const { return *reinterpret_cast<float*>(rows + b[x] + ((c * 4) ^ xb[x])); }
+};
+__device__ __forceinline__ Tf32A tf32_a(const FragLane& f, uint8_t* rows, int c) {
+    const float2 x = *reinterpret_cast<const float2*>(f.at_a(rows, c));
+    const float2 y = *reinterpret_cast<const float2*>(f.at_a(rows + 8 * 256, c));
     Tf32A a;
     a.h[0] = split_tf32(x.x, a.l[0]); a.h[1] = split_tf32(y.x, a.l[1]);
     a.h[2] = split_tf32(x.y, a.l[2]); a.h[3] = split_tf32(y.y, a.l[3]);
@@ -112,14 +132,14 @@ __device__ __forceinline__ Tf32A tf32_a(const float (&d)[4]) {
     a.h[2] = split_tf32(d[1], a.l[2]); a.h[3] = split_tf32(d[3], a.l[3]);
     return a;
 }
-// d[16 x 8 T] += A B, B the 8 x 8 T block at (r0, c0)
+// d[16 x 8 T] += A B, B the 8 x 8 T block at `rows`, column c
 template <int T>
-__device__ __forceinline__ void mma_tf32(float (&d)[T][4], const Tf32A& a, uint8_t* aH, uint8_t* aL, int b, int r0, int c0, int lane) {
+__device__ __forceinline__ void mma_tf32(float (&d)[T][4], const Tf32A& a, const FragLane& f, uint8_t* rows, int c) {
     uint32_t h[T][2], l[T][2];
 #pragma unroll
     for (int n = 0; n < T; ++n)
 #pragma unroll
-        for (int x = 0; x < 2; ++x) h[n][x] = split_tf32(*fel(aH, aL, b, r0 + 2 * (lane & 3) + x, c0 + n * 8 + (lane >> 2)), l[n][x]);
+        for (int x = 0; x < 2; ++x) h[n][x] = split_tf32(f.at_b(rows, c + n * 8, x), l[n][x]);
 #pragma unroll
     for (int n = 0; n < T; ++n) mma1688(d[n], a.h, h[n][0], h[n][1]);
 #pragma unroll
@@ -142,9 +162,14 @@ template <int NBK>
 __device__ __forceinline__ void merge_f32(uint8_t* aH, uint8_t* aL, int warp, int lane) {
     constexpr int NT = NBK;                       // 8-column tiles of the result per warp
     const int hw = warp >> 2, w4 = warp & 3;
-    const int b = NBK == 1 ? w4 >> 1 : w4 & 1, rb = NBK == 1 ? 0 : ((w4 >> 1) ^ hw);
-    const int base_a = NBK == 1 ? (w4 & 1) * 32 : 0, base_b = base_a + NBK * 16, row0 = base_b + rb * 16;
-    const int k_lo = NBK == 1 ? 0 : hw, col0 = base_a + hw * NBK * 8;   // A^-1 is lower triangular: columns col0.. need no earlier block
+    const int b = NBK == 1 ? w4 >> 1 : w4 & 1, rb = NBK == 1 ? 0 : ((w4 >> 1) ^ hw), odd = w4 & 1;
+    const FragLane f(lane);
+    // NBK = 1: a stripe's rows 0 - 15 (A) and 16 - 31; NBK = 2: its upper (A) and its lower stripe
+    const int ca = NBK == 1 ? odd * 32 : 0, cb = ca + NBK * 16;
+    uint8_t* rows_a = (NBK == 1 && odd ? aL : aH) + b * (kPanelB + 8192);
+    uint8_t* rows_b = (NBK == 1 ? rows_a + 16 * 256 : aL + b * (kPanelB + 8192));
+    uint8_t* strip = rows_b + rb * 16 * 256;
+    const int k_lo = NBK == 1 ? 0 : hw, col0 = ca + hw * NBK * 8;   // A^-1 is lower triangular: columns col0.. need no earlier block
     float m[NT][4], p1[NBK][2][4];
 #pragma unroll
     for (int k = 0; k < NBK; ++k)
@@ -154,29 +179,25 @@ __device__ __forceinline__ void merge_f32(uint8_t* aH, uint8_t* aL, int warp, in
     for (int x = 0; x < 4 * NT; ++x) m[x >> 2][x & 3] = 0.f;
 #pragma unroll 1
     for (int j = 0; j < 16 * (rb + 1); j += 8) {
-        const Tf32A a = tf32_a(aH, aL, b, row0, base_b + j, lane);
+        const Tf32A a = tf32_a(f, strip, cb + j);
 #pragma unroll
         for (int kb = 0; kb < NBK; ++kb) {
             if (kb < k_lo) continue;
-            mma_tf32(p1[kb], a, aH, aL, b, base_b + j, base_a + kb * 16, lane);
+            mma_tf32(p1[kb], a, f, rows_b + j * 256, ca + kb * 16);
         }
     }
 #pragma unroll
     for (int kb = 0; kb < NBK; ++kb) {
         if (kb < k_lo) continue;
 #pragma unroll
-        for (int k8 = 0; k8 < 2; ++k8) {
-            const Tf32A a = tf32_a(p1[kb][k8]);
-            mma_tf32(m, a, aH, aL, b, base_a + kb * 16 + k8 * 8, col0, lane);
-        }
+        for (int k8 = 0; k8 < 2; ++k8) mma_tf32(m, tf32_a(p1[kb][k8]), f, rows_a + (kb * 16 + k8 * 8) * 256, col0);
     }
     wsync();   // the other warps of the pair read C as well
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
         for (int y = 0; y < 2; ++y)
-            *reinterpret_cast<float2*>(fel(aH, aL, b, row0 + (lane >> 2) + 8 * y, col0 + n * 8 + 2 * (lane & 3))) =
-                make_float2(-m[n][2 * y], -m[n][2 * y + 1]);
+            *reinterpret_cast<float2*>(f.at_a(strip + 8 * y * 256, col0 + n * 8)) = make_float2(-m[n][2 * y], -m[n][2 * y + 1]);
 }
 // 16 x 16 diagonal blocks: half a warp each, a lane owns a column of the inverse and reads the rows all lanes of its half need.
 __device__ __forceinline__ void substitute16(uint8_t* aH, uint8_t* aL, int warp, int lane) {
