@@ -9,8 +9,8 @@
 //   dq = dQl + s dSd K + dXq W                   dk = dKr + s dSd^T Q + dXk^T W
 //   dw = -Y dKr - U dP^T + T~^T dU + dXq^T Q + dXk K + (dGm + dGm^T) W
 // A persistent CTA (one per SM) walks over chunks and runs these ~31 products per chunk as tcgen05 MMAs on swizzled
-// shared-memory tiles.  Eight worker warps turn accumulators (tensor memory, one row per thread) into the next operand
-// tiles; the first lane of a ninth warp requests every tile (TMA) and issues every product.  The two sides meet only
+// shared-memory tiles.  Sixteen worker warps turn accumulators (tensor memory, 32 columns of one row per thread) into the next
+// operand tiles; one lane of another warp requests every tile (TMA) and issues every product.  The two sides meet only
 // through mbarriers: the workers hand tiles over and go on (they wait for products, never for the issuer), the issuer
 // sends out first whatever does not depend on the read-out in progress, starts the next chunk's first products while
 // the current chunk's results are still leaving, and requests tiles the moment their slots are free.  dQl and dKr
@@ -24,9 +24,9 @@ using namespace tile;
 namespace {
 
 constexpr int kSlots = 7;
-constexpr int kChainThreads = 288;   // eight worker warps + the warp whose first lane loads tiles and issues products
+constexpr int kChainWorkers = 512, kChainThreads = kChainWorkers + 32;   // sixteen worker warps + the one that loads tiles and issues products
 constexpr uint32_t kBarOff = kSlots * kTileB;
-constexpr uint32_t kChainSmem = kBarOff + 64 + kT * 4 + kT * 4 + 1024;
+constexpr uint32_t kChainSmem = kBarOff + 64 + 3 * kT * 4 + 1024;
 
 template <int HD>
 __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __grid_constant__ ChainTensorMaps tm,
@@ -36,14 +36,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     uint64_t* bars = (uint64_t*)(smem + kBarOff);  // two for loads, two for product groups, two for the workers' hand-overs
     uint32_t* tmem_slot = (uint32_t*)(bars + 6);
     volatile uint32_t* abort_flag = (volatile uint32_t*)(tmem_slot + 1);
-    float* bt = (float*)(smem + kBarOff + 64);
-    float* t1 = bt + kT;
+    float* t1 = (float*)(smem + kBarOff + 64);
+    float* parts = t1 + kT;   // [2][128]
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row = (warp & 3) * 32 + lane, half = (warp >> 2) & 1;
+    const int row = (warp & 3) * 32 + lane, cg = (warp >> 2) & 3;   // a worker's row and which 32 of an accumulator's columns it has
 
     if (tid == 0) {
-        for (int i = 0; i < 6; ++i) mbar_init(&bars[i], i < 4 ? 1u : 256u);   // B_R0, B_R1: every worker arrives
+        for (int i = 0; i < 6; ++i) mbar_init(&bars[i], i < 4 ? 1u : (uint32_t)kChainWorkers);   // B_R0, B_R1: every worker arrives
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     enum { B_LOAD = 0, B_LOAD2, B_MMA, B_MMA2, B_R0, B_R1, B_COUNT };
     const int grid = (int)gridDim.x;
 
-    if (warp == 8) {
+    if (warp == kChainWorkers / 32) {
     if (elect_one()) {
     // ------------------------------------------------------------------ leader: TMA loads and every product
     bool ok = true;
@@ -193,9 +193,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
     bool ok = true;
     uint32_t ph_mma = 0, ph_mma2 = 0;
     float v[32];
+    uint32_t hi[16], lo[16];
     auto wsync = [&]() {
         __syncwarp();
-        asm volatile("bar.sync 1, 256;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(kChainWorkers) : "memory");
     };
     // lane 0 of every warp waits for the product group; the vote that follows releases the other lanes
     auto mma_wait = [&](int b = B_MMA) {
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         bool good = true;
         if (lane == 0) good = mbar_wait(&bars[b], ph, abort_flag, ST_CHAIN);
         ph ^= 1;
-        ok = barrier_and<1, 256>(good);
+        ok = barrier_and<1, kChainWorkers>(good);
         tc_fence_after_sync();
     };
     // tiles written by this thread become visible to the MMA unit, its accumulator reads are ordered, the leader learns
@@ -212,183 +213,141 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tc_fence_before_sync();
         mbar_arrive(&bars[b]);
     };
-    // accumulator [128][ncols] -> f(row values) -> bf16 tile
-    enum { M_NONE = 0, M_LOWER = 1, M_STRICT = 2 };
-    auto acc_to_tile = [&](uint32_t col, int ncols, uint8_t* dst, float mul, int mask) {
-        const int per = ncols / 2;
-        for (int c = 0; c < per / 32; ++c) {
-            const int c0 = half * per + c * 32;
-            tmem_row32(tl + col + c0, v);
+    // This thread's 32 columns of an accumulator's lower triangle.  `above` = columns minus rows of the warp's 32 x 32 block: > 0 nothing
+    // of it counts, < 0 everything, 0 it lies on the diagonal, which counts itself or not.
+    const int above = cg * 32 - (warp & 3) * 32;
+    auto read_lower = [&](uint32_t col, int diagonal) {
+        if (above > 0) {
 #pragma unroll
-            for (int x = 0; x < 32; ++x) {
-                const bool keep = mask == M_NONE || (mask == M_LOWER ? (c0 + x <= row) : (c0 + x < row));
-                v[x] = keep ? v[x] * mul : 0.f;
-            }
-            tile_store32(dst, row, c0, v);
+            for (int x = 0; x < 32; ++x) v[x] = 0.f;
+            return;
+        }
+        tmem_row32(tl + col + cg * 32, v);
+        if (above == 0) {
+#pragma unroll
+            for (int x = 0; x < 32; ++x) v[x] = x < lane + diagonal ? v[x] : 0.f;
         }
     };
-    // accumulator [128][128] -> f(value, column) -> hi or lo part of its bf16 pair -> tile
-    auto split_to_tile = [&](uint32_t col, uint8_t* dst, bool want_lo, auto&& f) {
-        for (int c = 0; c < 2; ++c) {
-            const int c0 = half * 64 + c * 32;
-            tmem_row32(tl + col + c0, v);
-#pragma unroll
-            for (int x = 0; x < 32; ++x) {
-                const float t = f(v[x], c0 + x);
-                const float h = __bfloat162float(__float2bfloat16_rn(t));
-                v[x] = want_lo ? t - h : h;
-            }
-            tile_store32(dst, row, c0, v);
-        }
-    };
-    // the same, both parts from one read of the accumulator
-    auto split_both = [&](uint32_t col, uint8_t* dst_hi, uint8_t* dst_lo, auto&& f) {
-        for (int c = 0; c < 2; ++c) {
-            const int c0 = half * 64 + c * 32;
-            uint32_t hi[16], lo[16];
-            tmem_row32(tl + col + c0, v);
-#pragma unroll
-            for (int x = 0; x < 32; ++x) v[x] = f(v[x], c0 + x);
-            split32(v, hi, lo);
-            tile_store_w16(dst_hi, row, c0, hi);
-            tile_store_w16(dst_lo, row, c0, lo);
-        }
-    };
-    auto f_dT = [&](float x, int col) { return col <= row ? x : 0.f; };
-    float inv_b = 0.f;   // 1 / beta of this thread's row
-    auto f_M = [&](float x, int col) { return x * inv_b; };
-    auto f_dGm = [&](float x, int col) { return col < row ? -bt[row] * x : 0.f; };
+    // A tile of the head dimension: its 32 columns from head_c0 on belong to this thread if `mine`.  At d = 64 two of the four column
+    // groups would have none; the second of two such tiles then goes to them.
+    auto has = [&](int which) { return HD == 128 || (cg >> 1) == which; };
+    const int head_c0 = (HD == 128 ? cg : cg & 1) * 32;
 
 #pragma unroll 1
     for (int chunk = blockIdx.x; chunk < nchunks; chunk += grid) {
         const int s_idx = chunk / p.N, pos = (chunk % p.N) * kT + row;   // slice and position of this thread's row
         const bool row_valid = pos < p.L;
         const size_t urow = (size_t)s_idx * p.L + pos;                   // row in the caller's [S][L][.] tensors
-        if (tid < kT) bt[tid] = beta_floor(row_valid ? p.beta[urow] : 0.f);   // first read after several barriers (phase 4)
-        mma_wait();                                                 // phase 0
+        const float beta = beta_floor(row_valid ? p.beta[urow] : 0.f);
+        mma_wait();                                                 // phase 0: -dXq
         if (!ok) break;
-        acc_to_tile(cA, kT, slot(0), -1.f, M_LOWER);                // dXq (over U)
+        read_lower(cA, 1);
+#pragma unroll
+        for (int x = 0; x < 32; ++x) v[x] = -v[x];
+        tile_store32(slot(0), row, cg * 32, v);                     // dXq (over U)
         publish(B_R0);
-        mma_wait();                                                 // phase 1
+        mma_wait();                                                 // phase 1: -dY, -dU
         if (!ok) break;
-        acc_to_tile(cA, kT, slot(5), -1.f, M_NONE);                 // dY (over dKr)
-        acc_to_tile(cB, HD, slot(6), -1.f, M_NONE);                 // dU (over dP)
+        tmem_row32(tl + cA + cg * 32, v);
+#pragma unroll
+        for (int x = 0; x < 32; ++x) v[x] = -v[x];
+        tile_store32(slot(5), row, cg * 32, v);                     // dY (over dKr)
+        if (has(0)) {
+            tmem_row32(tl + cB + head_c0, v);
+#pragma unroll
+            for (int x = 0; x < 32; ++x) v[x] = -v[x];
+            tile_store32(slot(6), row, head_c0, v);                 // dU (over dP)
+        }
         publish(B_R1);
         mma_wait();                                                 // phase 2
         if (!ok) break;
-        // dT stays in tensor memory (cA); its bf16 hi part goes over Xk now, the lo part follows once dU has been read
-        split_to_tile(cA, slot(2), false, f_dT);
+        // dT: its bf16 hi part goes over Xk now, the lo part follows once dU has been read
+        read_lower(cA, 1);
+        split32(v, hi, lo);
+        tile_store_w16(slot(2), row, cg * 32, hi);
         mma_wait(B_MMA2);                                           // phase 3
         if (!ok) break;
-        split_to_tile(cA, slot(6), true, f_dT);                     // dT lo (over dU)
+        tile_store_w16(slot(6), row, cg * 32, lo);                  // dT lo (over dU)
         publish(B_R0);
         // dXk leaves its columns while M is being computed; W W^T takes them over as soon as it has
-        acc_to_tile(cB, kT, slot(5), 1.f, M_STRICT);                // dXk (over dY)
+        read_lower(cB, 0);
+        tile_store32(slot(5), row, cg * 32, v);                     // dXk (over dY)
         publish(B_R1);
         mma_wait();                                                 // D M
         if (!ok) break;
-        inv_b = 1.f / bt[row];
-        {   // diagonal of M -> t1 (dbeta's column part)
-            const int c0 = (row >> 5) << 5;
-            if ((c0 >> 6) == half) {
-                tmem_row32(tl + cG + c0, v);
+        {   // M, hi (over dT hi) and lo (over dT lo); its diagonal is dbeta's column part
+            const float inv_b = 1.f / beta;
+            tmem_row32(tl + cG + cg * 32, v);
+#pragma unroll
+            for (int x = 0; x < 32; ++x) v[x] *= inv_b;
+            if (above == 0) {
 #pragma unroll
                 for (int x = 0; x < 32; ++x)
-                    if (c0 + x == row) t1[row] = v[x] * inv_b;
+                    if (x == lane) t1[row] = v[x];
             }
+            split32(v, hi, lo);
+            tile_store_w16(slot(2), row, cg * 32, hi);
+            tile_store_w16(slot(6), row, cg * 32, lo);
         }
-        split_both(cG, slot(2), slot(6), f_M);                      // M, hi (over dT hi) and lo (over dT lo)
         publish(B_R0);
         mma_wait();                                                 // dA and W W^T
         if (!ok) break;
-        float dbeta_row;
-        {   // dA = strictLower(-cA);  dbeta_r = t1_r + sum_c dA_rc (W W^T)_rc
-            float part = 0.f;
-            for (int c = 0; c < 2; ++c) {
-                const int c0 = half * 64 + c * 32;
+        float part = 0.f;
+        {   // dA = strictLower(-cA);  dbeta_r = t1_r + sum_c dA_rc (W W^T)_rc;  dGm = D dA, hi now, lo once dXk's slot is free
+            read_lower(cA, 0);
+            if (above <= 0) {
                 float gm[32];
-                tmem_row32(tl + cA + c0, v);
-                tmem_row32(tl + cB + c0, gm);
+                tmem_row32(tl + cB + cg * 32, gm);
 #pragma unroll
                 for (int x = 0; x < 32; ++x)
-                    if (c0 + x < row) part -= v[x] * gm[x];
+                    if (above < 0 || x < lane) part -= v[x] * gm[x];
             }
-            // the two threads of a row add their halves through shared memory
-            wsync();
-            if (half == 1) t1[row] += part;
-            wsync();
-            dbeta_row = t1[row] + part;
+#pragma unroll
+            for (int x = 0; x < 32; ++x) v[x] *= -beta;
+            split32(v, hi, lo);
+            tile_store_w16(slot(2), row, cg * 32, hi);
         }
-        split_to_tile(cA, slot(2), false, f_dGm);                   // dGm = D dA, hi
         publish(B_R1);
         // (global stores and loads come after a hand-over, never just before it: the hand-over waits for them)
-        if (half == 0 && row_valid) p.dbeta[urow] = dbeta_row;
-        // The dQl / dKr rows of the final sums are fetched while the products run.  At d = 128 a thread's half row is one
-        // 128-byte line: four lanes fetch four lines together, a quarter of each per instruction (whole lines per request
-        // instead of 32 scattered pieces, which held up the products' operand reads as well).
-        constexpr int NI = HD / 64;
-        uint32_t rq[4][8], rk[4][8];
-        uint4 pre_q[4], pre_k[4];
+        // The dQl / dKr rows of the final sums are fetched while the products run.
+        uint32_t rq[2][8], rk[2][8];
         {
-            const __nv_bfloat16* g_dql = p.dql + ((size_t)chunk * kT + row) * HD + half * (HD / 2);
-            const __nv_bfloat16* g_dkr = p.dkr + ((size_t)chunk * kT + row) * HD + half * (HD / 2);
-            if (HD == 128) {
-                gload_f32x32_issue(reinterpret_cast<const float*>(g_dql), rq);
-                gload_f32x32_issue(reinterpret_cast<const float*>(g_dkr), rk);
-            } else {
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    pre_q[x] = reinterpret_cast<const uint4*>(g_dql)[x];
-                    pre_k[x] = reinterpret_cast<const uint4*>(g_dkr)[x];
-                }
-            }
+            const size_t o = ((size_t)chunk * kT + row) * HD + head_c0;
+            if (has(0)) gload_bf16_issue(p.dql + o, rq);
+            if (has(1)) gload_bf16_issue(p.dkr + o, rk);
         }
+        // the four threads of a row add their parts through shared memory
+        if (cg >= 2) parts[(cg - 2) * kT + row] = part;
+        wsync();
+        if (cg < 2) part += parts[cg * kT + row];
+        if (cg == 1) parts[kT + row] = part;
+        wsync();
+        if (cg == 0 && row_valid) p.dbeta[urow] = t1[row] + (part + parts[kT + row]);
         mma_wait(B_MMA2);                                           // phase 5, first group: dXk's slot is free
         if (!ok) break;
-        split_to_tile(cA, slot(5), true, f_dGm);                    // dGm lo (over dXk)
+        tile_store_w16(slot(5), row, cg * 32, lo);                  // dGm lo (over dXk)
         publish(B_R0);
         mma_wait();                                                 // phase 5, second group
         if (!ok) break;
         // dq and dk are complete: they leave while the last two products run
-        {
-            float wq[32], wk[32];   // HD == 128: the fetched half rows, two bf16 per word
-            if (HD == 128) {
-                gload_f32x32_finish(rq, wq);
-                gload_f32x32_finish(rk, wk);
+        auto finish = [&](uint32_t col, const uint32_t (&fetched)[2][8], __nv_bfloat16* out) {
+            uint32_t w[16];
+            gload_bf16_finish(fetched, w);
+            tmem_row32(tl + col + head_c0, v);
+#pragma unroll
+            for (int x = 0; x < 16; ++x) {
+                v[2 * x] += __uint_as_float(w[x] << 16);
+                v[2 * x + 1] += __uint_as_float(w[x] & 0xffff0000u);
             }
-            auto add_row = [&](const float (&words)[32], const uint4 (&pre)[4], int c, float (&acc)[32]) {
-                if (HD == 128) {
-#pragma unroll
-                    for (int x = 0; x < 16; ++x) {
-                        const uint32_t u = __float_as_uint(words[16 * c + x]);
-                        acc[2 * x] += __uint_as_float(u << 16);
-                        acc[2 * x + 1] += __uint_as_float(u & 0xffff0000u);
-                    }
-                } else {
-                    float in[32];
-                    unpack_bf16x32(pre, in);
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) acc[x] += in[x];
-                }
-            };
-#pragma unroll
-            for (int c = 0; c < NI; ++c) {
-                const int c0 = half * (HD / 2) + c * 32;
-                tmem_row32(tl + cB + c0, v);
-                add_row(wq, pre_q, c, v);
-                gstore_bf16x32<true>(p.dq + urow * HD + c0, v, row_valid);
-                tmem_row32(tl + cG + c0, v);
-                add_row(wk, pre_k, c, v);
-                gstore_bf16x32<true>(p.dk + urow * HD + c0, v, row_valid);
-            }
-        }
+            gstore_bf16x32<true>(out + urow * HD + head_c0, v, row_valid);
+        };
+        if (has(0)) finish(cB, rq, p.dq);
+        if (has(1)) finish(cG, rk, p.dk);
         mma_wait(B_MMA2);                                           // the last of dw
         if (!ok) break;
-#pragma unroll
-        for (int c = 0; c < NI; ++c) {
-            const int c0 = half * (HD / 2) + c * 32;
-            tmem_row32(tl + cDW + c0, v);
-            gstore_bf16x32<true>(p.dw + urow * HD + c0, v, row_valid);
+        if (has(0)) {
+            tmem_row32(tl + cDW + head_c0, v);
+            gstore_bf16x32<true>(p.dw + urow * HD + head_c0, v, row_valid);
         }
         publish(B_R1);   // the next chunk's first products overwrite the accumulators read above
     }

@@ -153,6 +153,22 @@ __device__ __forceinline__ void gstore_bf16_w16(__nv_bfloat16* dst, const uint32
     if (odd ? ovalid : valid) st_global_32<CALLER>((uint8_t*)(odd ? other : mine) + 32 * (int)odd, first);
     if (odd ? valid : ovalid) st_global_32<CALLER>((uint8_t*)(odd ? mine : other) + 32 * (int)odd, second);
 }
+// The load, in two halves as above: 32-byte pieces go to the lanes of a pair so that an instruction covers 64 bytes of each row it touches.
+__device__ __forceinline__ void gload_bf16_issue(const __nv_bfloat16* src, uint32_t (&d)[2][8]) {
+    const bool odd = threadIdx.x & 1;
+    const unsigned long long mine = (unsigned long long)src, other = __shfl_xor_sync(0xffffffffu, mine, 1);
+    ld_global_v8((const uint8_t*)(odd ? other : mine) + 32 * (int)odd, d[0]);   // of the even lane's row
+    ld_global_v8((const uint8_t*)(odd ? mine : other) + 32 * (int)odd, d[1]);   // of the odd lane's row
+}
+__device__ __forceinline__ void gload_bf16_finish(const uint32_t (&d)[2][8], uint32_t (&w)[16]) {
+    const bool odd = threadIdx.x & 1;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        const uint32_t recv = __shfl_xor_sync(0xffffffffu, odd ? d[0][x] : d[1][x], 1);   // the other half of this lane's row
+        w[x] = odd ? recv : d[0][x];
+        w[8 + x] = odd ? d[1][x] : recv;
+    }
+}
 __device__ __forceinline__ void pack32(const float (&v)[32], uint32_t (&w)[16]) {
 #pragma unroll
     for (int x = 0; x < 16; ++x) w[x] = pack_bf16(v[2 * x], v[2 * x + 1]);
