@@ -162,6 +162,7 @@ struct LevelParams {
     int nseg, seg_chunks;         // key-side edge / suffix / apply-product kernels: ranges per slice (<= 1: none), chunks per range
     float* gq;                    // apply-product kernel: [S][Lp] gate terms of the rows (+= gtot[slice]), or nullptr
     const float* gtot;            // [S]
+    const float* reach;           // gated problems: chunks between the farthest kept pair of slice s at reach[s * N * 8], or nullptr = all levels
     const int *nkeep, *nvisit;    // version backward: chunk counts of a sweep shortened by block skipping ([S][N]), or nullptr
     uint32_t* status;
 };

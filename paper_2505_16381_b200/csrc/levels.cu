@@ -115,6 +115,13 @@ template <int HD> constexpr uint32_t kOffFused = 6 * kTS<HD>;
 template <int HD> constexpr uint32_t kOffVersion = kTS<HD> + 2 * kMS<HD>;
 template <int HD> constexpr uint32_t kOffSegment = 2 * kTS<HD> + 2 * kMS<HD>;
 template <int HD> constexpr uint32_t kOffBwd = 3 * kMS<HD> + 4 * kTS<HD> + (HD == 64 ? kPanelB : 0);   // (the panel after the last tile)
+// Is a run product of level l multiplied by anything in slice s?  A step of a version chain by a run of 2^l chunks belongs to a pair
+// of chunks that lie more than 2^l apart, so under block skipping the upper levels of a slice are left out: neither built nor
+// differentiated.  (2 x 16 x 8192 x 128 with a gate that reaches four chunks: levels 2 to 5 of 0 to 5: run products 95 -> 60 us for a pass,
+// their gradients 206 -> 180.)
+__device__ __forceinline__ bool level_used(const LevelParams& p, int s, int l) {
+    return !p.reach || p.reach[(size_t)s * p.N * 8] > (float)(1 << l);
+}
 constexpr uint32_t kOffKeys = 5 * kTileB, kOffSuffix = 4 * kTileB;
 constexpr uint32_t smem_bytes(uint32_t bars) { return bars + 64 + 1024; }
 // Loads of d x d matrices: maps with boxes of d rows.
@@ -127,12 +134,14 @@ __device__ __forceinline__ void tma_matrix(uint8_t* dst, const CUtensorMap* m, u
 // grid.x = S * cnt2.  Dy[l+1][b] = Dy[l][2b+1] Dy[l][2b] with hi/lo operands (three products).
 template <int HD>
 __global__ void __launch_bounds__(256, 1) dyadic_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
+    const int cnt2 = p.lv.dy_cnt[p.l + 1], cnt = p.lv.dy_cnt[p.l];
+    const int s = blockIdx.x / cnt2, b = blockIdx.x % cnt2;
+    grid_wait();   // (the reach)
+    if (!level_used(p, s, p.l + 1)) return;
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
     setup<128>(c, smem_raw, kOffDyadic<HD>);
     constexpr uint32_t M = kMS<HD>;
-    const int cnt2 = p.lv.dy_cnt[p.l + 1], cnt = p.lv.dy_cnt[p.l];
-    const int s = blockIdx.x / cnt2, b = blockIdx.x % cnt2;
     const long mat_lo = p.lv.dy_off[p.l] / (HD * HD) + (long)s * cnt + 2 * b;        // right factor; left is +1
     const long mat_out = p.lv.dy_off[p.l + 1] / (HD * HD) + (long)s * cnt2 + b;
     uint8_t* sm = c.smem;
@@ -181,13 +190,16 @@ __global__ void __launch_bounds__(256, 1) dyadic_fwd_kernel(const __grid_constan
 // 128..255) while A_2, A_3 and B_1 are made.  grid.x = S * groups, groups = ceil(cnt(l + 1) / 2^(fuse-1)).
 template <int HD>
 __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) dyadic_fused_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
+    const int half_w = 1 << (p.fuse - 1);                        // A products per group
+    const int groups = (p.lv.dy_cnt[p.l + 1] + half_w - 1) / half_w;
+    const int s = blockIdx.x / groups, g = blockIdx.x % groups;
+    grid_wait();   // (the reach)
+    if (!level_used(p, s, p.l + 1)) return;
+    const bool useB = level_used(p, s, p.l + 2), useC = level_used(p, s, p.l + 3);
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
     setup<256>(c, smem_raw, kOffFused<HD>);
     constexpr uint32_t T = kTS<HD>;
-    const int half_w = 1 << (p.fuse - 1);                        // A products per group
-    const int groups = (p.lv.dy_cnt[p.l + 1] + half_w - 1) / half_w;
-    const int s = blockIdx.x / groups, g = blockIdx.x % groups;
     uint8_t* sm = c.smem;
     auto mat = [&](int lvl, int idx) { return p.lv.dy_off[lvl] / (HD * HD) + (long)s * p.lv.dy_cnt[lvl] + idx; };
     // acc(col) = left (slots a, a + 1) x right (slots b, b + 1), the lo x lo term left out
@@ -229,9 +241,9 @@ __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) dyadic_fused_kernel(con
     const int l = p.l;
     const int a0 = g * half_w;                                   // first A product of this group (index at level l + 1)
     const int cntA = p.lv.dy_cnt[l + 1], cntB = p.lv.dy_cnt[l + 2], cntC = p.fuse >= 3 ? p.lv.dy_cnt[l + 3] : 0;
-    const bool hasA1 = a0 + 1 < cntA, hasB0 = (a0 >> 1) < cntB;
-    const bool more = p.fuse >= 3 && hasB0 && a0 + 2 < cntA;     // is there a second half of the tree?
-    const bool hasA3 = more && a0 + 3 < cntA, hasB1 = more && (a0 >> 1) + 1 < cntB, hasC = hasB1 && (a0 >> 2) < cntC;
+    const bool hasA1 = a0 + 1 < cntA, hasB0 = useB && (a0 >> 1) < cntB;
+    const bool more = p.fuse >= 3 && (a0 >> 1) < cntB && a0 + 2 < cntA;     // is there a second half of the tree?
+    const bool hasA3 = more && a0 + 3 < cntA, hasB1 = useB && more && (a0 >> 1) + 1 < cntB, hasC = useC && hasB1 && (a0 >> 2) < cntC;
     // The operands of A_k (level-l pair 2k+1, 2k) are requested as soon as their slots are free, on a barrier of their
     // own per parity of k: left factor into slots a, a + 1, right factor into b, b + 1.
     uint64_t* lbar[2] = {&c.bars[0], c.bars + 4};
@@ -263,29 +275,29 @@ __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) dyadic_fused_kernel(con
     wait_a(0);
     product(0, 0, 2);                                            // A_0
     if (hasA1) request_a2(1, 2);                                 // slots 2, 3 are free again
-    readout(0, l + 1, a0, true, 0);                              // A_0 -> slots 0, 1
+    readout(0, l + 1, a0, true, hasB0 ? 0 : -1);                 // A_0 -> slots 0, 1
     if (hasA1) {
         wait_a(1);
         product(0, 2, 4);                                        // A_1
-        readout(0, l + 1, a0 + 1, true, 2);                      // -> slots 2, 3
+        readout(0, l + 1, a0 + 1, true, hasB0 ? 2 : -1);         // -> slots 2, 3
     }
-    if (hasB0) {
-        product(more ? 128 : 0, 2, 0);                           // B_0 = A_1 A_0; it waits in columns 128.. if there is more
+    if (hasB0 || more) {
+        if (hasB0) product(more ? 128 : 0, 2, 0);                // B_0 = A_1 A_0; it waits in columns 128.. if there is more
         if (more) {                                              // every slot is free now
             request_a1(2, 2);
             request_a2(2, 0);
         }
         if (hasA3) request_a1(3, 4);
-        readout(more ? 128 : 0, l + 2, a0 >> 1, true, -1);
+        if (hasB0) readout(more ? 128 : 0, l + 2, a0 >> 1, true, -1);
         if (more) {
             wait_a(2);
             product(0, 0, 2);                                    // A_2
             if (hasA3) request_a2(3, 2);
-            readout(0, l + 1, a0 + 2, true, 0);                  // -> slots 0, 1
+            readout(0, l + 1, a0 + 2, true, hasB1 ? 0 : -1);     // -> slots 0, 1
             if (hasA3) {
                 wait_a(3);
                 product(0, 2, 4);                                // A_3
-                readout(0, l + 1, a0 + 3, true, 2);              // -> slots 2, 3
+                readout(0, l + 1, a0 + 3, true, hasB1 ? 2 : -1); // -> slots 2, 3
             }
             if (hasB1) {
                 product(0, 2, 0);                                // B_1 = A_3 A_2
@@ -572,7 +584,8 @@ __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) level_bwd_kernel(const 
             if (valid(ch)) return ch;
         return -1;
     };
-    const bool parent = l1 + 1 <= p.nlev - 2 && (b >> 1) >= 1 && (b >> 1) < p.lv.dy_cnt[l1 + 1];
+    if (l1 > 0 && !level_used(p, s, l1)) return;
+    const bool parent = l1 + 1 <= p.nlev - 2 && (b >> 1) >= 1 && (b >> 1) < p.lv.dy_cnt[l1 + 1] && level_used(p, s, l1 + 1);
     int ch = next_chunk(c0);
     __nv_bfloat16* out = p.ddy16 + (size_t)mat * HD * HD;
     if (ch < 0 && !parent) {   // nothing multiplies by this run product

@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(1024) gate_suffix_kernel(const float* __restri
 // query chunk keeps the key chunks up to the farthest one that fails this test.
 constexpr float kSkipMargin = 30.f;   // exp(-30) ~ 1e-13 per logit, far below bf16 resolution even summed over a long row
 
-// stats[tile] = {max|q|, max|k|, max G, min G, min s_ii over real rows, sum of log factors, 0, 0}
+// stats[tile] = {max|q|, max|k|, max G, min G, min s_ii over real rows, sum of log factors, 0, 0}; tile_ranges_kernel leaves the
+// distance of the slice's farthest kept pair, in chunks, in entry 6 of its first tile
 // A row takes hd/8 lanes (16-byte loads), so a warp works on 2 (hd = 128) or 4 (hd = 64) rows at a time.
 // Bound by its bytes, q, k and w once.  LPR lanes share a row, eight channels each.  The row's four sums are reduced together: at the
 // first two steps a lane gives away half of what it holds, so that it ends up with one of them (role 0: |q|^2, 1: |k|^2, 2: q k,
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(256) tile_stats_kernel(const __nv_bfloat16* __
 // chunks) computes the same pairs as the query-major sweeps, and every version a sweep asks for lies within the levels its
 // chunk reaches.  Also counts the kept pairs.  (Two kernels with one serial thread per query chunk and per slice took
 // 30 us at 32 slices x 64 chunks.)
-__global__ void __launch_bounds__(1024) tile_ranges_kernel(const float* __restrict__ stats, int* __restrict__ nkeep,
+__global__ void __launch_bounds__(1024) tile_ranges_kernel(float* stats, int* __restrict__ nkeep,
                                                            int* __restrict__ nvisit, unsigned long long* counters, int N,
                                                            float ascale) {
     grid_wait();
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(1024) tile_ranges_kernel(const float* __restri
     __syncthreads();
     if (warp == 0) {   // from the last chunk down: start(I) = min over I' >= I of the first kept chunk
         unsigned long long kept = 0;
-        int start = N;
+        int start = N, far = 0;
         for (int top = N; top > 0; top -= 32) {
             const int I = top - 1 - lane;
             int first = I >= 0 ? I - nk[I] + 1 : N;
@@ -271,13 +272,18 @@ __global__ void __launch_bounds__(1024) tile_ranges_kernel(const float* __restri
             first = min(first, start);
             if (I >= 0) {
                 nk[I] = I - first + 1;
+                far = max(far, I - first);
                 kept += (unsigned long long)nk[I];
             }
             start = __shfl_sync(0xffffffffu, first, 31);
         }
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, off);
+        for (int off = 16; off >= 1; off >>= 1) {
+            kept += __shfl_xor_sync(0xffffffffu, kept, off);
+            far = max(far, __shfl_xor_sync(0xffffffffu, far, off));
+        }
         if (lane == 0) {
+            stats[(size_t)sl * N * 8 + 6] = (float)far;
             atomicAdd(&counters[0], kept);
             atomicAdd(&counters[1], (unsigned long long)N * (N + 1) / 2);
         }
@@ -427,7 +433,7 @@ cudaError_t launch_gate_skip(const void* q, const void* k, const void* w, const 
     const cudaError_t e = hd == 64 ? launch<tile_stats_kernel<64>>(S * N, 256, 0, st, (const bf*)q, (const bf*)k, (const bf*)w, beta, G, stats, L, Lp, scale)
                                    : launch<tile_stats_kernel<128>>(S * N, 256, 0, st, (const bf*)q, (const bf*)k, (const bf*)w, beta, G, stats, L, Lp, scale);
     if (e != cudaSuccess) return e;
-    return launch<tile_ranges_kernel>(S, 1024, 0, st, (const float*)stats, nkeep, nvisit, counters, N, fabsf(scale));
+    return launch<tile_ranges_kernel>(S, 1024, 0, st, stats, nkeep, nvisit, counters, N, fabsf(scale));
 }
 
 cudaError_t launch_cache_rows(const void* v, void* vc, const float* G, float* gc, int S, int L, int Lp, int cap, int hd, cudaStream_t st) {

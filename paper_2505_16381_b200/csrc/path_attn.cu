@@ -226,7 +226,7 @@ static LevelParams level_params(const Plan& p, void* ws) {
     if (p.bwd) {
         lp.dqv = at<__nv_bfloat16>(ws, p.dQv); lp.dkv = at<__nv_bfloat16>(ws, p.dKv); lp.ddy16 = at<__nv_bfloat16>(ws, p.dDy);
     }
-    if (p.gate) { lp.nkeep = at<int>(ws, p.nkeep); lp.nvisit = at<int>(ws, p.nvisit); }   // block skipping (see run_gate_skip)
+    if (p.gate) { lp.nkeep = at<int>(ws, p.nkeep); lp.nvisit = at<int>(ws, p.nvisit); lp.reach = at<float>(ws, p.tstats) + 6; }   // block skipping (see run_gate_skip)
     lp.status = at<uint32_t>(ws, p.status);
     return lp;
 }
@@ -282,6 +282,7 @@ static int run_prep(const Plan& p, void* ws, const void* q, const void* k, const
     LevelTensorMaps tm;
     if (!make_level_maps(p, ws, tm)) { g_last_cuda_error = (int)cudaErrorUnknown; return PATH_ERR_LAUNCH; }
     LevelParams lp = level_params(p, ws);
+    if (edge_q) lp.reach = nullptr;               // chains that go on to the sequence's edges need every run product
     prof_mark(stg_lev, 0, st);
     for (int l = 0; l + 1 <= p.nlev - 2;) {       // run products of 2, 4, ... chunks, up to three levels per launch
         const int left = p.nlev - 2 - l;

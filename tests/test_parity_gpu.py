@@ -556,6 +556,17 @@ def test_gate_block_skipping_keeps_parity(binding, oracle, L, d, shift, expect):
         check(name, g[name].reshape(-1, *g[name].shape[2:]), r)
 
 
+@pytest.mark.parametrize("L,d,reach", [(1500, 64, 1), (1500, 128, 2), (1500, 64, 3), (1500, 128, 4), (1500, 64, 5), (1400, 128, 9),
+                                       (2300, 64, 2.4), (2300, 128, 4.4), (4300, 64, 16)])
+def test_gate_reach_at_the_edges_of_levels(binding, oracle, L, d, reach):
+    """Run products of a level are built only for slices with a kept pair more than 2^level chunks apart: a constant gate whose 30 nats
+    are used up after about `reach` chunks in the first head, twice as far in the second (slices differ)."""
+    inp = synth.make_inputs(1, 2, L, d, "bf16", gate=True, seed=4300 + L + d)
+    rate = torch.tensor([32.0 / (128 * reach), 16.0 / (128 * reach)])
+    inp["log_f"] = (-rate[None, :, None]).expand(1, 2, L).contiguous()
+    compare_all(binding, oracle, inp)
+
+
 def test_block_skipping_respects_large_logits_and_growing_transitions(binding, oracle):
     """Keys with a large norm, or transitions with |1 - beta |w|^2| > 1, can outweigh the gate: the bound must see both."""
     L, d = 1024, 64
