@@ -91,6 +91,17 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tma_tile(slot(5), &tm.dkr, &bars[B_LOAD2], HD, ch * kT);
         tma_rows(slot(4), &tm.w, &bars[B_LOAD2], HD, (ch % p.N) * kT, ch / p.N);
     };
+    // Tiles on their way into L2 before their slots are free: a load that has to come from memory holds the chain up for 2 to 3 thousand
+    // cycles.  Only where the copy engine has nothing to load meanwhile: it works requests off in order.  (As prefetch.global of
+    // worker threads or of a warp of their own they held up the next hand-over or the stores to shared memory.)  At d = 128, where
+    // the bytes themselves take as long as the chain, it changes nothing.  8 x 16 x 2048 x 64: 231 -> 216 us.
+    constexpr bool kPrefetch = HD == 64;
+    auto fetch = [&](const CUtensorMap* m, int ncols, int row0) {
+        for (int h = 0; h < ncols / 64; ++h) tma_prefetch_2d(m, h * 64, row0);
+    };
+    auto fetch_rows = [&](const CUtensorMap* m, int ch) {
+        for (int h = 0; h < HD / 64; ++h) tma_prefetch_3d(m, h * 64, (ch % p.N) * kT, ch / p.N);
+    };
     if ((int)blockIdx.x < nchunks) {
         first_loads_a(blockIdx.x);
         first_loads_b(blockIdx.x);
@@ -101,8 +112,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         // ---- phase 0: dXq = lower(-(dQl U^T + s dSd Y^T)) -> cA, while the previous chunk's results are still leaving
         // the other columns; then dw = -Y dKr - U dP^T
         if (!wait(B_LOAD)) break;
-        mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(1), sa(0), false);
-        mma<OP_MN, OP_K, K8, 128>(tmem + cA, sa(3), sa(2), true);
+        mma<OP_K, OP_K, KD, 128, true>(tmem + cA, sa(1), sa(0), false);
+        mma<OP_MN, OP_K, K8, 128, true>(tmem + cA, sa(3), sa(2), true);
         if (chunk != (int)blockIdx.x && !wait(B_R1)) break;                      // the previous chunk's dw has left cDW
         if (!wait(B_LOAD2)) break;
         mma<OP_K, OP_MN, K8, HD, true>(tmem + cDW, sa(2), sa(5), false);
@@ -113,12 +124,12 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         if (!wait(B_MMA)) break;
         mbar_expect_tx(&bars[B_LOAD], kTileB);
         tma_tile(slot(2), &tm.xq, &bars[B_LOAD], kT, r0);
-        mma<OP_K, OP_MN, KD, HD>(tmem + cB, sa(4), sa(6), false);           // W dP needs no new tile
+        mma<OP_K, OP_MN, KD, HD, true>(tmem + cB, sa(4), sa(6), false);     // W dP needs no new tile
         if (!wait(B_LOAD)) break;
-        mma<OP_MN, OP_MN, K8, HD>(tmem + cB, sa(2), sa(1), true);
+        mma<OP_MN, OP_MN, K8, HD, true>(tmem + cB, sa(2), sa(1), true);
         if (!wait(B_R0)) break;                                                  // dXq has left cA
-        mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(4), sa(5), false);
-        mma<OP_MN, OP_K, K8, 128>(tmem + cA, sa(2), sa(3), true);
+        mma<OP_K, OP_K, KD, 128, true>(tmem + cA, sa(4), sa(5), false);
+        mma<OP_MN, OP_K, K8, 128, true>(tmem + cA, sa(2), sa(3), true);
         umma_commit(&bars[B_MMA]);
         // ---- phase 2: dT = lower(dY Xk^T + dU W^T) -> cA, and phase 3 right behind it (the same dY and dU tiles and T~):
         // dXk = strictLower(T~^T dY) -> cB,  dw += T~^T dU.  (s dSd)^T is not needed again before phase 5, where it is
@@ -128,6 +139,22 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         tma_tile(slot(2), &tm.xk, &bars[B_LOAD], kT, r0);
         tma_tile(slot(1), &tm.th, &bars[B_LOAD], kT, r0);
         tma_tile(slot(3), &tm.tl, &bars[B_LOAD], kT, r0);
+        // (from here to phase 5 nothing is loaded: what phase 5 and the next chunk's first phases need)
+        if (kPrefetch) {
+            fetch_rows(&tm.q, chunk);
+            fetch_rows(&tm.k, chunk);
+        }
+        if (kPrefetch && chunk + grid < nchunks) {
+            const int ch = chunk + grid;
+            fetch(&tm.dql, HD, ch * kT);
+            fetch(&tm.u, HD, ch * kT);
+            fetch(&tm.dsdt, kT, ch * kT);
+            fetch(&tm.y, kT, ch * kT);
+            fetch(&tm.dp, HD, ch * HD);
+            fetch(&tm.dkr, HD, ch * kT);
+            fetch_rows(&tm.w, ch);
+            fetch(&tm.xq, kT, ch * kT);
+        }
         if (!wait(B_R1)) break;                                                  // dY, dU tiles
         mma<OP_K, OP_K, KD, 128>(tmem + cA, sa(6), sa(4), false);           // dU W^T needs no new tile
         if (!wait(B_LOAD)) break;
@@ -149,9 +176,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         mma<OP_K, OP_K, KD, 128>(tmem + cB, sa(4), sa(4), false);          // retires with the next group
         if (!wait(B_MMA)) break;
         if (!wait(B_R0)) break;                                                  // M hi, lo tiles
-        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(2), sa(1), false);
-        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(2), sa(3), true);
-        mma<OP_K, OP_K, K8, 128>(tmem + cA, sa(6), sa(1), true);
+        mma<OP_K, OP_K, K8, 128, true>(tmem + cA, sa(2), sa(1), false);
+        mma<OP_K, OP_K, K8, 128, true>(tmem + cA, sa(2), sa(3), true);
+        mma<OP_K, OP_K, K8, 128, true>(tmem + cA, sa(6), sa(1), true);
         umma_commit(&bars[B_MMA]);
         // ---- phase 5: dq -> cB, dk -> cG and the rest of dw, in three groups.  K, (s dSd)^T and Q replace T~ and M
         // lo.  First the products that need neither dGm nor the columns that dbeta still reads; when they have
@@ -184,7 +211,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         mma<OP_MN, OP_MN, K8, HD>(tmem + cDW, sa(5), sa(4), true);
         umma_commit(&bars[B_MMA2]);
         if (!wait(B_MMA2)) break;
-        if (next < nchunks) first_loads_b(next);                                 // and the other two
+        if (next < nchunks) {
+            first_loads_b(next);                                                 // and the other two
+            if (kPrefetch) {
+                fetch(&tm.xk, kT, next * kT);
+                fetch(&tm.th, kT, next * kT);
+                fetch(&tm.tl, kT, next * kT);
+            }
+        }
     }
     }
     __syncwarp();
@@ -238,24 +272,18 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         const int s_idx = chunk / p.N, pos = (chunk % p.N) * kT + row;   // slice and position of this thread's row
         const bool row_valid = pos < p.L;
         const size_t urow = (size_t)s_idx * p.L + pos;                   // row in the caller's [S][L][.] tensors
-        const float beta = beta_floor(row_valid ? p.beta[urow] : 0.f);
-        mma_wait();                                                 // phase 0: -dXq
+        const float beta = beta_floor(row_valid ? p.beta[urow] : 0.f), inv_b = 1.f / beta;
+        mma_wait();                                                 // phase 0
         if (!ok) break;
         read_lower(cA, 1);
-#pragma unroll
-        for (int x = 0; x < 32; ++x) v[x] = -v[x];
         tile_store32(slot(0), row, cg * 32, v);                     // dXq (over U)
         publish(B_R0);
-        mma_wait();                                                 // phase 1: -dY, -dU
+        mma_wait();                                                 // phase 1
         if (!ok) break;
         tmem_row32(tl + cA + cg * 32, v);
-#pragma unroll
-        for (int x = 0; x < 32; ++x) v[x] = -v[x];
         tile_store32(slot(5), row, cg * 32, v);                     // dY (over dKr)
         if (has(0)) {
             tmem_row32(tl + cB + head_c0, v);
-#pragma unroll
-            for (int x = 0; x < 32; ++x) v[x] = -v[x];
             tile_store32(slot(6), row, head_c0, v);                 // dU (over dP)
         }
         publish(B_R1);
@@ -276,14 +304,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         mma_wait();                                                 // D M
         if (!ok) break;
         {   // M, hi (over dT hi) and lo (over dT lo); its diagonal is dbeta's column part
-            const float inv_b = 1.f / beta;
             tmem_row32(tl + cG + cg * 32, v);
 #pragma unroll
             for (int x = 0; x < 32; ++x) v[x] *= inv_b;
             if (above == 0) {
+                float m = 0.f;
 #pragma unroll
-                for (int x = 0; x < 32; ++x)
-                    if (x == lane) t1[row] = v[x];
+                for (int x = 0; x < 32; ++x) m = x == lane ? v[x] : m;
+                t1[row] = m;
             }
             split32(v, hi, lo);
             tile_store_w16(slot(2), row, cg * 32, hi);
@@ -293,17 +321,17 @@ __global__ void __launch_bounds__(kChainThreads, 1) chunk_chain_kernel(const __g
         mma_wait();                                                 // dA and W W^T
         if (!ok) break;
         float part = 0.f;
-        {   // dA = strictLower(-cA);  dbeta_r = t1_r + sum_c dA_rc (W W^T)_rc;  dGm = D dA, hi now, lo once dXk's slot is free
+        {   // dA = strictLower(cA);  dbeta_r = t1_r + sum_c dA_rc (W W^T)_rc;  dGm = D dA, hi now, lo once dXk's slot is free
             read_lower(cA, 0);
             if (above <= 0) {
                 float gm[32];
                 tmem_row32(tl + cB + cg * 32, gm);
 #pragma unroll
                 for (int x = 0; x < 32; ++x)
-                    if (above < 0 || x < lane) part -= v[x] * gm[x];
+                    if (above < 0 || x < lane) part += v[x] * gm[x];
             }
 #pragma unroll
-            for (int x = 0; x < 32; ++x) v[x] *= -beta;
+            for (int x = 0; x < 32; ++x) v[x] *= beta;
             split32(v, hi, lo);
             tile_store_w16(slot(2), row, cg * 32, hi);
         }
