@@ -82,10 +82,11 @@ __device__ __forceinline__ void mma1688(float (&d)[4], const uint32_t (&a)[4], u
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// hi (x cut off), l = lo (the rest, rounded: 11 + 11 bits and a sign; the product cuts off what lies below them).
+// hi (x cut off), l = lo (the rest, rounded: 11 + 11 bits and a sign).  Both are tf32 values as they stand: that a product ignores what
+// lies below a tf32 number's bits is not promised.
 __device__ __forceinline__ uint32_t split_tf32(float x, uint32_t& l) {
     const uint32_t h = __float_as_uint(x) & 0xffffe000u;
-    l = __float_as_uint(x - __uint_as_float(h)) + 0x1000u;
+    l = (__float_as_uint(x - __uint_as_float(h)) + 0x1000u) & 0xffffe000u;
     return h;
 }
 // Element (r, c) of the float32 diagonal block b (64 x 64): rows 0 - 31 where the block's hi tile goes later, rows 32 - 63 at its lo
