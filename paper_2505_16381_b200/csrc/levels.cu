@@ -734,19 +734,20 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
             *reinterpret_cast<__nv_bfloat16*>(sm + oR + sw128_off(r, j >> 3) + (j & 7) * 2) = __float2bfloat16_rn(1.f);
         }
     }
-    uint64_t* lbar[2] = {&c.bars[0], c.bars + 4};
+    // (barrier and phase of a set are computed: as arrays with a changing index they lived in local memory, on the chain)
+    auto lbar = [&](int set) { return c.bars + 4 * set; };
     if (c.tid == 0) {
-        mbar_init(lbar[1], 1);
+        mbar_init(lbar(1), 1);
         mbar_fence_init();
     }
     __syncthreads();
     auto issue = [&](int J, int set) {
         const long mat = p.lv.dy_off[0] / (HD * HD) + (long)s * p.lv.dy_cnt[0] + J;
         uint8_t* t = sm + set * 3 * kTileB;
-        mbar_expect_tx(lbar[set], kTileBytes<HD> + 2 * kMatBytes<HD>);
-        tma_tile(t, &tm.kv, lbar[set], HD, (int)((long)s * p.Lp + (long)J * kT));   // version slot 0
-        tma_matrix<HD>(t + kTileB, &tm.dyh, lbar[set], mat);
-        tma_matrix<HD>(t + 2 * kTileB, &tm.dyl, lbar[set], mat);
+        mbar_expect_tx(lbar(set), kTileBytes<HD> + 2 * kMatBytes<HD>);
+        tma_tile(t, &tm.kv, lbar(set), HD, (int)((long)s * p.Lp + (long)J * kT));   // version slot 0
+        tma_matrix<HD>(t + kTileB, &tm.dyh, lbar(set), mat);
+        tma_matrix<HD>(t + 2 * kTileB, &tm.dyl, lbar(set), mat);
     };
     // Segments (key side, p.nseg > 1): blockIdx.z walks only the chunks [z * seg_chunks, (z+1) * seg_chunks) and leaves its keys
     // advanced to the end of THAT range (bf16, p.edge16) together with the range's product (p.pseg); a second pass
@@ -767,15 +768,13 @@ __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant
         if (p.kc) gstore_f32x32<true>(p.kc + ((size_t)s * p.cap + pos) * HD + col0 + c0, v, pos < p.L);
         if (p.edge16) gstore_bf16x32(p.edge16 + ((size_t)s * p.L + pos) * HD + col0 + c0, v, pos < p.L);
     };
-    uint32_t lph[2] = {0, 0};
 #pragma unroll 1
     for (int n = 0; n < cnt && c.ok; ++n) {
         const int set = n & 1;
         const bool more = n + 1 < cnt;
         // every range but the first also wants its whole product
         const bool update = more || (p.nseg > 1 && blockIdx.z > 0);
-        if (!mbar_wait(lbar[set], lph[set], c.abort_flag, ST_LEVELS)) c.ok = false;
-        lph[set] ^= 1;
+        if (!mbar_wait(lbar(set), (uint32_t)(n >> 1) & 1u, c.abort_flag, ST_LEVELS)) c.ok = false;
         publish();   // R; and the accumulators of this step have been read two steps ago
         if (leader(c)) {
             tc_fence_after_sync();
