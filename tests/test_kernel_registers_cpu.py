@@ -21,12 +21,13 @@ def stack_frames(source, tmp_path):
     return {(name, args): int(n) for name, args, n in found}
 
 
-@pytest.mark.parametrize("source,kernels", [
-    ("levels.cu", ["key_cache_kernel"]),
+@pytest.mark.parametrize("source,kernel,instances", [
+    ("levels.cu", "key_cache_kernel", ["Li64E", "Li128E"]),
+    ("chunk_chain.cu", "chunk_chain_kernel", ["Li64E"]),
 ])
-def test_no_stack_frame(source, kernels, tmp_path):
+def test_no_stack_frame(source, kernel, instances, tmp_path):
     frames = stack_frames(source, tmp_path)
-    for k in kernels:
-        mine = {n: b for n, b in frames.items() if n[0].endswith(k)}
-        assert len(mine) >= 2, (k, sorted(frames))
+    for i in instances:
+        mine = {n: b for n, b in frames.items() if n[0].endswith(kernel) and n[1].startswith(i)}
+        assert mine, (i, sorted(frames))
         assert not any(mine.values()), mine
