@@ -20,12 +20,13 @@
 // stores tiles.  They meet at mbarriers only.  Every result leaves by a TMA store from the tile that the workers have written anyway
 // (or write for that): no worker touches global memory but for beta.
 //
-// What bounds it.  d = 64: the inverse, about 17 k cycles per chunk, of which its merges take 7 k (mma.sync shares the tensor pipe
-// with the products: 2.6 k when nothing else runs).  d = 128: shared memory, which moves about 2 MB per chunk (operand reads of the
+// What bounds it.  d = 64: the inverse, of which its merges take 7 k cycles (mma.sync shares the tensor pipe
+// with the products: 2.6 k when nothing else runs); a chunk takes 19 k.  d = 128: shared memory, which moves about 2 MB per chunk (operand reads of the
 // products 1 MB, tiles in and out 0.4, the workers 0.6) = 16 k of 20 k cycles.  Both streams of code together have to fit the
 // instruction caches as well: warps went without instructions for 2.3 cycles per issue until the operand group was one loop, 0.7
-// since.  Times, before with one group of warps and one chunk at a time / now: B = 2, H = 16, L = 8192, d = 128, forward's instance
-// 220 / 180 us, backward's 238 / 195; 32 x 32768 x 128 928 / 750; 128 x 2048 x 64 185 / 166 and 199 / 180.
+// since.  And the registers of each role have to do: a few spilled ones cost as much as anything here (shared memory leaves no L1),
+// 13 - 18 % of the kernel at d = 64 and 2 % at d = 128.  Times, before with one group of warps and one chunk at a time / now: 2 x 16 x 8192 x 128,
+// forward's instance 220 / 175 us, backward's 238 / 197; 32 x 32768 x 128 928 / 740; 128 x 2048 x 64 185 / 135 and 199 / 150.
 // Tried: 32 x 32 blocks by substitution and a merge in float32 arithmetic (rows broadcast from shared memory: 4.3 k and 5.7 k
 // cycles, the loads' 128 bytes per cycle bound them); T~ from tensor memory at d = 128 too (Gm of the next chunk has to be ready
 // before T~: its W arrives too late, 750 -> 880 us).
@@ -256,6 +257,37 @@ __device__ __forceinline__ void invert_diagonal(uint8_t* aH, uint8_t* aL, const 
     scale32(d, bt + cb);
 }
 
+// Accumulators of one row, W columns from `taddr` on, times `scale` if there is one, as a bf16 pair; the pair into the two tiles.
+template <int W, bool SCALED>
+__device__ __forceinline__ void read_pair(uint32_t taddr, const float* scale, uint32_t (&hi)[W / 2], uint32_t (&lo)[W / 2]) {
+    uint32_t r[W];
+    if constexpr (W == 16) tmem_ld16(taddr, r);
+    else tmem_ld32(taddr, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int x = 0; x < W; x += 4) {
+        float4 v = make_float4(__uint_as_float(r[x]), __uint_as_float(r[x + 1]), __uint_as_float(r[x + 2]), __uint_as_float(r[x + 3]));
+        if (SCALED) {
+            const float4 b = *reinterpret_cast<const float4*>(scale + x);
+            v.x *= b.x; v.y *= b.y; v.z *= b.z; v.w *= b.w;
+        }
+        const uint32_t h0 = pack_bf16(v.x, v.y), h1 = pack_bf16(v.z, v.w);
+        hi[x / 2] = h0;
+        hi[x / 2 + 1] = h1;
+        lo[x / 2] = pack_bf16(v.x - __uint_as_float(h0 << 16), v.y - __uint_as_float(h0 & 0xffff0000u));
+        lo[x / 2 + 1] = pack_bf16(v.z - __uint_as_float(h1 << 16), v.w - __uint_as_float(h1 & 0xffff0000u));
+    }
+}
+template <int N>
+__device__ __forceinline__ void store_pair(uint8_t* aH, uint8_t* aL, int row, int c0, const uint32_t (&hi)[N], const uint32_t (&lo)[N]) {
+#pragma unroll
+    for (int x = 0; x < N; x += 4) {
+        const uint32_t at = (uint32_t)(c0 >> 6) * kPanelB + sw128_off((uint32_t)row, (uint32_t)((c0 & 63) >> 3) + x / 4);
+        *reinterpret_cast<uint4*>(aH + at) = make_uint4(hi[x], hi[x + 1], hi[x + 2], hi[x + 3]);
+        *reinterpret_cast<uint4*>(aL + at) = make_uint4(lo[x], lo[x + 1], lo[x + 2], lo[x + 3]);
+    }
+}
+
 // MODE: PREP_FWD = everything the forward needs; PREP_SAVE = also keeps the tiles of the chain rule (the backward's instance);
 // PREP_KEYS = the key side only (prompt key cache: Kright and the chunk products; no query is involved, so Xq, Xq U,
 // Qleft and the diagonal-correction operands are left out and q is not even loaded).
@@ -313,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
     auto col_u = [](uint32_t it) { return 384u - (it & 1) * 128u; };
 
     if (warp >= 2 * kWorkers / 32) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");   // 128 x 72 + 256 x 128 + 256 x 72 = 60416 of the 640 x 96
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");   // 128 x 80 + 256 x 120 + 256 x 80 = all of the 640 x 96 that the block starts with
         auto wait = [&](int b, uint32_t par) { return mbar_wait<true>(&bars[b], par, abort_flag, ST_PREP); };
         if (warp == 16 && elect_one()) {
             // -------------------------------------------------------------- products
@@ -521,7 +553,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
         __syncwarp();
     } else if (warp < kWorkers / 32) {
         // ------------------------------------------------------------------ inverse
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
         bool ok = true;
         // lane 0 of every warp waits; the vote that follows is also the barrier that releases the other lanes
         auto wwait = [&](int b, uint32_t par) {
@@ -599,64 +631,66 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
             fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&bars[R_ID]);
-            if (TMT && next < nchunks) {   // Gm of the next chunk leaves its columns to T~
-                if (!(ok = wwait(M_GM, par ^ 1))) break;
-                tc_fence_after_sync();
-                read_gm();
-            }
             // X = C A^-1 over C, then the block of T~ there: -B^-1 X D; a thread has 32 entries of a row in all of this.  T~ goes into
             // tensor memory (per 32 columns 16 of hi, 16 of lo) and / or over the tiles.
             const uint32_t cu = col_u(it) + half * 32;
             const int cd = (row & 64) + half * 32, co = half * 32 + 64 - (row & 64);   // its columns in the diagonal block and the other one
-            uint32_t hi[16], lo[16];
+            // Columns at a time.  At d = 64 the 64 entries of the next Gm or the 32 of d are live as well; 32 more spilled (183 / 152 us for
+            // the 2048 chunks of 8 x 16 x 2048 x 64).
+            constexpr int W = D64 ? 16 : 32;
             if (!(ok = wwait(M_IX, par))) break;
             tc_fence_after_sync();
             if (row >= 64) {
-                float v[32];
-                tmem_row32(tl + cu, v);
-                split32(v, hi, lo);
-                tile_store_w16(aH, row, half * 32, hi);
-                tile_store_w16(aL, row, half * 32, lo);
+#pragma unroll 1
+                for (int c = 0; c < 32; c += W) {
+                    uint32_t h[W / 2], l[W / 2];
+                    read_pair<W, false>(tl + cu + c, nullptr, h, l);
+                    store_pair(aH, aL, row, half * 32 + c, h, l);
+                }
             }
             fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&bars[R_IX]);
+            if (TMT && next < nchunks) {   // Gm of the next chunk leaves its columns to T~
+                if (!(ok = wwait(M_GM, par ^ 1))) break;
+                tc_fence_after_sync();
+                read_gm();
+            } else {   // (the entries end here in either case: 64 registers that are not carried through the inverse)
+#pragma unroll
+                for (int x = 0; x < 32; ++x) g[0][x] = g[1][x] = 0u;
+            }
+            uint32_t hi[16], lo[16];
             split32(d, hi, lo);
+            if (!(ok = wwait(M_IT, par))) break;
+            tc_fence_after_sync();
             if (TMT) {   // (everybody has read Gm: there was a vote since)
                 tmem_st16(tl + cG + cd, hi);
                 tmem_st16(tl + cG + cd + 16, lo);
             }
-            if (!(ok = wwait(M_IT, par))) break;
-            tc_fence_after_sync();
-            if (!TMT || SAVE) {
-                tile_store_w16(aH, row, cd, hi);
-                tile_store_w16(aL, row, cd, lo);
-            }
-            if (row >= 64) {
-                float v[32];
-                tmem_row32(tl + cu + 64, v);
-                scale32(v, bt + half * 32);
-                split32(v, hi, lo);
-                if (!TMT || SAVE) {
-                    tile_store_w16(aH, row, co, hi);
-                    tile_store_w16(aL, row, co, lo);
-                }
-            } else {
+            if (!TMT || SAVE) store_pair(aH, aL, row, cd, hi, lo);
+#pragma unroll 1
+            for (int c = 0; c < 32; c += W) {
+                uint32_t h[W / 2], l[W / 2];
+                if (row >= 64) {
+                    read_pair<W, true>(tl + cu + 64 + c, bt + half * 32 + c, h, l);
+                    if (!TMT || SAVE) store_pair(aH, aL, row, co + c, h, l);
+                } else {
 #pragma unroll
-                for (int x = 0; x < 16; ++x) hi[x] = lo[x] = 0u;
+                    for (int x = 0; x < W / 2; ++x) h[x] = l[x] = 0u;
+                }
+                if constexpr (TMT) {
+                    tmem_st8(tl + cG + co + c / 2, h);
+                    tmem_st8(tl + cG + co + 16 + c / 2, l);
+                }
             }
-            if (TMT) {
-                tmem_st16(tl + cG + co, hi);
-                tmem_st16(tl + cG + co + 16, lo);
-                tmem_st_wait();
-            }
+            if (TMT) tmem_st_wait();
             if (!TMT || SAVE) fence_proxy_async_smem();
             tc_fence_before_sync();
             mbar_arrive(&bars[R_TT]);
         }
     } else {
         // ------------------------------------------------------------------ operands and results
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         bool ok = true;
         uint32_t r[32];
         float v[32];

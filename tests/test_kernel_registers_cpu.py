@@ -21,13 +21,14 @@ def stack_frames(source, tmp_path):
     return {(name, args): int(n) for name, args, n in found}
 
 
-@pytest.mark.parametrize("source,kernel,instances", [
-    ("levels.cu", "key_cache_kernel", ["Li64E", "Li128E"]),
-    ("chunk_chain.cu", "chunk_chain_kernel", ["Li64E"]),
+@pytest.mark.parametrize("source,kernel,limits", [
+    ("levels.cu", "key_cache_kernel", {"Li64E": 0, "Li128E": 0}),
+    ("chunk_chain.cu", "chunk_chain_kernel", {"Li64E": 0}),
+    ("chunk_prep.cu", "chunk_prep_kernel", {"Li64E": 8, "Li128E": 0}),   # (8: one pointer that all roles of the block share)
 ])
-def test_no_stack_frame(source, kernel, instances, tmp_path):
+def test_stack_frames(source, kernel, limits, tmp_path):
     frames = stack_frames(source, tmp_path)
-    for i in instances:
-        mine = {n: b for n, b in frames.items() if n[0].endswith(kernel) and n[1].startswith(i)}
-        assert mine, (i, sorted(frames))
-        assert not any(mine.values()), mine
+    for instance, limit in limits.items():
+        mine = {n: b for n, b in frames.items() if n[0].endswith(kernel) and n[1].startswith(instance)}
+        assert mine, (instance, sorted(frames))
+        assert max(mine.values()) <= limit, mine
