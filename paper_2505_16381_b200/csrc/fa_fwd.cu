@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
     constexpr bool SEP = HD == 64;
     constexpr int kOff = CROSS ? 0 : 1;                        // stream 0's step index is n - kOff
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    // (Without the gate the integer form, whose accesses are generic: 1 - 4 % faster there by the compiler's schedule, 307 / 311 us at
+    // (Without the gate the integer form, whose accesses are generic: 1 % faster there by the compiler's schedule, 307 / 311 us at
     // 4 x 16 x 4096 x 128, while the gated instance takes 169 / 151 us at 2 x 16 x 8192 x 128.)
     uint8_t* smem = GATE ? align1024(smem_raw) : (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     if ((uint32_t)(smem - smem_raw) + FwdSmem::total > FwdSmem::alloc) {   // uniform over the CTA

@@ -99,7 +99,7 @@ static bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t c
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// bf16 matrix [rows][cols], box = [box_rows][64 cols], 128-byte swizzle (the low-rank layer's operands).
+// The same with a box of box_rows rows (d x d matrices: chunk, run and range products and their gradients; the low-rank layer's operands).
 static bool make_map_box(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;

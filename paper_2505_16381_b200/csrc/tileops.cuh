@@ -1,7 +1,7 @@
 // Building blocks of the per-chunk kernels: every matrix of the chunk-level algebra is a 128-row
 // bf16 tile in shared memory (row-major, 64-column panels, 128-byte swizzle), every product a tcgen05 MMA into
-// tensor memory issued by one thread, every result read back one row per thread (256 worker threads: two per row,
-// each taking half of the columns).
+// tensor memory issued by one thread, every result read back one row per thread (with 256 worker threads two share a row, each
+// taking half of the columns; with the 512 of the chain rule four).
 #pragma once
 #include "common.cuh"
 #include "tc5.cuh"
@@ -103,9 +103,9 @@ __device__ __forceinline__ void gstore_f32x32(float* dst, const float (&v)[32], 
         if (ok) st_global_32<CALLER>((uint8_t*)ptr + 32 * j, d);
     }
 }
-// The load in two halves, so that a caller can put other work between the request and the first use of the data.
-__device__ __forceinline__ void gload_f32x32_issue(const float* src, uint32_t (&d)[4][8], bool valid = true) {
+__device__ __forceinline__ void gload_f32x32(const float* src, float (&v)[32], bool valid = true) {
     const int j = threadIdx.x & 3;
+    uint32_t d[4][8], w[32];
     const unsigned long long mine = (unsigned long long)src;
     unsigned long long ptr[4];
     bool ok[4];
@@ -120,10 +120,6 @@ __device__ __forceinline__ void gload_f32x32_issue(const float* src, uint32_t (&
         for (int x = 0; x < 8; ++x) d[r][x] = 0u;
         if (ok[r]) ld_global_v8((const uint8_t*)ptr[r] + 32 * j, d[r]);
     }
-}
-__device__ __forceinline__ void gload_f32x32_finish(const uint32_t (&d)[4][8], float (&v)[32]) {
-    const int j = threadIdx.x & 3;
-    uint32_t w[32];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -131,11 +127,6 @@ __device__ __forceinline__ void gload_f32x32_finish(const uint32_t (&d)[4][8], f
     rot4_pieces(w, j);
 #pragma unroll
     for (int x = 0; x < 32; ++x) v[x] = __uint_as_float(w[x]);
-}
-__device__ __forceinline__ void gload_f32x32(const float* src, float (&v)[32], bool valid = true) {
-    uint32_t d[4][8];
-    gload_f32x32_issue(src, d, valid);
-    gload_f32x32_finish(d, v);
 }
 // 32 bf16 = 64 bytes per row: pairs of lanes.  `w`: the row segment as 16 packed words.
 template <bool CALLER = false>
@@ -153,7 +144,7 @@ __device__ __forceinline__ void gstore_bf16_w16(__nv_bfloat16* dst, const uint32
     if (odd ? ovalid : valid) st_global_32<CALLER>((uint8_t*)(odd ? other : mine) + 32 * (int)odd, first);
     if (odd ? valid : ovalid) st_global_32<CALLER>((uint8_t*)(odd ? mine : other) + 32 * (int)odd, second);
 }
-// The load, in two halves as above: 32-byte pieces go to the lanes of a pair so that an instruction covers 64 bytes of each row it touches.
+// The load, in two halves, so that a caller can put other work between the request and the first use of the data: 32-byte pieces go to the lanes of a pair so that an instruction covers 64 bytes of each row it touches.
 __device__ __forceinline__ void gload_bf16_issue(const __nv_bfloat16* src, uint32_t (&d)[2][8]) {
     const bool odd = threadIdx.x & 1;
     const unsigned long long mine = (unsigned long long)src, other = __shfl_xor_sync(0xffffffffu, mine, 1);
@@ -196,14 +187,6 @@ __device__ __forceinline__ void tile_store_w16(uint8_t* t, int row, int c0, cons
     for (int ch = 0; ch < 4; ++ch)
         *reinterpret_cast<uint4*>(panel + sw128_off((uint32_t)row, (uint32_t)(ch0 + ch))) =
             make_uint4(w[4 * ch], w[4 * ch + 1], w[4 * ch + 2], w[4 * ch + 3]);
-}
-__device__ __forceinline__ void tile_load_w16(const uint8_t* t, int row, int c0, uint32_t (&w)[16]) {
-    const uint8_t* panel = t + (c0 >> 6) * kPanelB;
-#pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-        const uint4 u = *reinterpret_cast<const uint4*>(panel + sw128_off((uint32_t)row, (uint32_t)(((c0 & 63) >> 3) + ch)));
-        w[4 * ch] = u.x; w[4 * ch + 1] = u.y; w[4 * ch + 2] = u.z; w[4 * ch + 3] = u.w;
-    }
 }
 __device__ __forceinline__ void unpack_bf16x32(const uint4 (&u4)[4], float (&v)[32]) {
 #pragma unroll
