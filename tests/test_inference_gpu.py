@@ -60,6 +60,29 @@ def test_prefill_cache_matches_oracle(binding, oracle, B, H, L, d, gate):
         assert np.abs(cache["gc"][:, :, :L].cpu().double().numpy() - G).max() <= 1e-4 * max(1.0, np.abs(G).max())
 
 
+ROUNDS = [0, 48, 49, 50, 98, 99, 147, 148, 149]   # 150 slices of 3 chunks: four rounds on 148 SMs, the last of six CTAs
+
+
+@pytest.mark.parametrize("S,L,d,gate,picked", [
+    (150, 300, 64, False, ROUNDS), (150, 300, 128, False, ROUNDS), (150, 300, 64, True, ROUNDS), (150, 300, 128, True, ROUNDS),
+    (14, 4200, 64, True, [0, 6, 13]), (14, 4200, 128, False, [0, 6, 13]),     # 33 chunks each, the walk in ranges
+])
+def test_prefill_cache_with_several_chunks_per_cta(binding, oracle, S, L, picked, d, gate):
+    """The chunk preparation hands tiles, accumulator columns and barrier phases from one chunk of a CTA to the next; its keys-only
+    instance does so without the query side's waits.  At least three chunks per CTA, slices from every round."""
+    inp = synth.make_inputs(1, S, L, d, "bf16", gate=gate, seed=90 + L + d)
+    dev = {n: (t.cuda() if torch.is_tensor(t) else t) for n, t in inp.items()}
+    cache = binding.alloc_cache(1, S, L, d, gate)
+    cache["kc"].fill_(float("nan"))
+    ws = binding.path_attn_prefill_cache(dev["k"], dev["v"], dev["w"], dev["beta"], cache, dev["log_f"])
+    assert binding.device_status(ws) == 0
+    ref = oracle.key_cache(*(f64(inp[n])[0, picked] for n in ("k", "w", "beta")))
+    got = cache["kc"][0, picked].cpu().double().numpy()
+    for g, r in zip(got, ref):
+        assert rel_fro(g, r) <= 1e-2 and np.abs(g - r).max() <= 2e-2 * max(1.0, np.abs(r).max())
+    assert torch.isfinite(cache["kc"]).all() and torch.equal(cache["vc"], dev["v"])
+
+
 @pytest.mark.parametrize("B,H,L0,T,d,gate,scale", [
     (1, 2, 0, 40, 64, False, 1.0),        # decoding from an empty cache
     (2, 2, 300, 33, 128, True, 1.0),      # crosses a 256-position block of the split

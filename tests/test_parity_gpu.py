@@ -556,14 +556,54 @@ def test_gate_block_skipping_keeps_parity(binding, oracle, L, d, shift, expect):
         check(name, g[name].reshape(-1, *g[name].shape[2:]), r)
 
 
-@pytest.mark.parametrize("L,d,reach", [(1500, 64, 1), (1500, 128, 2), (1500, 64, 3), (1500, 128, 4), (1500, 64, 5), (1400, 128, 9),
-                                       (2300, 64, 2.4), (2300, 128, 4.4), (4300, 64, 16)])
-def test_gate_reach_at_the_edges_of_levels(binding, oracle, L, d, reach):
-    """Run products of a level are built only for slices with a kept pair more than 2^level chunks apart: a constant gate whose 30 nats
-    are used up after about `reach` chunks in the first head, twice as far in the second (slices differ)."""
+def kept_ranges(inp, scale=1.0, margin=30.0):
+    """The block-skipping bound in float64: (chunk pairs kept, distance of the farthest kept pair of every slice, in chunks)."""
+    x = slices(inp, range(inp["q"].shape[0] * inp["q"].shape[1]))
+    S, L, _ = x["q"].shape
+    cut = [slice(a, min(a + 128, L)) for a in range(0, L, 128)]
+    kept, reach = 0, []
+    for s in range(S):
+        q, k, w, beta = (x[n][s] for n in ("q", "k", "w", "beta"))
+        G = np.cumsum(x["log_f"][s])
+        norm = lambda t: [np.sqrt((t[c] ** 2).sum(-1).max()) * 1.001 for c in cut]
+        qn, kn = norm(q), norm(k)
+        own = [(scale * (q[c] * k[c]).sum(-1)).min() for c in cut]
+        growth = np.log(np.maximum(1.0, np.abs(1.0 - beta * (w ** 2).sum(-1))))
+        growth = [growth[c].sum() * 1.001 + 1e-6 for c in cut]
+        first = []
+        for I in range(len(cut)):
+            grown, far = 0.0, I
+            for J in range(I, -1, -1):
+                grown += growth[J]
+                bound = abs(scale) * qn[I] * kn[J] * np.exp(grown) + G[cut[I]].max() - G[cut[J]].min()
+                if bound >= own[I] - 1e-3 * abs(own[I]) - margin:
+                    far = J
+            first.append(far)
+        first = np.minimum.accumulate(first[::-1])[::-1]     # ranges widened into a staircase
+        dist = np.arange(len(cut)) - first
+        kept += int((dist + 1).sum())
+        reach.append(int(dist.max()))
+    return kept, reach
+
+
+# `chunks`: after how many chunks a constant gate has used up about 30 nats in the first head (twice as many in the second);
+# `reach`: the farthest kept pair that this makes.  A level l is built for slices with a reach above 2^l: edges of levels 0 to 4, and with
+# 5 - 8 and 33 - 64 chunks a top level (1 and 4) that a launch of its own would build and no slice needs.
+@pytest.mark.parametrize("L,d,chunks,reach", [
+    (1500, 64, 1, [2, 2]), (1500, 128, 2, [2, 4]), (1500, 64, 3, [4, 6]), (1500, 128, 4, [4, 8]), (1500, 64, 5, [5, 10]),
+    (1400, 128, 9, [9, 10]), (2300, 64, 2.4, [3, 5]), (2300, 128, 4.4, [5, 9]), (4300, 64, 16, [17, 32]),
+    (700, 64, 0.8, [1, 2]), (1000, 128, 0.6, [1, 2]), (4300, 64, 7.7, [8, 16]), (4300, 128, 8, [8, 16]), (4300, 64, 8, [9, 17])])
+def test_gate_reach_at_the_edges_of_levels(binding, oracle, L, d, chunks, reach):
+    """Run products of a level are built only for slices with a kept pair more than 2^level chunks apart."""
     inp = synth.make_inputs(1, 2, L, d, "bf16", gate=True, seed=4300 + L + d)
-    rate = torch.tensor([32.0 / (128 * reach), 16.0 / (128 * reach)])
+    rate = torch.tensor([32.0 / (128 * chunks), 16.0 / (128 * chunks)])
     inp["log_f"] = (-rate[None, :, None]).expand(1, 2, L).contiguous()
+    kept, far = kept_ranges(inp)
+    assert far == reach
+    dev = to_dev(inp)
+    ws = binding.alloc_workspace(dev["q"], True, False)
+    binding.path_attn_fwd(dev["q"], dev["k"], dev["v"], dev["w"], dev["beta"], dev["log_f"], workspace=ws)
+    assert binding.skipped_chunk_pairs(ws)[0] == kept
     compare_all(binding, oracle, inp)
 
 
