@@ -118,10 +118,10 @@ template <int HD> constexpr uint32_t kOffBwd = 3 * kMS<HD> + 4 * kTS<HD> + (HD =
 // Is a run product of level l multiplied by anything in slice s?  A step of a version chain by a run of 2^l chunks belongs to a pair
 // of chunks that lie more than 2^l apart, so under block skipping the upper levels of a slice are left out: neither built nor
 // differentiated.  (2 x 16 x 8192 x 128 with a gate that reaches four chunks: levels 2 to 5 of 0 to 5: run products 95 -> 60 us for a pass,
-// their gradients 206 -> 180.)
-__device__ __forceinline__ bool level_used(const LevelParams& p, int s, int l) {
-    return !p.reach || p.reach[(size_t)s * p.N * 8] > (float)(1 << l);
-}
+// their gradients 206 -> 180.)  The distance is one load behind the wait for the kernels before, so it is requested early and asked late: level
+// 1, on whose products a small problem waits, is built in any case.
+__device__ __forceinline__ float slice_reach(const LevelParams& p, int s) { return p.reach ? p.reach[(size_t)s * p.N * 8] : INFINITY; }
+__device__ __forceinline__ bool level_used(float reach, int l) { return reach > (float)(1 << l); }
 constexpr uint32_t kOffKeys = 7 * kTileB, kOffSuffix = 4 * kTileB;
 constexpr uint32_t smem_bytes(uint32_t bars) { return bars + 64 + 1024; }
 // Loads of d x d matrices: maps with boxes of d rows.
@@ -136,11 +136,10 @@ template <int HD>
 __global__ void __launch_bounds__(256, 1) dyadic_fwd_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     const int cnt2 = p.lv.dy_cnt[p.l + 1], cnt = p.lv.dy_cnt[p.l];
     const int s = blockIdx.x / cnt2, b = blockIdx.x % cnt2;
-    grid_wait();   // (the reach)
-    if (!level_used(p, s, p.l + 1)) return;
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
     setup<128>(c, smem_raw, kOffDyadic<HD>);
+    if (p.l > 0 && !level_used(slice_reach(p, s), p.l + 1)) { teardown<128>(c, p.status); return; }
     constexpr uint32_t M = kMS<HD>;
     const long mat_lo = p.lv.dy_off[p.l] / (HD * HD) + (long)s * cnt + 2 * b;        // right factor; left is +1
     const long mat_out = p.lv.dy_off[p.l + 1] / (HD * HD) + (long)s * cnt2 + b;
@@ -193,12 +192,12 @@ __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) dyadic_fused_kernel(con
     const int half_w = 1 << (p.fuse - 1);                        // A products per group
     const int groups = (p.lv.dy_cnt[p.l + 1] + half_w - 1) / half_w;
     const int s = blockIdx.x / groups, g = blockIdx.x % groups;
-    grid_wait();   // (the reach)
-    if (!level_used(p, s, p.l + 1)) return;
-    const bool useB = level_used(p, s, p.l + 2), useC = level_used(p, s, p.l + 3);
     extern __shared__ uint8_t smem_raw[];
     Ctx c;
     setup<256>(c, smem_raw, kOffFused<HD>);
+    const float reach = slice_reach(p, s);
+    if (p.l > 0 && !level_used(reach, p.l + 1)) { teardown<256>(c, p.status); return; }
+    const bool useB = level_used(reach, p.l + 2), useC = level_used(reach, p.l + 3);
     constexpr uint32_t T = kTS<HD>;
     uint8_t* sm = c.smem;
     auto mat = [&](int lvl, int idx) { return p.lv.dy_off[lvl] / (HD * HD) + (long)s * p.lv.dy_cnt[lvl] + idx; };
@@ -561,6 +560,7 @@ __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) level_bwd_kernel(const 
     const int l1 = p.l, cnt = p.lv.dy_cnt[l1];
     grid_wait();   // (the block-skipping counts, and the zeros below)
     const int s = blockIdx.x / cnt, b = blockIdx.x % cnt;
+    const float reach = slice_reach(p, s);
     const long mat = p.lv.dy_off[l1] / (HD * HD) + (long)s * cnt + b;
     const int is_key = b & 1;
     // the chunks of this run's version steps and their common target level
@@ -584,12 +584,12 @@ __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) level_bwd_kernel(const 
             if (valid(ch)) return ch;
         return -1;
     };
-    if (l1 > 0 && !level_used(p, s, l1)) return;
-    const bool parent = l1 + 1 <= p.nlev - 2 && (b >> 1) >= 1 && (b >> 1) < p.lv.dy_cnt[l1 + 1] && level_used(p, s, l1 + 1);
+    if (l1 > 1 && !level_used(reach, l1)) return;
     int ch = next_chunk(c0);
+    const bool parent = l1 + 1 <= p.nlev - 2 && (b >> 1) >= 1 && (b >> 1) < p.lv.dy_cnt[l1 + 1] && level_used(reach, l1 + 1);
     __nv_bfloat16* out = p.ddy16 + (size_t)mat * HD * HD;
     if (ch < 0 && !parent) {   // nothing multiplies by this run product
-        if (b >= 1 || l1 == 0)
+        if (l1 == 0 || (b >= 1 && level_used(reach, l1)))
             for (int i = threadIdx.x; i < HD * HD / 8; i += 256) reinterpret_cast<uint4*>(out)[i] = make_uint4(0u, 0u, 0u, 0u);
         return;
     }
