@@ -108,7 +108,7 @@ def chunk_kernel_flops(d):
     of the bf16 pairs included), read off their product lists."""
     kd = d // 16
     prep = (3 * mma_flops(128, kd) + 2 * mma_flops(d, 8) + 3 * mma_flops(128, 8) + 3 * mma_flops(d, 8) +
-            2 * mma_flops(d, 8) + 2 * mma_flops(d, 8))
+            2 * mma_flops(d, 8) + 2 * mma_flops(d, 8) + 6 * mma_flops(64, 4))                                    # (last: the inverse's)
     chain = (mma_flops(128, kd) + mma_flops(128, 8) + mma_flops(d, 8) + mma_flops(d, kd) +                       # phase 0
              mma_flops(128, kd) + mma_flops(128, 8) + mma_flops(d, 8) + mma_flops(d, kd) + mma_flops(128, kd) +  # phase 1
              mma_flops(128, 8) + mma_flops(128, kd) +                                                            # phase 2
@@ -118,9 +118,25 @@ def chunk_kernel_flops(d):
     return prep, chain
 
 
+def _version_runs(N):
+    """Run products that some version-chain step multiplies by, as (level, index): chunks of one run share them."""
+    used = set()
+    for l2 in range(1, (N - 1).bit_length() if N > 1 else 0):
+        for c in range(N):
+            low, lowz = c & ((1 << l2) - 1), ~c & ((1 << l2) - 1)
+            if (c >> l2) & 1 and low:
+                l1 = low.bit_length() - 1
+                used.add((l1, ((c >> l2) << l2) >> l1))
+            if not (c >> l2) & 1 and lowz and (((c >> l2) + 1) << l2) <= N - 1:
+                l1 = lowz.bit_length() - 1
+                used.add((l1, (c >> l1) + 1))
+    return used
+
+
 def level_bytes(S, N, d):
-    """Algorithmic bytes of the level kernels (run products and version chains), forward and backward: every tile a
-    launch has to read or write once, counted from the step lists (t = 128 x d bf16 tile, m = d x d bf16 matrix)."""
+    """Algorithmic bytes of the level kernels (run products and version chains), forward and backward: every tile and matrix a
+    launch has to read or write, once (t = 128 x d bf16 tile, m = d x d bf16 matrix).  Up to 2^l chunks multiply by the same run
+    product; all but the first of these reads can come from L2."""
     t, m = CHUNK * d * 2, d * d * 2
     nq, nk, nlev = _version_steps(N)
     chains_q = sum(1 for c in range(N) if bin(c).count("1") >= 2)
@@ -135,11 +151,13 @@ def level_bytes(S, N, d):
         fuse = min(3, nlev - 2 - l)
         dy += 2 * runs(l + 1) * 2 * m + sum(runs(l + j) for j in range(1, fuse + 1)) * 2 * m
         l += fuse
-    fwd = S * (dy + (nq + nk) * (2 * m + t) + (chains_q + chains_k) * t)
+    fwd = S * (dy + len(_version_runs(N)) * 2 * m + (nq + nk) * t + (chains_q + chains_k) * t)
+    # backward, per version step: its gradient and its version in, the carry's target in and out; per run product: itself in, its
+    # gradient out, and the gradient of the level above in once for both its factors
     top = max(nlev - 2, 0)
     run_cnt = sum(runs(l) for l in range(0, top + 1))
-    parents = sum(runs(l) for l in range(0, top))
-    bwd = S * ((nq + nk) * 4 * t + run_cnt * 2 * m + parents * 2 * m)
+    above = sum(runs(l) for l in range(1, top + 1))
+    bwd = S * ((nq + nk) * 4 * t + run_cnt * 2 * m + above * m)
     return fwd, bwd
 
 
@@ -439,8 +457,8 @@ def run_ours(args, cfg):
     tf = lambda fl, t_ms: fl / (t_ms * 1e-3) / 1e12
     value = world * tf(f1 + b1, ms)
     # Work models of the stages.  Attention sweeps: executed FLOPs (tensor-bound).  Per-chunk kernels: BOTH their
-    # algorithmic bytes and their executed tensor-core FLOPs (they turn out to be bound by the latter).  Level
-    # kernels: algorithmic bytes.
+    # algorithmic bytes and their executed tensor-core FLOPs.  Level
+    # kernels: algorithmic bytes, each once.
     S, N = B * H, -(-L // CHUNK)
     nch = S * N
     diag = nch * 2 * CHUNK ** 3

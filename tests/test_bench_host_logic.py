@@ -26,6 +26,17 @@ def test_flop_models():
     assert (nq, nk) == (bq, bk)
 
 
+def test_level_bytes_count_every_run_product_once():
+    """32 x 256 chunks, d = 128: up to 2^l chunks multiply by one run product; charged to each of them the forward had 6.4 GB, more
+    than the copy rate moves in the time that the kernels take."""
+    import bench
+    runs = bench._version_runs(256)
+    nq, nk, _ = bench._version_steps(256)
+    assert all(b < 256 >> l for l, b in runs) and len(runs) < (nq + nk) / 3
+    fwd, bwd = bench.level_bytes(32, 256, 128)
+    assert 4.25e9 < fwd < 4.35e9 and fwd < bwd
+
+
 WORKER = r"""
 import os, sys
 sys.path.insert(0, {root!r})
