@@ -47,13 +47,13 @@ UNIT = "TFLOP/s"
 # DRAM bytes per launch PER (batch, head) SLICE at the C3 shape (L=4096, d=128), from the ncu captures at batch 1
 # (16 slices) summarised under profiles/; slices are independent, so a launch over S slices moves S times this.
 NCU_TRAFFIC_BYTES_PER_SLICE = {
-    "chunk_prep": 9.83e6,            # backward instance (the step's forward runs on the shared workspace)
-    "levels_fwd": 2.10e6 + 6.10e6,   # dyadic_fused (one launch for three levels) + version_fwd
-    "fa_fwd": 10.88e6,
-    "fa_bwd_dkv": 14.97e6,
+    "chunk_prep": 10.12e6,           # backward instance (the step's forward runs on the shared workspace)
+    "levels_fwd": 2.10e6 + 6.09e6,   # dyadic_fused (one launch for three levels) + version_fwd
+    "fa_fwd": 10.89e6,
+    "fa_bwd_dkv": 14.77e6,
     "fa_bwd_dq": 8.31e6,
-    "bwd_levels": 12.45e6,           # level_bwd (4 launches)
-    "bwd_chunk_chain": 15.58e6,
+    "bwd_levels": 12.49e6,           # level_bwd (4 launches)
+    "bwd_chunk_chain": 15.53e6,
 }
 
 # DRAM bytes per launch of frontend_bwd_kernel PER BATCH ROW at H=32, L=4096, d=64 with the gate, from the ncu capture at

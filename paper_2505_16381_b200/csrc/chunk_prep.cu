@@ -26,7 +26,7 @@
 // instruction caches as well: warps went without instructions for 2.3 cycles per issue until the operand group was one loop, 0.7
 // since.  And the registers of each role have to do: a few spilled ones cost as much as anything here (shared memory leaves no L1),
 // 13 - 18 % of the kernel at d = 64 and 2 % at d = 128.  Times, before with one group of warps and one chunk at a time / now: 2 x 16 x 8192 x 128,
-// forward's instance 220 / 175 us, backward's 238 / 197; 32 x 32768 x 128 928 / 740; 128 x 2048 x 64 185 / 135 and 199 / 150.
+// forward's instance 226 / 175 us, backward's 245 / 197; 32 x 32768 x 128 880 / 630; 128 x 2048 x 64 192 / 135 and 206 / 151.
 // Tried: 32 x 32 blocks by substitution and a merge in float32 arithmetic (rows broadcast from shared memory: 4.3 k and 5.7 k
 // cycles, the loads' 128 bytes per cycle bound them); T~ from tensor memory at d = 128 too (Gm of the next chunk has to be ready
 // before T~: its W arrives too late, 750 -> 880 us).

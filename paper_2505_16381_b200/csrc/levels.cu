@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(256, HD == 64 ? 2 : 1) level_bwd_kernel(const 
 //
 // The chain from step to step is P_J^T R -> its pair in shared memory -> the next product, and nothing else lies on it: the tiles of a
 // step are requested a whole step ahead (two sets of slots), and a step's keys are read out and stored while the next step's
-// products run (two sets of accumulators).  With one set of each a step took 4.6 k cycles: the walks of a prompt of 32 x 32768 x 128 take 338 instead of 427 us.
+// products run (two sets of accumulators).  With one set of each a step took 4.6 k cycles: the walks of a prompt of 32 x 32768 x 128 take 261 instead of 384 us (launch lists).
 template <int HD>
 __global__ void __launch_bounds__(256, 1) key_cache_kernel(const __grid_constant__ LevelTensorMaps tm, const LevelParams p) {
     extern __shared__ uint8_t smem_raw[];
