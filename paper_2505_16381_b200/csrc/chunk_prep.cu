@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(kThreads, 1) chunk_prep_kernel(const __grid_co
 
     tc_fence_before_sync();
     __syncthreads();
-    if (tid == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    report_abort(abort_flag, p.status);
     if (warp == 0) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 512);

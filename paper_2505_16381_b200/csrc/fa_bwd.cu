@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(384, 1) dkv_kernel(const __grid_constant__ Bwd
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (threadIdx.x == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    report_abort(abort_flag, p.status);
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 512);
@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(512, 1) dq_kernel(const __grid_constant__ BwdT
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (threadIdx.x == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    report_abort(abort_flag, p.status);
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 512);
@@ -1375,7 +1375,7 @@ __global__ void __launch_bounds__(512, 1) dkv64_kernel(const __grid_constant__ B
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (threadIdx.x == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    report_abort(abort_flag, p.status);
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 512);

@@ -538,7 +538,7 @@ fa_split_kernel(const __grid_constant__ FwdTensorMaps tm, const FwdParams p) {
 
     tc_fence_before_sync();
     __syncthreads();
-    if (threadIdx.x == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    report_abort(abort_flag, p.status);
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 512);
@@ -980,7 +980,7 @@ __global__ void __launch_bounds__(384, 1) fa_fwd_kernel(const __grid_constant__ 
 
     tc_fence_before_sync();
     __syncthreads();
-    if (threadIdx.x == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    report_abort(abort_flag, p.status);
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 512);

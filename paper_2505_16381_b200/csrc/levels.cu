@@ -56,7 +56,7 @@ template <int NCOLS>
 __device__ __forceinline__ void teardown(Ctx& c, uint32_t* status) {
     tc_fence_before_sync();
     __syncthreads();
-    if (c.tid == 0 && *c.abort_flag != 0) atomicCAS(status, 0u, *c.abort_flag);
+    report_abort(c.abort_flag, status);
     if (c.warp == 0) {
         tc_fence_after_sync();
         tmem_dealloc(c.tmem, NCOLS);

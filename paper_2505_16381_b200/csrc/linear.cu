@@ -384,7 +384,7 @@ __global__ void selftest_wait_kernel(uint32_t* status, long long ticks) {
     if (threadIdx.x == 0) {
         bool ok = tc5::mbar_try_wait(&bar, 0);
         if (!ok) ok = tc5::mbar_wait_slow(&bar, 0, abort_flag, ST_SELFTEST, ticks);
-        if (!ok && *abort_flag != 0) atomicCAS(status, 0u, *abort_flag);
+        if (!ok) tc5::report_abort(abort_flag, status);
     }
 }
 

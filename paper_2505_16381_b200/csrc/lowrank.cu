@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(192, 2) gemm_kernel(const __grid_constant__ CU
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (tid == 0 && *abort_flag != 0) atomicCAS(p.status, 0u, *abort_flag);
+    report_abort(abort_flag, p.status);
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 128);
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(192, R == 64 ? 2 : 1) wide_kernel(const __grid
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (tid == 0 && *abort_flag != 0) atomicCAS(status, 0u, *abort_flag);
+    report_abort(abort_flag, status);
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, 256);

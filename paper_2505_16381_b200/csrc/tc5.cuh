@@ -101,6 +101,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return mbar_wait_slow<PARKED>(bar, parity, abort_flag, code);
 }
 
+// The end of a CTA, after its last barrier.  If it gave up, copies and products that it issued may still be on their way into its shared and
+// tensor memory, which the next CTA is about to get: nothing is issued any more, so a pause of a tenth of a millisecond (they take
+// microseconds; what has been held up for a second is not worth more) outlasts them.
+__device__ __forceinline__ void report_abort(volatile uint32_t* abort_flag, uint32_t* status) {
+    const uint32_t code = *abort_flag;
+    if (code == 0) return;
+    if (threadIdx.x == 0) atomicCAS(status, 0u, code);
+    const long long t0 = clock64();
+    while (clock64() - t0 < kWaitTicks / 10000) {}
+}
+
 // Barrier ID over N threads (whole warps) + AND of `ok`.  Warps that meet at a named barrier leave a loop only on a vote like
 // this: if each went by its own waits, one whose wait ran out would be gone, and another, whose wait on the same barrier was
 // answered an instant later, would wait for it at the next named barrier for ever (that wait has no limit).  The instruction
